@@ -174,20 +174,58 @@ __global__ void bin_kernel(const SweepParams<T> *__restrict__ probs, int chains,
     if (threadIdx.x == 0 && complete) p.bcount[q] = nb;
 }
 
-// Sums over chains, in chain order, of the binning sums of one problem:
-// out[0][k][n] = sum of bin means, out[1][k][n] = sum of their squares.
-__global__ void bin_reduce_kernel(const double *__restrict__ acc1, const double *__restrict__ acc2, int chains,
-                                  int N, double *out)
+// Sums over chains of the columns of a chains x columns matrix.  A CTA takes
+// kColTile neighbouring columns (one or two 32-byte sectors of a row, so that
+// reads stay whole) and cuts the chains into kColRows groups, thread t = column
+// t mod 8, chains t/8, t/8 + 32, ...: the loads of a thread are independent and
+// the serial part is chains/32 additions.  What bounds these kernels is the FP64
+// pipe (one warp instruction per ~64 cycles and sub-partition); one thread per
+// column, serial over the chains, was bound by memory latency and left the GPU
+// idle: 7.08 ms for the score products of 4096 chains x 200 points x 8
+// parameters and 3.65 ms for the means of a result call.  The groups are added
+// in a fixed order, so a result does not depend on the schedule.
+constexpr int kColTile = 8;
+constexpr int kColThreads = 256;
+constexpr int kColRows = kColThreads / kColTile;
+
+// The CTA's sum of v over the row groups, per column, in every thread.
+__device__ __forceinline__ double column_total(double v, double (*part)[kColTile])
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;   // k * N + n
-    if (i >= kBinLevels * N) return;
+    v += __shfl_xor_sync(0xffffffffu, v, 8);
+    v += __shfl_xor_sync(0xffffffffu, v, 16);
+    __syncthreads();   // the previous use of part has been read
+    if ((threadIdx.x & 31) < kColTile) part[threadIdx.x >> 5][threadIdx.x & 7] = v;
+    __syncthreads();
+    double t = part[0][threadIdx.x & 7];
+    for (int k = 1; k < kColThreads / 32; ++k) t += part[k][threadIdx.x & 7];
+    return t;
+}
+
+// Sums over chains of the binning sums of one problem: out[0][k][n] = sum of the
+// bin means, out[1][k][n] = sum of their squares.  Levels without a bin yet are
+// zero and not read.
+__global__ void __launch_bounds__(kColThreads) bin_reduce_kernel(const double *__restrict__ acc1,
+                                                                 const double *__restrict__ acc2, const int *bcount,
+                                                                 int chains, int N, double *out)
+{
+    __shared__ double part[kColThreads / 32][kColTile];
+    const int cols = kBinLevels * N;
+    const int i = blockIdx.x * kColTile + (threadIdx.x & (kColTile - 1));   // k * N + n
+    const bool any = i < cols && (bcount[0] >> (i / N)) > 0;                // every chain has the same bins
     double a = 0.0, b = 0.0;
-    for (int q = 0; q < chains; ++q) {
-        a += acc1[(size_t)q * kBinLevels * N + i];
-        b += acc2[(size_t)q * kBinLevels * N + i];
+    if (any) {
+#pragma unroll 4
+        for (int q = threadIdx.x / kColTile; q < chains; q += kColRows) {
+            a += acc1[(size_t)q * cols + i];
+            b += acc2[(size_t)q * cols + i];
+        }
     }
-    out[i] = a;
-    out[(size_t)kBinLevels * N + i] = b;
+    a = column_total(a, part);
+    b = column_total(b, part);
+    if (i < cols && threadIdx.x < kColTile) {
+        out[i] = a;
+        out[(size_t)cols + i] = b;
+    }
 }
 
 // FP32 state: the sums of the open 64-sweep block added to the FP64 sums now
@@ -206,53 +244,106 @@ __global__ void fold_open_block_kernel(float *P1, float *P2, int ldP, double *S1
 }
 
 // Per grid point: mean over chains and kept sweeps, the spread of the chain
-// means (two passes) and the second moment.  P1, P2 (FP32 chain state; else
-// null): the kept-sweep sums of a 64-sweep block still open, added here.
-__global__ void reduce_kernel(const double *S1, const double *S2, const float *P1, const float *P2, int ldP,
-                              int chains, int N, double kept, double *mean, double *semsq, double *m2)
+// means (two passes; s1/kept - mu is formed as (s1 - kept mu)/kept, so that no
+// division is left per chain) and the second moment.  P1, P2 (FP32 chain state;
+// else null): the kept-sweep sums of a 64-sweep block still open, added here.
+__global__ void __launch_bounds__(kColThreads)
+reduce_kernel(const double *__restrict__ S1, const double *__restrict__ S2, const float *__restrict__ P1,
+              const float *__restrict__ P2, int ldP, int chains, int N, double kept, double *mean, double *semsq,
+              double *m2)
 {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    auto s1 = [&](int q) { return S1[(size_t)q * N + n] + (P1 ? (double)P1[(size_t)q * ldP + n] : 0.0); };
+    __shared__ double part[kColThreads / 32][kColTile];
+    const int n = blockIdx.x * kColTile + (threadIdx.x & (kColTile - 1));
+    const int q0 = threadIdx.x / kColTile;
+    const bool in = n < N;
     double a = 0.0, b = 0.0;
-    for (int q = 0; q < chains; ++q) {
-        a += s1(q);
-        b += S2[(size_t)q * N + n] + (P2 ? (double)P2[(size_t)q * ldP + n] : 0.0);
+    if (in) {
+#pragma unroll 4
+        for (int q = q0; q < chains; q += kColRows) {
+            a += S1[(size_t)q * N + n];
+            b += S2[(size_t)q * N + n];
+        }
+        if (P1) {
+#pragma unroll 4
+            for (int q = q0; q < chains; q += kColRows) {
+                a += (double)P1[(size_t)q * ldP + n];
+                b += (double)P2[(size_t)q * ldP + n];
+            }
+        }
     }
-    const double mu = a / (chains * kept);
+    a = column_total(a, part);
+    b = column_total(b, part);
+    const double mu = a / (chains * kept), centre = kept * mu;
     double v = 0.0;
-    for (int q = 0; q < chains; ++q) {
-        const double d = s1(q) / kept - mu;
-        v += d * d;
+    if (in) {
+#pragma unroll 4
+        for (int q = q0; q < chains; q += kColRows) {
+            const double d = (S1[(size_t)q * N + n] + (P1 ? (double)P1[(size_t)q * ldP + n] : 0.0)) - centre;
+            v += d * d;
+        }
     }
-    mean[n] = mu;
-    semsq[n] = chains > 1 ? v / ((double)(chains - 1) * chains) : NAN;
-    m2[n] = b / (chains * kept);
+    v = column_total(v, part);
+    if (in && threadIdx.x < kColTile) {
+        mean[n] = mu;
+        semsq[n] = chains > 1 ? v / (kept * kept) / ((double)(chains - 1) * chains) : NAN;
+        m2[n] = b / (chains * kept);
+    }
 }
 
 // ---------------------------------------------------------------------------
 // snapshot moments for the backward pass
 // ---------------------------------------------------------------------------
-// Sf[n] += sum over chains of f[q][n]
-template <class T>
-__global__ void colsum_kernel(const T *F, int ldF, int chains, int N, double *Sf)
-{
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    double a = 0.0;
-    for (int q = 0; q < chains; ++q) a += (double)F[(size_t)q * ldF + n];
-    Sf[n] += a;
-}
-
 // shift[n] = mean over chains of f[q][n] (the centre of all later snapshots)
 template <class T>
-__global__ void shift_kernel(const T *F, int ldF, int chains, int N, double *shift)
+__global__ void __launch_bounds__(kColThreads) shift_kernel(const T *__restrict__ F, int ldF, int chains, int N,
+                                                            double *shift)
 {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
+    __shared__ double part[kColThreads / 32][kColTile];
+    const int n = blockIdx.x * kColTile + (threadIdx.x & (kColTile - 1));
     double a = 0.0;
-    for (int q = 0; q < chains; ++q) a += (double)F[(size_t)q * ldF + n];
-    shift[n] = a / chains;
+    if (n < N) {
+#pragma unroll 4
+        for (int q = threadIdx.x / kColTile; q < chains; q += kColRows) a += (double)F[(size_t)q * ldF + n];
+    }
+    a = column_total(a, part);
+    if (n < N && threadIdx.x < kColTile) shift[n] = a / chains;
+}
+
+// Sums over chains of a centred snapshot D and of its products with the scores s:
+// CTAs with blockIdx.x = p < P add sum_q d[q][n] s[q][p] to Sfs[n][p] (and, the
+// first of them, sum_q s[q][p] to Ss[p]); those with blockIdx.x = P add the plain
+// sums to Sf[n].  One launch for all of them: 4096 chains x 200 points x 8
+// parameters took 7.08 + 0.47 ms with a thread per grid point.
+template <class T>
+__global__ void __launch_bounds__(kColThreads)
+moment_sums_kernel(const T *__restrict__ D, int ldD, const double *__restrict__ Sq, int chains, int N, int P,
+                   double *Sf, double *Sfs, double *Ss)
+{
+    __shared__ double part[kColThreads / 32][kColTile];
+    const int n = blockIdx.y * kColTile + (threadIdx.x & (kColTile - 1));
+    const int q0 = threadIdx.x / kColTile, p = blockIdx.x;
+    double a = 0.0;
+    if (p == P) {
+        if (n < N) {
+#pragma unroll 4
+            for (int q = q0; q < chains; q += kColRows) a += (double)D[(size_t)q * ldD + n];
+        }
+        a = column_total(a, part);
+        if (n < N && threadIdx.x < kColTile) Sf[n] += a;
+        return;
+    }
+    if (n < N) {
+#pragma unroll 4
+        for (int q = q0; q < chains; q += kColRows) a += (double)D[(size_t)q * ldD + n] * Sq[(size_t)q * P + p];
+    }
+    a = column_total(a, part);
+    if (n < N && threadIdx.x < kColTile) Sfs[(size_t)n * P + p] += a;
+    if (blockIdx.y == 0) {   // (uniform per CTA) the scores alone, the same in every column
+        double b = 0.0;
+        for (int q = q0; q < chains; q += kColRows) b += Sq[(size_t)q * P + p];
+        b = column_total(b, part);
+        if (threadIdx.x == 0) Ss[p] += b;
+    }
 }
 
 // D = F - shift (rows of chains, padding kept at zero)
@@ -276,25 +367,6 @@ __global__ void kshift_kernel(const double *Kth, const double *shift, int M, int
     kshift[i] = a;
 }
 
-// Sfs[n*P + p] += sum_q f[q][n] s[q][p]; Ss[p] += sum_q s[q][p] (thread n < P also does Ss).
-template <class T>
-__global__ void fs_kernel(const T *F, int ldF, const double *Sq, int chains, int N, int P, double *Sfs,
-                          double *Ss)
-{
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    for (int pi = 0; pi < P; ++pi) {
-        double a = 0.0, b = 0.0;
-        for (int q = 0; q < chains; ++q) {
-            const double s = Sq[(size_t)q * P + pi];
-            a += (double)F[(size_t)q * ldF + n] * s;
-            b += s;
-        }
-        Sfs[(size_t)n * P + pi] += a;
-        if (n == 0) Ss[pi] += b;
-    }
-}
-
 // Backward: u = Cov(fbar) v' from the snapshot moments (v' = v / w).
 // (the moments are of d = fbar - shift: the covariance is unchanged)
 __global__ void vjp_cov_kernel(const double *Sff, const double *Sf, double ns, const double *vp, int N, double *u)
@@ -309,20 +381,24 @@ __global__ void vjp_cov_kernel(const double *Sff, const double *Sf, double ns, c
     u[n] = a / ns - (Sf[n] / ns) * (mv / ns);
 }
 
-// Backward: g_theta[p] = Cov(v'^T fbar, s_p) - sum_n v_n <fbar_n> dw_pn / w_n^2.
+// Backward: g_theta[p] = Cov(v'^T fbar, s_p) - sum_n v_n <fbar_n> dw_pn / w_n^2, one warp per parameter.
 __global__ void vjp_theta_kernel(const double *Sfs, const double *Ss, const double *Sf, const double *shift,
                                  double ns, const double *vp, const double *v, const double *w, const double *dw,
                                  int N, int P, double *g)
 {
-    const int pi = blockIdx.x * blockDim.x + threadIdx.x;
-    if (pi >= P) return;
+    const int pi = blockIdx.x, lane = threadIdx.x;
     double c = 0.0, m = 0.0, t = 0.0;
-    for (int n = 0; n < N; ++n) {
+    for (int n = lane; n < N; n += 32) {
         c += vp[n] * Sfs[(size_t)n * P + pi];
         m += vp[n] * Sf[n];
         t += v[n] * (Sf[n] / ns + shift[n]) * dw[(size_t)pi * N + n] / (w[n] * w[n]);
     }
-    g[pi] = c / ns - (m / ns) * (Ss[pi] / ns) - t;
+    for (int off = 16; off; off >>= 1) {
+        c += __shfl_xor_sync(0xffffffffu, c, off);
+        m += __shfl_xor_sync(0xffffffffu, m, off);
+        t += __shfl_xor_sync(0xffffffffu, t, off);
+    }
+    if (lane == 0) g[pi] = c / ns - (m / ns) * (Ss[pi] / ns) - t;
 }
 
 // ---------------------------------------------------------------------------
@@ -330,6 +406,7 @@ __global__ void vjp_theta_kernel(const double *Sfs, const double *Ss, const doub
 // ---------------------------------------------------------------------------
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 int round_up_int(int x, int a) { return (x + a - 1) / a * a; }
+unsigned col_ctas(size_t cols) { return (unsigned)((cols + kColTile - 1) / kColTile); }   // CTAs of the column sums
 
 struct WsLayout {
     size_t counters, F, R, S1, S2, chi2;
@@ -1050,7 +1127,7 @@ int moment_update(asm_problem *p, const WsLayout &L, int chains)
     const T *Fraw = (const T *)(ws + L.F);
     double *shift = (double *)(ws + L.shift);
     if (p->nsnap == 0) {   // centre every snapshot on the first one's mean (keeps FP32 GEMMs accurate)
-        shift_kernel<T><<<(N + 127) / 128, 128, 0, p->stream>>>(Fraw, L.ldF, chains, N, shift);
+        shift_kernel<T><<<col_ctas(N), kColThreads, 0, p->stream>>>(Fraw, L.ldF, chains, N, shift);
         ++p->other_launches;
         if (p->P > 0) {
             kshift_kernel<<<(M * p->P + 127) / 128, 128, 0, p->stream>>>(p->d_Kth64, shift, M, N, p->P,
@@ -1067,8 +1144,7 @@ int moment_update(asm_problem *p, const WsLayout &L, int chains)
     const T *F = (const T *)(ws + L.D);
     // Sff += D^T D (FP32 partial sums over slices of chains in the mixed path, added in FP64)
     if (launch_gram(F, L.ldF, chains, N, (double *)(ws + L.Sff), p->stream) != cudaSuccess) return ASM_ERR_CUDA;
-    colsum_kernel<T><<<(N + 127) / 128, 128, 0, p->stream>>>(F, L.ldF, chains, N, (double *)(ws + L.Sf));
-    p->other_launches += 2;
+    ++p->other_launches;
     if (p->P > 0) {
         // Y = D K~_theta^T for every parameter at once, then the scores
         T *Y = (T *)(ws + L.Y);
@@ -1080,11 +1156,10 @@ int moment_update(asm_problem *p, const WsLayout &L, int chains)
             return ASM_ERR_CUDA;
         p->other_launches += 2;
     }
-    if (p->P > 0) {
-        fs_kernel<T><<<(N + 127) / 128, 128, 0, p->stream>>>(F, L.ldF, (const double *)(ws + L.Sq), chains, N, p->P,
-                                                             (double *)(ws + L.Sfs), (double *)(ws + L.Ss));
-        ++p->other_launches;
-    }
+    moment_sums_kernel<T><<<dim3((unsigned)p->P + 1, col_ctas(N)), kColThreads, 0, p->stream>>>(
+        F, L.ldF, (const double *)(ws + L.Sq), chains, N, p->P, (double *)(ws + L.Sf), (double *)(ws + L.Sfs),
+        (double *)(ws + L.Ss));
+    ++p->other_launches;
     if (cudaGetLastError() != cudaSuccess) return ASM_ERR_CUDA;
     p->nsnap += chains;
     return ASM_OK;
@@ -1902,7 +1977,7 @@ int asm_average(asm_problem *p, double *mean_A, double *sem_A, double *ess, doub
     char *ws = (char *)p->ws;
     ++p->other_launches;
     const bool open32 = p->precision != ASM_FP64;   // FP32 state: sums of the open 64-sweep block
-    reduce_kernel<<<(N + 127) / 128, 128, 0, p->stream>>>(
+    reduce_kernel<<<col_ctas(N), kColThreads, 0, p->stream>>>(
         (const double *)(ws + L.S1), (const double *)(ws + L.S2), open32 ? (const float *)(ws + L.P1) : nullptr,
         open32 ? (const float *)(ws + L.P2) : nullptr, L.ldF, p->chains, N, (double)p->kept, d, d + N, d + 2 * N);
     std::vector<double> h((size_t)3 * N);
@@ -1942,11 +2017,12 @@ int asm_mc_error(asm_problem *p, int k, double *ess, double *sem_fbar, double *s
     if (cudaMalloc(&d, sizeof(double) * (3 * (size_t)N + 2 * nk)) != cudaSuccess) return ASM_ERR_CUDA;
     const char *ws = (const char *)u->ws;
     const bool open32 = u->precision != ASM_FP64;
-    reduce_kernel<<<(N + 127) / 128, 128, 0, p->stream>>>(
+    reduce_kernel<<<col_ctas(N), kColThreads, 0, p->stream>>>(
         (const double *)(ws + L.S1), (const double *)(ws + L.S2), open32 ? (const float *)(ws + L.P1) : nullptr,
         open32 ? (const float *)(ws + L.P2) : nullptr, L.ldF, chains, N, (double)u->kept, d, d + N, d + 2 * N);
-    bin_reduce_kernel<<<(unsigned)((nk + 127) / 128), 128, 0, p->stream>>>(
-        (const double *)(ws + L.bacc1), (const double *)(ws + L.bacc2), chains, N, d + 3 * N);
+    bin_reduce_kernel<<<col_ctas(nk), kColThreads, 0, p->stream>>>(
+        (const double *)(ws + L.bacc1), (const double *)(ws + L.bacc2), (const int *)(ws + L.bcount), chains, N,
+        d + 3 * N);
     p->other_launches += 2;
     std::vector<double> h(3 * (size_t)N + 2 * nk);
     int nb = 0;
@@ -2016,7 +2092,7 @@ int asm_backward(asm_problem *p, const double *v, double *grad_G, double *grad_t
             return ASM_ERR_CUDA;
     }
     if (grad_theta) {
-        vjp_theta_kernel<<<(p->P + 31) / 32, 32, 0, p->stream>>>(
+        vjp_theta_kernel<<<p->P, 32, 0, p->stream>>>(
             (const double *)(ws + L.Sfs), (const double *)(ws + L.Ss), (const double *)(ws + L.Sf),
             (const double *)(ws + L.shift), ns, d_vp, d_v, p->d_w, p->d_dw, N, p->P, d_g);
         if (cudaGetLastError() != cudaSuccess ||
@@ -2132,7 +2208,7 @@ int asm_sample_noalloc(asm_problem *p, int chains, long burn_in, long sweeps, ui
     const WsLayout L = ws_layout(p, chains, precision);
     const char *ws = (const char *)p->ws;
     const bool open32 = precision != ASM_FP64;
-    reduce_kernel<<<(p->N + 127) / 128, 128, 0, p->stream>>>(
+    reduce_kernel<<<col_ctas(p->N), kColThreads, 0, p->stream>>>(
         (const double *)(ws + L.S1), (const double *)(ws + L.S2), open32 ? (const float *)(ws + L.P1) : nullptr,
         open32 ? (const float *)(ws + L.P2) : nullptr, L.ldF, chains, p->N, (double)sweeps, d_mean_fbar, d_sem2_fbar,
         d_m2_fbar);
