@@ -68,16 +68,18 @@ enum { ASM_FP64 = 0, ASM_MIXED = 1 };   /* precision of asm_sample */
 /* Environment variables the library reads (testing and tuning only; no result
  * depends on them, every chain does the same arithmetic under every launch
  * shape; values outside the ranges below are ignored):
- *   ASM_TEAM_LANES         8, 16 or 32: lanes per chain of a handle, read by
- *                          asm_setup (asm_tune replaces it);
+ *   ASM_TEAM_LANES         8, 16 or 32: lanes per chain of a handle, i.e. 4, 2 or
+ *                          1 chains per warp (with a gamma prior always 1), read
+ *                          by asm_setup (asm_tune replaces it);
  *   ASM_CONSUMERS_PER_CTA  1..7: chain warps per CTA of every sweep launch
  *                          (takes precedence over the heuristic and asm_tune);
  *   ASM_RING_DEPTH         2..48: stages of the move-record ring (default: as
  *                          many as shared memory holds, at most 48);
- *   ASM_RECORDS_PER_STAGE  1..8: consecutive move records per ring stage
- *                          (default 4: one barrier wait and release per stage);
+ *   ASM_RECORDS_PER_STAGE  1..8: move records of the largest block per ring stage
+ *                          (default 4: one barrier wait and release per stage;
+ *                          smaller blocks put more records in a stage);
  *   ASM_NO_U_STAGE         set: the block projections read U from global memory
- *                          instead of a shared-memory stage. */
+ *                          instead of the visit packet in shared memory. */
 
 typedef struct asm_problem asm_problem;  /* opaque, library-owned */
 
@@ -144,7 +146,7 @@ typedef struct {
     int64_t timeouts;           /* bounded device waits that gave up (0 in a valid run) */
     int64_t graph_replays;      /* refresh periods run as replays of the handle's CUDA graph */
     int64_t tc_refreshes;       /* residual refreshes run on the tensor cores (3xTF32) */
-    int32_t team_lanes;         /* lanes per chain of the last sweep launch */
+    int32_t team_lanes;         /* lanes per chain of the last sweep launch: 32 / (chains per warp) */
     int32_t consumers_per_cta;  /* chain warps per CTA of the last sweep launch */
     int32_t ctas;               /* CTAs of the last sweep launch (persistent) */
     int32_t work_items;         /* (problem, chain group) items of the last sweep launch */
@@ -193,7 +195,8 @@ int asm_partition_hierarchy(int N, int *n_levels, int *level_nblocks, int *block
 int asm_problem_count(const asm_problem *p);
 
 /* Autotuner of the sweep launch (no counterpart in the paper).  Times every
- * candidate shape -- lanes per chain S in {32, 16, 8} times chain warps per
+ * candidate shape -- lanes per chain S in {32, 16, 8} (a warp runs 32/S chains
+ * that share every row it loads) times chain warps per
  * CTA in {heuristic, 2, 3, 4, 5, 6, 7} times the register budget (kernels
  * compiled for one CTA per SM, up to 255 registers per thread, or for two,
  * 128), where it fits -- on one warm-up and three

@@ -8,9 +8,12 @@
 
 namespace asmgb {
 
-// Rows of every block's mode data are padded to a multiple of this many
-// elements so that any team size S <= 32 with 16-byte vectors stays in the row.
+// Rows of a block's mode data are padded so that 32 lanes of whole vectors stay in
+// the row: 64 elements for blocks of up to 64 points, else a multiple of 128.
+constexpr int kRowAlignSmall = 64;
 constexpr int kRowAlign = 128;
+// Elements reserved for the block descriptor at the head of a visit packet.
+constexpr int kPacketHeader = 32;
 // Residual refresh period of the sweep loop (sweeps).
 constexpr int kRefreshPeriod = 64;
 
@@ -20,26 +23,23 @@ struct BlockDesc {
     int start;       // first grid point of the block
     int n;           // block width n_b
     int np;          // modes with a U column: min(M, n_b)
-    int rs;          // row stride of V/R rows (multiple of kRowAlign)
-    long long offV;  // V: n rows
-    long long offR;  // R = -1/V (NaN where V is left out): n + 1 rows, the last all-NaN
-    long long offd;  // d, invd: n values
-    long long offU;  // Ut: np x M (mode-major); Um: M x np (grid-major)
+    int nz;          // moves from this one on have no U column and d = 0 (flat)
+    int rs;          // row stride of V/R rows
+    int recstride;   // elements per move record (2 rs + 4)
+    int usr;         // row stride of U in the packet (odd: conflict-free column reads)
+    int last;        // 1: the last block of its level
+    long long offU;    // Ut: np x M (mode-major); Um: M x np (grid-major)
     long long offRec;  // move records of the block: n records of recstride elements
-    int recstride;     // elements per record (2 rs + 16)
-    int usr;           // row stride of the staging copy of U (odd: conflict-free column reads)
-    long long offUs;   // staging copy of U: np rows of usr elements, 16-byte aligned
+    long long offPk;   // visit packet: header, R row of mode 0 (rs), U (np rows of usr); 16-byte aligned
 };
+static_assert(sizeof(BlockDesc) <= kPacketHeader * sizeof(float), "the packet's header holds the descriptor");
 
-// Device-side problem data in one precision T.
+// Device-side problem data in one precision T (R = -1/V, NaN where V is left out of the bounds).
 template <class T>
 struct ProblemData {
-    const T *V, *R;          // mode rows V and R = -1/V (NaN where V is left out of the bounds)
-    const T *d, *invd;       // singular values and their reciprocals (0 for zero modes)
-    const T *meta;           // per mode, 16 bytes: {d, 1/d} (FP32: {d, 1/d, 0, 0})
-    const T *rec;            // per move j: {V_j, R_{j+1} (rs each), d_j, 1/d_j, |K~_b V_j|}
-    const T *Ut, *Um;        // U in two layouts
-    const T *Us;             // U mode-major with odd row stride, copied to shared memory per block visit
+    const T *rec;            // per move j: {V_j, R_{j+1} (rs each), d_j, 1/d_j, |K~_b V_j|, 0}
+    const T *pk;             // visit packets
+    const T *Ut, *Um;        // U in two layouts, for blocks whose U does not fit a packet slot
 };
 
 struct Counters {            // device counters, first bytes of the workspace
@@ -100,31 +100,29 @@ struct SweepParams {
 
 // What every problem of one launch shares: the CTA shape and the
 // shared-memory plan (the union of the problems' needs).  The move records
-// of a CTA's item flow through a ring of `depth` stages filled by one
-// producer warp with bulk copies (TMA engine); `full` barriers signal a
-// landed record, `empty` barriers collect the consumer warps' releases.
+// of a CTA's item flow through a ring of `depth` stages and its visit packets
+// through `pslots` slots, filled by one producer warp with bulk copies (TMA
+// engine); `full` barriers signal landed bytes, `empty` barriers collect the
+// consumer warps' releases.
 struct LaunchShape {
-    int S;                            // lanes per chain (power of two, <= 32)
+    int C;                            // chains per warp
     int consumers;                    // consumer warps per CTA (the producer is one more)
     int depth;                        // stages in the ring
-    int off_full, off_empty, off_stages;  // byte offsets in dynamic shared memory
     int stage_bytes;                  // bytes per stage (>= rps of the largest records)
-    int rps;                          // move records per stage (consecutive moves of one block)
+    int rps;                          // the largest block's move records per stage
+    int pslots, pbytes;               // visit packets: slots and bytes of one
+    int off_bars, off_packets, off_stages;  // byte offsets in dynamic shared memory
     int cpad;                         // shared-memory stride of the c/w buffers (>= max np)
     int mpad;                         // shared-memory stride of the residual (>= max M)
-    int npad;                         // shared-memory sums of the kept sweeps per team (>= max N;
-                                      // 0: the kept sweeps are added to the FP64 sums directly)
-    int team_words;                   // shared-memory elements per team: 2 cpad + mpad + 8 S + 2 npad
+    int fpad;                         // chain state in shared memory (>= max N; 0: in global memory)
+    int npad;                         // shared-memory sums of the kept sweeps per chain (>= max N;
+                                      // 0: in the workspace)
+    int team_words;                   // shared-memory elements per chain
     int n_items;                      // (problem, chain group) work items
     int minb;                         // register budget: 1 or 2 CTAs per SM
     int prior;                        // 1: kernels with the gamma prior's acceptance step
     int wait_limit;                   // polls before a bounded mbarrier wait gives up
     int stall;                        // test of the failure path: the producer issues no records
-    // U of the visited block in shared memory (two stages filled by the producer with
-    // one bulk copy per block visit; 0: the projections read U from global memory)
-    int ubytes;                       // bytes per stage (blocks whose U is larger read global memory)
-    int off_ubuf;                     // byte offset of the two stages
-    int off_ubar;                     // byte offset of their full[2] and empty[2] barriers
 };
 
 // Per-launch control block in device memory: the work queue and the launch's
@@ -137,29 +135,46 @@ struct RunCtrl {
     long long burn_in;                // absolute sweep index where accumulation starts
 };
 
-// A work item: problem index and chain group (consumers x 32/S chains).
+// A work item: problem index and chain group (consumers x C chains).
 struct WorkItem {
     int problem, group;
 };
 
-// Launchers (asm_sweep_{f32,f64}{,_m2}.cu).  kv: 16-byte vectors per lane.
+// Launchers (asm_sweep_*.cu).  kv: 16-byte vectors per lane and chain, a power of two.
 // Persistent: `ctas` CTAs of (consumers + 1) warps pull work items from
-// ctrl->queue (reset to 0 before the launch).  One problem (batch = false):
-// its parameters p0 travel by value in the launch; several (batch = true):
-// work item problems index the device array probs.  _m1 kernels budget the
-// registers for one CTA per SM (up to 255 per thread), _m2 for two (128).
-#define ASM_DECLARE_SWEEP_LAUNCHER(T, NAME)                                                                   \
-    cudaError_t launch_sweeps_##NAME(const SweepParams<T> &p0, const SweepParams<T> *probs, const WorkItem *items, \
-                                     RunCtrl *ctrl, const LaunchShape &shape, int kv, bool batch, int ctas,     \
-                                     cudaStream_t s);                                                          \
-    int sweep_ctas_per_sm_##NAME(const LaunchShape &shape, int kv, bool batch);
-ASM_DECLARE_SWEEP_LAUNCHER(float, f32_m1)
-ASM_DECLARE_SWEEP_LAUNCHER(float, f32_m2)
-ASM_DECLARE_SWEEP_LAUNCHER(double, f64_m1)
-ASM_DECLARE_SWEEP_LAUNCHER(double, f64_m2)
-ASM_DECLARE_SWEEP_LAUNCHER(float, f32_prior)     // with the gamma prior, one CTA per SM
+// ctrl->queue (reset to 0 before the launch); work item problems index the
+// device array probs.  _cC: C chains per warp; _m1 kernels budget the registers
+// for one CTA per SM (up to 255 per thread), _m2 for two (128).  A kv that a
+// launcher has no kernel for gives cudaErrorInvalidValue, and 0 CTAs per SM.
+#define ASM_DECLARE_SWEEP_LAUNCHER(T, NAME)                                                                     \
+    cudaError_t launch_sweeps_##NAME(const SweepParams<T> *probs, const WorkItem *items, RunCtrl *ctrl,         \
+                                     const LaunchShape &shape, int kv, int ctas, cudaStream_t s);               \
+    int sweep_ctas_per_sm_##NAME(const LaunchShape &shape, int kv);
+ASM_DECLARE_SWEEP_LAUNCHER(float, f32_c1_m1)
+ASM_DECLARE_SWEEP_LAUNCHER(float, f32_c2_m1)
+ASM_DECLARE_SWEEP_LAUNCHER(float, f32_c4_m1)
+ASM_DECLARE_SWEEP_LAUNCHER(float, f32_c1_m2)
+ASM_DECLARE_SWEEP_LAUNCHER(float, f32_c2_m2)
+ASM_DECLARE_SWEEP_LAUNCHER(float, f32_c4_m2)
+ASM_DECLARE_SWEEP_LAUNCHER(float, f32_prior)     // with the gamma prior: one chain per warp, one CTA per SM
+ASM_DECLARE_SWEEP_LAUNCHER(double, f64_c1_m1)
+ASM_DECLARE_SWEEP_LAUNCHER(double, f64_c2_m1)
+ASM_DECLARE_SWEEP_LAUNCHER(double, f64_c4_m1)
+ASM_DECLARE_SWEEP_LAUNCHER(double, f64_c1_m2)
+ASM_DECLARE_SWEEP_LAUNCHER(double, f64_c2_m2)
+ASM_DECLARE_SWEEP_LAUNCHER(double, f64_c4_m2)
 ASM_DECLARE_SWEEP_LAUNCHER(double, f64_prior)
 #undef ASM_DECLARE_SWEEP_LAUNCHER
+#define ASM_DEFINE_SWEEP_LAUNCHER(T, NAME, C, MINB, PRIOR, ...)                                                 \
+    cudaError_t launch_sweeps_##NAME(const SweepParams<T> *probs, const WorkItem *items, RunCtrl *ctrl,         \
+                                     const LaunchShape &shape, int kv, int ctas, cudaStream_t s)                \
+    {                                                                                                           \
+        return SweepDispatch<T, C, MINB, PRIOR, __VA_ARGS__>::launch(probs, items, ctrl, shape, kv, ctas, s);   \
+    }                                                                                                           \
+    int sweep_ctas_per_sm_##NAME(const LaunchShape &shape, int kv)                                              \
+    {                                                                                                           \
+        return SweepDispatch<T, C, MINB, PRIOR, __VA_ARGS__>::per_sm(shape, kv);                                \
+    }
 // Tensor-core residual refresh of the mixed path (asm_refresh_tc.cu): grid of
 // (chain tiles of 128) x n_problems x (the largest k split) CTAs; max_bn = the
 // largest refresh_tc_bn(M).
@@ -193,10 +208,6 @@ cudaError_t launch_scores(const double *R, int ldR, const double *Y, const doubl
                           double *Sq, cudaStream_t s);
 cudaError_t launch_vjp_G(const double *KtT, const double *L, const double *u, int M, int N, double *y,
                          cudaStream_t s);
-// CTAs of the persistent kernel that fit one SM at this shape (shared memory included).
-int sweep_ctas_per_sm_f32(const LaunchShape &shape, int kv, bool batch);
-int sweep_ctas_per_sm_f64(const LaunchShape &shape, int kv, bool batch);
-// Largest supported kv per precision.
 // Polls of a bounded mbarrier wait before it gives up (each poll may suspend
 // the thread briefly); a run that gives up counts a timeout and its results
 // are reported as ASM_ERR_TIMEOUT.
@@ -214,9 +225,14 @@ constexpr int kStepTraceMax = 4096;
 constexpr int kMaxConsumers = 7;
 // Deepest ring of move records (stages) a launch may use.
 constexpr int kMaxRingDepth = 48;
-// Move records per ring stage (one barrier wait and one release per stage).
+// Move records of the largest block per ring stage (one barrier wait and one release
+// per stage); smaller blocks put up to kMaxRecordsPerStage in a stage of that size.
 constexpr int kRecordsPerStage = 4;
-constexpr int kMaxKvF32 = 16;   // 64 floats per lane
-constexpr int kMaxKvF64 = 32;   // 64 doubles per lane
+constexpr int kMaxRecordsPerStage = 16;
+// Most slots of the ring of visit packets.
+constexpr int kMaxPacketSlots = 8;
+// Largest kv (16-byte vectors per lane and chain): 64 elements per lane.
+constexpr int kMaxKvF32 = 16;
+constexpr int kMaxKvF64 = 32;
 
 }  // namespace asmgb

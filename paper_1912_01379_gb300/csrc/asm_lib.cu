@@ -426,8 +426,7 @@ struct WsLayout {
 
 // device buffers of one precision
 struct PrecBuffers {
-    void *V = nullptr, *R = nullptr, *d = nullptr, *invd = nullptr, *meta = nullptr,
-         *rec = nullptr, *Ut = nullptr, *Um = nullptr, *Us = nullptr;
+    void *rec = nullptr, *pk = nullptr, *Ut = nullptr, *Um = nullptr;
     void *prior_am1 = nullptr;   // a_n - 1 of the gamma prior (nullptr: flat)
 };
 
@@ -438,7 +437,7 @@ struct asm_problem {
     std::vector<double> w;
     double f0 = 0.0;
     int max_nb = 0, max_np = 0;
-    long long totV = 0, totR = 0, totd = 0, totU = 0, totRec = 0, totUs = 0;
+    long long totU = 0, totRec = 0, totPk = 0;
     int max_rec = 0;   // largest record (elements)
     // device
     int *d_level_first = nullptr, *d_level_nblocks = nullptr;
@@ -462,7 +461,8 @@ struct asm_problem {
     void *ws_all = nullptr;   // the caller's workspace (header + every problem's section)
     void *ws = nullptr;       // this problem's section of it
     size_t ws_bytes = 0;
-    int chains = 0, precision = -1, team = 32;
+    int chains = 0, precision = -1;
+    int team = 0;   // lanes per chain, 32 / (chains per warp): 32, 16 or 8 (0: the built-in heuristic)
     long long sweeps_done = 0, kept = 0;
     long long kept_since = 0;   // every sweep from this one on has been accumulated
     unsigned long long seed = 0;
@@ -478,18 +478,15 @@ struct asm_problem {
     cudaGraphExec_t gexec = nullptr;
     struct GraphKey {
         const void *ws_all = nullptr;
-        int chains = 0, precision = -1, kv = 0, ctas = 0, S = 0, consumers = 0, depth = 0, n_items = 0, minb = 0,
-            ubytes = 0, rps = 0, npad = 0;
+        int chains = 0, precision = -1, kv = 0, ctas = 0, C = 0, consumers = 0, depth = 0, n_items = 0, minb = 0,
+            pbytes = 0, pslots = 0, rps = 0, npad = 0, fpad = 0;
         size_t refresh_smem = 0;
-        unsigned long long seed = 0, problem_id = 0, chain_offset = 0;
         bool operator==(const GraphKey &o) const
         {
             return ws_all == o.ws_all && chains == o.chains && precision == o.precision && kv == o.kv &&
-                   ctas == o.ctas && S == o.S && consumers == o.consumers && depth == o.depth &&
-                   n_items == o.n_items && minb == o.minb && ubytes == o.ubytes && rps == o.rps && npad == o.npad &&
-                   refresh_smem == o.refresh_smem &&
-                   seed == o.seed &&
-                   problem_id == o.problem_id && chain_offset == o.chain_offset;
+                   ctas == o.ctas && C == o.C && consumers == o.consumers && depth == o.depth &&
+                   n_items == o.n_items && minb == o.minb && pbytes == o.pbytes && pslots == o.pslots &&
+                   rps == o.rps && npad == o.npad && fpad == o.fpad && refresh_smem == o.refresh_smem;
         }
     } gkey;
     long long graph_replays = 0, tc_refreshes = 0;
@@ -598,7 +595,7 @@ int upload(void **dst, const std::vector<T> &src)
 
 void free_prec(PrecBuffers &b)
 {
-    void *ptrs[] = {b.V, b.R, b.d, b.invd, b.meta, b.rec, b.Ut, b.Um, b.Us, b.prior_am1};
+    void *ptrs[] = {b.rec, b.pk, b.Ut, b.Um, b.prior_am1};
     for (void *x : ptrs)
         if (x) cudaFree(x);
     b = PrecBuffers{};
@@ -848,58 +845,52 @@ done:
     return rc;
 }
 
-// Host-side mode rows for one precision, then upload.
+// Host-side mode records and visit packets for one precision, then upload.
 template <class T>
 int build_precision(asm_problem *p, const HostFactors &hf, PrecBuffers &out)
 {
     const int M = p->M;
     const T nan = std::numeric_limits<T>::quiet_NaN();
-    constexpr int MW = 16 / sizeof(T);
-    std::vector<T> V(p->totV, T(0)), R(p->totR, nan), d(p->totd, T(0)),
-        invd(p->totd, T(0)), meta((size_t)p->totd * MW, T(0)), rec(std::max<long long>(p->totRec, 1), T(0)),
-        Ut(std::max<long long>(p->totU, 1), T(0)),
-        Um(std::max<long long>(p->totU, 1), T(0)),
-        Us(p->totUs + 4, T(0));   // + 4: a copy rounded up to 16 bytes stays inside
+    std::vector<T> rec(p->totRec, T(0)), pk(p->totPk + 4, T(0)),   // + 4: a copy rounded up to 16 bytes stays inside
+        Ut(std::max<long long>(p->totU, 1), T(0)), Um(std::max<long long>(p->totU, 1), T(0));
     for (int b = 0; b < p->n_blocks; ++b) {
         const BlockDesc &B = p->blocks[b];
         const std::vector<double> &hd = hf.d[b], &hV = hf.V[b], &hU = hf.U[b];
-        for (int j = 0; j < B.n; ++j) {
+        // R_j = -1/V_j; NaN where V is left out of the bounds, in the padding and past the last mode
+        auto bounds_row = [&](int j, T *r) {
+            for (int i = 0; i < B.rs; ++i) r[i] = nan;
+            if (j >= B.n) return;
             const double *v = &hV[(size_t)j * B.n];
             double vmax = 0.0;
             for (int i = 0; i < B.n; ++i) vmax = std::max(vmax, std::fabs(v[i]));
-            for (int i = 0; i < B.n; ++i) {
-                V[B.offV + (size_t)j * B.rs + i] = (T)v[i];
-                if (std::fabs(v[i]) < 0x1p-40 * vmax) continue;   // left out of the bounds
-                R[B.offR + (size_t)j * B.rs + i] = (T)(-1.0 / v[i]);
-            }
-            d[B.offd + j] = (T)hd[j];
-            invd[B.offd + j] = hd[j] > 0.0 ? (T)(1.0 / hd[j]) : T(0);
-            meta[(size_t)(B.offd + j) * MW] = d[B.offd + j];
-            meta[(size_t)(B.offd + j) * MW + 1] = invd[B.offd + j];
-        }
+            for (int i = 0; i < B.n; ++i)
+                if (!(std::fabs(v[i]) < 0x1p-40 * vmax)) r[i] = (T)(-1.0 / v[i]);
+        };
         for (int j = 0; j < B.np; ++j)
             for (int m = 0; m < M; ++m) {
                 Ut[B.offU + (size_t)j * M + m] = (T)hU[(size_t)j * M + m];
                 Um[B.offU + (size_t)m * B.np + j] = (T)hU[(size_t)j * M + m];
-                Us[B.offUs + (size_t)j * B.usr + m] = (T)hU[(size_t)j * M + m];
             }
-        // move records: {V_j, R_{j+1}, d_j, 1/d_j, dres_j}
+        // move records: {V_j, R_{j+1}, d_j, 1/d_j, dres_j, 0}
         for (int j = 0; j < B.n; ++j) {
             T *r = &rec[B.offRec + (size_t)j * B.recstride];
-            for (int i = 0; i < B.rs; ++i) {
-                r[i] = V[B.offV + (size_t)j * B.rs + i];
-                r[B.rs + i] = R[B.offR + (size_t)(j + 1) * B.rs + i];
-            }
-            r[2 * B.rs] = d[B.offd + j];
-            r[2 * B.rs + 1] = invd[B.offd + j];
+            for (int i = 0; i < B.n; ++i) r[i] = (T)hV[(size_t)j * B.n + i];
+            bounds_row(j + 1, r + B.rs);
+            r[2 * B.rs] = (T)hd[j];
+            r[2 * B.rs + 1] = hd[j] > 0.0 ? (T)(1.0 / hd[j]) : T(0);
             r[2 * B.rs + 2] = (T)hf.dres[b][j];
         }
+        // visit packet: descriptor, R_0, U with odd row stride
+        T *k = &pk[B.offPk];
+        std::memcpy(k, &B, sizeof(B));
+        bounds_row(0, k + kPacketHeader);
+        for (int j = 0; j < B.np; ++j)
+            for (int m = 0; m < M; ++m)
+                k[kPacketHeader + B.rs + (size_t)j * B.usr + m] = (T)hU[(size_t)j * M + m];
     }
     int rc;
-    if ((rc = upload(&out.V, V)) || (rc = upload(&out.R, R)) ||
-        (rc = upload(&out.d, d)) || (rc = upload(&out.invd, invd)) || (rc = upload(&out.meta, meta)) || (rc = upload(&out.rec, rec)) ||
-        (rc = upload(&out.Ut, Ut)) ||
-        (rc = upload(&out.Um, Um)) || (rc = upload(&out.Us, Us)))
+    if ((rc = upload(&out.rec, rec)) || (rc = upload(&out.pk, pk)) || (rc = upload(&out.Ut, Ut)) ||
+        (rc = upload(&out.Um, Um)))
         return rc;
     return ASM_OK;
 }
@@ -950,13 +941,10 @@ SweepParams<T> make_params(asm_problem *p, const PrecBuffers &b, const WsLayout 
     sp.level_first = p->d_level_first;
     sp.level_nblocks = p->d_level_nblocks;
     sp.blocks = p->d_blocks;
-    sp.pd.V = (const T *)b.V;
-    sp.pd.R = (const T *)b.R;
-    sp.pd.d = (const T *)b.d;
-    sp.pd.invd = (const T *)b.invd;
+    sp.pd.rec = (const T *)b.rec;
+    sp.pd.pk = (const T *)b.pk;
     sp.pd.Ut = (const T *)b.Ut;
     sp.pd.Um = (const T *)b.Um;
-    sp.pd.Us = (const T *)b.Us;
     char *ws = (char *)p->ws;
     sp.F = (T *)(ws + L.F);
     sp.ldF = L.ldF;
@@ -969,8 +957,6 @@ SweepParams<T> make_params(asm_problem *p, const PrecBuffers &b, const WsLayout 
     sp.problem_id = p->problem_id;
     sp.chain_offset = p->chain_offset;
     sp.counters = (Counters *)(ws + L.counters);
-    sp.pd.meta = (const T *)b.meta;
-    sp.pd.rec = (const T *)b.rec;
     sp.KtT = p->d_KtT;
     sp.Khi = p->d_Khi;
     sp.Klo = p->d_Klo;
@@ -995,125 +981,163 @@ SweepParams<T> make_params(asm_problem *p, const PrecBuffers &b, const WsLayout 
     return sp;
 }
 
-// Shared memory of the sweep kernel: per team c, w, r~ and the uniforms of a
-// window of 4S moves (draws and prior acceptances); the ring's `full`
-// and `empty` barriers and `depth` record stages.  Consumer warps per CTA:
-// enough that the CTAs about cover the SMs once (all chains of an SM then
-// share one ring), or the tuned count.  CTAs per SM: as many as the work
-// needs and the registers allow (the persistent kernel queues the rest); the
-// ring is as deep as the shared memory left to each of them.  For a batch the
-// shape covers the largest problem.
-int ctas_per_sm(int precision, const LaunchShape &sh, int kv, bool batch)
+// The sweep kernels of one (precision, chains per warp, register budget, prior).
+struct SweepFns {
+    cudaError_t (*launch64)(const SweepParams<double> *, const WorkItem *, RunCtrl *, const LaunchShape &, int, int,
+                            cudaStream_t);
+    cudaError_t (*launch32)(const SweepParams<float> *, const WorkItem *, RunCtrl *, const LaunchShape &, int, int,
+                            cudaStream_t);
+    int (*per_sm)(const LaunchShape &, int);
+    cudaError_t launch(const SweepParams<double> *p, const WorkItem *it, RunCtrl *c, const LaunchShape &sh, int kv,
+                       int ctas, cudaStream_t s) const { return launch64(p, it, c, sh, kv, ctas, s); }
+    cudaError_t launch(const SweepParams<float> *p, const WorkItem *it, RunCtrl *c, const LaunchShape &sh, int kv,
+                       int ctas, cudaStream_t s) const { return launch32(p, it, c, sh, kv, ctas, s); }
+};
+
+SweepFns sweep_fns(int precision, const LaunchShape &sh)
 {
-    if (precision == ASM_FP64)
-        return sh.prior ? sweep_ctas_per_sm_f64_prior(sh, kv, batch)
-               : sh.minb == 2 ? sweep_ctas_per_sm_f64_m2(sh, kv, batch) : sweep_ctas_per_sm_f64_m1(sh, kv, batch);
-    return sh.prior ? sweep_ctas_per_sm_f32_prior(sh, kv, batch)
-           : sh.minb == 2 ? sweep_ctas_per_sm_f32_m2(sh, kv, batch) : sweep_ctas_per_sm_f32_m1(sh, kv, batch);
+    const int ci = sh.C == 1 ? 0 : sh.C == 2 ? 1 : 2;
+#define F64(NAME) SweepFns{launch_sweeps_##NAME, nullptr, sweep_ctas_per_sm_##NAME}
+#define F32(NAME) SweepFns{nullptr, launch_sweeps_##NAME, sweep_ctas_per_sm_##NAME}
+    static const SweepFns f64[2][3] = {{F64(f64_c1_m1), F64(f64_c2_m1), F64(f64_c4_m1)},
+                                       {F64(f64_c1_m2), F64(f64_c2_m2), F64(f64_c4_m2)}};
+    static const SweepFns f32[2][3] = {{F32(f32_c1_m1), F32(f32_c2_m1), F32(f32_c4_m1)},
+                                       {F32(f32_c1_m2), F32(f32_c2_m2), F32(f32_c4_m2)}};
+    if (precision == ASM_FP64) return sh.prior ? F64(f64_prior) : f64[sh.minb == 2][ci];
+    return sh.prior ? F32(f32_prior) : f32[sh.minb == 2][ci];
+#undef F64
+#undef F32
 }
 
+// What the shared-memory plan of a launch depends on (the largest of its problems').
+struct PlanNeeds {
+    int max_rec = 0, max_np = 1, max_M = 1, max_N = 1;   // elements
+    int head = 0;                    // bytes of the largest packet without U
+    std::vector<int> packets;        // bytes of every block's packet with U
+};
+
+// Shared memory of the sweep kernel: per chain c, w, r~ and the uniforms of a window of
+// 128 moves (with a prior as many for the acceptances), the barriers, the packet slots
+// and the record stages.  Consumer warps per CTA: enough that the CTAs about cover the
+// SMs once (all chains of an SM then share one ring), or the tuned count.  CTAs per SM:
+// as many as the work needs and the registers allow (the persistent kernel queues the
+// rest).  What the budget leaves goes, in this order, to: a ring of at least
+// kMinStages stages (fewer records to a stage where the records are long, before fewer
+// consumers); U of the visited blocks in the packets; the sums of the kept sweeps; the chain
+// states; a ring of kRingRecords of the largest records; more packet slots; the
+// rest of the ring.  For a batch the shape covers the largest problem.
 template <class T>
-bool plan_shape(LaunchShape &sh, int S, int max_rec, int max_np, int max_M, long long total_warps, int kv,
-                bool batch, int want_consumers, int minb, bool prior, const std::vector<int> &ublk_bytes,
-                int max_N_sum)
+bool plan_shape(LaunchShape &sh, int C, const PlanNeeds &nd, long long chains, int kv, int want_consumers, int minb,
+                bool prior)
 {
     sh.minb = prior ? 1 : minb;   // the prior's kernels exist for one CTA per SM
     sh.prior = prior ? 1 : 0;
+    sh.C = C;
     sh.wait_limit = kWaitLimit;
     sh.stall = 0;
     constexpr int kSMs = 152;
-    constexpr int kMinRingRecords = 8;   // the U stages may not squeeze the ring below this many records
-    const int TW = 32 / S;
-    const int prec = sizeof(T) == 8 ? ASM_FP64 : ASM_MIXED;
-    sh.S = S;
-    sh.cpad = round_up_int(std::max(max_np, 1), 32);
-    sh.mpad = round_up_int(std::max(max_M, 1), 32);
-    sh.npad = 0;
+    constexpr int kMinStages = 3;
+    constexpr int kRingRecords = 24;
+    const long long total_warps = (chains + C - 1) / C;
+    sh.cpad = round_up_int(std::max(nd.max_np, 1), 32);
+    sh.mpad = round_up_int(std::max(nd.max_M, 1), 32);
     int consumers = want_consumers > 0
                         ? want_consumers
                         : (int)std::min<long long>(kMaxConsumers,
                                                    std::max<long long>(1, (total_warps + kSMs - 1) / kSMs));
-    if (const char *e = std::getenv("ASM_CONSUMERS_PER_CTA")) {   // tuning override
-        const int c = std::atoi(e);
-        if (c >= 1 && c <= kMaxConsumers) consumers = c;
-    }
-    sh.rps = kRecordsPerStage;
-    if (const char *e = std::getenv("ASM_RECORDS_PER_STAGE")) {   // tuning override
-        const int r = std::atoi(e);
-        if (r >= 1 && r <= 8) sh.rps = r;
-    }
-    // fewer records per stage where a ring of four stages would not fit (long records: FP64
-    // state on large blocks)
-    auto stage_of = [&](int rps) { return (int)align_up((size_t)rps * max_rec * sizeof(T), 128); };
-    while (sh.rps > 1 && 4 * (size_t)stage_of(sh.rps) > 200 * 1024) --sh.rps;
-    sh.stage_bytes = stage_of(sh.rps);
-    const int kMinRing = std::max(2, (kMinRingRecords + sh.rps - 1) / sh.rps);
-    // per-team state, then the ring's barriers (full, empty: 8 bytes per stage each), the
-    // U stages' barriers (4 x 8 bytes, padded to 128) and the U stages
-    constexpr int kBarBytes = 8 * kMaxRingDepth;
-    auto words = [&](int npad) { return 2 * sh.cpad + sh.mpad + 8 * S + 2 * npad; };
-    auto fixed = [&](int c) {
-        return align_up((size_t)c * TW * words(sh.npad) * sizeof(T), 128) + 2 * kBarBytes + 128;
+    auto env = [](const char *name, int lo, int hi, int dflt) {   // tuning overrides
+        const char *e = std::getenv(name);
+        const int v = e ? std::atoi(e) : 0;
+        return e && v >= lo && v <= hi ? v : dflt;
     };
-    int max_depth = kMaxRingDepth;
-    if (const char *e = std::getenv("ASM_RING_DEPTH")) {            // tuning override
-        const int d = std::atoi(e);
-        if (d >= 2 && d <= kMaxRingDepth) max_depth = d;
-    }
-    bool stage_u = std::getenv("ASM_NO_U_STAGE") == nullptr;       // tuning override
+    consumers = env("ASM_CONSUMERS_PER_CTA", 1, kMaxConsumers, consumers);
+    const int want_rps = env("ASM_RECORDS_PER_STAGE", 1, 8, kRecordsPerStage);
+    const int max_depth = env("ASM_RING_DEPTH", 2, kMaxRingDepth, kMaxRingDepth);
+    const bool stage_u = std::getenv("ASM_NO_U_STAGE") == nullptr;
+    constexpr size_t kBarBytes = 8 * (2 * kMaxRingDepth + 2 * kMaxPacketSlots);
+    const size_t head = align_up((size_t)nd.head, 128);
+    auto stage_of = [&](int rps) { return align_up((size_t)rps * nd.max_rec * sizeof(T), 128); };
     for (; consumers >= 1; --consumers) {
         LaunchShape probe = sh;   // no dynamic shared memory: the register limit alone
         probe.consumers = consumers;
         probe.depth = 0;
         probe.off_stages = 0;
-        probe.ubytes = 0;
-        const int by_regs = std::max(1, ctas_per_sm(prec, probe, kv, batch));
+        const int by_regs = sweep_fns(sizeof(T) == 8 ? ASM_FP64 : ASM_MIXED, probe).per_sm(probe, kv);
+        if (by_regs < 1) return false;   // no kernel for this tile
         const long long ctas = (total_warps + consumers - 1) / consumers;
         const int per_sm = (int)std::min<long long>(by_regs, std::max<long long>(1, (ctas + kSMs - 1) / kSMs));
-        const size_t budget = std::min<size_t>(220 * 1024 / per_sm, 227 * 1024);
-        // FP32 chain state: the kept sweeps' sums of one launch (at most one refresh period)
-        // in shared memory, added to the FP64 sums once per launch, where they fit
-        sh.npad = 0;
-        if (sizeof(T) == 4 && max_N_sum > 0 && std::getenv("ASM_NO_SMEM_SUMS") == nullptr) {
-            sh.npad = round_up_int(max_N_sum, 32);
-            if (fixed(consumers) + (size_t)kMinRing * sh.stage_bytes > budget) sh.npad = 0;
-        }
-        // U stages: as large as the largest block U that leaves room for a ring of kMinRing
-        size_t ub = 0;
-        if (stage_u) {
-            const size_t room = budget > fixed(consumers) + (size_t)kMinRing * sh.stage_bytes
-                                    ? (budget - fixed(consumers) - (size_t)kMinRing * sh.stage_bytes) / 2
-                                    : 0;
-            for (int b : ublk_bytes) {
+        const size_t budget = std::min<size_t>(220 * 1024 / per_sm, 224 * 1024);
+        const int base_words = 2 * sh.cpad + sh.mpad + (prior ? 256 : 128);
+        const size_t per_word = (size_t)consumers * C * sizeof(T);
+        size_t used = per_word * base_words + kBarBytes + 256 + 2 * head;
+        const int min_stages = std::min(kMinStages, max_depth);
+        int rps = want_rps;
+        while (rps > 1 && used + min_stages * stage_of(rps) > budget) --rps;
+        int depth = min_stages;
+        if (used + depth * stage_of(rps) > budget) depth = 2;
+        if (used + depth * stage_of(rps) > budget) continue;
+        used += depth * stage_of(rps);
+        size_t slot = head;
+        if (stage_u)
+            for (int b : nd.packets) {
                 const size_t bb = align_up((size_t)b, 128);
-                if (bb <= room && bb > ub) ub = bb;
+                if (bb > slot && used + 2 * (bb - head) <= budget) slot = bb;
             }
+        used += 2 * (slot - head);
+        const int nr = round_up_int(nd.max_N, 32);
+        sh.npad = sh.fpad = 0;
+        if (sizeof(T) == 4 && std::getenv("ASM_NO_SMEM_SUMS") == nullptr && used + 2 * per_word * nr <= budget) {
+            sh.npad = nr;
+            used += 2 * per_word * nr;
         }
-        int depth = max_depth;
-        while (depth > 2 && fixed(consumers) + 2 * ub + (size_t)depth * sh.stage_bytes > budget) --depth;
-        if (fixed(consumers) + 2 * ub + (size_t)depth * sh.stage_bytes <= budget || consumers == 1) {
-            if (fixed(consumers) + 2 * ub + (size_t)depth * sh.stage_bytes > 227 * 1024) return false;
-            sh.consumers = consumers;
-            sh.depth = depth;
-            sh.ubytes = (int)ub;
-            sh.team_words = words(sh.npad);
-            sh.off_full = (int)align_up((size_t)consumers * TW * sh.team_words * sizeof(T), 128);
-            sh.off_empty = sh.off_full + kBarBytes;
-            sh.off_ubar = sh.off_full + 2 * kBarBytes;
-            sh.off_ubuf = sh.off_ubar + 128;
-            sh.off_stages = sh.off_ubuf + 2 * (int)ub;
-            return true;
+        if (used + per_word * nr <= budget) {
+            sh.fpad = nr;
+            used += per_word * nr;
         }
+        auto deepen = [&](int records) {
+            while (depth < max_depth && depth * rps < records && used + stage_of(rps) <= budget) {
+                ++depth;
+                used += stage_of(rps);
+            }
+        };
+        deepen(kRingRecords);
+        int slots = 2;
+        while (slots < kMaxPacketSlots && used + slot <= budget) {
+            ++slots;
+            used += slot;
+        }
+        deepen(max_depth * rps);
+        sh.consumers = consumers;
+        sh.rps = rps;
+        sh.stage_bytes = (int)stage_of(rps);
+        sh.depth = depth;
+        sh.pslots = slots;
+        sh.pbytes = (int)slot;
+        sh.team_words = base_words + sh.fpad + 2 * sh.npad;
+        sh.off_bars = (int)align_up(per_word * sh.team_words, 128);
+        sh.off_packets = (int)align_up(sh.off_bars + kBarBytes, 128);
+        sh.off_stages = sh.off_packets + slots * (int)slot;
+        return true;
     }
     return false;
 }
 
-int pick_kv(int max_nb, int vec, int S, int kmax)
+int pick_kv(int max_nb, int vec, int kmax)
 {
-    int need = (max_nb + vec * S - 1) / (vec * S);
+    const int need = (max_nb + vec * 32 - 1) / (vec * 32);
     int kv = 1;
     while (kv < need) kv <<= 1;
     return kv <= kmax ? kv : -1;
+}
+
+// Chains per warp and register budget of a launch that is not tuned.
+void pick_shape(bool f64, int kv, long long chains, int &C, int &minb)
+{
+    C = 1;
+    minb = 1;
+    (void)f64;
+    (void)kv;
+    (void)chains;
 }
 
 // Snapshot of all chains into the moments of the backward pass (every
@@ -1196,41 +1220,38 @@ int run_all(asm_problem *h, int chains, long long s_begin, long long s_end, long
     const RunLayout RL = run_layout(h, chains, h->precision);
     char *base = (char *)h->ws_all;
     std::vector<SweepParams<T>> probs;
-    int max_rec = 0, max_np = 1, max_M = 1, max_nb = 1, max_N = 1;
+    PlanNeeds nd;
+    int max_nb = 1;
+    bool prior = false;   // any problem with a gamma prior: the kernels with the acceptance step
     for (asm_problem *u : us) {
         const WsLayout L = ws_layout(u, chains, h->precision);
-        probs.push_back(make_params<T>(u, sizeof(T) == 8 ? u->b64 : u->b32, L, chains));
-        max_rec = std::max(max_rec, u->max_rec);
-        max_np = std::max(max_np, u->max_np);
-        max_M = std::max(max_M, u->M);
+        const PrecBuffers &pb = sizeof(T) == 8 ? u->b64 : u->b32;
+        probs.push_back(make_params<T>(u, pb, L, chains));
+        prior = prior || pb.prior_am1 != nullptr;
+        nd.max_rec = std::max(nd.max_rec, u->max_rec);
+        nd.max_np = std::max(nd.max_np, u->max_np);
+        nd.max_M = std::max(nd.max_M, u->M);
+        nd.max_N = std::max(nd.max_N, u->N);
         max_nb = std::max(max_nb, u->max_nb);
-        max_N = std::max(max_N, u->N);
+        for (const BlockDesc &B : u->blocks) {
+            nd.head = std::max(nd.head, (int)((kPacketHeader + B.rs) * sizeof(T)));
+            const long long whole = (kPacketHeader + B.rs + (long long)B.np * B.usr) * (long long)sizeof(T);
+            if (whole < 220 * 1024) nd.packets.push_back((int)((whole + 15) / 16 * 16));
+        }
     }
-    // bytes of every block's U in its staging layout (np rows of usr elements, 16-byte multiple)
-    std::vector<int> ublk;
-    for (asm_problem *u : us)
-        for (const BlockDesc &B : u->blocks)
-            ublk.push_back((int)(((size_t)B.np * B.usr * sizeof(T) + 15) / 16 * 16));
-    const int S = h->team;
+    std::sort(nd.packets.begin(), nd.packets.end());
     const int vec = 16 / (int)sizeof(T);
-    const int kv = pick_kv(max_nb, vec, S, sizeof(T) == 8 ? kMaxKvF64 : kMaxKvF32);
+    const int kv = pick_kv(max_nb, vec, sizeof(T) == 8 ? kMaxKvF64 : kMaxKvF32);
     if (kv < 0) return ASM_ERR_TOO_LARGE;
-    const int TW = 32 / S;
-    const long long warps_per_unit = (chains + TW - 1) / TW;
-    const bool batch = !h->kids.empty();
-    const long long total_warps = warps_per_unit * (long long)us.size();
-    // register budget: one CTA per SM (up to 255 registers) while one CTA of
-    // consumers per SM holds every chain; two CTAs (128 registers) when there
-    // are more chains than that, except for FP64 with wide blocks, whose chain
-    // state would spill
-    int minb = total_warps > 152LL * kMaxConsumers && !(sizeof(T) == 8 && kv >= 16) ? 2 : 1;
+    const long long all_chains = (long long)chains * (long long)us.size();
+    int C = 1, minb = 1;
+    pick_shape(sizeof(T) == 8, kv, all_chains, C, minb);
+    if (h->team) C = 32 / h->team;
+    if (prior) C = 1;
     if (h->tuned_minb) minb = h->tuned_minb;
-    bool prior = false;   // any problem with a gamma prior: the kernels with the acceptance step
-    for (asm_problem *u : us) prior = prior || (sizeof(T) == 8 ? u->b64.prior_am1 : u->b32.prior_am1) != nullptr;
     LaunchShape sh{};
-    if (!plan_shape<T>(sh, S, max_rec, max_np, max_M, total_warps, kv, batch, h->tuned_consumers, minb, prior, ublk,
-                       max_N))
-        return ASM_ERR_TOO_LARGE;
+    if (!plan_shape<T>(sh, C, nd, all_chains, kv, h->tuned_consumers, minb, prior)) return ASM_ERR_TOO_LARGE;
+    const SweepFns fns = sweep_fns(h->precision, sh);
     bool stall = h->test_stall;
     for (asm_problem *u : us) stall = stall || u->test_stall;
     if (stall) {   // failure-path test: no records, short waits
@@ -1244,19 +1265,20 @@ int run_all(asm_problem *h, int chains, long long s_begin, long long s_end, long
         return (long long)us[a]->N * us[a]->max_nb > (long long)us[b]->N * us[b]->max_nb;
     });
     std::vector<WorkItem> items;
-    const int groups = (int)((warps_per_unit + sh.consumers - 1) / sh.consumers);
+    const int per_item = sh.consumers * sh.C;   // chains
+    const int groups = (chains + per_item - 1) / per_item;
     for (int k : order)
         for (int g = 0; g < groups; ++g) items.push_back(WorkItem{k, g});
     sh.n_items = (int)items.size();
-    const int per_sm = ctas_per_sm(h->precision, sh, kv, batch);
+    const int per_sm = fns.per_sm(sh, kv);
     if (per_sm <= 0) return ASM_ERR_CUDA;
     const int ctas = (int)std::min<long long>(sh.n_items, 152LL * per_sm);
-    h->last_team = sh.S;
+    h->last_team = 32 / sh.C;
     h->last_consumers = sh.consumers;
     h->last_ctas = ctas;
     h->last_items = sh.n_items;
     h->last_minb = sh.minb;
-    const size_t rsmem = sizeof(double) * (size_t)max_N;
+    const size_t rsmem = sizeof(double) * (size_t)nd.max_N;
     if (const int rc = refresh_smem(refresh_all_kernel<T>, rsmem); rc != ASM_OK) return rc;
     // the mixed path refreshes on the tensor cores (3xTF32) unless asked for FP64 CUDA cores
     const bool tc = sizeof(T) == 4 && !h->refresh_fp64;
@@ -1275,17 +1297,7 @@ int run_all(asm_problem *h, int chains, long long s_begin, long long s_end, long
                         h->stream) != cudaSuccess)
         return ASM_ERR_CUDA;
     const unsigned n_refresh = (unsigned)(us.size() * chains);
-    const SweepParams<T> &p0 = probs[0];   // a single problem's parameters travel by value
-    auto sweep = [&](cudaStream_t st) {
-        if constexpr (sizeof(T) == 8)
-            return sh.prior ? launch_sweeps_f64_prior(p0, d_probs, d_items, ctrl, sh, kv, batch, ctas, st)
-                   : sh.minb == 2 ? launch_sweeps_f64_m2(p0, d_probs, d_items, ctrl, sh, kv, batch, ctas, st)
-                                  : launch_sweeps_f64_m1(p0, d_probs, d_items, ctrl, sh, kv, batch, ctas, st);
-        else
-            return sh.prior ? launch_sweeps_f32_prior(p0, d_probs, d_items, ctrl, sh, kv, batch, ctas, st)
-                   : sh.minb == 2 ? launch_sweeps_f32_m2(p0, d_probs, d_items, ctrl, sh, kv, batch, ctas, st)
-                                  : launch_sweeps_f32_m1(p0, d_probs, d_items, ctrl, sh, kv, batch, ctas, st);
-    };
+    auto sweep = [&](cudaStream_t st) { return fns.launch(d_probs, d_items, ctrl, sh, kv, ctas, st); };
     auto binning = [&](cudaStream_t st) {
         bin_kernel<T><<<n_refresh, 128, 0, st>>>(d_probs, chains, ctrl);
         return cudaGetLastError();
@@ -1296,7 +1308,7 @@ int run_all(asm_problem *h, int chains, long long s_begin, long long s_end, long
     auto refresh = [&](cudaStream_t st) {
         if constexpr (sizeof(T) == 4) {
             if (tc) {
-                cudaError_t e = launch_refresh_ref(d_probs, (int)us.size(), chains, max_N, max_M, st);
+                cudaError_t e = launch_refresh_ref(d_probs, (int)us.size(), chains, nd.max_N, nd.max_M, st);
                 if (e == cudaSuccess) e = launch_refresh_tc(d_probs, (int)us.size(), chains, max_bn, max_parts, true, st);
                 if (e == cudaSuccess && max_parts > 1) e = launch_refresh_finish(d_probs, (int)us.size(), chains, true, st);
                 return e;
@@ -1321,18 +1333,17 @@ int run_all(asm_problem *h, int chains, long long s_begin, long long s_end, long
             key.precision = h->precision;
             key.kv = kv;
             key.ctas = ctas;
-            key.S = sh.S;
+            key.C = sh.C;
             key.consumers = sh.consumers;
             key.depth = sh.depth;
             key.n_items = sh.n_items;
             key.minb = sh.minb + 4 * sh.prior + 8 * sh.stall;
-            key.ubytes = sh.ubytes;
+            key.pbytes = sh.pbytes;
+            key.pslots = sh.pslots;
             key.rps = sh.rps;
             key.npad = sh.npad;
+            key.fpad = sh.fpad;
             key.refresh_smem = tc ? refresh_tc_smem(max_bn) + 1 : rsmem;
-            key.seed = p0.seed;   // by value in a single problem's launch
-            key.problem_id = p0.problem_id;
-            key.chain_offset = p0.chain_offset;
             if (!h->gexec || !(h->gkey == key)) {
                 drop_graph(h);
                 if (!h->cap_stream && cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking) != cudaSuccess)
@@ -1511,7 +1522,7 @@ int asm_setup(const asm_desc *ds, asm_problem **out)
         nb += ds->level_nblocks[l];
     }
     p->n_blocks = nb;
-    long long oV = 0, oR = 0, od = 0, oU = 0, oRec = 0, oUs = 0;
+    long long oU = 0, oRec = 0, oPk = 0;
     for (int l = 0; l < ds->n_levels; ++l) {
         const int *st = ds->block_start + p->level_first[l];
         for (int b = 0; b < ds->level_nblocks[l]; ++b) {
@@ -1521,22 +1532,21 @@ int asm_setup(const asm_desc *ds, asm_problem **out)
             B.start = s0;
             B.n = s1 - s0;
             B.np = std::min(M, B.n);
-            B.rs = round_up_int(B.n, kRowAlign);
-            B.offV = oV; oV += (long long)B.n * B.rs;
-            B.offR = oR; oR += (long long)(B.n + 1) * B.rs;
-            B.offd = od; od += B.n;
+            B.nz = B.n;   // lowered when the singular values are known
+            B.rs = B.n <= kRowAlignSmall ? kRowAlignSmall : round_up_int(B.n, kRowAlign);
+            B.last = b + 1 == ds->level_nblocks[l];
             B.offU = oU; oU += (long long)B.np * M;
             B.usr = M | 1;
-            B.offUs = oUs; oUs += ((long long)B.np * B.usr + 3) / 4 * 4;   // 16-byte aligned in both precisions
-            B.recstride = 2 * B.rs + 16;   // elements; 16 holds the mode data in both precisions
+            B.recstride = 2 * B.rs + 4;   // elements; the mode data take 3
             B.offRec = oRec; oRec += (long long)B.n * B.recstride;
+            B.offPk = oPk; oPk += (kPacketHeader + B.rs + (long long)B.np * B.usr + 3) / 4 * 4;   // 16-byte aligned
             p->max_rec = std::max(p->max_rec, B.recstride);
             p->blocks.push_back(B);
             p->max_nb = std::max(p->max_nb, B.n);
             p->max_np = std::max(p->max_np, B.np);
         }
     }
-    p->totV = oV; p->totR = oR; p->totd = od; p->totU = oU; p->totRec = oRec; p->totUs = oUs;
+    p->totU = oU; p->totRec = oRec; p->totPk = oPk;
     p->w.assign(N, 1.0);
     if (ds->w) {
         if (!all_finite(ds->w, N)) { asm_destroy(p); return ASM_ERR_NONFINITE; }
@@ -1589,6 +1599,11 @@ int asm_setup(const asm_desc *ds, asm_problem **out)
         if (rc != ASM_OK) { asm_destroy(p); return rc; }
     }
     complete_residual_update(p, hf);
+    // the tail of a block's moves that are flat in its exact null space
+    for (int b = 0; b < nb; ++b) {
+        BlockDesc &B = p->blocks[b];
+        while (B.nz > B.np && hf.d[b][B.nz - 1] == 0.0) --B.nz;
+    }
     if (given && ds->C) {
         if (!all_finite(ds->C, (size_t)M * M)) { asm_destroy(p); return ASM_ERR_NONFINITE; }
         rc = device_cholesky(ds->C, M, &p->d_L);
@@ -1884,10 +1899,14 @@ int asm_tune(asm_problem *p, int chains, int precision, void *d_workspace, size_
     int best_team = team0, best_cons = cons0, best_minb = minb0, rc = ASM_OK;
     float best = 0.f;
     bool any = false;
+    bool prior = false;
+    for (asm_problem *u : units_of(p))
+        prior = prior || (precision == ASM_FP64 ? u->b64.prior_am1 : u->b32.prior_am1) != nullptr;
     const int teams[] = {32, 16, 8};
     const int conss[] = {0, 2, 3, 4, 5, 6, 7};   // 0: the built-in heuristic
     for (int trial = 0; trial < 3 * 7 * 2; ++trial) {
         const int S = teams[trial / 14], c = conss[(trial / 2) % 7], mb = 1 + trial % 2;
+        if (prior && (S != 32 || mb != 1)) continue;   // its kernels: one chain per warp, one CTA per SM
         {
             p->team = S;
             p->tuned_consumers = c;

@@ -1,14 +1,16 @@
 // asm_sweep.cuh -- the chain kernel of blocked modes sampling (Ghanem & Koch,
 // arXiv:1912.01379, Sec. IV.B-C) for sm_103a.
 //
-// Layout.  A team of S lanes (S a power of two, S <= 32) runs one chain; a warp
-// runs 32/S chains.  While a block is visited, the team keeps the block's part
-// of the chain state f in registers: lane s holds the 16-byte vectors
-// k*S + s (k < KV) of the block.  Mode rows (V, and the masked reciprocals
-// R = -1/V that give the bounds of Eq. modeLimits) are read as 16-byte vectors
-// from a CTA-shared ring of move records; every chain of the same problem reads
-// the same rows at the same time.  The tracked residual r~ = g~ - K~ f and the block's
-// projections c_j = U_j^T r~ live in shared memory.
+// Layout.  A warp runs C chains (1, 2 or 4) of one problem.  While a block is
+// visited, the block's part of each chain's state f is in registers, spread over
+// the 32 lanes in 16-byte vectors (8-byte ones for small blocks).  Mode rows (V,
+// and the masked reciprocals R = -1/V that give the bounds of Eq. modeLimits) are
+// read as vectors from a CTA-shared ring of move records, once for the warp's C
+// chains; every chain of the same problem reads the same rows at the same time.
+// A block visit starts from its packet in shared memory (block descriptor, bounds
+// row of the first mode, U_b).  The tracked residual r~ = g~ - K~ f and the
+// block's projections c_j = U_j^T r~ live in shared memory, the chain state too
+// where it fits.
 //
 // One move of mode j (Sec. IV.B, "sample e_i' from a univariate Gaussian ...
 // truncated to the interval for which f' >= 0"):
@@ -63,29 +65,21 @@ template <> __device__ __forceinline__ float uniform_from<float>(unsigned long l
 }
 
 // --------------------------------------------------------------------------
-// precision-overloaded math (CUDA math library calls)
+// math by precision (CUDA math library calls)
 // --------------------------------------------------------------------------
 __device__ __forceinline__ double m_fma(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float m_fma(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double m_max(double a, double b) { return fmax(a, b); }
 __device__ __forceinline__ float m_max(float a, float b) { return fmaxf(a, b); }
-__device__ __forceinline__ double m_min(double a, double b) { return fmin(a, b); }
 __device__ __forceinline__ float m_min(float a, float b) { return fminf(a, b); }
-__device__ __forceinline__ double m_phi(double x) { return normcdf(x); }
 __device__ __forceinline__ float m_phi(float x) { return normcdff(x); }
-__device__ __forceinline__ double m_phiinv(double p) { return normcdfinv(p); }
 __device__ __forceinline__ float m_phiinv(float p) { return normcdfinvf(p); }
-__device__ __forceinline__ double m_erfcx(double x) { return erfcx(x); }
 __device__ __forceinline__ float m_erfcx(float x) { return erfcxf(x); }
 __device__ __forceinline__ double m_log(double x) { return log(x); }
 __device__ __forceinline__ float m_log(float x) { return logf(x); }
-__device__ __forceinline__ double m_log1p(double x) { return log1p(x); }
 __device__ __forceinline__ float m_log1p(float x) { return log1pf(x); }
-__device__ __forceinline__ double m_exp(double x) { return exp(x); }
 __device__ __forceinline__ float m_exp(float x) { return expf(x); }
-__device__ __forceinline__ double m_expm1(double x) { return expm1(x); }
 __device__ __forceinline__ float m_expm1(float x) { return expm1f(x); }
-__device__ __forceinline__ double m_abs(double x) { return fabs(x); }
 __device__ __forceinline__ float m_abs(float x) { return fabsf(x); }
 
 template <class T> struct TailTraits;
@@ -116,41 +110,39 @@ template <> struct TailTraits<float> {
 // and, below, y = -Phi^{-1}(q) - a with q = (1-u)Q(a) + uQ(b): accurate to a
 // few ulp of a, which FP32 keeps; in FP64 the offset form refines it so that y
 // keeps its relative accuracy however small it is.
-template <class T>
-__device__ __forceinline__ T right_tail(T a, T w, T u, int &capped)
+__device__ __forceinline__ float right_tail(float a, float w, float u, int &capped)
 {
-    const T b = a + w;
-    const T kRsqrt2 = T(0.70710678118654752440);
-    const T kSqrtPiOver2 = T(1.25331413731550025121);
-    constexpr bool kRefine = sizeof(T) == 8;
-    T y;
-    if (a < T(5)) {
-        const T qa = m_phi(-a);
-        const T qb = isinf(b) ? T(0) : m_phi(-b);
-        const T q = (T(1) - u) * qa + u * qb;
+    const float b = a + w;
+    const float kRsqrt2 = 0.70710678118654752440f;
+    const float kSqrtPiOver2 = 1.25331413731550025121f;
+    float y;
+    if (a < 5.0f) {
+        const float qa = m_phi(-a);
+        const float qb = isinf(b) ? 0.0f : m_phi(-b);
+        const float q = (1.0f - u) * qa + u * qb;
         y = -m_phiinv(q) - a;
     }
-    if (a >= T(5) || (kRefine && a > T(0))) {
-        const T exa = m_erfcx(a * kRsqrt2);
-        T r = T(0), em = T(-1);
+    if (a >= 5.0f) {
+        const float exa = m_erfcx(a * kRsqrt2);
+        float r = 0.0f, em = -1.0f;
         if (!isinf(b)) {
-            const T lr = m_log(m_erfcx(b * kRsqrt2) / exa) - T(0.5) * w * (a + b);
+            const float lr = m_log(m_erfcx(b * kRsqrt2) / exa) - 0.5f * w * (a + b);
             r = m_exp(lr);
             em = m_expm1(lr);
         }
-        const T dt = r < T(0.5) ? m_log((T(1) - u) + u * r) : m_log1p(u * em);
-        if (a >= T(5)) y = -dt / a;
+        const float dt = r < 0.5f ? m_log((1.0f - u) + u * r) : m_log1p(u * em);
+        y = -dt / a;
         int it = 0;
-        for (; it < TailTraits<T>::nmax; ++it) {
-            const T exy = m_erfcx((a + y) * kRsqrt2);
-            const T g = m_log(exy / exa) - y * (a + T(0.5) * y) - dt;
-            const T step = -g * exy * kSqrtPiOver2;   // g / g', g' = -sqrt(2/pi)/erfcx
+        for (; it < TailTraits<float>::nmax; ++it) {
+            const float exy = m_erfcx((a + y) * kRsqrt2);
+            const float g = m_log(exy / exa) - y * (a + 0.5f * y) - dt;
+            const float step = -g * exy * kSqrtPiOver2;   // g / g', g' = -sqrt(2/pi)/erfcx
             y -= step;
-            if (m_abs(step) <= TailTraits<T>::tol * (y + T(1) / a)) break;
+            if (m_abs(step) <= TailTraits<float>::tol * (y + 1.0f / a)) break;
         }
-        if (it == TailTraits<T>::nmax) ++capped;
+        if (it == TailTraits<float>::nmax) ++capped;
     }
-    y = m_max(y, T(0));
+    y = m_max(y, 0.0f);
     y = m_min(y, w);
     return y;
 }
@@ -184,16 +176,15 @@ template <> struct GaussLegendre<float> {
 
 // I(t) = int_0^t exp(-a s - s^2/2) ds (the CDF of N(0,1) on [a, a+w] from a,
 // unnormalised) by Gauss-Legendre; accurate while t (|a| + t) <= 1/2.
-template <class T>
-__device__ __forceinline__ T narrow_cdf(T a, T t)
+__device__ __forceinline__ float narrow_cdf(float a, float t)
 {
-    using GL = GaussLegendre<T>;
-    const T h = T(0.5) * t;
-    T acc = T(0);
+    using GL = GaussLegendre<float>;
+    const float h = 0.5f * t;
+    float acc = 0.0f;
 #pragma unroll
     for (int i = 0; i < GL::half; ++i) {
-        const T s1 = h * (T(1) - GL::x(i)), s2 = h * (T(1) + GL::x(i));
-        acc += GL::w(i) * (m_exp(-s1 * (a + T(0.5) * s1)) + m_exp(-s2 * (a + T(0.5) * s2)));
+        const float s1 = h * (1.0f - GL::x(i)), s2 = h * (1.0f + GL::x(i));
+        acc += GL::w(i) * (m_exp(-s1 * (a + 0.5f * s1)) + m_exp(-s2 * (a + 0.5f * s2)));
     }
     return h * acc;
 }
@@ -212,26 +203,25 @@ __device__ __forceinline__ T narrow_cdf(T a, T t)
 // start's, which is below w^2/12 relative, and one step leaves at most 1.5e-7
 // relative over the narrow regime with w <= 0.2 (measured against the root of
 // a 64-point rule at 4 million (a, w, u)), below the FP32 tolerance.
-template <class T>
-__device__ __forceinline__ T narrow_offset(T a, T w, T u, int &capped)
+__device__ __forceinline__ float narrow_offset(float a, float w, float u, int &capped)
 {
-    using GL = GaussLegendre<T>;
-    const T lam = a + T(0.5) * w;
-    const T x = lam * w;
-    T t = m_abs(x) < T(1e-3) ? u * w * (T(1) - T(0.5) * x * (T(1) - u))   // the series for small lam w
+    using GL = GaussLegendre<float>;
+    const float lam = a + 0.5f * w;
+    const float x = lam * w;
+    float t = m_abs(x) < 1e-3f ? u * w * (1.0f - 0.5f * x * (1.0f - u))   // the series for small lam w
                              : -m_log1p(u * m_expm1(-x)) / lam;
-    t = m_min(m_max(t, T(0)), w);
-    if (sizeof(T) == 4 && w * w <= T(4e-7)) return t;
-    const T target = u * narrow_cdf(a, w);
-    if (sizeof(T) == 4 && w <= T(0.2)) {
-        const T step = (narrow_cdf(a, t) - target) / m_exp(-t * (a + T(0.5) * t));
-        return m_min(m_max(t - step, T(0)), w);
+    t = m_min(m_max(t, 0.0f), w);
+    if (w * w <= 4e-7f) return t;
+    const float target = u * narrow_cdf(a, w);
+    if (w <= 0.2f) {
+        const float step = (narrow_cdf(a, t) - target) / m_exp(-t * (a + 0.5f * t));
+        return m_min(m_max(t - step, 0.0f), w);
     }
     int it = 0;
     for (; it < GL::nmax; ++it) {
-        const T step = (narrow_cdf(a, t) - target) / m_exp(-t * (a + T(0.5) * t));
-        t = m_min(m_max(t - step, T(0)), w);
-        if (m_abs(step) <= GL::tol * t || t == T(0)) break;
+        const float step = (narrow_cdf(a, t) - target) / m_exp(-t * (a + 0.5f * t));
+        t = m_min(m_max(t - step, 0.0f), w);
+        if (m_abs(step) <= GL::tol * t || t == 0.0f) break;
     }
     if (it == GL::nmax) ++capped;
     return t;
@@ -241,53 +231,39 @@ __device__ __forceinline__ T narrow_offset(T a, T w, T u, int &capped)
 // In standard units x = d delta - c the interval is [a, b] = [d lo - c, d hi - c].
 // Each branch returns delta in the form that keeps delta - lo (or hi - delta)
 // accurate relative to hi - lo.
-template <class T>
-__device__ __forceinline__ T tn_step(T c, T d, T invd, T lo, T hi, T u, int &capped)
+__device__ __forceinline__ float tn_step(float c, float d, float invd, float lo, float hi, float u, int &capped)
 {
-    const T a = m_fma(lo, d, -c);
-    const T b = m_fma(hi, d, -c);
-    const T wid = (hi - lo) * d;
-    T delta;
-    if (isfinite(wid) && wid * (m_abs(a) + wid) <= T(0.5)) {
+    const float a = m_fma(lo, d, -c);
+    const float b = m_fma(hi, d, -c);
+    const float wid = (hi - lo) * d;
+    float delta;
+    if (isfinite(wid) && wid * (m_abs(a) + wid) <= 0.5f) {
         delta = lo + invd * narrow_offset(a, wid, u, capped);
-    } else if (a >= T(0)) {
+    } else if (a >= 0.0f) {
         delta = lo + invd * right_tail(a, wid, u, capped);
-    } else if (b <= T(0)) {
-        delta = hi - invd * right_tail(-b, wid, T(1) - u, capped);
-    } else if (a < -TailTraits<T>::far && b > TailTraits<T>::far) {
+    } else if (b <= 0.0f) {
+        delta = hi - invd * right_tail(-b, wid, 1.0f - u, capped);
+    } else if (a < -TailTraits<float>::far && b > TailTraits<float>::far) {
         // the truncation is below the resolution of u: the untruncated inverse CDF
-        const T x = u <= T(0.5) ? m_phiinv(u) : -m_phiinv(T(1) - u);
+        const float x = u <= 0.5f ? m_phiinv(u) : -m_phiinv(1.0f - u);
         delta = (x + c) * invd;
     } else {
-        const T p = (T(1) - u) * m_phi(a) + u * m_phi(b);
-        T x;
-        if (p <= T(0.5)) {
+        const float p = (1.0f - u) * m_phi(a) + u * m_phi(b);
+        float x;
+        if (p <= 0.5f) {
             x = m_phiinv(p);
         } else {
-            x = -m_phiinv((T(1) - u) * m_phi(-a) + u * m_phi(-b));
+            x = -m_phiinv((1.0f - u) * m_phi(-a) + u * m_phi(-b));
         }
         delta = (x + c) * invd;
     }
     return m_min(m_max(delta, lo), hi);
 }
 
-// --------------------------------------------------------------------------
-// 16-byte vector loads through the read-only path
-// --------------------------------------------------------------------------
+// elements of a 16-byte vector
 template <class T> struct VecOf;
 template <> struct VecOf<float> { static constexpr int n = 4; };
 template <> struct VecOf<double> { static constexpr int n = 2; };
-
-__device__ __forceinline__ void ldv(const float *p, float (&o)[4])
-{
-    const float4 v = __ldg(reinterpret_cast<const float4 *>(p));
-    o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
-}
-__device__ __forceinline__ void ldv(const double *p, double (&o)[2])
-{
-    const double2 v = __ldg(reinterpret_cast<const double2 *>(p));
-    o[0] = v.x; o[1] = v.y;
-}
 
 // Bound keys.  With x >= +0 and R = -1/V (NaN where V is left out of the
 // bounds), t = x R is <= -0 exactly when V > 0 (a lower-bound candidate for
@@ -316,100 +292,87 @@ template <> struct BoundKey<double> {
     static __device__ __forceinline__ double lo_of(S k) { return __longlong_as_double(k); }
     static __device__ __forceinline__ double hi_of(U k) { return __longlong_as_double((long long)k); }
 };
-template <class T>
-__device__ __forceinline__ void key_update(typename BoundKey<T>::S &lk, typename BoundKey<T>::U &hk, T t)
+// max(x, +0) (NaN gives +0).  FP64 as an integer test of the high word: a DSETP
+// would occupy the FP64 pipe, which issues one warp instruction per 64 cycles and
+// sub-partition, for as long as the fused multiply-add itself.
+__device__ __forceinline__ float clamp0(float x) { return fmaxf(x, 0.0f); }
+__device__ __forceinline__ double clamp0(double x)
 {
-    const typename BoundKey<T>::S k = BoundKey<T>::bits(t);
-    lk = k < lk ? k : lk;
-    const typename BoundKey<T>::U ku = (typename BoundKey<T>::U)k;
-    hk = ku < hk ? ku : hk;
+    return (unsigned)__double2hiint(x) <= 0x7ff00000u ? x : 0.0;
 }
 
-// One 16-byte chunk of the pass: x = max(f + delta V, +0), f = x, and the keys
-// of t = x R into two accumulator pairs (even and odd element), so that the
-// chain of integer minima is half as long.  The minima are exact, so the keys
-// do not depend on the grouping.  FP32: the products and the fused
-// multiply-adds in packed pairs (one instruction per two elements, each
-// element rounded as by the scalar instruction).
+// One vector of the pass: x = max(f + delta V, +0), f = x, and the keys of t = x R.
+// The minima are exact, so the keys do not depend on the grouping.  FP32: the
+// products and the fused multiply-adds in packed pairs (one instruction per two
+// elements, each element rounded as by the scalar instruction), and three-way
+// minima (0.63 issue slots of an SM per warp instruction against 0.41 for a
+// two-way one that takes half as many elements).
 template <class T>
 struct Keys {
-    typename BoundKey<T>::S l0, l1;
-    typename BoundKey<T>::U h0, h1;
+    typename BoundKey<T>::S l;
+    typename BoundKey<T>::U h;
     __device__ __forceinline__ void reset()
     {
-        l0 = l1 = BoundKey<T>::lo0;
-        h0 = h1 = BoundKey<T>::hi0;
+        l = BoundKey<T>::lo0;
+        h = BoundKey<T>::hi0;
     }
     __device__ __forceinline__ void fold(typename BoundKey<T>::S &lk, typename BoundKey<T>::U &hk) const
     {
-        lk = l1 < l0 ? l1 : l0;
-        hk = h1 < h0 ? h1 : h0;
+        lk = l;
+        hk = h;
+    }
+    __device__ __forceinline__ void take(T t)
+    {
+        const typename BoundKey<T>::S k = BoundKey<T>::bits(t);
+        const typename BoundKey<T>::U u = (typename BoundKey<T>::U)k;
+        l = k < l ? k : l;
+        h = u < h ? u : h;
     }
 };
-__device__ __forceinline__ void pass_chunk(float (&f)[4], float delta, const float (&vv)[4], const float (&rr)[4],
+__device__ __forceinline__ void take2(Keys<float> &kk, float2 t)
+{
+    const int a = __float_as_int(t.x), b = __float_as_int(t.y);
+    kk.l = __vimin3_s32(kk.l, a, b);
+    kk.h = __vimin3_u32(kk.h, (unsigned)a, (unsigned)b);
+}
+template <int VE>
+__device__ __forceinline__ void pass_chunk(float (&f)[VE], float delta, const float (&vv)[VE], const float (&rr)[VE],
                                            Keys<float> &kk)
 {
     const float2 d2 = make_float2(delta, delta);
-    float2 a = __ffma2_rn(d2, make_float2(vv[0], vv[1]), make_float2(f[0], f[1]));
-    float2 b = __ffma2_rn(d2, make_float2(vv[2], vv[3]), make_float2(f[2], f[3]));
-    a.x = fmaxf(a.x, 0.0f);
-    a.y = fmaxf(a.y, 0.0f);
-    b.x = fmaxf(b.x, 0.0f);
-    b.y = fmaxf(b.y, 0.0f);
-    f[0] = a.x; f[1] = a.y; f[2] = b.x; f[3] = b.y;
-    const float2 ta = __fmul2_rn(a, make_float2(rr[0], rr[1]));
-    const float2 tb = __fmul2_rn(b, make_float2(rr[2], rr[3]));
-    key_update<float>(kk.l0, kk.h0, ta.x);
-    key_update<float>(kk.l1, kk.h1, ta.y);
-    key_update<float>(kk.l0, kk.h0, tb.x);
-    key_update<float>(kk.l1, kk.h1, tb.y);
+#pragma unroll
+    for (int v = 0; v < VE; v += 2) {
+        float2 a = __ffma2_rn(d2, make_float2(vv[v], vv[v + 1]), make_float2(f[v], f[v + 1]));
+        a.x = clamp0(a.x);
+        a.y = clamp0(a.y);
+        f[v] = a.x;
+        f[v + 1] = a.y;
+        take2(kk, __fmul2_rn(a, make_float2(rr[v], rr[v + 1])));
+    }
 }
-__device__ __forceinline__ void pass_chunk(double (&f)[2], double delta, const double (&vv)[2],
-                                           const double (&rr)[2], Keys<double> &kk)
+template <int VE>
+__device__ __forceinline__ void pass_chunk(double (&f)[VE], double delta, const double (&vv)[VE], const double (&rr)[VE],
+                                           Keys<double> &kk)
 {
-    double x0 = fmax(fma(delta, vv[0], f[0]), 0.0);
-    double x1 = fmax(fma(delta, vv[1], f[1]), 0.0);
-    f[0] = x0;
-    f[1] = x1;
-    key_update<double>(kk.l0, kk.h0, x0 * rr[0]);
-    key_update<double>(kk.l1, kk.h1, x1 * rr[1]);
+#pragma unroll
+    for (int v = 0; v < VE; ++v) {
+        f[v] = clamp0(fma(delta, vv[v], f[v]));
+        kk.take(f[v] * rr[v]);
+    }
 }
 // Keys alone (the first mode of a block: f is unchanged, t = f R).
-__device__ __forceinline__ void key_chunk(const float (&f)[4], const float (&rr)[4], Keys<float> &kk)
+template <int VE>
+__device__ __forceinline__ void key_chunk(const float (&f)[VE], const float (&rr)[VE], Keys<float> &kk)
 {
-    const float2 ta = __fmul2_rn(make_float2(f[0], f[1]), make_float2(rr[0], rr[1]));
-    const float2 tb = __fmul2_rn(make_float2(f[2], f[3]), make_float2(rr[2], rr[3]));
-    key_update<float>(kk.l0, kk.h0, ta.x);
-    key_update<float>(kk.l1, kk.h1, ta.y);
-    key_update<float>(kk.l0, kk.h0, tb.x);
-    key_update<float>(kk.l1, kk.h1, tb.y);
-}
-__device__ __forceinline__ void key_chunk(const double (&f)[2], const double (&rr)[2], Keys<double> &kk)
-{
-    key_update<double>(kk.l0, kk.h0, f[0] * rr[0]);
-    key_update<double>(kk.l1, kk.h1, f[1] * rr[1]);
-}
-
-// The lane's bound keys of a block's first mode from f (>= +0, so that
-// max(f + 0 V, +0) = f and the pass reduces to the products) and that mode's R
-// row, read from global memory.
-template <class T, int KV>
-__device__ __forceinline__ void first_keys(const T (&f)[KV][VecOf<T>::n], const T *__restrict__ rrow, int kcnt,
-                                           int sl, int S, typename BoundKey<T>::S &lk,
-                                           typename BoundKey<T>::U &hk)
-{
-    constexpr int VEC = VecOf<T>::n;
-    Keys<T> kk;
-    kk.reset();
 #pragma unroll
-    for (int k = 0; k < KV; ++k) {
-        if (k < kcnt) {
-            T rr[VEC];
-            ldv(rrow + VEC * (k * S + sl), rr);
-            key_chunk(f[k], rr, kk);
-        }
-    }
-    kk.fold(lk, hk);
+    for (int v = 0; v < VE; v += 2)
+        take2(kk, __fmul2_rn(make_float2(f[v], f[v + 1]), make_float2(rr[v], rr[v + 1])));
+}
+template <int VE>
+__device__ __forceinline__ void key_chunk(const double (&f)[VE], const double (&rr)[VE], Keys<double> &kk)
+{
+#pragma unroll
+    for (int v = 0; v < VE; ++v) kk.take(f[v] * rr[v]);
 }
 
 // --------------------------------------------------------------------------
@@ -459,13 +422,6 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long *bar, unsigned pari
         if (mbar_try_wait(bar, parity)) return true;
     return false;
 }
-// Consumer-side wait: a non-blocking test first (the record has usually
-// landed long before it is needed), then the suspending wait, bounded.
-__device__ __forceinline__ bool mbar_wait_ready(unsigned long long *bar, unsigned parity, int limit)
-{
-    if (mbar_test_wait(bar, parity)) return true;
-    return mbar_wait(bar, parity, limit);
-}
 __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned bytes, unsigned long long *bar)
 {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
@@ -482,80 +438,287 @@ __device__ __forceinline__ void fence_mbar_init()
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 
-
-// Team-wide bounds from the lanes' keys: signed and unsigned integer minima
-// (FP32: one redux instruction each; FP64: a butterfly of shuffles).
-__device__ __forceinline__ void team_bounds(int lk, unsigned hk, float &lo, float &hi, int S, int team_base)
+// The warp's bounds from the lanes' keys: signed and unsigned integer minima,
+// one redux instruction each (24 cycles, 26 for a pair in flight; with half-warp
+// masks 168, which is why a chain always spans the warp).  FP64: the minimum of
+// the high words, then of the low words of the lanes that hold it (a butterfly
+// of 64-bit shuffles took five dependent steps of ~45 cycles).
+template <int C>
+__device__ __forceinline__ void warp_bounds(const int (&lk)[C], const unsigned (&hk)[C], float (&lo)[C], float (&hi)[C])
 {
-    const unsigned mask = S == 32 ? 0xffffffffu : (((1u << S) - 1u) << team_base);
-    lo = __int_as_float(__reduce_min_sync(mask, lk));
-    hi = __uint_as_float(__reduce_min_sync(mask, hk));
-}
-__device__ __forceinline__ void team_bounds(long long lk, unsigned long long hk, double &lo, double &hi, int S, int)
-{
-    for (int off = 1; off < S; off <<= 1) {
-        const long long l2 = __shfl_xor_sync(0xffffffffu, lk, off);
-        const unsigned long long h2 = __shfl_xor_sync(0xffffffffu, hk, off);
-        lk = l2 < lk ? l2 : lk;
-        hk = h2 < hk ? h2 : hk;
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+        lo[c] = __int_as_float(__reduce_min_sync(0xffffffffu, lk[c]));
+        hi[c] = __uint_as_float(__reduce_min_sync(0xffffffffu, hk[c]));
     }
-    lo = __longlong_as_double(lk);
-    hi = __longlong_as_double((long long)hk);
+}
+template <int C>
+__device__ __forceinline__ void warp_bounds(const long long (&lk)[C], const unsigned long long (&hk)[C], double (&lo)[C],
+                                            double (&hi)[C])
+{
+    int lh[C];
+    unsigned hh[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+        lh[c] = __reduce_min_sync(0xffffffffu, (int)(lk[c] >> 32));
+        hh[c] = __reduce_min_sync(0xffffffffu, (unsigned)(hk[c] >> 32));
+    }
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+        const unsigned ll = __reduce_min_sync(0xffffffffu, (int)(lk[c] >> 32) == lh[c] ? (unsigned)lk[c] : 0xffffffffu);
+        const unsigned hl =
+            __reduce_min_sync(0xffffffffu, (unsigned)(hk[c] >> 32) == hh[c] ? (unsigned)hk[c] : 0xffffffffu);
+        lo[c] = __hiloint2double(lh[c], (int)ll);
+        hi[c] = __hiloint2double((int)hh[c], (int)hl);
+    }
 }
 
-// 16-byte vector loads from shared memory
+// lo < hi for bounds that come from keys: lo is -0 or below, hi +0 or above, neither
+// is NaN, so they differ unless both are zeros.  FP64 as an integer test: a DSETP would
+// occupy the FP64 pipe for 64 cycles.
+__device__ __forceinline__ bool open_interval(float lo, float hi) { return hi > lo; }
+__device__ __forceinline__ bool open_interval(double lo, double hi)
+{
+    return ((__double_as_longlong(lo) | __double_as_longlong(hi)) << 1) != 0;
+}
+__device__ __forceinline__ bool is_zero(float x) { return x == 0.0f; }
+__device__ __forceinline__ bool is_zero(double x) { return (__double_as_longlong(x) << 1) == 0; }
+__device__ __forceinline__ bool is_finite(float x) { return isfinite(x); }
+__device__ __forceinline__ bool is_finite(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+
+// vector loads from shared memory: VE elements, naturally aligned
 __device__ __forceinline__ void lds_v(const float *p, float (&o)[4])
 {
     const float4 v = *reinterpret_cast<const float4 *>(p);
     o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
+}
+__device__ __forceinline__ void lds_v(const float *p, float (&o)[2])
+{
+    const float2 v = *reinterpret_cast<const float2 *>(p);
+    o[0] = v.x; o[1] = v.y;
 }
 __device__ __forceinline__ void lds_v(const double *p, double (&o)[2])
 {
     const double2 v = *reinterpret_cast<const double2 *>(p);
     o[0] = v.x; o[1] = v.y;
 }
+__device__ __forceinline__ void lds_v(const double *p, double (&o)[1]) { o[0] = *p; }
 
-// f += delta * V (clamped at +0) and the lane's bound keys of the next mode,
-// rows read from a shared-memory stage.
-// The caller loads chunk 0 (v0, r0) ahead of the draw; kcnt >= 1.  The pass
-// covers chunks 0 .. KK-1; with CHK each is tested against kcnt, without it
-// all KK are present (kcnt == KK), so the loop has no branch.
-template <class T, int KV, int KK = KV, bool CHK = true>
-__device__ __forceinline__ void fused_pass_smem(T (&f)[KV][VecOf<T>::n], T delta, const T (&v0)[VecOf<T>::n],
-                                                const T (&r0)[VecOf<T>::n], const T *vrow, const T *rrow,
-                                                int kcnt, int sl, int S, typename BoundKey<T>::S &lk,
-                                                typename BoundKey<T>::U &hk)
+// The mode data of a record: d_j, 1/d_j, dres_j.
+__device__ __forceinline__ void lds_mode(const float *p, float &d, float &invd, float &dres)
 {
-    constexpr int VEC = VecOf<T>::n;
-    static_assert(KK >= 1 && KK <= KV, "chunk count");
-    Keys<T> kk;
-    kk.reset();
-#pragma unroll
-    for (int k = 0; k < KK; ++k) {
-        if (!CHK || k < kcnt) {
-            const int idx = VEC * (k * S + sl);
-            if (k == 0) {
-                pass_chunk(f[0], delta, v0, r0, kk);
-            } else {
-                T vv[VEC], rr[VEC];
-                lds_v(vrow + idx, vv);
-                lds_v(rrow + idx, rr);
-                pass_chunk(f[k], delta, vv, rr, kk);
-            }
-        }
-    }
-    kk.fold(lk, hk);
+    const float4 v = *reinterpret_cast<const float4 *>(p);
+    d = v.x; invd = v.y; dres = v.z;
+}
+__device__ __forceinline__ void lds_mode(const double *p, double &d, double &invd, double &dres)
+{
+    const double2 v = *reinterpret_cast<const double2 *>(p);
+    d = v.x; invd = v.y;
+    dres = p[2];
 }
 
 // --------------------------------------------------------------------------
-// Position in the stream of moves of a launch (sweep, level, block, mode).
+// The draw by a team of lanes.  A warp holds C chains; every lane of the G = 32/C
+// lanes of a chain's team has the same arguments.
+//
+// FP32: each lane draws for its team's chain, so C draws cost one.
+//
+// FP64: one warp instruction of the FP64 pipe takes 64 cycles of a sub-partition
+// whether one lane is active or all are, so the draw's independent function
+// values go to different lanes: the eight exponentials of the quadrature (and,
+// where the team is wide enough, those of the target's quadrature and of the
+// density that Newton's step divides by) are one exponential, and the pairs
+// Phi(a), Phi(b) and erfcx(a), erfcx(b) one call each.  Sums are formed from
+// the lanes' values in the order of the scalar code, so the draw is the same
+// bit for bit.
 // --------------------------------------------------------------------------
-struct MoveCursor {
+template <int G>
+__device__ __forceinline__ float tn_step_team(float c, float d, float invd, float lo, float hi, float u, bool open,
+                                              int, int &capped)
+{
+    return open ? tn_step(c, d, invd, lo, hi, u, capped) : 0.0f;
+}
+
+template <int G>
+struct TeamLanes {
+    unsigned mask;   // lanes of the warp that run this path (whole teams)
+    int base, gl;    // first lane of the team, lane within the team
+    __device__ __forceinline__ double from(double v, int l) const { return __shfl_sync(mask, v, base + l); }
+};
+
+// 1 - x or 1 + x of the quadrature node of a lane: lanes 2i, 2i + 1 of eight take node i.
+__device__ __forceinline__ double gl_node(int lane)
+{
+    using GL = GaussLegendre<double>;
+    const int i = (lane >> 1) & 3;
+    const double lo = i == 0 ? 1.0 - GL::x(0) : i == 1 ? 1.0 - GL::x(1) : i == 2 ? 1.0 - GL::x(2) : 1.0 - GL::x(3);
+    const double hi = i == 0 ? 1.0 + GL::x(0) : i == 1 ? 1.0 + GL::x(1) : i == 2 ? 1.0 + GL::x(2) : 1.0 + GL::x(3);
+    return (lane & 1) ? hi : lo;
+}
+
+// sum_i w_i (e_{2i} + e_{2i+1}) from the exponentials held by lanes first .. first + 7 of the team.
+template <int G>
+__device__ __forceinline__ double gl_sum(const TeamLanes<G> &tl, double e, int first)
+{
+    using GL = GaussLegendre<double>;
+    const double pair = e + __shfl_xor_sync(tl.mask, e, 1);
+    double acc = 0.0;
+#pragma unroll
+    for (int i = 0; i < GL::half; ++i) acc = fma(GL::w(i), tl.from(pair, first + 2 * i), acc);
+    return acc;
+}
+
+template <int G>
+__device__ __forceinline__ double narrow_offset_team(double a, double w, double u, const TeamLanes<G> &tl, int &capped)
+{
+    using GL = GaussLegendre<double>;
+    const double lam = a + 0.5 * w;
+    const double x = lam * w;
+    double t = fabs(x) < 1e-3 ? u * w * (1.0 - 0.5 * x * (1.0 - u)) : -log1p(u * expm1(-x)) / lam;
+    t = fmin(fmax(t, 0.0), w);
+    const double node = gl_node(tl.gl);
+    double target = 0.0;
+    bool live = true;
+    for (int it = 0; it < GL::nmax; ++it) {
+        // lanes 0-7: the nodes of I(t); lane 8 (teams of 16 and 32): the density at t;
+        // the first time also I(w) for the target, on lanes 16-23 of a team of 32
+        double acc, den;   // I(t) = t/2 acc
+        if (G == 32) {
+            const bool at_w = it == 0 && (tl.gl & 16);
+            const double h = 0.5 * (at_w ? w : t);
+            const double s = tl.gl == 8 ? t : h * node;
+            const double e = exp(-s * fma(0.5, s, a));
+            if (it == 0) target = __dmul_rn(u, __dmul_rn(0.5 * w, gl_sum<G>(tl, e, 16)));
+            den = tl.from(e, 8);
+            acc = gl_sum<G>(tl, e, 0);
+        } else {
+            if (it == 0) {
+                const double s = 0.5 * w * node;
+                target = __dmul_rn(u, __dmul_rn(0.5 * w, gl_sum<G>(tl, exp(-s * fma(0.5, s, a)), 0)));
+            }
+            const double s = G > 8 && tl.gl == 8 ? t : 0.5 * t * node;
+            const double e = exp(-s * fma(0.5, s, a));
+            den = G > 8 ? tl.from(e, G > 8 ? 8 : 0) : exp(-t * fma(0.5, t, a));
+            acc = gl_sum<G>(tl, e, 0);
+        }
+        if (live) {
+            const double step = (__dmul_rn(0.5 * t, acc) - target) / den;
+            t = fmin(fmax(t - step, 0.0), w);
+            if (fabs(step) <= GL::tol * t || t == 0.0) live = false;
+        }
+        if (!__any_sync(tl.mask, live)) break;
+    }
+    if (live) ++capped;
+    return t;
+}
+
+// f(x0) and f(x1) from one call: the even lanes take x0, the odd ones x1.
+template <int G, class F>
+__device__ __forceinline__ void pair_of(F f, double x0, double x1, const TeamLanes<G> &tl, double &y0, double &y1)
+{
+    const double y = f((tl.gl & 1) ? x1 : x0);
+    y0 = tl.from(y, 0);
+    y1 = tl.from(y, 1);
+}
+
+template <int G>
+__device__ __forceinline__ double right_tail_team(double a, double w, double u, TeamLanes<G> tl, int &capped)
+{
+    const double b = a + w;
+    const double kRsqrt2 = 0.70710678118654752440;
+    const double kSqrtPiOver2 = 1.25331413731550025121;
+    double y = 0.0;
+    const unsigned all = tl.mask, near = __ballot_sync(all, a < 5.0), refine = __ballot_sync(all, a > 0.0);
+    if (a < 5.0) {
+        double qa, qb;
+        tl.mask = near;
+        pair_of<G>([](double z) { return normcdf(z); }, -a, -b, tl, qa, qb);
+        if (isinf(b)) qb = 0.0;
+        const double q = (1.0 - u) * qa + u * qb;
+        y = -normcdfinv(q) - a;
+    }
+    if (a > 0.0) {
+        double exa, exb;
+        tl.mask = refine;
+        pair_of<G>([](double z) { return erfcx(z); }, a * kRsqrt2, b * kRsqrt2, tl, exa, exb);
+        double r = 0.0, lr = 0.0;
+        if (!isinf(b)) {
+            lr = log(exb / exa) - 0.5 * w * (a + b);
+            r = exp(lr);
+        }
+        const double dt = r < 0.5 ? log((1.0 - u) + u * r) : log1p(u * expm1(lr));
+        if (a >= 5.0) y = -dt / a;
+        int it = 0;
+        for (; it < TailTraits<double>::nmax; ++it) {
+            const double exy = erfcx((a + y) * kRsqrt2);
+            const double g = log(exy / exa) - y * (a + 0.5 * y) - dt;
+            const double step = -g * exy * kSqrtPiOver2;   // g / g', g' = -sqrt(2/pi)/erfcx
+            y -= step;
+            if (fabs(step) <= TailTraits<double>::tol * (y + 1.0 / a)) break;
+        }
+        if (it == TailTraits<double>::nmax) ++capped;
+    }
+    y = fmax(y, 0.0);
+    y = fmin(y, w);
+    return y;
+}
+
+// tn_step for the chains of a warp, FP64 (called by the whole warp; teams whose
+// interval is not open return 0).
+template <int G>
+__device__ __forceinline__ double tn_step_team(double c, double d, double invd, double lo, double hi, double u, bool open,
+                                               int lane, int &capped)
+{
+    TeamLanes<G> tl;
+    tl.base = lane & ~(G - 1);
+    tl.gl = lane & (G - 1);
+    const double a = fma(lo, d, -c);
+    const double b = fma(hi, d, -c);
+    const double wid = (hi - lo) * d;
+    const bool narrow = open && is_finite(wid) && wid * (fabs(a) + wid) <= 0.5;
+    const bool right = open && !narrow && a >= 0.0;
+    const bool left = open && !narrow && !right && b <= 0.0;
+    const bool middle = open && !narrow && !right && !left;
+    const bool untruncated = middle && a < -TailTraits<double>::far && b > TailTraits<double>::far;
+    double delta = 0.0;
+    const unsigned mn = __ballot_sync(0xffffffffu, narrow), mt = __ballot_sync(0xffffffffu, right || left),
+                   mc = __ballot_sync(0xffffffffu, middle && !untruncated);
+    if (narrow) {
+        tl.mask = mn;
+        delta = lo + invd * narrow_offset_team<G>(a, wid, u, tl, capped);
+    } else if (right || left) {
+        tl.mask = mt;
+        const double y = right_tail_team<G>(right ? a : -b, wid, right ? u : 1.0 - u, tl, capped);
+        delta = right ? lo + invd * y : hi - invd * y;
+    } else if (untruncated) {
+        // the truncation is below the resolution of u: the untruncated inverse CDF
+        const double x = u <= 0.5 ? normcdfinv(u) : -normcdfinv(1.0 - u);
+        delta = (x + c) * invd;
+    } else if (middle) {
+        double pa, pb, x;
+        tl.mask = mc;
+        pair_of<G>([](double z) { return normcdf(z); }, a, b, tl, pa, pb);
+        const double p = fma(1.0 - u, pa, __dmul_rn(u, pb));
+        tl.mask = __ballot_sync(mc, p > 0.5);
+        if (p > 0.5) {
+            double na, nb;
+            pair_of<G>([](double z) { return normcdf(z); }, -a, -b, tl, na, nb);
+            x = -normcdfinv(fma(u, nb, __dmul_rn(1.0 - u, na)));
+        } else {
+            x = normcdfinv(p);
+        }
+        delta = (x + c) * invd;
+    }
+    return open ? fmin(fmax(delta, lo), hi) : 0.0;
+}
+
+// --------------------------------------------------------------------------
+// Position in the stream of blocks and moves of a launch (sweep, level, block).
+// --------------------------------------------------------------------------
+struct BlockCursor {
     long long s, s_end;     // sweep, end of the launch's range
-    int bi, j;              // block within the level, mode within the block
-    int nb;                 // blocks of the level
+    int bi, nb;             // block within the level, blocks of the level
     const BlockDesc *bd;    // blocks of the level
-    BlockDesc B;            // the current block (a copy)
     bool done;
 };
 
@@ -564,26 +727,16 @@ struct SweepRange {
     long long sweep0, nsweeps, burn_in;
 };
 
-// A warp's position in the record ring: records seen (g), stage and phase
-// (kept incrementally: no division per move).
+// A warp's position in the record ring and in the ring of visit packets (kept
+// incrementally: no division per move).
 struct RingPos {
-    unsigned g;             // stages in this launch (< 2^32: one launch is at most 64 sweeps)
+    unsigned g;             // record stages so far in this launch
     int slot;
     unsigned phase;
-    unsigned ug;            // block visits whose U went through the two U stages
+    unsigned pg;            // visit packets so far
+    int pslot;
+    unsigned pphase;
 };
-
-// Bytes of block B's U in its staging layout, and whether it goes through the U stages.
-template <class T>
-__device__ __forceinline__ unsigned u_stage_bytes(const BlockDesc &B)
-{
-    return (unsigned)((((size_t)B.np * B.usr * sizeof(T)) + 15) / 16 * 16);
-}
-template <class T>
-__device__ __forceinline__ bool u_staged(const LaunchShape &sh, const BlockDesc &B)
-{
-    return sh.ubytes > 0 && u_stage_bytes<T>(B) <= (unsigned)sh.ubytes;
-}
 
 __device__ __forceinline__ void ring_next(RingPos &r, int depth)
 {
@@ -592,6 +745,33 @@ __device__ __forceinline__ void ring_next(RingPos &r, int depth)
         r.slot = 0;
         r.phase ^= 1u;
     }
+}
+__device__ __forceinline__ void packet_next(RingPos &r, int slots)
+{
+    ++r.pg;
+    if (++r.pslot == slots) {
+        r.pslot = 0;
+        r.pphase ^= 1u;
+    }
+}
+
+// Bytes of a block's visit packet: header and first bounds row alone, or with U where it fits a slot.
+template <class T>
+__device__ __forceinline__ unsigned packet_bytes(const LaunchShape &sh, const BlockDesc &B)
+{
+    const unsigned whole = (unsigned)((kPacketHeader + B.rs + (long long)B.np * B.usr) * (long long)sizeof(T) + 15) & ~15u;
+    return whole <= (unsigned)sh.pbytes ? whole : (unsigned)((kPacketHeader + B.rs) * sizeof(T));
+}
+template <class T>
+__device__ __forceinline__ bool u_staged(const LaunchShape &sh, const BlockDesc &B)
+{
+    return packet_bytes<T>(sh, B) > (unsigned)((kPacketHeader + B.rs) * sizeof(T));
+}
+// Records of a block per ring stage.
+template <class T>
+__device__ __forceinline__ int records_per_stage(const LaunchShape &sh, const BlockDesc &B)
+{
+    return min(kMaxRecordsPerStage, sh.stage_bytes / (int)(B.recstride * sizeof(T)));
 }
 
 __device__ __forceinline__ int level_of_sweep(long long s, unsigned long long seed, unsigned long long pid,
@@ -604,25 +784,18 @@ __device__ __forceinline__ int level_of_sweep(long long s, unsigned long long se
 }
 
 template <class T>
-__device__ __forceinline__ void cursor_start_sweep(MoveCursor &c, const SweepParams<T> &p)
+__device__ __forceinline__ void cursor_start_sweep(BlockCursor &c, const SweepParams<T> &p)
 {
     const int level = level_of_sweep(c.s, p.seed, p.problem_id, p.n_levels);
     c.nb = p.level_nblocks[level];
     c.bd = p.blocks + p.level_first[level];
     c.bi = 0;
-    c.j = 0;
-    c.B = c.bd[0];
 }
 
 template <class T>
-__device__ __forceinline__ void cursor_advance(MoveCursor &c, const SweepParams<T> &p, int n = 1)
+__device__ __forceinline__ void cursor_advance(BlockCursor &c, const SweepParams<T> &p)
 {
-    if ((c.j += n) < c.B.n) return;
-    c.j = 0;
-    if (++c.bi < c.nb) {
-        c.B = c.bd[c.bi];
-        return;
-    }
+    if (++c.bi < c.nb) return;
     if (++c.s >= c.s_end) {
         c.done = true;
         return;
@@ -630,10 +803,6 @@ __device__ __forceinline__ void cursor_advance(MoveCursor &c, const SweepParams<
     cursor_start_sweep(c, p);
 }
 
-__device__ __forceinline__ void mbar_arrive(unsigned long long *bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
-}
 // Arrival by lane 0 of the warp only, as a predicated instruction (no branch).
 __device__ __forceinline__ void mbar_arrive_lane0(unsigned long long *bar, int lane)
 {
@@ -644,100 +813,628 @@ __device__ __forceinline__ void mbar_arrive_lane0(unsigned long long *bar, int l
         "r"(lane)
         : "memory");
 }
+// Wait of a whole warp: true once the phase has completed, decided warp-wide.
+__device__ __forceinline__ bool warp_wait(unsigned long long *bar, unsigned parity, int limit)
+{
+    bool ok = mbar_test_wait(bar, parity);
+    if (__any_sync(0xffffffffu, !ok)) {
+        ok = ok || mbar_wait(bar, parity, limit);
+        if (__any_sync(0xffffffffu, !ok)) return false;
+    }
+    return true;
+}
+
+// Shared-memory regions of a CTA.
+struct Regions {
+    unsigned long long *full, *empty, *pfull, *pempty;
+    unsigned char *stages, *packets;
+};
 
 // --------------------------------------------------------------------------
-// The producer warp: one bulk copy per stage of up to sh.rps consecutive move
-// records of one block into the ring, after every consumer warp has released
-// the slot's previous stage.  The ring position runs on across the CTA's items.
+// The producer warp.  Per block visit one bulk copy of the visit packet (block
+// descriptor, bounds row of the first mode, U where it fits) into the next
+// packet slot, then the block's move records, as many to a ring stage as fit,
+// one bulk copy per stage; each after every consumer warp has released the
+// slot's previous contents.  The ring positions run on across the CTA's items.
 // --------------------------------------------------------------------------
 template <class T>
 __device__ __forceinline__ void produce(const SweepParams<T> &p, const LaunchShape &sh, const SweepRange &rg,
-                                        unsigned long long *full, unsigned long long *empty,
-                                        unsigned char *stages, unsigned long long *ufull, unsigned long long *uempty,
-                                        unsigned char *ubuf, RingPos &rp, bool &failed)
+                                        const Regions &R, RingPos &rp, bool &failed)
 {
     if ((threadIdx.x & 31) != 0 || rg.nsweeps <= 0 || failed || sh.stall) return;
-    const int D = sh.depth;
-    MoveCursor c;
+    const int D = sh.depth, P = sh.pslots;
+    BlockCursor c;
     c.s = rg.sweep0;
     c.s_end = rg.sweep0 + rg.nsweeps;
     c.done = false;
     cursor_start_sweep(c, p);
-    const unsigned g0 = rp.g, ug0 = rp.ug;
-    while (!c.done) {
-        // a block visit starts: its U into the next U stage (after that stage's previous
-        // U has been released by every consumer warp)
-        if (c.j == 0 && u_staged<T>(sh, c.B)) {
-            const unsigned us = rp.ug & 1u;
-            if (rp.ug >= 2u && !mbar_wait(uempty + us, ((rp.ug >> 1) & 1u) ^ 1u, sh.wait_limit)) {
-                failed = true;
-                break;
-            }
-            const unsigned ubytes = u_stage_bytes<T>(c.B);
-            mbar_expect_tx(ufull + us, ubytes);
-            bulk_g2s(ubuf + (size_t)us * sh.ubytes, p.pd.Us + c.B.offUs, ubytes, ufull + us);
-            ++rp.ug;
-        }
-        // the slot's previous stage (phase ^ 1) must have been released
-        if (rp.g >= (unsigned)D && !mbar_wait(empty + rp.slot, rp.phase ^ 1u, sh.wait_limit)) {
+    const unsigned g0 = rp.g, pg0 = rp.pg;
+    BlockDesc next = c.bd[c.bi];
+    bool done = false;
+    while (!done && !failed) {
+        const BlockDesc B = next;
+        cursor_advance(c, p);
+        if (!c.done) next = c.bd[c.bi];   // in flight while this block's copies are issued
+        if (rp.pg >= (unsigned)P && !mbar_wait(R.pempty + rp.pslot, rp.pphase ^ 1u, sh.wait_limit)) {
             failed = true;
             break;
         }
-        const int nrec = min(sh.rps, c.B.n - c.j);   // records of this stage (a stage stays in its block)
-        const unsigned bytes = (unsigned)(nrec * c.B.recstride * sizeof(T));
-        mbar_expect_tx(full + rp.slot, bytes);
-        bulk_g2s(stages + (size_t)rp.slot * sh.stage_bytes, p.pd.rec + c.B.offRec + (size_t)c.j * c.B.recstride,
-                 bytes, full + rp.slot);
-        ring_next(rp, D);
-        cursor_advance(c, p, nrec);
+        const unsigned pbytes = packet_bytes<T>(sh, B);
+        mbar_expect_tx(R.pfull + rp.pslot, pbytes);
+        bulk_g2s(R.packets + (size_t)rp.pslot * sh.pbytes, p.pd.pk + B.offPk, pbytes, R.pfull + rp.pslot);
+        packet_next(rp, P);
+        const int rps = records_per_stage<T>(sh, B);
+        for (int j = 0; j < B.n; j += rps) {
+            if (rp.g >= (unsigned)D && !mbar_wait(R.empty + rp.slot, rp.phase ^ 1u, sh.wait_limit)) {
+                failed = true;
+                break;
+            }
+            const unsigned bytes = (unsigned)(min(rps, B.n - j) * B.recstride * sizeof(T));
+            mbar_expect_tx(R.full + rp.slot, bytes);
+            bulk_g2s(R.stages + (size_t)rp.slot * sh.stage_bytes, p.pd.rec + B.offRec + (size_t)j * B.recstride, bytes,
+                     R.full + rp.slot);
+            ring_next(rp, D);
+        }
+        done = c.done;
     }
     if (failed) {
         // the copies already issued must land before the CTA may exit
-        const unsigned g = rp.g;
-        const unsigned from = g > g0 + (unsigned)D ? g - D : g0;
-        for (unsigned k = from; k < g; ++k)
-            mbar_wait(full + (k % (unsigned)D), (k / (unsigned)D) & 1u, sh.wait_limit);
-        const unsigned ufrom = rp.ug > ug0 + 2u ? rp.ug - 2u : ug0;
-        for (unsigned k = ufrom; k < rp.ug; ++k) mbar_wait(ufull + (k & 1u), (k >> 1) & 1u, sh.wait_limit);
+        const unsigned from = rp.g > g0 + (unsigned)D ? rp.g - D : g0;
+        for (unsigned k = from; k < rp.g; ++k)
+            mbar_wait(R.full + (k % (unsigned)D), (k / (unsigned)D) & 1u, sh.wait_limit);
+        const unsigned pfrom = rp.pg > pg0 + (unsigned)P ? rp.pg - P : pg0;
+        for (unsigned k = pfrom; k < rp.pg; ++k)
+            mbar_wait(R.pfull + (k % (unsigned)P), (k / (unsigned)P) & 1u, sh.wait_limit);
         atomicAdd(&p.counters->timeouts, 1ull);
     }
 }
 
+// The C chains of a consumer warp: shared memory and state of each.
+template <class T, int C>
+struct WarpChains {
+    long long q[C];        // local chain (idle ones shadow the last chain and write nothing)
+    bool active[C];
+    T *sm;                 // chain 0's shared memory; chain c at sm + c * team_words
+    int tw;
+    int off_w, off_r, off_u, off_f, off_p;   // words: c at 0, w, r~, uniforms, f, sums
+    __device__ __forceinline__ T *c_(int c) const { return sm + (size_t)c * tw; }
+    __device__ __forceinline__ T *w_(int c) const { return c_(c) + off_w; }
+    __device__ __forceinline__ T *r_(int c) const { return c_(c) + off_r; }
+    __device__ __forceinline__ T *u_(int c) const { return c_(c) + off_u; }
+};
+
+// Move counts of a warp's chains in one launch (at most 64 sweeps).
+template <int C>
+struct MoveCounts {
+    unsigned deg[C], zero[C], bad[C], rej[C];
+    int capped;
+};
+
+// c = U_b^T r~ for the warp's chains: partial sum i of eight takes the terms m = i mod 8
+// in increasing m, the rest goes to sum 0, then a fixed tree; so the sums are the same from
+// shared or global memory, for any C.  Blocks of up to eight modes spread the eight
+// partial sums over lanes (four modes at a time): with a lane per mode most lanes idle.
+template <class T, int C, int KVC, bool WIDE>
+__device__ __forceinline__ void project_entry(const WarpChains<T, C> &wc, const T *Us, const T *Um, int np, int usr, int M,
+                                              int lane)
+{
+    constexpr int VEC = VecOf<T>::n;
+    if (Us && np <= 8) {
+        const int i = lane & 7;
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const T *r = wc.r_(c);
+            for (int j0 = 0; j0 < np; j0 += 4) {
+                const int j = j0 + (lane >> 3);
+                const T *u = Us + (size_t)min(j, np - 1) * usr;
+                T a = T(0);
+                int m = 0;
+#pragma unroll 4
+                for (; m + 7 < M; m += 8) a = m_fma(u[m + i], r[m + i], a);
+                if (i == 0)
+                    for (; m < M; ++m) a = m_fma(u[m], r[m], a);
+                a += __shfl_xor_sync(0xffffffffu, a, 1);
+                a += __shfl_xor_sync(0xffffffffu, a, 2);
+                a += __shfl_xor_sync(0xffffffffu, a, 4);
+                if (i == 0 && j < np) wc.c_(c)[j] = a;
+            }
+        }
+        return;
+    }
+    if (Us) {
+        constexpr int JJ = C == 1 ? 2 : 1;   // modes of a lane at a time
+        for (int j = lane; j < np; j += 32 * JJ) {
+            T a[C * JJ][8];
+#pragma unroll
+            for (int x = 0; x < C * JJ; ++x)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) a[x][i] = T(0);
+            const T *u[JJ];
+#pragma unroll
+            for (int x = 0; x < JJ; ++x) u[x] = Us + (size_t)(j + 32 * x < np ? j + 32 * x : j) * usr;
+            int m = 0;
+            for (; m + 7 < M; m += 8) {
+#pragma unroll
+                for (int v = 0; v < 8; v += VEC) {
+                    T r[C][VEC];
+#pragma unroll
+                    for (int c = 0; c < C; ++c) lds_v(wc.r_(c) + m + v, r[c]);
+#pragma unroll
+                    for (int k = 0; k < VEC; ++k)
+#pragma unroll
+                        for (int x = 0; x < JJ; ++x) {
+                            const T uu = u[x][m + v + k];
+#pragma unroll
+                            for (int c = 0; c < C; ++c) a[c * JJ + x][v + k] = m_fma(uu, r[c][k], a[c * JJ + x][v + k]);
+                        }
+                }
+            }
+            for (; m < M; ++m)
+#pragma unroll
+                for (int c = 0; c < C; ++c)
+#pragma unroll
+                    for (int x = 0; x < JJ; ++x) a[c * JJ + x][0] = m_fma(u[x][m], wc.r_(c)[m], a[c * JJ + x][0]);
+#pragma unroll
+            for (int c = 0; c < C; ++c)
+#pragma unroll
+                for (int x = 0; x < JJ; ++x) {
+                    const T(&b)[8] = a[c * JJ + x];
+                    if (x == 0 || j + 32 * x < np)
+                        wc.c_(c)[j + 32 * x] = ((b[0] + b[1]) + (b[2] + b[3])) + ((b[4] + b[5]) + (b[6] + b[7]));
+                }
+        }
+        return;
+    }
+    // U in global memory (grid-major): sixteen loads in flight, eight in the 128-register kernels of wide tiles
+    constexpr int NL = WIDE || KVC <= 8 ? 16 : 8;
+    for (int j = lane; j < np; j += 32) {
+        T a[C][8];
+#pragma unroll
+        for (int c = 0; c < C; ++c)
+#pragma unroll
+            for (int i = 0; i < 8; ++i) a[c][i] = T(0);
+        int m = 0;
+        for (; m + NL - 1 < M; m += NL) {
+            T x[NL];
+#pragma unroll
+            for (int i = 0; i < NL; ++i) x[i] = __ldg(Um + (size_t)(m + i) * np + j);
+#pragma unroll
+            for (int i = 0; i < NL; ++i)
+#pragma unroll
+                for (int c = 0; c < C; ++c) a[c][i & 7] = m_fma(x[i], wc.r_(c)[m + i], a[c][i & 7]);
+        }
+        for (; m + 7 < M; m += 8) {
+            T x[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) x[i] = __ldg(Um + (size_t)(m + i) * np + j);
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int c = 0; c < C; ++c) a[c][i] = m_fma(x[i], wc.r_(c)[m + i], a[c][i]);
+        }
+        for (; m < M; ++m) {
+            const T x = __ldg(Um + (size_t)m * np + j);
+#pragma unroll
+            for (int c = 0; c < C; ++c) a[c][0] = m_fma(x, wc.r_(c)[m], a[c][0]);
+        }
+#pragma unroll
+        for (int c = 0; c < C; ++c)
+            wc.c_(c)[j] = ((a[c][0] + a[c][1]) + (a[c][2] + a[c][3])) + ((a[c][4] + a[c][5]) + (a[c][6] + a[c][7]));
+    }
+}
+
+// r~ -= U_b w for the warp's chains (lanes split the data points; partial sum i of eight
+// takes the modes j = i mod 8 as at entry).
+template <class T, int C, int KVC, bool WIDE>
+__device__ __forceinline__ void project_exit(const WarpChains<T, C> &wc, const T *Us, const T *Ut, int np, int usr, int M,
+                                             int lane)
+{
+    constexpr int VEC = VecOf<T>::n;
+    constexpr int MM = C == 1 ? 2 : 1;   // data points of a lane at a time
+    if (Us) {
+        for (int m = lane; m < M; m += 32 * MM) {
+            T a[C * MM][8];
+#pragma unroll
+            for (int x = 0; x < C * MM; ++x)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) a[x][i] = T(0);
+            int mm[MM];
+#pragma unroll
+            for (int x = 0; x < MM; ++x) mm[x] = m + 32 * x < M ? m + 32 * x : m;
+            int j = 0;
+            for (; j + 7 < np; j += 8) {
+                const T *u = Us + (size_t)j * usr;
+#pragma unroll
+                for (int v = 0; v < 8; v += VEC) {
+                    T w[C][VEC];
+#pragma unroll
+                    for (int c = 0; c < C; ++c) lds_v(wc.w_(c) + j + v, w[c]);
+#pragma unroll
+                    for (int k = 0; k < VEC; ++k)
+#pragma unroll
+                        for (int x = 0; x < MM; ++x) {
+                            const T uu = u[(v + k) * usr + mm[x]];
+#pragma unroll
+                            for (int c = 0; c < C; ++c) a[c * MM + x][v + k] = m_fma(uu, w[c][k], a[c * MM + x][v + k]);
+                        }
+                }
+            }
+            for (; j < np; ++j)
+#pragma unroll
+                for (int c = 0; c < C; ++c)
+#pragma unroll
+                    for (int x = 0; x < MM; ++x)
+                        a[c * MM + x][0] = m_fma(Us[(size_t)j * usr + mm[x]], wc.w_(c)[j], a[c * MM + x][0]);
+#pragma unroll
+            for (int c = 0; c < C; ++c)
+#pragma unroll
+                for (int x = 0; x < MM; ++x) {
+                    const T(&b)[8] = a[c * MM + x];
+                    if (x == 0 || m + 32 * x < M)
+                        wc.r_(c)[m + 32 * x] -= ((b[0] + b[1]) + (b[2] + b[3])) + ((b[4] + b[5]) + (b[6] + b[7]));
+                }
+        }
+        return;
+    }
+    constexpr int NL = WIDE || KVC <= 8 ? 16 : 8;
+    for (int m = lane; m < M; m += 32) {
+        T a[C][8];
+#pragma unroll
+        for (int c = 0; c < C; ++c)
+#pragma unroll
+            for (int i = 0; i < 8; ++i) a[c][i] = T(0);
+        int j = 0;
+        for (; j + NL - 1 < np; j += NL) {
+            T x[NL];
+#pragma unroll
+            for (int i = 0; i < NL; ++i) x[i] = __ldg(Ut + (size_t)(j + i) * M + m);
+#pragma unroll
+            for (int i = 0; i < NL; ++i)
+#pragma unroll
+                for (int c = 0; c < C; ++c) a[c][i & 7] = m_fma(x[i], wc.w_(c)[j + i], a[c][i & 7]);
+        }
+        for (; j + 7 < np; j += 8) {
+            T x[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) x[i] = __ldg(Ut + (size_t)(j + i) * M + m);
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int c = 0; c < C; ++c) a[c][i] = m_fma(x[i], wc.w_(c)[j + i], a[c][i]);
+        }
+        for (; j < np; ++j) {
+            const T x = __ldg(Ut + (size_t)j * M + m);
+#pragma unroll
+            for (int c = 0; c < C; ++c) a[c][0] = m_fma(x, wc.w_(c)[j], a[c][0]);
+        }
+#pragma unroll
+        for (int c = 0; c < C; ++c)
+            wc.r_(c)[m] -= ((a[c][0] + a[c][1]) + (a[c][2] + a[c][3])) + ((a[c][4] + a[c][5]) + (a[c][6] + a[c][7]));
+    }
+}
+
 // --------------------------------------------------------------------------
-// A consumer warp: its team(s) of S lanes run the chains of chain group
-// `group` (consumers x 32/S chains) of problem p for the launch's sweeps.
-// WIDE: the block entry/exit projections keep sixteen loads in flight instead
-// of eight (same accumulation order); it pays in the kernels budgeted for two
-// CTAs per SM and costs a little in the 255-register ones.
+// The moves of one block visit.  Lane l holds the elements VE (32 k + l) + v of
+// the block, k < KK, v < VE, of each of the warp's C chains.  VE = VEC (16-byte
+// vectors), or half of that for blocks of at most 16 VEC points, whose rows
+// would fill only half the lanes.  KC = KK chunks known to be present, or 0: each
+// of KV is tested (uniformly) against kcnt.
 // --------------------------------------------------------------------------
-template <class T, int KV, bool PRIOR, bool WIDE>
-__device__ __forceinline__ void consume(const SweepParams<T> &p, const LaunchShape &sh, const SweepRange &rg,
-                                        int group, unsigned char *smem_raw, unsigned long long *full,
-                                        unsigned long long *empty, unsigned char *stages, unsigned long long *ufull,
-                                        unsigned long long *uempty, unsigned char *ubuf, RingPos &rp, bool &failed)
+template <class T, int KV, int C, bool PRIOR, int KC, int VE>
+struct Visit {
+    static constexpr int KK = KC ? KC : KV;
+    static constexpr bool CHK = KC == 0;
+    using KS = typename BoundKey<T>::S;
+    using KU = typename BoundKey<T>::U;
+
+    static __device__ __forceinline__ void pass(T (&f)[C][KK][VE], const T (&delta)[C], const T (&v0)[VE], const T (&r0)[VE],
+                                                const T *st, int rs, int kcnt, int lane, KS (&lk)[C], KU (&hk)[C])
+    {
+        Keys<T> kk[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) kk[c].reset();
+#pragma unroll
+        for (int k = 0; k < KK; ++k) {
+            if (!CHK || k < kcnt) {
+                T vv[VE], rr[VE];
+                if (k) {
+                    lds_v(st + VE * (32 * k + lane), vv);
+                    lds_v(st + rs + VE * (32 * k + lane), rr);
+                }
+#pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    if (k) pass_chunk(f[c][k], delta[c], vv, rr, kk[c]);
+                    else pass_chunk(f[c][0], delta[c], v0, r0, kk[c]);
+                }
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < C; ++c) kk[c].fold(lk[c], hk[c]);
+    }
+
+    // false: a bounded wait gave up
+    static __device__ __forceinline__ bool run(const SweepParams<T> &p, const LaunchShape &sh, const Regions &R, RingPos &rp,
+                                               const WarpChains<T, C> &wc, MoveCounts<C> &n, const BlockDesc &B,
+                                               const T *pk, const T *Us, long long s, bool keep, bool trace, int &win,
+                                               int &win_end, int lane, T (&sd2)[C], T (&sf2)[C])
+    {
+        const int kcnt = (B.n + 32 * VE - 1) / (32 * VE);
+        const int bn = B.n, bstart = B.start, rs = B.rs, recstride = B.recstride, np = B.np;
+        T f[C][KK][VE];
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const T *Fq = sh.fpad ? wc.c_(c) + wc.off_f : p.F + (size_t)wc.q[c] * p.ldF;
+#pragma unroll
+            for (int k = 0; k < KK; ++k)
+#pragma unroll
+                for (int v = 0; v < VE; ++v) {
+                    const int nl = VE * (32 * k + lane) + v;
+                    f[c][k][v] = nl < bn ? Fq[bstart + nl] : T(0);
+                }
+        }
+        // keys of the block's first mode: f >= +0, so that the pass reduces to the products
+        KS lk[C];
+        KU hk[C];
+        {
+            Keys<T> kk[C];
+#pragma unroll
+            for (int c = 0; c < C; ++c) kk[c].reset();
+#pragma unroll
+            for (int k = 0; k < KK; ++k) {
+                if (!CHK || k < kcnt) {
+                    T rr[VE];
+                    lds_v(pk + kPacketHeader + VE * (32 * k + lane), rr);
+#pragma unroll
+                    for (int c = 0; c < C; ++c) key_chunk(f[c][k], rr, kk[c]);
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < C; ++c) kk[c].fold(lk[c], hk[c]);
+        }
+        const int rps = records_per_stage<T>(sh, B);
+        const int nz = B.nz;       // moves from nz on are flat and leave the residual alone
+        int jr = 0;                // record of move j within its ring stage
+        const T *stb = nullptr;    // the stage holding move j's record
+        for (int j = 0; j < bn;) {
+            // uniform of move t: word t%4 of Philox(ctr = {t/4, s, q, problem}); the 128
+            // uniforms of a window come from one Philox call per lane and chain
+            const int t0 = bstart + j;
+            if (t0 >= win_end) {
+                win = t0 & ~127;
+                win_end = win + 128;
+                __syncwarp();   // the previous window is read by every lane
+#pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    unsigned long long c0 = (unsigned long long)(win >> 2) + (unsigned long long)lane;
+                    unsigned long long c1 = (unsigned long long)s, c2 = (unsigned long long)wc.q[c] + p.chain_offset,
+                                       c3 = p.problem_id;
+                    philox4x64_10(c0, c1, c2, c3, p.seed, 0ull);
+                    T *usm = wc.u_(c);
+                    usm[4 * lane] = uniform_from<T>(c0);
+                    usm[4 * lane + 1] = uniform_from<T>(c1);
+                    usm[4 * lane + 2] = uniform_from<T>(c2);
+                    usm[4 * lane + 3] = uniform_from<T>(c3);
+                    if constexpr (PRIOR) {   // acceptance uniforms: ctr {t/4, s, q, problem xor 2^63}
+                        c0 = (unsigned long long)(win >> 2) + (unsigned long long)lane;
+                        c1 = (unsigned long long)s;
+                        c2 = (unsigned long long)wc.q[c] + p.chain_offset;
+                        c3 = p.problem_id ^ (1ull << 63);
+                        philox4x64_10(c0, c1, c2, c3, p.seed, 0ull);
+                        usm[128 + 4 * lane] = uniform_from<T>(c0);
+                        usm[128 + 4 * lane + 1] = uniform_from<T>(c1);
+                        usm[128 + 4 * lane + 2] = uniform_from<T>(c2);
+                        usm[128 + 4 * lane + 3] = uniform_from<T>(c3);
+                    }
+                }
+                __syncwarp();
+            }
+            if (jr == 0) {   // the stage of the next record: usually landed long ago
+                if (!warp_wait(R.full + rp.slot, rp.phase, sh.wait_limit)) return false;
+                stb = reinterpret_cast<const T *>(R.stages + (size_t)rp.slot * sh.stage_bytes);
+            }
+            // this segment's moves: up to the end of the window, of the stage, of the modes
+            // that need more than their rows, or of the block
+            const int jbeg = j;
+            int jend = min(min(bn, win_end - bstart), j + (rps - jr));
+            const T *st = stb + (size_t)jr * recstride;
+            const T *up = wc.u_(0) + (bstart - win);
+            if (!PRIOR && j >= nz) {
+                // flat moves in the block's null space: bounds, a uniform and the pass
+                unsigned opened[C];
+#pragma unroll
+                for (int c = 0; c < C; ++c) opened[c] = 0u;
+#pragma unroll 1
+                for (; j < jend; ++j, st += recstride) {
+                    T u[C], v0[VE], r0[VE], lo[C], hi[C], delta[C];
+#pragma unroll
+                    for (int c = 0; c < C; ++c) u[c] = up[j + c * wc.tw];
+                    lds_v(st + VE * lane, v0);
+                    lds_v(st + rs + VE * lane, r0);
+                    warp_bounds<C>(lk, hk, lo, hi);
+#pragma unroll
+                    for (int c = 0; c < C; ++c) {
+                        const bool open = open_interval(lo[c], hi[c]);
+                        delta[c] = open ? m_fma(u[c], hi[c] - lo[c], lo[c]) : T(0);
+                        opened[c] += open ? 1u : 0u;
+                    }
+                    pass(f, delta, v0, r0, st, rs, kcnt, lane, lk, hk);
+                }
+#pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    n.zero[c] += opened[c];
+                    n.deg[c] += (unsigned)(j - jbeg) - opened[c];
+                }
+            } else {
+                if (!PRIOR) jend = min(jend, nz);
+#pragma unroll 1
+                for (; j < jend; ++j, st += recstride) {
+                    T u[C], v0[VE], r0[VE], lo[C], hi[C], delta[C], dj, ij, dres;
+                    // chunk 0 of the pass and the mode's data do not depend on the bounds: loaded first
+                    lds_mode(st + 2 * rs, dj, ij, dres);
+#pragma unroll
+                    for (int c = 0; c < C; ++c) u[c] = up[j + c * wc.tw];
+                    lds_v(st + VE * lane, v0);
+                    lds_v(st + rs + VE * lane, r0);
+                    warp_bounds<C>(lk, hk, lo, hi);
+                    // degenerate interval: no move; zero mode: flat on [lo, hi] (both bounds
+                    // finite: set-up rejects zero modes that do not change sign); else the
+                    // truncated Gaussian.  The branch is on the record's d_j, the same for all
+                    // chains and known long before the bounds.
+                    if (is_zero(dj)) {
+#pragma unroll
+                        for (int c = 0; c < C; ++c) {
+                            const bool open = open_interval(lo[c], hi[c]);
+                            delta[c] = open ? m_fma(u[c], hi[c] - lo[c], lo[c]) : T(0);
+                            n.zero[c] += open ? 1u : 0u;
+                            n.deg[c] += open ? 0u : 1u;
+                        }
+                    } else {
+                        constexpr int G = 32 / C;
+                        T l = lo[0], h = hi[0], uu = u[0];
+                        const T *cs = wc.c_(0);
+#pragma unroll
+                        for (int c = 1; c < C; ++c) {
+                            const bool mine = lane / G == c;
+                            l = mine ? lo[c] : l;
+                            h = mine ? hi[c] : h;
+                            uu = mine ? u[c] : uu;
+                            cs = mine ? wc.c_(c) : cs;
+                        }
+                        const T cj = j < np ? cs[j] : T(0);
+                        T dl = tn_step_team<G>(cj, dj, ij, l, h, uu, open_interval(l, h), lane, n.capped);
+#pragma unroll
+                        for (int c = 0; c < C; ++c) {
+                            const T x = C == 1 ? dl : __shfl_sync(0xffffffffu, dl, c * G);
+                            const bool fin = is_finite(x);
+                            n.bad[c] += fin ? 0u : 1u;
+                            n.deg[c] += open_interval(lo[c], hi[c]) ? 0u : 1u;
+                            delta[c] = fin ? x : T(0);
+                        }
+                    }
+                    if constexpr (PRIOR) if (delta[0] != T(0)) {
+                        // gamma prior (Eq. compat): the draw is a proposal, accepted with
+                        // probability min(1, prod ((f + delta V)_+ / f)^(a - 1)) over the block
+                        T lsum = T(0);
+                        unsigned zflags = 0u;   // 1: a proposed value is 0, 2: a current value is 0
+#pragma unroll
+                        for (int k = 0; k < KK; ++k) {
+                            if (!CHK || k < kcnt) {
+                                T vv[VE];
+                                if (k == 0) {
+#pragma unroll
+                                    for (int v = 0; v < VE; ++v) vv[v] = v0[v];
+                                } else {
+                                    lds_v(st + VE * (32 * k + lane), vv);
+                                }
+#pragma unroll
+                                for (int v = 0; v < VE; ++v) {
+                                    const int nl = VE * (32 * k + lane) + v;
+                                    if (nl < bn) {
+                                        const T am1 = __ldg(p.prior_am1 + bstart + nl);
+                                        if (am1 != T(0)) {
+                                            const T x0 = f[0][k][v];
+                                            const T x1 = m_max(m_fma(delta[0], vv[v], x0), T(0));
+                                            if (x1 == T(0)) zflags |= 1u;
+                                            else if (x0 == T(0)) zflags |= 2u;
+                                            else lsum += am1 * (m_log(x1) - m_log(x0));
+                                        }
+                                    }
+                                }
+                            }
+                        }
+                        for (int off = 1; off < 32; off <<= 1) {
+                            lsum += __shfl_xor_sync(0xffffffffu, lsum, off);
+                            zflags |= __shfl_xor_sync(0xffffffffu, zflags, off);
+                        }
+                        const T lr = (zflags & 1u) ? -CUDART_INF_F : (zflags & 2u) ? CUDART_INF_F : lsum;
+                        const T ua = up[128 + j];
+                        if (!(m_log(ua) < lr)) {
+                            delta[0] = T(0);
+                            ++n.rej[0];
+                        }
+                    }
+                    pass(f, delta, v0, r0, st, rs, kcnt, lane, lk, hk);
+                    // the residual moves by K~_b V_j delta = dres_j delta U_j (dres = d for a
+                    // Gaussian mode, |K~_b V_j| for one sampled flat); all lanes store the same
+                    if (j < np) {
+#pragma unroll
+                        for (int c = 0; c < C; ++c) wc.w_(c)[j] = dres * delta[c];
+                    }
+                }
+            }
+            // release the stage to the producer after its last record (one arrival per warp)
+            jr += j - jbeg;
+            if (jr == rps || j == bn) {
+                __syncwarp();
+                mbar_arrive_lane0(R.empty + rp.slot, lane);
+                ring_next(rp, sh.depth);
+                jr = 0;
+            }
+        }
+        // write the block back and accumulate the kept sweep
+        constexpr bool psums = sizeof(T) == 4;
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            T *Fq = sh.fpad ? wc.c_(c) + wc.off_f : p.F + (size_t)wc.q[c] * p.ldF;
+            const bool write = wc.active[c];
+#pragma unroll
+            for (int k = 0; k < KK; ++k)
+#pragma unroll
+                for (int v = 0; v < VE; ++v) {
+                    const int nl = VE * (32 * k + lane) + v;
+                    if (write && nl < bn) {
+                        const int i = bstart + nl;
+                        if (trace) {
+                            const T old = Fq[i], dlt = f[c][k][v] - old;
+                            sd2[c] = m_fma(dlt, dlt, sd2[c]);
+                            sf2[c] = m_fma(old, old, sf2[c]);
+                        }
+                        Fq[i] = f[c][k][v];
+                        if (keep) {
+                            if constexpr (psums) {
+                                T *p1 = sh.npad ? wc.c_(c) + wc.off_p : reinterpret_cast<T *>(p.P1) + (size_t)wc.q[c] * p.ldF;
+                                T *p2 = sh.npad ? p1 + sh.npad : reinterpret_cast<T *>(p.P2) + (size_t)wc.q[c] * p.ldF;
+                                p1[i] += f[c][k][v];
+                                p2[i] = m_fma(f[c][k][v], f[c][k][v], p2[i]);
+                            } else {
+                                const double x = (double)f[c][k][v];
+                                p.S1[(size_t)wc.q[c] * p.N + i] += x;
+                                p.S2[(size_t)wc.q[c] * p.N + i] += x * x;
+                            }
+                        }
+                    }
+                    // one chunk's sums at a time: keeps the compiler from holding every
+                    // chunk's loaded sums in registers at once (the widest tiles spilled)
+                    if (v + 1 == VE) asm volatile("" ::: "memory");
+                }
+        }
+        return true;
+    }
+};
+
+// --------------------------------------------------------------------------
+// A consumer warp: its C chains of chain group `group` (consumers x C chains) of
+// problem p for the launch's sweeps.
+// --------------------------------------------------------------------------
+template <class T, int KV, int C, bool PRIOR, bool WIDE>
+__device__ __forceinline__ void consume(const SweepParams<T> &p, const LaunchShape &sh, const SweepRange &rg, int group,
+                                        unsigned char *smem_raw, const Regions &R, RingPos &rp, bool &failed)
 {
     constexpr int VEC = VecOf<T>::n;
     if (failed) return;
     const int lane = threadIdx.x & 31;
     const int wcta = threadIdx.x >> 5;
-    const int D = sh.depth;
-    const int S = sh.S;
-    const int TW = 32 / S;
-    const int team = lane / S;
-    const int sl = lane - team * S;
-    const int team_base = team * S;
-    const long long gwarp = (long long)group * sh.consumers + wcta;
-    const long long q_raw = gwarp * TW + team;
-    const bool active = q_raw < p.chains;
-    const long long q = active ? q_raw : (long long)p.chains - 1;  // idle teams shadow a real chain, write nothing
-
-    // per team in shared memory: c (cpad), w (cpad), r~ (mpad), the uniforms of the
-    // current window of 4S moves and, where they fit (npad > 0), the sums of f and f^2
-    // over this launch's kept sweeps (FP32; at most one refresh period of terms)
-    T *csm = reinterpret_cast<T *>(smem_raw) + (size_t)(wcta * TW + team) * sh.team_words;
-    T *wsm = csm + sh.cpad;
-    T *rsm = wsm + sh.cpad;
-    T *usm = rsm + sh.mpad;   // 4S uniforms of the draws, then 4S of the prior's acceptances
+    WarpChains<T, C> wc;
+    // per chain in shared memory: c (cpad), w (cpad), r~ (mpad), the uniforms of the current
+    // window of 128 moves (with a prior 128 more) and, where they fit, the chain state (fpad)
+    // and the sums of f and f^2 over this launch's kept sweeps (FP32, npad each)
+    wc.tw = sh.team_words;
+    wc.sm = reinterpret_cast<T *>(smem_raw) + (size_t)(wcta * C) * sh.team_words;
+    wc.off_w = sh.cpad;
+    wc.off_r = 2 * sh.cpad;
+    wc.off_u = 2 * sh.cpad + sh.mpad;
+    wc.off_f = wc.off_u + (PRIOR ? 256 : 128);
+    wc.off_p = wc.off_f + sh.fpad;
     // FP32 chain state: the kept-sweep sums of the current kBinSweeps-sweep block (aligned
     // to absolute sweep indices) in FP32, added to the FP64 sums when the block closes.
     // Between launches they wait in the workspace (P1, P2); during one they live in shared
@@ -746,395 +1443,132 @@ __device__ __forceinline__ void consume(const SweepParams<T> &p, const LaunchSha
     // FP64 chain state: straight into the FP64 sums.
     constexpr bool psums = sizeof(T) == 4;
     const bool kept_here = psums && rg.burn_in < rg.sweep0 + rg.nsweeps;
-    T *P1q = psums ? reinterpret_cast<T *>(p.P1) + (size_t)q * p.ldF : nullptr;
-    T *P2q = psums ? reinterpret_cast<T *>(p.P2) + (size_t)q * p.ldF : nullptr;
-    T *p1sm = sh.npad ? usm + 8 * S : P1q;
-    T *p2sm = sh.npad ? p1sm + sh.npad : P2q;
-    if (kept_here && sh.npad)
-        for (int n = sl; n < p.N; n += S) {
-            p1sm[n] = P1q[n];
-            p2sm[n] = P2q[n];
+    MoveCounts<C> n;
+    n.capped = 0;
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+        const long long q_raw = ((long long)group * sh.consumers + wcta) * C + c;
+        wc.active[c] = q_raw < p.chains;
+        wc.q[c] = wc.active[c] ? q_raw : (long long)p.chains - 1;   // idle chains shadow a real one, write nothing
+        n.deg[c] = n.zero[c] = n.bad[c] = n.rej[c] = 0u;
+        const T *Rq = p.R + (size_t)wc.q[c] * p.ldR;
+        for (int m = lane; m < p.M; m += 32) wc.r_(c)[m] = Rq[m];
+        if (sh.fpad) {
+            const T *Fq = p.F + (size_t)wc.q[c] * p.ldF;
+            T *fs = wc.c_(c) + wc.off_f;
+            for (int i = lane; i < p.N; i += 32) fs[i] = Fq[i];
         }
-    T *Rq = p.R + (size_t)q * p.ldR;
-    for (int m = sl; m < p.M; m += S) rsm[m] = Rq[m];
-    T *Fq = p.F + (size_t)q * p.ldF;
-    double *S1q = p.S1 + (size_t)q * p.N;
-    double *S2q = p.S2 + (size_t)q * p.N;
+        if (kept_here && sh.npad) {
+            const T *P1q = reinterpret_cast<const T *>(p.P1) + (size_t)wc.q[c] * p.ldF;
+            const T *P2q = reinterpret_cast<const T *>(p.P2) + (size_t)wc.q[c] * p.ldF;
+            T *p1 = wc.c_(c) + wc.off_p;
+            for (int i = lane; i < p.N; i += 32) {
+                p1[i] = P1q[i];
+                p1[sh.npad + i] = P2q[i];
+            }
+        }
+    }
     __syncwarp();
 
-    T f[KV][VEC];
-    unsigned n_deg = 0, n_zero = 0, n_bad = 0, n_rej = 0;   // per launch: at most 64 sweeps of moves
     const bool trace = p.steptrace != nullptr;   // step-size trace of Fig. MCsteps (diagnostic)
-    int capped = 0;
     const long long s_end = rg.sweep0 + rg.nsweeps;
     for (long long s = rg.sweep0; s < s_end && !failed; ++s) {
-        // level of this sweep: same for every chain of the problem (Sec. IV.C)
-        const int level = level_of_sweep(s, p.seed, p.problem_id, p.n_levels);
         const bool keep = s >= rg.burn_in;
-        int win = 0, win_end = -1;  // window [win, win_end) of moves whose uniforms are in usm
-        const int nb = p.level_nblocks[level];
-        const BlockDesc *bd = p.blocks + p.level_first[level];
-        T sd2 = T(0), sf2 = T(0);   // this lane's |f(s+1) - f(s)|^2 and |f(s)|^2 (trace only)
-
-        for (int bi = 0; bi < nb && !failed; ++bi) {
-            const BlockDesc B = bd[bi];
-            const int kcnt = (B.n + VEC * S - 1) / (VEC * S);
-            // entry: the block's f into registers
+        int win = 0, win_end = -1;  // window [win, win_end) of moves whose uniforms are in shared memory
+        T sd2[C], sf2[C];           // this lane's |f(s+1) - f(s)|^2 and |f(s)|^2 (trace only)
 #pragma unroll
-            for (int k = 0; k < KV; ++k)
-#pragma unroll
-                for (int v = 0; v < VEC; ++v) {
-                    const int nl = VEC * (k * S + sl) + v;
-                    f[k][v] = (k < kcnt && nl < B.n) ? Fq[B.start + nl] : T(0);
-                }
-            // U of this block: from its U stage once the producer's copy has landed, else
-            // from global memory
-            const bool ust = u_staged<T>(sh, B);
-            const T *Us = nullptr;
-            if (ust) {
-                bool ok = mbar_test_wait(ufull + (rp.ug & 1u), (rp.ug >> 1) & 1u);
-                if (__any_sync(0xffffffffu, !ok)) {
-                    ok = ok || mbar_wait(ufull + (rp.ug & 1u), (rp.ug >> 1) & 1u, sh.wait_limit);
-                    if (__any_sync(0xffffffffu, !ok)) {   // decided warp-wide
-                        failed = true;
-                        break;
-                    }
-                }
-                Us = reinterpret_cast<const T *>(ubuf + (size_t)(rp.ug & 1u) * sh.ubytes);
+        for (int c = 0; c < C; ++c) sd2[c] = sf2[c] = T(0);
+        // the sweep's blocks, as the packets bring them: the producer draws the level, the same
+        // for every chain of the problem (Sec. IV.C), and the last block of a level says so
+        for (bool last = false; !last;) {
+            if (!warp_wait(R.pfull + rp.pslot, rp.pphase, sh.wait_limit)) {
+                failed = true;
+                break;
             }
-            // c = U_b^T r~ (lanes split the modes; eight (WIDE: sixteen) loads in flight, eight
-            // partial sums, partial sum i taking the terms m = i mod 8 in increasing m; the
-            // same sums in the same order from the U stage)
-            const T *Um = p.pd.Um + B.offU;
-            if (ust) {
-                // two of the lane's modes at a time (j, j + S): two independent chains of sums
-                // (one at a time in the widest register tiles, whose registers hold f)
-                for (int j = sl; j < B.np; j += (KV <= 8 ? 2 : 1) * S) {
-                    const bool two = KV <= 8 && j + S < B.np;
-                    const T *u = Us + (size_t)j * B.usr;
-                    const T *u2 = Us + (size_t)(two ? j + S : j) * B.usr;
-                    T a[8], b[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) a[i] = b[i] = T(0);
-                    int m = 0;
-                    for (; m + 7 < p.M; m += 8) {
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const T r = rsm[m + i];
-                            a[i] = m_fma(u[m + i], r, a[i]);
-                            b[i] = m_fma(u2[m + i], r, b[i]);
-                        }
-                    }
-                    for (; m < p.M; ++m) {
-                        a[0] = m_fma(u[m], rsm[m], a[0]);
-                        b[0] = m_fma(u2[m], rsm[m], b[0]);
-                    }
-                    csm[j] = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
-                    if (two) csm[j + S] = ((b[0] + b[1]) + (b[2] + b[3])) + ((b[4] + b[5]) + (b[6] + b[7]));
-                }
-            } else
-            for (int j = sl; j < B.np; j += S) {
-                T a[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) a[i] = T(0);
-                int m = 0;
-                if constexpr (WIDE) {
-                    for (; m + 15 < p.M; m += 16) {
-                        T x[16];
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) x[i] = __ldg(Um + (size_t)(m + i) * B.np + j);
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) a[i & 7] = m_fma(x[i], rsm[m + i], a[i & 7]);
-                    }
-                }
-                for (; m + 7 < p.M; m += 8) {
-                    T x[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) x[i] = __ldg(Um + (size_t)(m + i) * B.np + j);
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) a[i] = m_fma(x[i], rsm[m + i], a[i]);
-                }
-                for (; m < p.M; ++m) a[0] = m_fma(__ldg(Um + (size_t)m * B.np + j), rsm[m], a[0]);
-                csm[j] = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
+            const T *pk = reinterpret_cast<const T *>(R.packets + (size_t)rp.pslot * sh.pbytes);
+            const BlockDesc &B = *reinterpret_cast<const BlockDesc *>(pk);
+            last = B.last != 0;
+            const T *Us = u_staged<T>(sh, B) ? pk + kPacketHeader + B.rs : nullptr;
+            project_entry<T, C, KV * C, WIDE>(wc, Us, p.pd.Um + B.offU, B.np, B.usr, p.M, lane);
+            __syncwarp();
+            bool ok;
+            if (B.n <= 16 * VEC)
+                ok = Visit<T, KV, C, PRIOR, 1, VEC / 2>::run(p, sh, R, rp, wc, n, B, pk, Us, s, keep, trace, win, win_end,
+                                                             lane, sd2, sf2);
+            else if (KV == 1 || B.n <= 32 * VEC)
+                ok = Visit<T, KV, C, PRIOR, 1, VEC>::run(p, sh, R, rp, wc, n, B, pk, Us, s, keep, trace, win, win_end, lane,
+                                                         sd2, sf2);
+            else if (KV == 2 || B.n > 32 * VEC * (KV - 1))
+                ok = Visit<T, KV, C, PRIOR, KV, VEC>::run(p, sh, R, rp, wc, n, B, pk, Us, s, keep, trace, win, win_end, lane,
+                                                          sd2, sf2);
+            else
+                ok = Visit<T, KV, C, PRIOR, 0, VEC>::run(p, sh, R, rp, wc, n, B, pk, Us, s, keep, trace, win, win_end, lane,
+                                                         sd2, sf2);
+            if (!ok) {
+                failed = true;
+                break;
             }
             __syncwarp();
-
-            typename BoundKey<T>::S lk;
-            typename BoundKey<T>::U hk;
-            first_keys<T, KV>(f, p.pd.R + B.offR, kcnt, sl, S, lk, hk);  // keys of mode 0
-            // The block's moves.  Where the lane's chunk count is 1 (blocks of at most
-            // VEC*S points) or KV (every chunk present) it is a compile-time constant and
-            // the move loop tests no chunk; the uniforms are refilled once per window of
-            // 4S moves, outside the loop over the window's moves.
-            auto block_moves = [&](auto chunks) {
-                constexpr int KC = decltype(chunks)::value;   // 0: kcnt chunks, each tested
-                constexpr int KK = KC ? KC : KV;
-                constexpr bool CHK = KC == 0;
-                int jr = 0;                        // record of move j within its ring stage
-                const T *stb = nullptr;            // the stage holding move j's record
-                for (int j = 0; j < B.n && !failed;) {
-                    // uniform of move t: word t%4 of Philox(ctr = {t/4, s, q, problem}); the 4S
-                    // uniforms of a window come from one Philox call per lane (lane sl: ctr
-                    // win/4 + sl, moves win + 4 sl + 0..3)
-                    const int t0 = B.start + j;
-                    if (t0 >= win_end) {
-                        win = (t0 / (4 * S)) * (4 * S);
-                        win_end = win + 4 * S;
-                        unsigned long long c0 = (unsigned long long)(win >> 2) + (unsigned long long)sl;
-                        unsigned long long c1 = (unsigned long long)s, c2 = (unsigned long long)q + p.chain_offset,
-                                           c3 = p.problem_id;
-                        philox4x64_10(c0, c1, c2, c3, p.seed, 0ull);
-                        __syncwarp();   // the previous window is read by every lane
-                        usm[4 * sl] = uniform_from<T>(c0);
-                        usm[4 * sl + 1] = uniform_from<T>(c1);
-                        usm[4 * sl + 2] = uniform_from<T>(c2);
-                        usm[4 * sl + 3] = uniform_from<T>(c3);
-                        if constexpr (PRIOR) {   // acceptance uniforms: ctr {t/4, s, q, problem xor 2^63}
-                            c0 = (unsigned long long)(win >> 2) + (unsigned long long)sl;
-                            c1 = (unsigned long long)s;
-                            c2 = (unsigned long long)q + p.chain_offset;
-                            c3 = p.problem_id ^ (1ull << 63);
-                            philox4x64_10(c0, c1, c2, c3, p.seed, 0ull);
-                            usm[4 * S + 4 * sl] = uniform_from<T>(c0);
-                            usm[4 * S + 4 * sl + 1] = uniform_from<T>(c1);
-                            usm[4 * S + 4 * sl + 2] = uniform_from<T>(c2);
-                            usm[4 * S + 4 * sl + 3] = uniform_from<T>(c3);
-                        }
-                        __syncwarp();
-                    }
-                    // the stage of the next record: usually landed long ago (one test, one vote
-                    // per stage of sh.rps moves)
-                    if (jr == 0) {
-                        bool ok = mbar_test_wait(full + rp.slot, rp.phase);
-                        if (__any_sync(0xffffffffu, !ok)) {
-                            ok = ok || mbar_wait(full + rp.slot, rp.phase, sh.wait_limit);
-                            if (__any_sync(0xffffffffu, !ok)) {   // decided warp-wide
-                                failed = true;
-                                break;
-                            }
-                        }
-                        stb = reinterpret_cast<const T *>(stages + (size_t)rp.slot * sh.stage_bytes);
-                    }
-                    // this segment's moves: up to the end of the window, of the stage or of the block
-                    const int jbeg = j, jend = min(min(B.n, win_end - B.start), j + (sh.rps - jr));
-                    const T *st = stb + (size_t)jr * B.recstride;
-                    for (; j < jend; ++j, st += B.recstride) {
-                        // what does not depend on the bounds first: c_j and the uniform
-                        const T cj = j < B.np ? csm[j] : T(0);
-                        const int t = B.start + j;
-                        const T u = usm[t - win];
-                        const T dj = st[2 * B.rs], ij = st[2 * B.rs + 1];
-                        T v0[VEC], r0[VEC];   // chunk 0 of the pass: independent of the draw, loaded first
-                        lds_v(st + VEC * sl, v0);
-                        lds_v(st + B.rs + VEC * sl, r0);
-
-                        T lo, hi;
-                        team_bounds(lk, hk, lo, hi, S, team_base);
-                        // degenerate interval: no move; zero mode: flat on [lo, hi] (both bounds
-                        // finite: set-up rejects zero modes that do not change sign); else the
-                        // truncated Gaussian.  The branch is on the record's d_j, which is known
-                        // long before the bounds, so the flat path is one FMA and a select.
-                        const bool open = hi > lo;
-                        T delta;
-                        if (dj == T(0)) {
-                            delta = open ? m_fma(u, hi - lo, lo) : T(0);
-                            n_zero += open ? 1u : 0u;
-                        } else {
-                            delta = open ? tn_step<T>(cj, dj, ij, lo, hi, u, capped) : T(0);
-                            const bool fin = isfinite(delta);
-                            n_bad += fin ? 0u : 1u;
-                            delta = fin ? delta : T(0);
-                        }
-                        n_deg += open ? 0u : 1u;
-                        if constexpr (PRIOR) if (delta != T(0)) {
-                            // gamma prior (Eq. compat): the draw is a proposal, accepted with
-                            // probability min(1, prod ((f + delta V)_+ / f)^(a - 1)) over the block
-                            T lsum = T(0);
-                            unsigned zflags = 0u;   // 1: a proposed value is 0, 2: a current value is 0
-#pragma unroll
-                            for (int k = 0; k < KV; ++k) {
-                                if (k < kcnt) {
-                                    T vv[VEC];
-                                    if (k == 0) {
-#pragma unroll
-                                        for (int v = 0; v < VEC; ++v) vv[v] = v0[v];
-                                    } else {
-                                        lds_v(st + VEC * (k * S + sl), vv);
-                                    }
-#pragma unroll
-                                    for (int v = 0; v < VEC; ++v) {
-                                        const int nl = VEC * (k * S + sl) + v;
-                                        if (nl < B.n) {
-                                            const T am1 = __ldg(p.prior_am1 + B.start + nl);
-                                            if (am1 != T(0)) {
-                                                const T x0 = f[k][v];
-                                                const T x1 = m_max(m_fma(delta, vv[v], x0), T(0));
-                                                if (x1 == T(0)) zflags |= 1u;
-                                                else if (x0 == T(0)) zflags |= 2u;
-                                                else lsum += am1 * (m_log(x1) - m_log(x0));
-                                            }
-                                        }
-                                    }
-                                }
-                            }
-                            for (int off = 1; off < S; off <<= 1) {
-                                lsum += __shfl_xor_sync(0xffffffffu, lsum, off);
-                                zflags |= __shfl_xor_sync(0xffffffffu, zflags, off);
-                            }
-                            const T lr = (zflags & 1u) ? -CUDART_INF_F : (zflags & 2u) ? CUDART_INF_F : lsum;
-                            const T ua = usm[4 * S + (t - win)];
-                            if (!(m_log(ua) < lr)) {
-                                delta = T(0);
-                                ++n_rej;
-                            }
-                        }
-                        fused_pass_smem<T, KV, KK, CHK>(f, delta, v0, r0, st, st + B.rs, kcnt, sl, S, lk, hk);
-                        // the residual moves by K~_b V_j delta = dres_j delta U_j (dres = d for a
-                        // Gaussian mode, |K~_b V_j| for one sampled flat)
-                        if (j < B.np && sl == 0) wsm[j] = st[2 * B.rs + 2] * delta;
-                    }
-                    // release the stage to the producer after its last record (one arrival per warp)
-                    jr += j - jbeg;
-                    if (jr == sh.rps || j == B.n) {
-                        __syncwarp();
-                        mbar_arrive_lane0(empty + rp.slot, lane);
-                        ring_next(rp, D);
-                        jr = 0;
-                    }
-                }
-            };
-            if (kcnt == 1) {
-                block_moves(std::integral_constant<int, 1>{});
-            } else if constexpr (KV > 1) {
-                if (kcnt == KV)
-                    block_moves(std::integral_constant<int, KV>{});
-                else
-                    block_moves(std::integral_constant<int, 0>{});
-            }
-            if (failed) break;
+            project_exit<T, C, KV * C, WIDE>(wc, Us, p.pd.Ut + B.offU, B.np, B.usr, p.M, lane);
+            // release the packet to the producer (one arrival per warp)
             __syncwarp();
-            // exit: r~ -= U_b w (lanes split the data points; eight (WIDE: sixteen) loads in
-            // flight, eight partial sums as at entry; the same from the U stage)
-            const T *Ut = p.pd.Ut + B.offU;
-            if (ust) {
-                // two of the lane's data points at a time (m, m + S; one in the widest tiles)
-                for (int m = sl; m < p.M; m += (KV <= 8 ? 2 : 1) * S) {
-                    const bool two = KV <= 8 && m + S < p.M;
-                    const int m2 = two ? m + S : m;
-                    T a[8], b[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) a[i] = b[i] = T(0);
-                    int j = 0;
-                    for (; j + 7 < B.np; j += 8) {
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const T w = wsm[j + i];
-                            const T *u = Us + (size_t)(j + i) * B.usr;
-                            a[i] = m_fma(u[m], w, a[i]);
-                            b[i] = m_fma(u[m2], w, b[i]);
-                        }
-                    }
-                    for (; j < B.np; ++j) {
-                        a[0] = m_fma(Us[(size_t)j * B.usr + m], wsm[j], a[0]);
-                        b[0] = m_fma(Us[(size_t)j * B.usr + m2], wsm[j], b[0]);
-                    }
-                    rsm[m] -= ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
-                    if (two) rsm[m + S] -= ((b[0] + b[1]) + (b[2] + b[3])) + ((b[4] + b[5]) + (b[6] + b[7]));
-                }
-                // release the U stage to the producer (one arrival per warp)
-                __syncwarp();
-                mbar_arrive_lane0(uempty + (rp.ug & 1u), lane);
-                ++rp.ug;
-            } else
-            for (int m = sl; m < p.M; m += S) {
-                T a[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) a[i] = T(0);
-                int j = 0;
-                if constexpr (WIDE) {
-                    for (; j + 15 < B.np; j += 16) {
-                        T x[16];
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) x[i] = __ldg(Ut + (size_t)(j + i) * p.M + m);
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) a[i & 7] = m_fma(x[i], wsm[j + i], a[i & 7]);
-                    }
-                }
-                for (; j + 7 < B.np; j += 8) {
-                    T x[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) x[i] = __ldg(Ut + (size_t)(j + i) * p.M + m);
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) a[i] = m_fma(x[i], wsm[j + i], a[i]);
-                }
-                for (; j < B.np; ++j) a[0] = m_fma(__ldg(Ut + (size_t)j * p.M + m), wsm[j], a[0]);
-                rsm[m] -= ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
-            }
-            // write the block back and accumulate the kept sweep
-#pragma unroll
-            for (int k = 0; k < KV; ++k)
-#pragma unroll
-                for (int v = 0; v < VEC; ++v) {
-                    const int nl = VEC * (k * S + sl) + v;
-                    if (active && k < kcnt && nl < B.n) {
-                        const int n = B.start + nl;
-                        if (trace) {
-                            const T old = Fq[n], dlt = f[k][v] - old;
-                            sd2 = m_fma(dlt, dlt, sd2);
-                            sf2 = m_fma(old, old, sf2);
-                        }
-                        Fq[n] = f[k][v];
-                        if (keep) {
-                            if constexpr (psums) {
-                                p1sm[n] += f[k][v];
-                                p2sm[n] = m_fma(f[k][v], f[k][v], p2sm[n]);
-                            } else {
-                                const double x = (double)f[k][v];
-                                S1q[n] += x;
-                                S2q[n] += x * x;
-                            }
-                        }
-                    }
-                    // one chunk's sums at a time: keeps the compiler from holding every
-                    // chunk's loaded sums in registers at once (the widest tiles spilled)
-                    if (v + 1 == VEC) asm volatile("" ::: "memory");
-                }
-            __syncwarp();
+            mbar_arrive_lane0(R.pempty + rp.pslot, lane);
+            packet_next(rp, sh.pslots);
         }
         if (trace && !failed) {   // Delta_s = |f(s+1) - f(s)| / |f(s)| of this chain, summed over chains
-            for (int off = 1; off < S; off <<= 1) {
-                sd2 += __shfl_xor_sync(0xffffffffu, sd2, off);
-                sf2 += __shfl_xor_sync(0xffffffffu, sf2, off);
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                T a = sd2[c], b = sf2[c];
+                for (int off = 1; off < 32; off <<= 1) {
+                    a += __shfl_xor_sync(0xffffffffu, a, off);
+                    b += __shfl_xor_sync(0xffffffffu, b, off);
+                }
+                if (wc.active[c] && lane == 0 && s < p.trace_cap && b > T(0))
+                    atomicAdd(p.steptrace + s, sqrt((double)a / (double)b));
             }
-            if (active && sl == 0 && s < p.trace_cap && sf2 > T(0))
-                atomicAdd(p.steptrace + s, sqrt((double)sd2 / (double)sf2));
         }
     }
     if (failed) {
         if (lane == 0) atomicAdd(&p.counters->timeouts, 1ull);
         return;
     }
-    if (active) {
-        for (int m = sl; m < p.M; m += S) Rq[m] = rsm[m];
-        if (kept_here) {
-            if ((rg.sweep0 + rg.nsweeps) % kBinSweeps == 0) {   // the block closes: into the FP64 sums
-                for (int n = sl; n < p.N; n += S) {
-                    S1q[n] += (double)p1sm[n];
-                    S2q[n] += (double)p2sm[n];
-                    P1q[n] = P2q[n] = T(0);
-                }
-            } else if (sh.npad) {   // the block continues in a later launch
-                for (int n = sl; n < p.N; n += S) {
-                    P1q[n] = p1sm[n];
-                    P2q[n] = p2sm[n];
+    __syncwarp();
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+        if (wc.active[c]) {
+            T *Rq = p.R + (size_t)wc.q[c] * p.ldR;
+            for (int m = lane; m < p.M; m += 32) Rq[m] = wc.r_(c)[m];
+            if (sh.fpad) {
+                T *Fq = p.F + (size_t)wc.q[c] * p.ldF;
+                const T *fs = wc.c_(c) + wc.off_f;
+                for (int i = lane; i < p.N; i += 32) Fq[i] = fs[i];
+            }
+            if (kept_here) {
+                T *P1q = reinterpret_cast<T *>(p.P1) + (size_t)wc.q[c] * p.ldF;
+                T *P2q = reinterpret_cast<T *>(p.P2) + (size_t)wc.q[c] * p.ldF;
+                const T *p1 = sh.npad ? wc.c_(c) + wc.off_p : P1q;
+                const T *p2 = sh.npad ? p1 + sh.npad : P2q;
+                if (s_end % kBinSweeps == 0) {   // the block closes: into the FP64 sums
+                    for (int i = lane; i < p.N; i += 32) {
+                        p.S1[(size_t)wc.q[c] * p.N + i] += (double)p1[i];
+                        p.S2[(size_t)wc.q[c] * p.N + i] += (double)p2[i];
+                        P1q[i] = P2q[i] = T(0);
+                    }
+                } else if (sh.npad) {   // the block continues in a later launch
+                    for (int i = lane; i < p.N; i += 32) {
+                        P1q[i] = p1[i];
+                        P2q[i] = p2[i];
+                    }
                 }
             }
         }
-        if (sl == 0) {
-            if (n_deg) atomicAdd(&p.counters->degenerate, (unsigned long long)n_deg);
-            if (n_zero) atomicAdd(&p.counters->zero_mode, (unsigned long long)n_zero);
-            if (n_bad) atomicAdd(&p.counters->nonfinite, (unsigned long long)n_bad);
-            if (n_rej) atomicAdd(&p.counters->prior_rejections, (unsigned long long)n_rej);
+        // counters: the solver's cap is counted by the lanes of a chain's team alike
+        const int capped = __shfl_sync(0xffffffffu, n.capped, c * (32 / C));
+        if (wc.active[c] && lane == 0) {
+            if (n.deg[c]) atomicAdd(&p.counters->degenerate, (unsigned long long)n.deg[c]);
+            if (n.zero[c]) atomicAdd(&p.counters->zero_mode, (unsigned long long)n.zero[c]);
+            if (n.bad[c]) atomicAdd(&p.counters->nonfinite, (unsigned long long)n.bad[c]);
+            if (n.rej[c]) atomicAdd(&p.counters->prior_rejections, (unsigned long long)n.rej[c]);
             if (capped) atomicAdd(&p.counters->tail_capped, (unsigned long long)capped);
         }
     }
@@ -1143,36 +1577,34 @@ __device__ __forceinline__ void consume(const SweepParams<T> &p, const LaunchSha
 // --------------------------------------------------------------------------
 // the persistent sweep kernel: the sweeps [ctrl->sweep0, + ctrl->nsweeps) of
 // every work item (problem, chain group).  Warps 0 .. consumers-1 run chains;
-// warp `consumers` produces the move records.  CTAs pull items from
-// ctrl->queue.  One problem (BATCH = false): its parameters are the launch's
-// grid constant p0.  Several: each item's parameters are copied from probs
-// into shared memory.
+// warp `consumers` produces visit packets and move records.  CTAs pull items
+// from ctrl->queue; an item's parameters are copied from probs into shared memory.
 // --------------------------------------------------------------------------
-template <class T, int KV, bool BATCH, int MINB, bool PRIOR>
-__global__ void __launch_bounds__(32 * (kMaxConsumers + 1), MINB) sweep_kernel(const __grid_constant__ SweepParams<T> p0,
-                                                    const SweepParams<T> *__restrict__ probs,
-                                                    const WorkItem *__restrict__ items, RunCtrl *ctrl,
-                                                    const __grid_constant__ LaunchShape shape)
+template <class T, int KV, int C, int MINB, bool PRIOR>
+__global__ void __launch_bounds__(32 * (kMaxConsumers + 1), MINB)
+sweep_kernel(const SweepParams<T> *__restrict__ probs, const WorkItem *__restrict__ items, RunCtrl *ctrl,
+             const __grid_constant__ LaunchShape shape)
 {
     __shared__ SweepParams<T> sp;
     __shared__ SweepRange rg;
     __shared__ int s_item;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    unsigned long long *full = reinterpret_cast<unsigned long long *>(smem_raw + shape.off_full);
-    unsigned long long *empty = reinterpret_cast<unsigned long long *>(smem_raw + shape.off_empty);
-    unsigned char *stages = smem_raw + shape.off_stages;
-    unsigned long long *ufull = reinterpret_cast<unsigned long long *>(smem_raw + shape.off_ubar);
-    unsigned long long *uempty = ufull + 2;
-    unsigned char *ubuf = smem_raw + shape.off_ubuf;
+    Regions R;
+    R.full = reinterpret_cast<unsigned long long *>(smem_raw + shape.off_bars);
+    R.empty = R.full + kMaxRingDepth;
+    R.pfull = R.empty + kMaxRingDepth;
+    R.pempty = R.pfull + kMaxPacketSlots;
+    R.packets = smem_raw + shape.off_packets;
+    R.stages = smem_raw + shape.off_stages;
     const int wcta = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
         for (int i = 0; i < shape.depth; ++i) {
-            mbar_init(full + i, 1);
-            mbar_init(empty + i, (unsigned)shape.consumers);
+            mbar_init(R.full + i, 1);
+            mbar_init(R.empty + i, (unsigned)shape.consumers);
         }
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(ufull + i, 1);
-            mbar_init(uempty + i, (unsigned)shape.consumers);
+        for (int i = 0; i < shape.pslots; ++i) {
+            mbar_init(R.pfull + i, 1);
+            mbar_init(R.pempty + i, (unsigned)shape.consumers);
         }
         fence_mbar_init();
         fence_proxy_async_smem();
@@ -1180,7 +1612,7 @@ __global__ void __launch_bounds__(32 * (kMaxConsumers + 1), MINB) sweep_kernel(c
         rg.nsweeps = ctrl->nsweeps;
         rg.burn_in = ctrl->burn_in;
     }
-    RingPos rp{0u, 0, 0u, 0u};
+    RingPos rp{0u, 0, 0u, 0u, 0, 0u};
     bool failed = false;
     for (;;) {
         if (threadIdx.x == 0) s_item = atomicAdd(&ctrl->queue, 1);
@@ -1188,70 +1620,59 @@ __global__ void __launch_bounds__(32 * (kMaxConsumers + 1), MINB) sweep_kernel(c
         const int it = s_item;
         if (it >= shape.n_items) break;
         const WorkItem w = items[it];
-        if constexpr (BATCH) {
-            if (threadIdx.x == 0) sp = probs[w.problem];
-            __syncthreads();
-        }
-        const SweepParams<T> &p = BATCH ? sp : p0;
+        static_assert(sizeof(SweepParams<T>) % 8 == 0, "copied in 8-byte words");
+        for (int i = threadIdx.x; i < (int)(sizeof(SweepParams<T>) / 8); i += blockDim.x)
+            reinterpret_cast<unsigned long long *>(&sp)[i] =
+                reinterpret_cast<const unsigned long long *>(probs + w.problem)[i];
+        __syncthreads();
         if (wcta == shape.consumers)
-            produce(p, shape, rg, full, empty, stages, ufull, uempty, ubuf, rp, failed);
+            produce(sp, shape, rg, R, rp, failed);
         else
-            consume<T, KV, PRIOR, (MINB > 1)>(p, shape, rg, w.group, smem_raw, full, empty, stages, ufull, uempty,
-                                             ubuf, rp, failed);
+            consume<T, KV, C, PRIOR, (MINB > 1)>(sp, shape, rg, w.group, smem_raw, R, rp, failed);
         __syncthreads();   // the item is finished before sp and s_item change
     }
 }
 
-template <class T, int KV, bool BATCH, int MINB, bool PRIOR>
-cudaError_t launch_sweep_kernel(const SweepParams<T> &p0, const SweepParams<T> *probs, const WorkItem *items,
-                                RunCtrl *ctrl, const LaunchShape &shape, int ctas, cudaStream_t stream)
-{
-    const size_t smem = (size_t)shape.off_stages + (size_t)shape.depth * shape.stage_bytes;
-    cudaError_t e = cudaFuncSetAttribute(sweep_kernel<T, KV, BATCH, MINB, PRIOR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-    sweep_kernel<T, KV, BATCH, MINB, PRIOR><<<(unsigned)ctas, 32 * (shape.consumers + 1), smem, stream>>>(p0, probs, items, ctrl,
-                                                                                             shape);
-    return cudaGetLastError();
-}
-
-template <class T, int KV, bool BATCH, int MINB, bool PRIOR>
-int sweep_ctas_per_sm(const LaunchShape &shape)
-{
-    const size_t smem = (size_t)shape.off_stages + (size_t)shape.depth * shape.stage_bytes;
-    if (cudaFuncSetAttribute(sweep_kernel<T, KV, BATCH, MINB, PRIOR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
-        return 0;
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, sweep_kernel<T, KV, BATCH, MINB, PRIOR>, 32 * (shape.consumers + 1),
-                                                      smem) != cudaSuccess)
-        return 0;
-    return n;
-}
-
-// dispatch over the register tile (kv) and the batch flag, for one residency
-// MINB (CTAs per SM the registers are budgeted for) and prior flag
-template <class T, int MINB, bool PRIOR, int... KVs>
-struct SweepDispatch {
-    static cudaError_t launch(const SweepParams<T> &p0, const SweepParams<T> *probs, const WorkItem *items,
-                              RunCtrl *ctrl, const LaunchShape &shape, int kv, bool batch, int ctas, cudaStream_t s)
+template <class T, int KV, int C, int MINB, bool PRIOR>
+struct SweepKernel {
+    static size_t smem(const LaunchShape &sh) { return (size_t)sh.off_stages + (size_t)sh.depth * sh.stage_bytes; }
+    static cudaError_t launch(const SweepParams<T> *probs, const WorkItem *items, RunCtrl *ctrl, const LaunchShape &sh,
+                              int ctas, cudaStream_t stream)
     {
-        cudaError_t e = cudaErrorInvalidValue;
-        ((kv == KVs ? (e = batch ? launch_sweep_kernel<T, KVs, true, MINB, PRIOR>(p0, probs, items, ctrl, shape, ctas, s)
-                                 : launch_sweep_kernel<T, KVs, false, MINB, PRIOR>(p0, probs, items, ctrl, shape, ctas, s),
-                       0)
-                    : 0),
-         ...);
-        return e;
+        const cudaError_t e = cudaFuncSetAttribute(sweep_kernel<T, KV, C, MINB, PRIOR>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(sh));
+        if (e != cudaSuccess) return e;
+        sweep_kernel<T, KV, C, MINB, PRIOR>
+            <<<(unsigned)ctas, 32 * (sh.consumers + 1), smem(sh), stream>>>(probs, items, ctrl, sh);
+        return cudaGetLastError();
     }
-    static int per_sm(const LaunchShape &shape, int kv, bool batch)
+    static int per_sm(const LaunchShape &sh)
     {
         int n = 0;
-        ((kv == KVs ? (n = batch ? sweep_ctas_per_sm<T, KVs, true, MINB, PRIOR>(shape)
-                                 : sweep_ctas_per_sm<T, KVs, false, MINB, PRIOR>(shape),
-                       0)
-                    : 0),
-         ...);
+        if (cudaFuncSetAttribute(sweep_kernel<T, KV, C, MINB, PRIOR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)smem(sh)) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, sweep_kernel<T, KV, C, MINB, PRIOR>,
+                                                          32 * (sh.consumers + 1), smem(sh)) != cudaSuccess)
+            return 0;
+        return n;
+    }
+};
+
+// dispatch over the register tile (kv) for one chain count per warp, residency MINB
+// (CTAs per SM the registers are budgeted for) and prior flag
+template <class T, int C, int MINB, bool PRIOR, int... KVs>
+struct SweepDispatch {
+    static cudaError_t launch(const SweepParams<T> *probs, const WorkItem *items, RunCtrl *ctrl, const LaunchShape &sh,
+                              int kv, int ctas, cudaStream_t s)
+    {
+        cudaError_t e = cudaErrorInvalidValue;
+        ((kv == KVs ? (e = SweepKernel<T, KVs, C, MINB, PRIOR>::launch(probs, items, ctrl, sh, ctas, s), 0) : 0), ...);
+        return e;
+    }
+    static int per_sm(const LaunchShape &sh, int kv)
+    {
+        int n = 0;
+        ((kv == KVs ? (n = SweepKernel<T, KVs, C, MINB, PRIOR>::per_sm(sh), 0) : 0), ...);
         return n;
     }
 };
