@@ -23,10 +23,10 @@ struct BlockDesc {
     int start;       // first grid point of the block
     int n;           // block width n_b
     int np;          // modes with a U column: min(M, n_b)
-    int nz;          // moves from this one on have no U column and d = 0 (flat)
+    int ng, nz;      // modes before ng are Gaussian (d > 0), from nz on flat (d = 0 in this precision)
     int rs;          // row stride of V/R rows
-    int recstride;   // elements per move record (2 rs + 4)
-    int usr;         // row stride of U in the packet (odd: conflict-free column reads)
+    int recstride;   // elements per move record: 2 rs + 4
+    int usr;         // row stride of U in the packet: M | 1 (odd: conflict-free column reads)
     int last;        // 1: the last block of its level
     long long offU;    // Ut: np x M (mode-major); Um: M x np (grid-major)
     long long offRec;  // move records of the block: n records of recstride elements

@@ -882,7 +882,10 @@ int build_precision(asm_problem *p, const HostFactors &hf, PrecBuffers &out)
         }
         // visit packet: descriptor, R_0, U with odd row stride
         T *k = &pk[B.offPk];
-        std::memcpy(k, &B, sizeof(B));
+        BlockDesc D = B;   // with this precision's runs of Gaussian and flat modes
+        while (D.ng < B.n && (T)hd[D.ng] != T(0)) ++D.ng;
+        for (D.nz = B.n; D.nz > D.ng && (T)hd[D.nz - 1] == T(0);) --D.nz;
+        std::memcpy(k, &D, sizeof(D));
         bounds_row(0, k + kPacketHeader);
         for (int j = 0; j < B.np; ++j)
             for (int m = 0; m < M; ++m)
@@ -1532,7 +1535,6 @@ int asm_setup(const asm_desc *ds, asm_problem **out)
             B.start = s0;
             B.n = s1 - s0;
             B.np = std::min(M, B.n);
-            B.nz = B.n;   // lowered when the singular values are known
             B.rs = B.n <= kRowAlignSmall ? kRowAlignSmall : round_up_int(B.n, kRowAlign);
             B.last = b + 1 == ds->level_nblocks[l];
             B.offU = oU; oU += (long long)B.np * M;
@@ -1599,11 +1601,6 @@ int asm_setup(const asm_desc *ds, asm_problem **out)
         if (rc != ASM_OK) { asm_destroy(p); return rc; }
     }
     complete_residual_update(p, hf);
-    // the tail of a block's moves that are flat in its exact null space
-    for (int b = 0; b < nb; ++b) {
-        BlockDesc &B = p->blocks[b];
-        while (B.nz > B.np && hf.d[b][B.nz - 1] == 0.0) --B.nz;
-    }
     if (given && ds->C) {
         if (!all_finite(ds->C, (size_t)M * M)) { asm_destroy(p); return ASM_ERR_NONFINITE; }
         rc = device_cholesky(ds->C, M, &p->d_L);

@@ -98,55 +98,6 @@ template <> struct TailTraits<float> {
     static constexpr float far = 10.0f;
 };
 
-// x ~ N(0,1) restricted to [a, a + w], a >= 0, 0 < w <= inf, by Q(x) = (1-u)Q(a) + uQ(b),
-// b = a + w.  The width comes in as w, formed from the interval's ends before they are
-// standardised: b - a of two standardised ends far in the tail cancels (a = 35 and
-// w = 0.03 leave w with a relative error of 2^-24 a / w = 7e-5 in FP32).
-// Returns the offset y = x - a.  The equation in y,
-//   log Q(a + y) - log Q(a) = dt,  dt = log((1-u) + u Q(b)/Q(a)),
-// is solved by Newton's method on log Q (concave, so the iterates are monotone
-// after the first step), with Q(b)/Q(a) formed through erfcx to keep narrow
-// intervals accurate.  The start is the exponential tail's inverse for a >= 5
-// and, below, y = -Phi^{-1}(q) - a with q = (1-u)Q(a) + uQ(b): accurate to a
-// few ulp of a, which FP32 keeps; in FP64 the offset form refines it so that y
-// keeps its relative accuracy however small it is.
-__device__ __forceinline__ float right_tail(float a, float w, float u, int &capped)
-{
-    const float b = a + w;
-    const float kRsqrt2 = 0.70710678118654752440f;
-    const float kSqrtPiOver2 = 1.25331413731550025121f;
-    float y;
-    if (a < 5.0f) {
-        const float qa = m_phi(-a);
-        const float qb = isinf(b) ? 0.0f : m_phi(-b);
-        const float q = (1.0f - u) * qa + u * qb;
-        y = -m_phiinv(q) - a;
-    }
-    if (a >= 5.0f) {
-        const float exa = m_erfcx(a * kRsqrt2);
-        float r = 0.0f, em = -1.0f;
-        if (!isinf(b)) {
-            const float lr = m_log(m_erfcx(b * kRsqrt2) / exa) - 0.5f * w * (a + b);
-            r = m_exp(lr);
-            em = m_expm1(lr);
-        }
-        const float dt = r < 0.5f ? m_log((1.0f - u) + u * r) : m_log1p(u * em);
-        y = -dt / a;
-        int it = 0;
-        for (; it < TailTraits<float>::nmax; ++it) {
-            const float exy = m_erfcx((a + y) * kRsqrt2);
-            const float g = m_log(exy / exa) - y * (a + 0.5f * y) - dt;
-            const float step = -g * exy * kSqrtPiOver2;   // g / g', g' = -sqrt(2/pi)/erfcx
-            y -= step;
-            if (m_abs(step) <= TailTraits<float>::tol * (y + 1.0f / a)) break;
-        }
-        if (it == TailTraits<float>::nmax) ++capped;
-    }
-    y = m_max(y, 0.0f);
-    y = m_min(y, w);
-    return y;
-}
-
 // Gauss-Legendre rule on [-1, 1] (symmetric half: nodes x > 0 and weights;
 // values of numpy.polynomial.legendre.leggauss).  8 points for FP64 (relative
 // error ~2e-16 on the narrow intervals below), 4 points for FP32 (~2e-10).
@@ -173,92 +124,6 @@ template <> struct GaussLegendre<float> {
     static constexpr float tol = 4e-7f;
     static constexpr int nmax = 12;
 };
-
-// I(t) = int_0^t exp(-a s - s^2/2) ds (the CDF of N(0,1) on [a, a+w] from a,
-// unnormalised) by Gauss-Legendre; accurate while t (|a| + t) <= 1/2.
-__device__ __forceinline__ float narrow_cdf(float a, float t)
-{
-    using GL = GaussLegendre<float>;
-    const float h = 0.5f * t;
-    float acc = 0.0f;
-#pragma unroll
-    for (int i = 0; i < GL::half; ++i) {
-        const float s1 = h * (1.0f - GL::x(i)), s2 = h * (1.0f + GL::x(i));
-        acc += GL::w(i) * (m_exp(-s1 * (a + 0.5f * s1)) + m_exp(-s2 * (a + 0.5f * s2)));
-    }
-    return h * acc;
-}
-
-// Narrow interval (w (|a| + w) <= 1/2, the Gaussian nearly flat across it):
-// solve I(t) = u I(w) by Newton's method.  The start is the inverse CDF of the
-// exponential law whose rate is the log-density's slope at the interval's
-// midpoint, lam = a + w/2: the neglected curvature changes the log-density by
-// at most w^2/8 across the interval, so one or two steps converge where the
-// flat start t = u w needed four.  The offset t from the lower end keeps its
-// relative accuracy however narrow the interval is.
-// In FP32 the start is the answer when w^2 / 8, the curvature's bound on the
-// relative error of the exponential law's CDF, lies below 2^-23 (w <= 6e-4: the
-// weak modes whose intervals are a tiny fraction of their Gaussian's width),
-// and one Newton step is when w <= 0.2: Newton's error is quadratic in the
-// start's, which is below w^2/12 relative, and one step leaves at most 1.5e-7
-// relative over the narrow regime with w <= 0.2 (measured against the root of
-// a 64-point rule at 4 million (a, w, u)), below the FP32 tolerance.
-__device__ __forceinline__ float narrow_offset(float a, float w, float u, int &capped)
-{
-    using GL = GaussLegendre<float>;
-    const float lam = a + 0.5f * w;
-    const float x = lam * w;
-    float t = m_abs(x) < 1e-3f ? u * w * (1.0f - 0.5f * x * (1.0f - u))   // the series for small lam w
-                             : -m_log1p(u * m_expm1(-x)) / lam;
-    t = m_min(m_max(t, 0.0f), w);
-    if (w * w <= 4e-7f) return t;
-    const float target = u * narrow_cdf(a, w);
-    if (w <= 0.2f) {
-        const float step = (narrow_cdf(a, t) - target) / m_exp(-t * (a + 0.5f * t));
-        return m_min(m_max(t - step, 0.0f), w);
-    }
-    int it = 0;
-    for (; it < GL::nmax; ++it) {
-        const float step = (narrow_cdf(a, t) - target) / m_exp(-t * (a + 0.5f * t));
-        t = m_min(m_max(t - step, 0.0f), w);
-        if (m_abs(step) <= GL::tol * t || t == 0.0f) break;
-    }
-    if (it == GL::nmax) ++capped;
-    return t;
-}
-
-// delta ~ N(c/d, 1/d^2) restricted to [lo, hi] (lo < hi), by the inverse CDF at u.
-// In standard units x = d delta - c the interval is [a, b] = [d lo - c, d hi - c].
-// Each branch returns delta in the form that keeps delta - lo (or hi - delta)
-// accurate relative to hi - lo.
-__device__ __forceinline__ float tn_step(float c, float d, float invd, float lo, float hi, float u, int &capped)
-{
-    const float a = m_fma(lo, d, -c);
-    const float b = m_fma(hi, d, -c);
-    const float wid = (hi - lo) * d;
-    float delta;
-    if (isfinite(wid) && wid * (m_abs(a) + wid) <= 0.5f) {
-        delta = lo + invd * narrow_offset(a, wid, u, capped);
-    } else if (a >= 0.0f) {
-        delta = lo + invd * right_tail(a, wid, u, capped);
-    } else if (b <= 0.0f) {
-        delta = hi - invd * right_tail(-b, wid, 1.0f - u, capped);
-    } else if (a < -TailTraits<float>::far && b > TailTraits<float>::far) {
-        // the truncation is below the resolution of u: the untruncated inverse CDF
-        const float x = u <= 0.5f ? m_phiinv(u) : -m_phiinv(1.0f - u);
-        delta = (x + c) * invd;
-    } else {
-        const float p = (1.0f - u) * m_phi(a) + u * m_phi(b);
-        float x;
-        if (p <= 0.5f) {
-            x = m_phiinv(p);
-        } else {
-            x = -m_phiinv((1.0f - u) * m_phi(-a) + u * m_phi(-b));
-        }
-        delta = (x + c) * invd;
-    }
-    return m_min(m_max(delta, lo), hi);
-}
 
 // elements of a 16-byte vector
 template <class T> struct VecOf;
@@ -473,6 +338,13 @@ __device__ __forceinline__ void warp_bounds(const long long (&lk)[C], const unsi
     }
 }
 
+// A value that is the same in all lanes, broadcast so that the compiler knows it too.
+// Loop bounds and branch conditions read from shared memory count as divergent
+// otherwise: every loop then carries reconvergence and every redux or shuffle a
+// warp synchronisation.
+template <class I>
+__device__ __forceinline__ I uni(I x) { return __shfl_sync(0xffffffffu, x, 0); }
+
 // lo < hi for bounds that come from keys: lo is -0 or below, hi +0 or above, neither
 // is NaN, so they differ unless both are zeros.  FP64 as an integer test: a DSETP would
 // occupy the FP64 pipe for 64 cycles.
@@ -518,33 +390,217 @@ __device__ __forceinline__ void lds_mode(const double *p, double &d, double &inv
 }
 
 // --------------------------------------------------------------------------
-// The draw by a team of lanes.  A warp holds C chains; every lane of the G = 32/C
-// lanes of a chain's team has the same arguments.
+// The draw: delta ~ N(c/d, 1/d^2) restricted to [lo, hi] (lo < hi), by the inverse
+// CDF at u.  In standard units x = d delta - c the interval is [a, b] =
+// [d lo - c, d hi - c].  Each branch returns delta in the form that keeps delta - lo
+// (or hi - delta) accurate relative to hi - lo.
 //
-// FP32: each lane draws for its team's chain, so C draws cost one.
+// Narrow interval, w (|a| + w) <= 1/2 with w = b - a (the Gaussian nearly flat across
+// it): the offset t from a solves I(t) = u I(w), I(t) = int_0^t exp(-a s - s^2/2) ds by
+// Gauss-Legendre (accurate while t (|a| + t) <= 1/2), by Newton's method.  The start is
+// the inverse CDF of the exponential law whose rate is the log-density's slope at the
+// interval's midpoint, lam = a + w/2: the neglected curvature changes the log-density by
+// at most w^2/8 across the interval, so one or two steps converge where the flat start
+// t = u w needed four.  The offset keeps its relative accuracy however narrow the
+// interval is.  In FP32 the start is the answer when w^2 / 8, the curvature's bound on
+// the relative error of the exponential law's CDF, lies below 2^-23 (w <= 6e-4: the weak
+// modes whose intervals are a tiny fraction of their Gaussian's width), and one Newton
+// step is when w <= 0.2: Newton's error is quadratic in the start's, which is below
+// w^2/12 relative, and one step leaves at most 1.5e-7 relative over the narrow regime
+// with w <= 0.2 (measured against the root of a 64-point rule at 4 million (a, w, u)),
+// below the FP32 tolerance.
 //
-// FP64: one warp instruction of the FP64 pipe takes 64 cycles of a sub-partition
-// whether one lane is active or all are, so the draw's independent function
-// values go to different lanes: the eight exponentials of the quadrature (and,
-// where the team is wide enough, those of the target's quadrature and of the
-// density that Newton's step divides by) are one exponential, and the pairs
-// Phi(a), Phi(b) and erfcx(a), erfcx(b) one call each.  Sums are formed from
-// the lanes' values in the order of the scalar code, so the draw is the same
-// bit for bit.
+// Tail, x in [a, a + w], a >= 0, 0 < w <= inf, by Q(x) = (1-u)Q(a) + uQ(b), b = a + w.
+// The width comes in as w, formed from the interval's ends before they are
+// standardised: b - a of two standardised ends far in the tail cancels (a = 35 and
+// w = 0.03 leave w with a relative error of 2^-24 a / w = 7e-5 in FP32).  The equation
+// in the offset y = x - a,
+//   log Q(a + y) - log Q(a) = dt,  dt = log((1-u) + u Q(b)/Q(a)),
+// is solved by Newton's method on log Q (concave, so the iterates are monotone after the
+// first step), with Q(b)/Q(a) formed through erfcx to keep narrow intervals accurate.
+// The start is the exponential tail's inverse for a >= 5 and, below,
+// y = -Phi^{-1}(q) - a with q = (1-u)Q(a) + uQ(b): accurate to a few ulp of a, which
+// FP32 keeps; in FP64 the offset form refines it so that y keeps its relative accuracy
+// however small it is.  Otherwise x is the normal quantile of (1-u) Phi(a) + u Phi(b),
+// taken from the side with the smaller mass.
+//
+// A warp holds C chains; every lane of the G = 32/C lanes of a chain's team has the same
+// arguments, so the C draws of a move cost one.  The draw's independent function values
+// go to different lanes: the pairs Phi(a), Phi(b) and erfcx(a), erfcx(b) are one call
+// each, and in FP64 the exponentials of the quadratures at t and at w and of the density
+// that Newton's step divides by are one exponential.  A warp instruction of the FP64 pipe
+// takes 64 cycles of a sub-partition whether one lane is active or all are, so that is a
+// quarter of the time of the scalar form (plain modes FP64, 50 points, 16 chains: 0.403
+// -> 0.168 ms a sweep); in FP32 it shortens the instruction stream (the hierarchy of 64
+// points, 1024 chains: 0.092 -> 0.071 ms a sweep).  Sums are formed from
+// the lanes' values in one order for every team width, and products that could be fused
+// either way are written out, so that a draw does not depend on C.
 // --------------------------------------------------------------------------
-template <int G>
-__device__ __forceinline__ float tn_step_team(float c, float d, float invd, float lo, float hi, float u, bool open,
-                                              int, int &capped)
-{
-    return open ? tn_step(c, d, invd, lo, hi, u, capped) : 0.0f;
-}
-
 template <int G>
 struct TeamLanes {
     unsigned mask;   // lanes of the warp that run this path (whole teams)
     int base, gl;    // first lane of the team, lane within the team
-    __device__ __forceinline__ double from(double v, int l) const { return __shfl_sync(mask, v, base + l); }
+    template <class T>
+    __device__ __forceinline__ T from(T v, int l) const { return __shfl_sync(mask, v, base + l); }
 };
+
+// f(x0) and f(x1) from one call: the even lanes take x0, the odd ones x1.
+template <int G, class T, class F>
+__device__ __forceinline__ void pair_of(F f, T x0, T x1, const TeamLanes<G> &tl, T &y0, T &y1)
+{
+    const T y = f((tl.gl & 1) ? x1 : x0);
+    y0 = tl.from(y, 0);
+    y1 = tl.from(y, 1);
+}
+
+// ---- FP32 ----------------------------------------------------------------
+
+// n / d, correctly rounded, from r = the correctly rounded 1 / d (Markstein 1990: the
+// remainder is exact in a fused multiply-add; the second step makes it correct where the
+// first product was off by more than an ulp).  For d well inside the normal range.
+__device__ __forceinline__ float div_by(float n, float d, float r)
+{
+    const float q0 = __fmul_rn(n, r);
+    const float q1 = __fmaf_rn(__fmaf_rn(-q0, d, n), r, q0);
+    return __fmaf_rn(__fmaf_rn(-q1, d, n), r, q1);
+}
+
+// I(t) / (t/2) by the quadrature.
+__device__ __forceinline__ float narrow_sum(float a, float t)
+{
+    using GL = GaussLegendre<float>;
+    const float h = 0.5f * t;
+    float acc = 0.0f;
+#pragma unroll
+    for (int i = 0; i < GL::half; ++i) {
+        const float s1 = h * (1.0f - GL::x(i)), s2 = h * (1.0f + GL::x(i));
+        acc = fmaf(GL::w(i), m_exp(-s1 * (a + 0.5f * s1)) + m_exp(-s2 * (a + 0.5f * s2)), acc);
+    }
+    return acc;
+}
+
+// The offset in a narrow interval.  Every lane evaluates the whole quadrature: four
+// exponentials in flight together are no slower than one and the shuffles that would
+// spread and collect them, and those of the target do not wait for the start.
+__device__ __forceinline__ float narrow_offset(float a, float w, float u, int &capped)
+{
+    using GL = GaussLegendre<float>;
+    const float lam = a + 0.5f * w;
+    const float x = lam * w;
+    float t = m_abs(x) < 1e-3f ? u * w * (1.0f - 0.5f * x * (1.0f - u))   // the series for small lam w
+                               : -m_log1p(u * m_expm1(-x)) / lam;
+    t = m_min(m_max(t, 0.0f), w);
+    if (w * w <= 4e-7f) return t;
+    const float target = __fmul_rn(u, __fmul_rn(0.5f * w, narrow_sum(a, w)));
+    int it = 0;
+    for (; it < GL::nmax; ++it) {
+        const float step = fmaf(0.5f * t, narrow_sum(a, t), -target) / m_exp(-t * (a + 0.5f * t));
+        t = m_min(m_max(t - step, 0.0f), w);
+        if (w <= 0.2f || m_abs(step) <= GL::tol * t || t == 0.0f) break;
+    }
+    if (it == GL::nmax) ++capped;
+    return t;
+}
+
+// The offset in a tail beyond a = 5.
+template <int G>
+__device__ __forceinline__ float far_tail_team(float a, float w, float u, const TeamLanes<G> &tl, int &capped)
+{
+    const float b = a + w;
+    const float kRsqrt2 = 0.70710678118654752440f;
+    const float kSqrtPiOver2 = 1.25331413731550025121f;
+    float exa, exb;
+    pair_of<G>([](float z) { return m_erfcx(z); }, a * kRsqrt2, b * kRsqrt2, tl, exa, exb);
+    float r = 0.0f, lr = 0.0f;
+    if (!isinf(b)) {
+        lr = m_log(exb / exa) - 0.5f * w * (a + b);
+        r = m_exp(lr);
+    }
+    const float dt = r < 0.5f ? m_log((1.0f - u) + u * r) : m_log1p(u * m_expm1(lr));
+    float y = -dt / a;
+    const float inva = 1.0f / a, invx = __frcp_rn(exa);
+    const bool plain = exa > 1e-25f;
+    int it = 0;
+    for (; it < TailTraits<float>::nmax; ++it) {
+        const float exy = m_erfcx((a + y) * kRsqrt2);
+        const float ratio = plain ? div_by(exy, exa, invx) : exy / exa;
+        const float g = m_log(ratio) - y * (a + 0.5f * y) - dt;
+        const float step = -g * exy * kSqrtPiOver2;   // g / g', g' = -sqrt(2/pi)/erfcx
+        y -= step;
+        if (m_abs(step) <= TailTraits<float>::tol * (y + inva)) break;
+    }
+    if (it == TailTraits<float>::nmax) ++capped;
+    return m_min(m_max(y, 0.0f), w);
+}
+
+// The draw for the chains of a warp, FP32 (called by the whole warp; teams whose
+// interval is not open return 0).  The branches that go through the normal quantile
+// (the centre, tails nearer than 5, the interval that does not truncate) share one call
+// of Phi for both ends and one quantile: the draw is most of the instructions of a
+// workload with many Gaussian modes, and inlined per branch it overran the
+// instruction cache.
+template <int G>
+__device__ __forceinline__ float draw_team(float c, float d, float invd, float lo, float hi, float u, bool open,
+                                              int lane, int &capped)
+{
+    TeamLanes<G> tl;
+    tl.base = lane & ~(G - 1);
+    tl.gl = lane & (G - 1);
+    const float a = m_fma(lo, d, -c);
+    const float b = m_fma(hi, d, -c);
+    const float wid = (hi - lo) * d;
+    const bool narrow = open && isfinite(wid) && wid * (m_abs(a) + wid) <= 0.5f;
+    const bool right = !narrow && a >= 0.0f, left = !narrow && !right && b <= 0.0f, tail = right || left;
+    const float ta = right ? a : -b, tu = right ? u : 1.0f - u;   // the tail's near end and uniform
+    const bool far = open && tail && ta >= 5.0f, quantile = open && !narrow && !far;
+    const unsigned mn = __ballot_sync(0xffffffffu, narrow), mf = __ballot_sync(0xffffffffu, far),
+                   mq = __ballot_sync(0xffffffffu, quantile);
+    float delta = 0.0f;
+    if (G == 32 ? mn != 0u : narrow) {   // one chain: uniform branches
+        delta = lo + invd * narrow_offset(a, wid, u, capped);
+    } else if (G == 32 ? mf != 0u : far) {
+        tl.mask = mf;
+        const float y = far_tail_team<G>(ta, wid, tu, tl, capped);
+        delta = right ? lo + invd * y : hi - invd * y;
+    } else if (G == 32 ? mq != 0u : quantile) {
+        // both ends beyond: the truncation is below the resolution of u
+        const bool untruncated = !tail && a < -TailTraits<float>::far && b > TailTraits<float>::far;
+        float q = u <= 0.5f ? u : 1.0f - u;
+        bool neg = u > 0.5f;
+        tl.mask = __ballot_sync(mq, !untruncated);
+        if (!untruncated) {
+            const float tb = ta + wid;
+            float A = tail ? -ta : a, B = tail ? -tb : b;
+            const float v = tail ? tu : u;
+            neg = tail;
+            for (;;) {
+                float pa, pb;
+                pair_of<G>([](float z) { return m_phi(z); }, A, B, tl, pa, pb);
+                if (tail && isinf(tb)) pb = 0.0f;
+                // the larger half of the centre is taken from the other side: q and its mirror image
+                // (1-v) pa + v pb; the mirror image rounds the other product first
+                const bool mirror = neg && !tail;
+                q = fmaf(mirror ? v : 1.0f - v, mirror ? pb : pa, __fmul_rn(mirror ? 1.0f - v : v, mirror ? pa : pb));
+                const bool again = !neg && q > 0.5f;
+                tl.mask = __ballot_sync(tl.mask, again);
+                if (!again) break;
+                A = -a;
+                B = -b;
+                neg = true;
+            }
+        }
+        const float z = m_phiinv(q), x = neg ? -z : z;
+        if (tail) {
+            const float y = m_min(m_max(x - ta, 0.0f), wid);
+            delta = right ? lo + invd * y : hi - invd * y;
+        } else {
+            delta = (x + c) * invd;
+        }
+    }
+    return open ? m_min(m_max(delta, lo), hi) : 0.0f;
+}
+
+// ---- FP64 ----------------------------------------------------------------
 
 // 1 - x or 1 + x of the quadrature node of a lane: lanes 2i, 2i + 1 of eight take node i.
 __device__ __forceinline__ double gl_node(int lane)
@@ -612,15 +668,6 @@ __device__ __forceinline__ double narrow_offset_team(double a, double w, double 
     return t;
 }
 
-// f(x0) and f(x1) from one call: the even lanes take x0, the odd ones x1.
-template <int G, class F>
-__device__ __forceinline__ void pair_of(F f, double x0, double x1, const TeamLanes<G> &tl, double &y0, double &y1)
-{
-    const double y = f((tl.gl & 1) ? x1 : x0);
-    y0 = tl.from(y, 0);
-    y1 = tl.from(y, 1);
-}
-
 template <int G>
 __device__ __forceinline__ double right_tail_team(double a, double w, double u, TeamLanes<G> tl, int &capped)
 {
@@ -663,10 +710,10 @@ __device__ __forceinline__ double right_tail_team(double a, double w, double u, 
     return y;
 }
 
-// tn_step for the chains of a warp, FP64 (called by the whole warp; teams whose
+// The draw for the chains of a warp, FP64 (called by the whole warp; teams whose
 // interval is not open return 0).
 template <int G>
-__device__ __forceinline__ double tn_step_team(double c, double d, double invd, double lo, double hi, double u, bool open,
+__device__ __forceinline__ double draw_team(double c, double d, double invd, double lo, double hi, double u, bool open,
                                                int lane, int &capped)
 {
     TeamLanes<G> tl;
@@ -769,9 +816,9 @@ __device__ __forceinline__ bool u_staged(const LaunchShape &sh, const BlockDesc 
 }
 // Records of a block per ring stage.
 template <class T>
-__device__ __forceinline__ int records_per_stage(const LaunchShape &sh, const BlockDesc &B)
+__device__ __forceinline__ int records_per_stage(const LaunchShape &sh, int recstride)
 {
-    return min(kMaxRecordsPerStage, sh.stage_bytes / (int)(B.recstride * sizeof(T)));
+    return min(kMaxRecordsPerStage, sh.stage_bytes / (int)(recstride * sizeof(T)));
 }
 
 __device__ __forceinline__ int level_of_sweep(long long s, unsigned long long seed, unsigned long long pid,
@@ -863,7 +910,7 @@ __device__ __forceinline__ void produce(const SweepParams<T> &p, const LaunchSha
         mbar_expect_tx(R.pfull + rp.pslot, pbytes);
         bulk_g2s(R.packets + (size_t)rp.pslot * sh.pbytes, p.pd.pk + B.offPk, pbytes, R.pfull + rp.pslot);
         packet_next(rp, P);
-        const int rps = records_per_stage<T>(sh, B);
+        const int rps = records_per_stage<T>(sh, B.recstride);
         for (int j = 0; j < B.n; j += rps) {
             if (rp.g >= (unsigned)D && !mbar_wait(R.empty + rp.slot, rp.phase ^ 1u, sh.wait_limit)) {
                 failed = true;
@@ -1152,14 +1199,70 @@ struct Visit {
         for (int c = 0; c < C; ++c) kk[c].fold(lk[c], hk[c]);
     }
 
+    // The residual moves by K~_b V_j delta = dres_j delta U_j (dres = d for a Gaussian mode,
+    // |K~_b V_j| for one sampled flat); all lanes store the same.
+    static __device__ __forceinline__ void store_w(const WarpChains<T, C> &wc, int j, int np, T dres, const T (&delta)[C])
+    {
+        if (j < np) {
+#pragma unroll
+            for (int c = 0; c < C; ++c) wc.w_(c)[j] = dres * delta[c];
+        }
+    }
+
+    // Gamma prior (Eq. compat): the draw is a proposal, accepted with probability
+    // min(1, prod ((f + delta V)_+ / f)^(a - 1)) over the block.
+    static __device__ __forceinline__ void prior_step(const SweepParams<T> &p, const T (&f)[C][KK][VE], T (&delta)[C],
+                                                      const T (&v0)[VE], const T *st, T ua, int bn, int bstart, int kcnt,
+                                                      int lane, unsigned (&rej)[C])
+    {
+        if (delta[0] == T(0)) return;
+        T lsum = T(0);
+        unsigned zflags = 0u;   // 1: a proposed value is 0, 2: a current value is 0
+#pragma unroll
+        for (int k = 0; k < KK; ++k) {
+            if (!CHK || k < kcnt) {
+                T vv[VE];
+                if (k == 0) {
+#pragma unroll
+                    for (int v = 0; v < VE; ++v) vv[v] = v0[v];
+                } else {
+                    lds_v(st + VE * (32 * k + lane), vv);
+                }
+#pragma unroll
+                for (int v = 0; v < VE; ++v) {
+                    const int nl = VE * (32 * k + lane) + v;
+                    if (nl < bn) {
+                        const T am1 = __ldg(p.prior_am1 + bstart + nl);
+                        if (am1 != T(0)) {
+                            const T x0 = f[0][k][v];
+                            const T x1 = m_max(m_fma(delta[0], vv[v], x0), T(0));
+                            if (x1 == T(0)) zflags |= 1u;
+                            else if (x0 == T(0)) zflags |= 2u;
+                            else lsum += am1 * (m_log(x1) - m_log(x0));
+                        }
+                    }
+                }
+            }
+        }
+        for (int off = 1; off < 32; off <<= 1) {
+            lsum += __shfl_xor_sync(0xffffffffu, lsum, off);
+            zflags |= __shfl_xor_sync(0xffffffffu, zflags, off);
+        }
+        const T lr = (zflags & 1u) ? -CUDART_INF_F : (zflags & 2u) ? CUDART_INF_F : lsum;
+        if (!(m_log(ua) < lr)) {
+            delta[0] = T(0);
+            ++rej[0];
+        }
+    }
+
     // false: a bounded wait gave up
     static __device__ __forceinline__ bool run(const SweepParams<T> &p, const LaunchShape &sh, const Regions &R, RingPos &rp,
                                                const WarpChains<T, C> &wc, MoveCounts<C> &n, const BlockDesc &B,
                                                const T *pk, const T *Us, long long s, bool keep, bool trace, int &win,
                                                int &win_end, int lane, T (&sd2)[C], T (&sf2)[C])
     {
-        const int kcnt = (B.n + 32 * VE - 1) / (32 * VE);
-        const int bn = B.n, bstart = B.start, rs = B.rs, recstride = B.recstride, np = B.np;
+        const int bn = uni(B.n), bstart = uni(B.start), rs = uni(B.rs), np = uni(B.np), recstride = 2 * rs + 4;
+        const int kcnt = (bn + 32 * VE - 1) / (32 * VE);
         T f[C][KK][VE];
 #pragma unroll
         for (int c = 0; c < C; ++c) {
@@ -1191,8 +1294,10 @@ struct Visit {
 #pragma unroll
             for (int c = 0; c < C; ++c) kk[c].fold(lk[c], hk[c]);
         }
-        const int rps = records_per_stage<T>(sh, B);
-        const int nz = B.nz;       // moves from nz on are flat and leave the residual alone
+        const int rps = records_per_stage<T>(sh, recstride);
+        // modes j < ng are Gaussian, those from nz on flat; in between both occur (never, when
+        // the singular values are sorted)
+        const int ng = uni(B.ng), nz = uni(B.nz);
         int jr = 0;                // record of move j within its ring stage
         const T *stb = nullptr;    // the stage holding move j's record
         for (int j = 0; j < bn;) {
@@ -1232,32 +1337,44 @@ struct Visit {
                 if (!warp_wait(R.full + rp.slot, rp.phase, sh.wait_limit)) return false;
                 stb = reinterpret_cast<const T *>(R.stages + (size_t)rp.slot * sh.stage_bytes);
             }
-            // this segment's moves: up to the end of the window, of the stage, of the modes
-            // that need more than their rows, or of the block
+            // this segment's moves: up to the end of the window, of the stage, of the modes of
+            // one kind or of the block
             const int jbeg = j;
             int jend = min(min(bn, win_end - bstart), j + (rps - jr));
             const T *st = stb + (size_t)jr * recstride;
             const T *up = wc.u_(0) + (bstart - win);
-            if (!PRIOR && j >= nz) {
-                // flat moves in the block's null space: bounds, a uniform and the pass
+            bool flat = j >= nz;
+            if (j < ng) {
+                jend = min(jend, ng);
+            } else if (!flat) {   // a mode between: one move, by its own d
+                jend = j + 1;
+                flat = uni((int)is_zero(st[2 * rs])) != 0;
+            }
+            if (flat) {
                 unsigned opened[C];
 #pragma unroll
                 for (int c = 0; c < C; ++c) opened[c] = 0u;
 #pragma unroll 1
                 for (; j < jend; ++j, st += recstride) {
                     T u[C], v0[VE], r0[VE], lo[C], hi[C], delta[C];
+                    // chunk 0 of the pass and the mode's data do not depend on the bounds: loaded first
+                    const T dres = st[2 * rs + 2];
 #pragma unroll
                     for (int c = 0; c < C; ++c) u[c] = up[j + c * wc.tw];
                     lds_v(st + VE * lane, v0);
                     lds_v(st + rs + VE * lane, r0);
                     warp_bounds<C>(lk, hk, lo, hi);
+                    // degenerate interval: no move; else flat on [lo, hi] (both bounds finite:
+                    // set-up rejects zero modes that do not change sign)
 #pragma unroll
                     for (int c = 0; c < C; ++c) {
                         const bool open = open_interval(lo[c], hi[c]);
                         delta[c] = open ? m_fma(u[c], hi[c] - lo[c], lo[c]) : T(0);
                         opened[c] += open ? 1u : 0u;
                     }
+                    if constexpr (PRIOR) prior_step(p, f, delta, v0, st, up[128 + j], bn, bstart, kcnt, lane, n.rej);
                     pass(f, delta, v0, r0, st, rs, kcnt, lane, lk, hk);
+                    store_w(wc, j, np, dres, delta);
                 }
 #pragma unroll
                 for (int c = 0; c < C; ++c) {
@@ -1265,101 +1382,40 @@ struct Visit {
                     n.deg[c] += (unsigned)(j - jbeg) - opened[c];
                 }
             } else {
-                if (!PRIOR) jend = min(jend, nz);
 #pragma unroll 1
                 for (; j < jend; ++j, st += recstride) {
                     T u[C], v0[VE], r0[VE], lo[C], hi[C], delta[C], dj, ij, dres;
-                    // chunk 0 of the pass and the mode's data do not depend on the bounds: loaded first
                     lds_mode(st + 2 * rs, dj, ij, dres);
 #pragma unroll
                     for (int c = 0; c < C; ++c) u[c] = up[j + c * wc.tw];
                     lds_v(st + VE * lane, v0);
                     lds_v(st + rs + VE * lane, r0);
                     warp_bounds<C>(lk, hk, lo, hi);
-                    // degenerate interval: no move; zero mode: flat on [lo, hi] (both bounds
-                    // finite: set-up rejects zero modes that do not change sign); else the
-                    // truncated Gaussian.  The branch is on the record's d_j, the same for all
-                    // chains and known long before the bounds.
-                    if (is_zero(dj)) {
+                    // degenerate interval: no move; else the truncated Gaussian
+                    constexpr int G = 32 / C;
+                    T l = lo[0], h = hi[0], uu = u[0];
+                    const T *cs = wc.c_(0);
 #pragma unroll
-                        for (int c = 0; c < C; ++c) {
-                            const bool open = open_interval(lo[c], hi[c]);
-                            delta[c] = open ? m_fma(u[c], hi[c] - lo[c], lo[c]) : T(0);
-                            n.zero[c] += open ? 1u : 0u;
-                            n.deg[c] += open ? 0u : 1u;
-                        }
-                    } else {
-                        constexpr int G = 32 / C;
-                        T l = lo[0], h = hi[0], uu = u[0];
-                        const T *cs = wc.c_(0);
-#pragma unroll
-                        for (int c = 1; c < C; ++c) {
-                            const bool mine = lane / G == c;
-                            l = mine ? lo[c] : l;
-                            h = mine ? hi[c] : h;
-                            uu = mine ? u[c] : uu;
-                            cs = mine ? wc.c_(c) : cs;
-                        }
-                        const T cj = j < np ? cs[j] : T(0);
-                        T dl = tn_step_team<G>(cj, dj, ij, l, h, uu, open_interval(l, h), lane, n.capped);
-#pragma unroll
-                        for (int c = 0; c < C; ++c) {
-                            const T x = C == 1 ? dl : __shfl_sync(0xffffffffu, dl, c * G);
-                            const bool fin = is_finite(x);
-                            n.bad[c] += fin ? 0u : 1u;
-                            n.deg[c] += open_interval(lo[c], hi[c]) ? 0u : 1u;
-                            delta[c] = fin ? x : T(0);
-                        }
+                    for (int c = 1; c < C; ++c) {
+                        const bool mine = lane / G == c;
+                        l = mine ? lo[c] : l;
+                        h = mine ? hi[c] : h;
+                        uu = mine ? u[c] : uu;
+                        cs = mine ? wc.c_(c) : cs;
                     }
-                    if constexpr (PRIOR) if (delta[0] != T(0)) {
-                        // gamma prior (Eq. compat): the draw is a proposal, accepted with
-                        // probability min(1, prod ((f + delta V)_+ / f)^(a - 1)) over the block
-                        T lsum = T(0);
-                        unsigned zflags = 0u;   // 1: a proposed value is 0, 2: a current value is 0
+                    const T cj = j < np ? cs[j] : T(0);
+                    const T dl = draw_team<G>(cj, dj, ij, l, h, uu, open_interval(l, h), lane, n.capped);
 #pragma unroll
-                        for (int k = 0; k < KK; ++k) {
-                            if (!CHK || k < kcnt) {
-                                T vv[VE];
-                                if (k == 0) {
-#pragma unroll
-                                    for (int v = 0; v < VE; ++v) vv[v] = v0[v];
-                                } else {
-                                    lds_v(st + VE * (32 * k + lane), vv);
-                                }
-#pragma unroll
-                                for (int v = 0; v < VE; ++v) {
-                                    const int nl = VE * (32 * k + lane) + v;
-                                    if (nl < bn) {
-                                        const T am1 = __ldg(p.prior_am1 + bstart + nl);
-                                        if (am1 != T(0)) {
-                                            const T x0 = f[0][k][v];
-                                            const T x1 = m_max(m_fma(delta[0], vv[v], x0), T(0));
-                                            if (x1 == T(0)) zflags |= 1u;
-                                            else if (x0 == T(0)) zflags |= 2u;
-                                            else lsum += am1 * (m_log(x1) - m_log(x0));
-                                        }
-                                    }
-                                }
-                            }
-                        }
-                        for (int off = 1; off < 32; off <<= 1) {
-                            lsum += __shfl_xor_sync(0xffffffffu, lsum, off);
-                            zflags |= __shfl_xor_sync(0xffffffffu, zflags, off);
-                        }
-                        const T lr = (zflags & 1u) ? -CUDART_INF_F : (zflags & 2u) ? CUDART_INF_F : lsum;
-                        const T ua = up[128 + j];
-                        if (!(m_log(ua) < lr)) {
-                            delta[0] = T(0);
-                            ++n.rej[0];
-                        }
+                    for (int c = 0; c < C; ++c) {
+                        const T x = C == 1 ? dl : __shfl_sync(0xffffffffu, dl, c * G);
+                        const bool fin = is_finite(x);
+                        n.bad[c] += fin ? 0u : 1u;
+                        n.deg[c] += open_interval(lo[c], hi[c]) ? 0u : 1u;
+                        delta[c] = fin ? x : T(0);
                     }
+                    if constexpr (PRIOR) prior_step(p, f, delta, v0, st, up[128 + j], bn, bstart, kcnt, lane, n.rej);
                     pass(f, delta, v0, r0, st, rs, kcnt, lane, lk, hk);
-                    // the residual moves by K~_b V_j delta = dres_j delta U_j (dres = d for a
-                    // Gaussian mode, |K~_b V_j| for one sampled flat); all lanes store the same
-                    if (j < np) {
-#pragma unroll
-                        for (int c = 0; c < C; ++c) wc.w_(c)[j] = dres * delta[c];
-                    }
+                    store_w(wc, j, np, dres, delta);
                 }
             }
             // release the stage to the producer after its last record (one arrival per warp)
@@ -1423,7 +1479,7 @@ __device__ __forceinline__ void consume(const SweepParams<T> &p, const LaunchSha
     constexpr int VEC = VecOf<T>::n;
     if (failed) return;
     const int lane = threadIdx.x & 31;
-    const int wcta = threadIdx.x >> 5;
+    const int wcta = uni((int)(threadIdx.x >> 5));
     WarpChains<T, C> wc;
     // per chain in shared memory: c (cpad), w (cpad), r~ (mpad), the uniforms of the current
     // window of 128 moves (with a prior 128 more) and, where they fit, the chain state (fpad)
@@ -1471,9 +1527,10 @@ __device__ __forceinline__ void consume(const SweepParams<T> &p, const LaunchSha
     __syncwarp();
 
     const bool trace = p.steptrace != nullptr;   // step-size trace of Fig. MCsteps (diagnostic)
-    const long long s_end = rg.sweep0 + rg.nsweeps;
-    for (long long s = rg.sweep0; s < s_end && !failed; ++s) {
-        const bool keep = s >= rg.burn_in;
+    const long long s_begin = uni(rg.sweep0), s_end = s_begin + uni(rg.nsweeps), burn_in = uni(rg.burn_in);
+    const int M = uni(p.M);
+    for (long long s = s_begin; s < s_end && !failed; ++s) {
+        const bool keep = s >= burn_in;
         int win = 0, win_end = -1;  // window [win, win_end) of moves whose uniforms are in shared memory
         T sd2[C], sf2[C];           // this lane's |f(s+1) - f(s)|^2 and |f(s)|^2 (trace only)
 #pragma unroll
@@ -1487,18 +1544,19 @@ __device__ __forceinline__ void consume(const SweepParams<T> &p, const LaunchSha
             }
             const T *pk = reinterpret_cast<const T *>(R.packets + (size_t)rp.pslot * sh.pbytes);
             const BlockDesc &B = *reinterpret_cast<const BlockDesc *>(pk);
-            last = B.last != 0;
-            const T *Us = u_staged<T>(sh, B) ? pk + kPacketHeader + B.rs : nullptr;
-            project_entry<T, C, KV * C, WIDE>(wc, Us, p.pd.Um + B.offU, B.np, B.usr, p.M, lane);
+            last = uni(B.last) != 0;
+            const int bn = uni(B.n), np = uni(B.np), usr = M | 1;
+            const T *Us = uni((int)u_staged<T>(sh, B)) ? pk + kPacketHeader + B.rs : nullptr;
+            project_entry<T, C, KV * C, WIDE>(wc, Us, p.pd.Um + B.offU, np, usr, M, lane);
             __syncwarp();
             bool ok;
-            if (B.n <= 16 * VEC)
+            if (bn <= 16 * VEC)
                 ok = Visit<T, KV, C, PRIOR, 1, VEC / 2>::run(p, sh, R, rp, wc, n, B, pk, Us, s, keep, trace, win, win_end,
                                                              lane, sd2, sf2);
-            else if (KV == 1 || B.n <= 32 * VEC)
+            else if (KV == 1 || bn <= 32 * VEC)
                 ok = Visit<T, KV, C, PRIOR, 1, VEC>::run(p, sh, R, rp, wc, n, B, pk, Us, s, keep, trace, win, win_end, lane,
                                                          sd2, sf2);
-            else if (KV == 2 || B.n > 32 * VEC * (KV - 1))
+            else if (KV == 2 || bn > 32 * VEC * (KV - 1))
                 ok = Visit<T, KV, C, PRIOR, KV, VEC>::run(p, sh, R, rp, wc, n, B, pk, Us, s, keep, trace, win, win_end, lane,
                                                           sd2, sf2);
             else
@@ -1509,7 +1567,7 @@ __device__ __forceinline__ void consume(const SweepParams<T> &p, const LaunchSha
                 break;
             }
             __syncwarp();
-            project_exit<T, C, KV * C, WIDE>(wc, Us, p.pd.Ut + B.offU, B.np, B.usr, p.M, lane);
+            project_exit<T, C, KV * C, WIDE>(wc, Us, p.pd.Ut + B.offU, np, usr, M, lane);
             // release the packet to the producer (one arrival per warp)
             __syncwarp();
             mbar_arrive_lane0(R.pempty + rp.pslot, lane);
