@@ -225,9 +225,12 @@ constexpr int kStepTraceMax = 4096;
 constexpr int kMaxConsumers = 7;
 // Deepest ring of move records (stages) a launch may use.
 constexpr int kMaxRingDepth = 48;
-// Move records of the largest block per ring stage (one barrier wait and one release
-// per stage); smaller blocks put up to kMaxRecordsPerStage in a stage of that size.
+// Move records of the largest block per ring stage: up to kMaxLargeRecords where shared
+// memory allows, at least kRecordsPerStage while three stages fit (a stage costs a consumer
+// its wait, its release and the start of its loop); smaller blocks put up to
+// kMaxRecordsPerStage in a stage of that size.
 constexpr int kRecordsPerStage = 4;
+constexpr int kMaxLargeRecords = 8;
 constexpr int kMaxRecordsPerStage = 16;
 // Most slots of the ring of visit packets.
 constexpr int kMaxPacketSlots = 8;

@@ -1019,48 +1019,88 @@ struct PlanNeeds {
     std::vector<int> packets;        // bytes of every block's packet with U
 };
 
+// Chains per warp (C) and chain warps per CTA (w) of a launch: the pair with the shortest
+// estimated run.  The chains of a warp share its row loads and its draws but also its issue
+// slots, and up to four warps have a sub-partition each, so a CTA's time (in units of C = 1,
+// w = 7) is kCta[C][w] below: blocked modes, N = 400, one CTA per SM, FP32 (1.0 = 0.083 ms a sweep;
+// FP64 scales alike, 1.0 = 1.32 ms).  A problem's items then take ceil(items / SMs) waves, those of
+// a batch (uneven, longest first) the longest item or the mean load of an SM and part of the longest.  So one chain per warp up to one wave
+// of 1064 chains, two up to 2128, four beyond, except where a last wave would be nearly empty (ms a
+// sweep for C = 1, 2, 4: 1024 chains 0.083, 0.106, 0.150; 2048: 0.163, 0.134, 0.162; 5000: 0.402,
+// 0.384, 0.438; 8192: 0.642, 0.522, 0.469), and few chains per warp where a batch's largest problem
+// bounds its time (8 problems x 256 chains: 0.31, 0.40, 0.50).  One CTA per SM: with two (128
+// registers per thread) no size was faster.  c, w > 0: given.
+struct ShapeChoice {
+    int C, consumers;
+};
+ShapeChoice pick_shape(bool f64, int kv, int chains, const std::vector<double> &cost, int c, int w)
+{
+    static const double kCta[3][kMaxConsumers] = {{0.79, 0.79, 0.80, 0.82, 0.96, 0.98, 1.00},
+                                                  {1.17, 1.17, 1.19, 1.27, 1.51, 1.56, 1.60},
+                                                  {1.76, 1.78, 1.85, 1.95, 2.65, 2.68, 2.80}};
+    constexpr double kSMs = 152.0;
+    ShapeChoice best{c > 0 ? c : 1, w > 0 ? w : 1};
+    double best_t = 0.0;
+    double longest = 0.0, total = 0.0;
+    for (double x : cost) {
+        longest = std::max(longest, x);
+        total += x;
+    }
+    for (int i = 0; i < 3; ++i) {
+        const int C = 1 << i;
+        if (c > 0 ? C != c : (C == 2 && kv > 16) || (C == 4 && kv > (f64 ? 4 : 8))) continue;   // the widest tiles: no registers
+        for (int x = 1; x <= kMaxConsumers; ++x) {
+            if (w > 0 ? x != w : cost.size() > 1 && x < 4) continue;   // a batch's small CTAs would share SMs
+            const double items = (double)((chains + x * C - 1) / (x * C));
+            const double load = cost.size() == 1
+                                    ? std::ceil(items / kSMs) * longest
+                                    : std::max(longest, (items + 0.5) * total / kSMs + 0.3 * longest);
+            const double t = load * kCta[i][x - 1];
+            if (best_t == 0.0 || t < best_t) {
+                best = {C, x};
+                best_t = t;
+            }
+        }
+    }
+    return best;
+}
+
 // Shared memory of the sweep kernel: per chain c, w, r~ and the uniforms of a window of
 // 128 moves (with a prior as many for the acceptances), the barriers, the packet slots
-// and the record stages.  Consumer warps per CTA: enough that the CTAs about cover the
-// SMs once (all chains of an SM then share one ring), or the tuned count.  CTAs per SM:
-// as many as the work needs and the registers allow (the persistent kernel queues the
-// rest).  What the budget leaves goes, in this order, to: a ring of at least
+// and the record stages.  CTAs per SM: as many as the work needs and the registers allow
+// (the persistent kernel queues the rest).  What the budget leaves goes, in this order, to: a ring of at least
 // kMinStages stages (fewer records to a stage where the records are long, before fewer
 // consumers); U of the visited blocks in the packets; the sums of the kept sweeps; the chain
 // states; a ring of kRingRecords of the largest records; more packet slots; the
 // rest of the ring.  For a batch the shape covers the largest problem.
 template <class T>
-bool plan_shape(LaunchShape &sh, int C, const PlanNeeds &nd, long long chains, int kv, int want_consumers, int minb,
+bool plan_shape(LaunchShape &sh, const ShapeChoice &pick, const PlanNeeds &nd, long long chains, int kv, int minb,
                 bool prior)
 {
+    const int C = pick.C;
     sh.minb = prior ? 1 : minb;   // the prior's kernels exist for one CTA per SM
     sh.prior = prior ? 1 : 0;
     sh.C = C;
     sh.wait_limit = kWaitLimit;
     sh.stall = 0;
-    constexpr int kSMs = 152;
+    constexpr long long kSMs = 152;
     constexpr int kMinStages = 3;
     constexpr int kRingRecords = 24;
     const long long total_warps = (chains + C - 1) / C;
     sh.cpad = round_up_int(std::max(nd.max_np, 1), 32);
     sh.mpad = round_up_int(std::max(nd.max_M, 1), 32);
-    int consumers = want_consumers > 0
-                        ? want_consumers
-                        : (int)std::min<long long>(kMaxConsumers,
-                                                   std::max<long long>(1, (total_warps + kSMs - 1) / kSMs));
     auto env = [](const char *name, int lo, int hi, int dflt) {   // tuning overrides
         const char *e = std::getenv(name);
         const int v = e ? std::atoi(e) : 0;
         return e && v >= lo && v <= hi ? v : dflt;
     };
-    consumers = env("ASM_CONSUMERS_PER_CTA", 1, kMaxConsumers, consumers);
-    const int want_rps = env("ASM_RECORDS_PER_STAGE", 1, 8, kRecordsPerStage);
+    const int want_rps = env("ASM_RECORDS_PER_STAGE", 1, 8, 0);
     const int max_depth = env("ASM_RING_DEPTH", 2, kMaxRingDepth, kMaxRingDepth);
     const bool stage_u = std::getenv("ASM_NO_U_STAGE") == nullptr;
     constexpr size_t kBarBytes = 8 * (2 * kMaxRingDepth + 2 * kMaxPacketSlots);
     const size_t head = align_up((size_t)nd.head, 128);
     auto stage_of = [&](int rps) { return align_up((size_t)rps * nd.max_rec * sizeof(T), 128); };
-    for (; consumers >= 1; --consumers) {
+    for (int consumers = pick.consumers; consumers >= 1; --consumers) {
         LaunchShape probe = sh;   // no dynamic shared memory: the register limit alone
         probe.consumers = consumers;
         probe.depth = 0;
@@ -1073,8 +1113,15 @@ bool plan_shape(LaunchShape &sh, int C, const PlanNeeds &nd, long long chains, i
         const int base_words = 2 * sh.cpad + sh.mpad + (prior ? 256 : 128);
         const size_t per_word = (size_t)consumers * C * sizeof(T);
         size_t used = per_word * base_words + kBarBytes + 256 + 2 * head;
+        const int nr = round_up_int(nd.max_N, 32);
         const int min_stages = std::min(kMinStages, max_depth);
         int rps = want_rps;
+        if (rps == 0) {   // as many as leave room for everything else, at least kRecordsPerStage
+            size_t extras = per_word * nr * (sizeof(T) == 4 ? 3 : 1);
+            if (stage_u && !nd.packets.empty()) extras += 2 * (align_up((size_t)nd.packets.back(), 128) - head);
+            for (rps = kMaxLargeRecords; rps > kRecordsPerStage; --rps)
+                if (used + extras + min_stages * stage_of(rps) <= budget) break;
+        }
         while (rps > 1 && used + min_stages * stage_of(rps) > budget) --rps;
         int depth = min_stages;
         if (used + depth * stage_of(rps) > budget) depth = 2;
@@ -1087,7 +1134,6 @@ bool plan_shape(LaunchShape &sh, int C, const PlanNeeds &nd, long long chains, i
                 if (bb > slot && used + 2 * (bb - head) <= budget) slot = bb;
             }
         used += 2 * (slot - head);
-        const int nr = round_up_int(nd.max_N, 32);
         sh.npad = sh.fpad = 0;
         if (sizeof(T) == 4 && std::getenv("ASM_NO_SMEM_SUMS") == nullptr && used + 2 * per_word * nr <= budget) {
             sh.npad = nr;
@@ -1131,16 +1177,6 @@ int pick_kv(int max_nb, int vec, int kmax)
     int kv = 1;
     while (kv < need) kv <<= 1;
     return kv <= kmax ? kv : -1;
-}
-
-// Chains per warp and register budget of a launch that is not tuned.
-void pick_shape(bool f64, int kv, long long chains, int &C, int &minb)
-{
-    C = 1;
-    minb = 1;
-    (void)f64;
-    (void)kv;
-    (void)chains;
 }
 
 // Snapshot of all chains into the moments of the backward pass (every
@@ -1239,7 +1275,7 @@ int run_all(asm_problem *h, int chains, long long s_begin, long long s_end, long
         for (const BlockDesc &B : u->blocks) {
             nd.head = std::max(nd.head, (int)((kPacketHeader + B.rs) * sizeof(T)));
             const long long whole = (kPacketHeader + B.rs + (long long)B.np * B.usr) * (long long)sizeof(T);
-            if (whole < 220 * 1024) nd.packets.push_back((int)((whole + 15) / 16 * 16));
+            if (whole < 110 * 1024) nd.packets.push_back((int)((whole + 15) / 16 * 16));
         }
     }
     std::sort(nd.packets.begin(), nd.packets.end());
@@ -1247,13 +1283,18 @@ int run_all(asm_problem *h, int chains, long long s_begin, long long s_end, long
     const int kv = pick_kv(max_nb, vec, sizeof(T) == 8 ? kMaxKvF64 : kMaxKvF32);
     if (kv < 0) return ASM_ERR_TOO_LARGE;
     const long long all_chains = (long long)chains * (long long)us.size();
-    int C = 1, minb = 1;
-    pick_shape(sizeof(T) == 8, kv, all_chains, C, minb);
-    if (h->team) C = 32 / h->team;
-    if (prior) C = 1;
-    if (h->tuned_minb) minb = h->tuned_minb;
+    int want_consumers = h->tuned_consumers;
+    if (const char *e = std::getenv("ASM_CONSUMERS_PER_CTA")) {   // tuning override
+        const int v = std::atoi(e);
+        if (v >= 1 && v <= kMaxConsumers) want_consumers = v;
+    }
+    std::vector<double> cost;   // relative time of a problem's sweep: wide blocks cost more per move
+    for (asm_problem *u : us) cost.push_back((double)u->N * (1.0 + u->max_nb / 2000.0));
+    const ShapeChoice pick =
+        pick_shape(sizeof(T) == 8, kv, chains, cost, prior ? 1 : h->team ? 32 / h->team : 0, want_consumers);
+    const int minb = h->tuned_minb ? h->tuned_minb : 1;
     LaunchShape sh{};
-    if (!plan_shape<T>(sh, C, nd, all_chains, kv, h->tuned_consumers, minb, prior)) return ASM_ERR_TOO_LARGE;
+    if (!plan_shape<T>(sh, pick, nd, all_chains, kv, minb, prior)) return ASM_ERR_TOO_LARGE;
     const SweepFns fns = sweep_fns(h->precision, sh);
     bool stall = h->test_stall;
     for (asm_problem *u : us) stall = stall || u->test_stall;

@@ -950,10 +950,11 @@ struct WarpChains {
     __device__ __forceinline__ T *u_(int c) const { return c_(c) + off_u; }
 };
 
-// Move counts of a warp's chains in one launch (at most 64 sweeps).
+// Move counts of a warp's chains in one launch (at most 64 sweeps): degenerate Gaussian
+// moves, flat moves made, non-finite steps, rejections; and the flat moves in all.
 template <int C>
 struct MoveCounts {
-    unsigned deg[C], zero[C], bad[C], rej[C];
+    unsigned deg[C], zero[C], bad[C], rej[C], flat;
     int capped;
 };
 
@@ -1298,14 +1299,18 @@ struct Visit {
         // modes j < ng are Gaussian, those from nz on flat; in between both occur (never, when
         // the singular values are sorted)
         const int ng = uni(B.ng), nz = uni(B.nz);
-        int jr = 0;                // record of move j within its ring stage
-        const T *stb = nullptr;    // the stage holding move j's record
+        // flat moves are unrolled where one chain's latency is the limit and runs are long
+        // (blocked modes, 1024 chains: 0.0850 -> 0.0808 ms a sweep); not in the kernels for blocks
+        // of one vector, whose time is draws and whose code has to stay small (hierarchy: 0.0688 by
+        // 1, 0.0744 by 4), nor with several chains, which fill the pipes (4096 chains: 0.1125, 0.1173)
+        constexpr int kUnroll = PRIOR || C > 1 || KV == 1 ? 1 : KK <= 2 ? 4 : KK <= 4 ? 2 : 1;
         for (int j = 0; j < bn;) {
-            // uniform of move t: word t%4 of Philox(ctr = {t/4, s, q, problem}); the 128
-            // uniforms of a window come from one Philox call per lane and chain
-            const int t0 = bstart + j;
-            if (t0 >= win_end) {
-                win = t0 & ~127;
+            // one ring stage of moves [j, jstage)
+            const int t0 = bstart + j, jstage = min(j + rps, bn);
+            // uniform of move t: word t%4 of Philox(ctr = {t/4, s, q, problem}); 128 of them, from
+            // the stage's first move on, come from one Philox call per lane and chain
+            if (bstart + jstage > win_end) {
+                win = t0 & ~3;
                 win_end = win + 128;
                 __syncwarp();   // the previous window is read by every lane
 #pragma unroll
@@ -1333,99 +1338,87 @@ struct Visit {
                 }
                 __syncwarp();
             }
-            if (jr == 0) {   // the stage of the next record: usually landed long ago
-                if (!warp_wait(R.full + rp.slot, rp.phase, sh.wait_limit)) return false;
-                stb = reinterpret_cast<const T *>(R.stages + (size_t)rp.slot * sh.stage_bytes);
-            }
-            // this segment's moves: up to the end of the window, of the stage, of the modes of
-            // one kind or of the block
-            const int jbeg = j;
-            int jend = min(min(bn, win_end - bstart), j + (rps - jr));
-            const T *st = stb + (size_t)jr * recstride;
             const T *up = wc.u_(0) + (bstart - win);
-            bool flat = j >= nz;
-            if (j < ng) {
-                jend = min(jend, ng);
-            } else if (!flat) {   // a mode between: one move, by its own d
-                jend = j + 1;
-                flat = uni((int)is_zero(st[2 * rs])) != 0;
-            }
-            if (flat) {
-                unsigned opened[C];
+            // the stage has usually landed long ago
+            if (!warp_wait(R.full + rp.slot, rp.phase, sh.wait_limit)) return false;
+            const T *st = reinterpret_cast<const T *>(R.stages + (size_t)rp.slot * sh.stage_bytes);
+            while (j < jstage) {
+                // moves of one kind
+                const int jbeg = j;
+                int jend = jstage;
+                bool flat = j >= nz;
+                if (j < ng) {
+                    jend = min(jstage, ng);
+                } else if (!flat) {   // a mode between: one move, by its own d
+                    jend = j + 1;
+                    flat = uni((int)is_zero(st[2 * rs])) != 0;
+                }
+                if (flat) {
+#pragma unroll kUnroll
+                    for (; j < jend; ++j, st += recstride) {
+                        T u[C], v0[VE], r0[VE], lo[C], hi[C], delta[C];
+                        // chunk 0 of the pass and the mode's data do not depend on the bounds: loaded first
+                        const T dres = st[2 * rs + 2];
 #pragma unroll
-                for (int c = 0; c < C; ++c) opened[c] = 0u;
+                        for (int c = 0; c < C; ++c) u[c] = up[j + c * wc.tw];
+                        lds_v(st + VE * lane, v0);
+                        lds_v(st + rs + VE * lane, r0);
+                        warp_bounds<C>(lk, hk, lo, hi);
+                        // degenerate interval: no move; else flat on [lo, hi] (both bounds finite:
+                        // set-up rejects zero modes that do not change sign)
+#pragma unroll
+                        for (int c = 0; c < C; ++c) {
+                            const bool open = open_interval(lo[c], hi[c]);
+                            delta[c] = open ? m_fma(u[c], hi[c] - lo[c], lo[c]) : T(0);
+                            n.zero[c] += open ? 1u : 0u;
+                        }
+                        if constexpr (PRIOR) prior_step(p, f, delta, v0, st, up[128 + j], bn, bstart, kcnt, lane, n.rej);
+                        pass(f, delta, v0, r0, st, rs, kcnt, lane, lk, hk);
+                        store_w(wc, j, np, dres, delta);
+                    }
+                    n.flat += (unsigned)(j - jbeg);
+                } else {
 #pragma unroll 1
-                for (; j < jend; ++j, st += recstride) {
-                    T u[C], v0[VE], r0[VE], lo[C], hi[C], delta[C];
-                    // chunk 0 of the pass and the mode's data do not depend on the bounds: loaded first
-                    const T dres = st[2 * rs + 2];
+                    for (; j < jend; ++j, st += recstride) {
+                        T u[C], v0[VE], r0[VE], lo[C], hi[C], delta[C], dj, ij, dres;
+                        lds_mode(st + 2 * rs, dj, ij, dres);
 #pragma unroll
-                    for (int c = 0; c < C; ++c) u[c] = up[j + c * wc.tw];
-                    lds_v(st + VE * lane, v0);
-                    lds_v(st + rs + VE * lane, r0);
-                    warp_bounds<C>(lk, hk, lo, hi);
-                    // degenerate interval: no move; else flat on [lo, hi] (both bounds finite:
-                    // set-up rejects zero modes that do not change sign)
+                        for (int c = 0; c < C; ++c) u[c] = up[j + c * wc.tw];
+                        lds_v(st + VE * lane, v0);
+                        lds_v(st + rs + VE * lane, r0);
+                        warp_bounds<C>(lk, hk, lo, hi);
+                        // degenerate interval: no move; else the truncated Gaussian
+                        constexpr int G = 32 / C;
+                        T l = lo[0], h = hi[0], uu = u[0];
+                        const T *cs = wc.c_(0);
 #pragma unroll
-                    for (int c = 0; c < C; ++c) {
-                        const bool open = open_interval(lo[c], hi[c]);
-                        delta[c] = open ? m_fma(u[c], hi[c] - lo[c], lo[c]) : T(0);
-                        opened[c] += open ? 1u : 0u;
+                        for (int c = 1; c < C; ++c) {
+                            const bool mine = lane / G == c;
+                            l = mine ? lo[c] : l;
+                            h = mine ? hi[c] : h;
+                            uu = mine ? u[c] : uu;
+                            cs = mine ? wc.c_(c) : cs;
+                        }
+                        const T cj = j < np ? cs[j] : T(0);
+                        const T dl = draw_team<G>(cj, dj, ij, l, h, uu, open_interval(l, h), lane, n.capped);
+#pragma unroll
+                        for (int c = 0; c < C; ++c) {
+                            const T x = C == 1 ? dl : __shfl_sync(0xffffffffu, dl, c * G);
+                            const bool fin = is_finite(x);
+                            n.bad[c] += fin ? 0u : 1u;
+                            n.deg[c] += open_interval(lo[c], hi[c]) ? 0u : 1u;
+                            delta[c] = fin ? x : T(0);
+                        }
+                        if constexpr (PRIOR) prior_step(p, f, delta, v0, st, up[128 + j], bn, bstart, kcnt, lane, n.rej);
+                        pass(f, delta, v0, r0, st, rs, kcnt, lane, lk, hk);
+                        store_w(wc, j, np, dres, delta);
                     }
-                    if constexpr (PRIOR) prior_step(p, f, delta, v0, st, up[128 + j], bn, bstart, kcnt, lane, n.rej);
-                    pass(f, delta, v0, r0, st, rs, kcnt, lane, lk, hk);
-                    store_w(wc, j, np, dres, delta);
-                }
-#pragma unroll
-                for (int c = 0; c < C; ++c) {
-                    n.zero[c] += opened[c];
-                    n.deg[c] += (unsigned)(j - jbeg) - opened[c];
-                }
-            } else {
-#pragma unroll 1
-                for (; j < jend; ++j, st += recstride) {
-                    T u[C], v0[VE], r0[VE], lo[C], hi[C], delta[C], dj, ij, dres;
-                    lds_mode(st + 2 * rs, dj, ij, dres);
-#pragma unroll
-                    for (int c = 0; c < C; ++c) u[c] = up[j + c * wc.tw];
-                    lds_v(st + VE * lane, v0);
-                    lds_v(st + rs + VE * lane, r0);
-                    warp_bounds<C>(lk, hk, lo, hi);
-                    // degenerate interval: no move; else the truncated Gaussian
-                    constexpr int G = 32 / C;
-                    T l = lo[0], h = hi[0], uu = u[0];
-                    const T *cs = wc.c_(0);
-#pragma unroll
-                    for (int c = 1; c < C; ++c) {
-                        const bool mine = lane / G == c;
-                        l = mine ? lo[c] : l;
-                        h = mine ? hi[c] : h;
-                        uu = mine ? u[c] : uu;
-                        cs = mine ? wc.c_(c) : cs;
-                    }
-                    const T cj = j < np ? cs[j] : T(0);
-                    const T dl = draw_team<G>(cj, dj, ij, l, h, uu, open_interval(l, h), lane, n.capped);
-#pragma unroll
-                    for (int c = 0; c < C; ++c) {
-                        const T x = C == 1 ? dl : __shfl_sync(0xffffffffu, dl, c * G);
-                        const bool fin = is_finite(x);
-                        n.bad[c] += fin ? 0u : 1u;
-                        n.deg[c] += open_interval(lo[c], hi[c]) ? 0u : 1u;
-                        delta[c] = fin ? x : T(0);
-                    }
-                    if constexpr (PRIOR) prior_step(p, f, delta, v0, st, up[128 + j], bn, bstart, kcnt, lane, n.rej);
-                    pass(f, delta, v0, r0, st, rs, kcnt, lane, lk, hk);
-                    store_w(wc, j, np, dres, delta);
                 }
             }
-            // release the stage to the producer after its last record (one arrival per warp)
-            jr += j - jbeg;
-            if (jr == rps || j == bn) {
-                __syncwarp();
-                mbar_arrive_lane0(R.empty + rp.slot, lane);
-                ring_next(rp, sh.depth);
-                jr = 0;
-            }
+            // release the stage to the producer (one arrival per warp)
+            __syncwarp();
+            mbar_arrive_lane0(R.empty + rp.slot, lane);
+            ring_next(rp, sh.depth);
         }
         // write the block back and accumulate the kept sweep
         constexpr bool psums = sizeof(T) == 4;
@@ -1501,6 +1494,7 @@ __device__ __forceinline__ void consume(const SweepParams<T> &p, const LaunchSha
     const bool kept_here = psums && rg.burn_in < rg.sweep0 + rg.nsweeps;
     MoveCounts<C> n;
     n.capped = 0;
+    n.flat = 0u;
 #pragma unroll
     for (int c = 0; c < C; ++c) {
         const long long q_raw = ((long long)group * sh.consumers + wcta) * C + c;
@@ -1623,7 +1617,8 @@ __device__ __forceinline__ void consume(const SweepParams<T> &p, const LaunchSha
         // counters: the solver's cap is counted by the lanes of a chain's team alike
         const int capped = __shfl_sync(0xffffffffu, n.capped, c * (32 / C));
         if (wc.active[c] && lane == 0) {
-            if (n.deg[c]) atomicAdd(&p.counters->degenerate, (unsigned long long)n.deg[c]);
+            const unsigned deg = n.deg[c] + (n.flat - n.zero[c]);
+            if (deg) atomicAdd(&p.counters->degenerate, (unsigned long long)deg);
             if (n.zero[c]) atomicAdd(&p.counters->zero_mode, (unsigned long long)n.zero[c]);
             if (n.bad[c]) atomicAdd(&p.counters->nonfinite, (unsigned long long)n.bad[c]);
             if (n.rej[c]) atomicAdd(&p.counters->prior_rejections, (unsigned long long)n.rej[c]);
