@@ -78,8 +78,9 @@ enum { ASM_FP64 = 0, ASM_MIXED = 1 };   /* precision of asm_sample */
  *   ASM_RECORDS_PER_STAGE  1..8: move records of the largest block per ring stage
  *                          (default 4: one barrier wait and release per stage;
  *                          smaller blocks put more records in a stage);
- *   ASM_NO_U_STAGE         set: the block projections read U from global memory
- *                          instead of the visit packet in shared memory. */
+ *   ASM_NO_U_STAGE         set: U of every block is streamed through the record
+ *                          ring for the projections instead of coming with the
+ *                          block's visit packet. */
 
 typedef struct asm_problem asm_problem;  /* opaque, library-owned */
 
@@ -150,7 +151,7 @@ typedef struct {
     int32_t consumers_per_cta;  /* chain warps per CTA of the last sweep launch */
     int32_t ctas;               /* CTAs of the last sweep launch (persistent) */
     int32_t work_items;         /* (problem, chain group) items of the last sweep launch */
-    int32_t min_blocks;         /* CTAs per SM the last sweep launch's registers were budgeted for (1, 2) */
+    int32_t min_blocks;         /* CTAs per SM the sweep kernel's registers are budgeted for (1) */
     int32_t reserved_;
     int64_t prior_rejections;   /* moves whose proposal the gamma prior rejected */
 } asm_stats;
@@ -197,9 +198,7 @@ int asm_problem_count(const asm_problem *p);
 /* Autotuner of the sweep launch (no counterpart in the paper).  Times every
  * candidate shape -- lanes per chain S in {32, 16, 8} (a warp runs 32/S chains
  * that share every row it loads) times chain warps per
- * CTA in {heuristic, 2, 3, 4, 5, 6, 7} times the register budget (kernels
- * compiled for one CTA per SM, up to 255 registers per thread, or for two,
- * 128), where it fits -- on one warm-up and three
+ * CTA in {heuristic, 2, 3, 4, 5, 6, 7}, where it fits -- on one warm-up and three
  * timed sweeps of fresh trial chains in the caller's workspace (same layout
  * and size rule as asm_sample), and keeps the fastest for later asm_sample
  * calls on p.  The shape changes no result: every chain does the same
@@ -207,7 +206,8 @@ int asm_problem_count(const asm_problem *p);
  * are overwritten, so the next asm_sample must start fresh chains
  * (ASM_SAMPLE_CONTINUE then fails with ASM_ERR_STATE).  Synchronises
  * `stream`.  team_out / consumers_out / min_blocks_out (may be NULL) receive
- * the choice (consumers 0 = the built-in heuristic; min_blocks 1 or 2). */
+ * the choice (consumers 0 = the built-in heuristic; min_blocks, the CTAs per
+ * SM that the kernel's registers are budgeted for, is 1). */
 int asm_tune(asm_problem *p, int chains, int precision, void *d_workspace, size_t workspace_bytes,
              void *stream, int *team_out, int *consumers_out, int *min_blocks_out);
 

@@ -15,9 +15,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libasm_gb300.so")
-UNITS = ["asm_sweep_f32_c1.cu", "asm_sweep_f32_c2.cu", "asm_sweep_f32_c4.cu", "asm_sweep_f32_m2.cu",
-         "asm_sweep_f32_prior.cu", "asm_sweep_f64_c1.cu", "asm_sweep_f64_c2.cu", "asm_sweep_f64_c4.cu",
-         "asm_sweep_f64_m2.cu", "asm_sweep_f64_prior.cu", "asm_lib.cu", "asm_refresh_tc.cu", "asm_ceiling.cu",
+UNITS = ["asm_sweep_f32_c1.cu", "asm_sweep_f32_c2.cu", "asm_sweep_f32_c4.cu", "asm_sweep_f32_prior.cu", "asm_sweep_f64_c1.cu", "asm_sweep_f64_c2.cu", "asm_sweep_f64_c4.cu",
+         "asm_sweep_f64_prior.cu", "asm_lib.cu", "asm_refresh_tc.cu", "asm_ceiling.cu",
          "asm_moments.cu"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc" if os.path.exists("/usr/local/cuda/bin/nvcc") else "nvcc")
 FLAGS = ["-std=c++17", "-O3", "-gencode", "arch=compute_103a,code=sm_103a", "-lineinfo",

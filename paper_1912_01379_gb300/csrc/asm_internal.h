@@ -28,7 +28,8 @@ struct BlockDesc {
     int recstride;   // elements per move record: 2 rs + 4
     int usr;         // row stride of U in the packet: M | 1 (odd: conflict-free column reads)
     int last;        // 1: the last block of its level
-    long long offU;    // Ut: np x M (mode-major); Um: M x np (grid-major)
+    long long offUe, offUx;   // U in tiles of 32 columns for the streamed projections: entry
+                              // (columns are modes, M rows each), exit (data points, np rows)
     long long offRec;  // move records of the block: n records of recstride elements
     long long offPk;   // visit packet: header, R row of mode 0 (rs), U (np rows of usr); 16-byte aligned
 };
@@ -39,7 +40,7 @@ template <class T>
 struct ProblemData {
     const T *rec;            // per move j: {V_j, R_{j+1} (rs each), d_j, 1/d_j, |K~_b V_j|, 0}
     const T *pk;             // visit packets
-    const T *Ut, *Um;        // U in two layouts, for blocks whose U does not fit a packet slot
+    const T *Ue, *Ux;        // U in two tilings, for blocks whose U does not fit a packet slot
 };
 
 struct Counters {            // device counters, first bytes of the workspace
@@ -119,7 +120,6 @@ struct LaunchShape {
                                       // 0: in the workspace)
     int team_words;                   // shared-memory elements per chain
     int n_items;                      // (problem, chain group) work items
-    int minb;                         // register budget: 1 or 2 CTAs per SM
     int prior;                        // 1: kernels with the gamma prior's acceptance step
     int wait_limit;                   // polls before a bounded mbarrier wait gives up
     int stall;                        // test of the failure path: the producer issues no records
@@ -143,37 +143,31 @@ struct WorkItem {
 // Launchers (asm_sweep_*.cu).  kv: 16-byte vectors per lane and chain, a power of two.
 // Persistent: `ctas` CTAs of (consumers + 1) warps pull work items from
 // ctrl->queue (reset to 0 before the launch); work item problems index the
-// device array probs.  _cC: C chains per warp; _m1 kernels budget the registers
-// for one CTA per SM (up to 255 per thread), _m2 for two (128).  A kv that a
-// launcher has no kernel for gives cudaErrorInvalidValue, and 0 CTAs per SM.
+// device array probs.  _cC: C chains per warp.  The registers are budgeted for one
+// CTA per SM (up to 255 per thread).  A kv that a launcher has no kernel for gives
+// cudaErrorInvalidValue, and 0 CTAs per SM.
 #define ASM_DECLARE_SWEEP_LAUNCHER(T, NAME)                                                                     \
     cudaError_t launch_sweeps_##NAME(const SweepParams<T> *probs, const WorkItem *items, RunCtrl *ctrl,         \
                                      const LaunchShape &shape, int kv, int ctas, cudaStream_t s);               \
     int sweep_ctas_per_sm_##NAME(const LaunchShape &shape, int kv);
-ASM_DECLARE_SWEEP_LAUNCHER(float, f32_c1_m1)
-ASM_DECLARE_SWEEP_LAUNCHER(float, f32_c2_m1)
-ASM_DECLARE_SWEEP_LAUNCHER(float, f32_c4_m1)
-ASM_DECLARE_SWEEP_LAUNCHER(float, f32_c1_m2)
-ASM_DECLARE_SWEEP_LAUNCHER(float, f32_c2_m2)
-ASM_DECLARE_SWEEP_LAUNCHER(float, f32_c4_m2)
-ASM_DECLARE_SWEEP_LAUNCHER(float, f32_prior)     // with the gamma prior: one chain per warp, one CTA per SM
-ASM_DECLARE_SWEEP_LAUNCHER(double, f64_c1_m1)
-ASM_DECLARE_SWEEP_LAUNCHER(double, f64_c2_m1)
-ASM_DECLARE_SWEEP_LAUNCHER(double, f64_c4_m1)
-ASM_DECLARE_SWEEP_LAUNCHER(double, f64_c1_m2)
-ASM_DECLARE_SWEEP_LAUNCHER(double, f64_c2_m2)
-ASM_DECLARE_SWEEP_LAUNCHER(double, f64_c4_m2)
+ASM_DECLARE_SWEEP_LAUNCHER(float, f32_c1)
+ASM_DECLARE_SWEEP_LAUNCHER(float, f32_c2)
+ASM_DECLARE_SWEEP_LAUNCHER(float, f32_c4)
+ASM_DECLARE_SWEEP_LAUNCHER(float, f32_prior)     // with the gamma prior: one chain per warp
+ASM_DECLARE_SWEEP_LAUNCHER(double, f64_c1)
+ASM_DECLARE_SWEEP_LAUNCHER(double, f64_c2)
+ASM_DECLARE_SWEEP_LAUNCHER(double, f64_c4)
 ASM_DECLARE_SWEEP_LAUNCHER(double, f64_prior)
 #undef ASM_DECLARE_SWEEP_LAUNCHER
-#define ASM_DEFINE_SWEEP_LAUNCHER(T, NAME, C, MINB, PRIOR, ...)                                                 \
+#define ASM_DEFINE_SWEEP_LAUNCHER(T, NAME, C, PRIOR, ...)                                                       \
     cudaError_t launch_sweeps_##NAME(const SweepParams<T> *probs, const WorkItem *items, RunCtrl *ctrl,         \
                                      const LaunchShape &shape, int kv, int ctas, cudaStream_t s)                \
     {                                                                                                           \
-        return SweepDispatch<T, C, MINB, PRIOR, __VA_ARGS__>::launch(probs, items, ctrl, shape, kv, ctas, s);   \
+        return SweepDispatch<T, C, PRIOR, __VA_ARGS__>::launch(probs, items, ctrl, shape, kv, ctas, s);         \
     }                                                                                                           \
     int sweep_ctas_per_sm_##NAME(const LaunchShape &shape, int kv)                                              \
     {                                                                                                           \
-        return SweepDispatch<T, C, MINB, PRIOR, __VA_ARGS__>::per_sm(shape, kv);                                \
+        return SweepDispatch<T, C, PRIOR, __VA_ARGS__>::per_sm(shape, kv);                                      \
     }
 // Tensor-core residual refresh of the mixed path (asm_refresh_tc.cu): grid of
 // (chain tiles of 128) x n_problems x (the largest k split) CTAs; max_bn = the

@@ -426,7 +426,7 @@ struct WsLayout {
 
 // device buffers of one precision
 struct PrecBuffers {
-    void *rec = nullptr, *pk = nullptr, *Ut = nullptr, *Um = nullptr;
+    void *rec = nullptr, *pk = nullptr, *Ue = nullptr, *Ux = nullptr;
     void *prior_am1 = nullptr;   // a_n - 1 of the gamma prior (nullptr: flat)
 };
 
@@ -437,7 +437,7 @@ struct asm_problem {
     std::vector<double> w;
     double f0 = 0.0;
     int max_nb = 0, max_np = 0;
-    long long totU = 0, totRec = 0, totPk = 0;
+    long long totUe = 0, totUx = 0, totRec = 0, totPk = 0;
     int max_rec = 0;   // largest record (elements)
     // device
     int *d_level_first = nullptr, *d_level_nblocks = nullptr;
@@ -472,26 +472,25 @@ struct asm_problem {
     bool have_run = false;
     // launch shape chosen by asm_tune (0: the built-in heuristic)
     int tuned_consumers = 0;
-    int tuned_minb = 0;   // CTAs per SM the registers are budgeted for (0: heuristic)
     // one refresh period (advance the range, sweep, refresh) as a CUDA graph
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t gexec = nullptr;
     struct GraphKey {
         const void *ws_all = nullptr;
-        int chains = 0, precision = -1, kv = 0, ctas = 0, C = 0, consumers = 0, depth = 0, n_items = 0, minb = 0,
+        int chains = 0, precision = -1, kv = 0, ctas = 0, C = 0, consumers = 0, depth = 0, n_items = 0, kind = 0,
             pbytes = 0, pslots = 0, rps = 0, npad = 0, fpad = 0;
         size_t refresh_smem = 0;
         bool operator==(const GraphKey &o) const
         {
             return ws_all == o.ws_all && chains == o.chains && precision == o.precision && kv == o.kv &&
                    ctas == o.ctas && C == o.C && consumers == o.consumers && depth == o.depth &&
-                   n_items == o.n_items && minb == o.minb && pbytes == o.pbytes && pslots == o.pslots &&
+                   n_items == o.n_items && kind == o.kind && pbytes == o.pbytes && pslots == o.pslots &&
                    rps == o.rps && npad == o.npad && fpad == o.fpad && refresh_smem == o.refresh_smem;
         }
     } gkey;
     long long graph_replays = 0, tc_refreshes = 0;
     bool refresh_fp64 = false;   // mixed path: FP64 CUDA-core refresh instead of the tensor cores
-    int last_team = 0, last_consumers = 0, last_ctas = 0, last_items = 0, last_minb = 0;   // last sweep launch
+    int last_team = 0, last_consumers = 0, last_ctas = 0, last_items = 0;   // last sweep launch
     bool no_graph = false;    // direct launches only (the allocation-free entry point)
     bool trace = false;       // ASM_SAMPLE_STEP_TRACE: the step-size trace of every sweep
     bool test_stall = false;  // ASM_FLAG_TEST_STALL: the failure path under test
@@ -595,7 +594,7 @@ int upload(void **dst, const std::vector<T> &src)
 
 void free_prec(PrecBuffers &b)
 {
-    void *ptrs[] = {b.rec, b.pk, b.Ut, b.Um, b.prior_am1};
+    void *ptrs[] = {b.rec, b.pk, b.Ue, b.Ux, b.prior_am1};
     for (void *x : ptrs)
         if (x) cudaFree(x);
     b = PrecBuffers{};
@@ -845,14 +844,17 @@ done:
     return rc;
 }
 
-// Host-side mode records and visit packets for one precision, then upload.
+// Columns of a block's entry tiles (the kernel's entry_width).
+int entry_cols(int np) { return np > 16 ? 32 : np > 8 ? 16 : np > 4 ? 8 : 4; }
+
+// Host-side mode records, visit packets and U tiles for one precision, then upload.
 template <class T>
 int build_precision(asm_problem *p, const HostFactors &hf, PrecBuffers &out)
 {
     const int M = p->M;
     const T nan = std::numeric_limits<T>::quiet_NaN();
     std::vector<T> rec(p->totRec, T(0)), pk(p->totPk + 4, T(0)),   // + 4: a copy rounded up to 16 bytes stays inside
-        Ut(std::max<long long>(p->totU, 1), T(0)), Um(std::max<long long>(p->totU, 1), T(0));
+        Ue(p->totUe, T(0)), Ux(p->totUx, T(0));
     for (int b = 0; b < p->n_blocks; ++b) {
         const BlockDesc &B = p->blocks[b];
         const std::vector<double> &hd = hf.d[b], &hV = hf.V[b], &hU = hf.U[b];
@@ -866,10 +868,13 @@ int build_precision(asm_problem *p, const HostFactors &hf, PrecBuffers &out)
             for (int i = 0; i < B.n; ++i)
                 if (!(std::fabs(v[i]) < 0x1p-40 * vmax)) r[i] = (T)(-1.0 / v[i]);
         };
+        // U in tiles of columns: element (row, column) of tile t at t K width + row width + column
+        const int we = entry_cols(B.np);
         for (int j = 0; j < B.np; ++j)
             for (int m = 0; m < M; ++m) {
-                Ut[B.offU + (size_t)j * M + m] = (T)hU[(size_t)j * M + m];
-                Um[B.offU + (size_t)m * B.np + j] = (T)hU[(size_t)j * M + m];
+                const T x = (T)hU[(size_t)j * M + m];
+                Ue[B.offUe + ((size_t)(j / 32) * M + m) * we + j % 32] = x;
+                Ux[B.offUx + ((size_t)(m / 32) * B.np + j) * 32 + m % 32] = x;
             }
         // move records: {V_j, R_{j+1}, d_j, 1/d_j, dres_j, 0}
         for (int j = 0; j < B.n; ++j) {
@@ -892,8 +897,8 @@ int build_precision(asm_problem *p, const HostFactors &hf, PrecBuffers &out)
                 k[kPacketHeader + B.rs + (size_t)j * B.usr + m] = (T)hU[(size_t)j * M + m];
     }
     int rc;
-    if ((rc = upload(&out.rec, rec)) || (rc = upload(&out.pk, pk)) || (rc = upload(&out.Ut, Ut)) ||
-        (rc = upload(&out.Um, Um)))
+    if ((rc = upload(&out.rec, rec)) || (rc = upload(&out.pk, pk)) || (rc = upload(&out.Ue, Ue)) ||
+        (rc = upload(&out.Ux, Ux)))
         return rc;
     return ASM_OK;
 }
@@ -946,8 +951,8 @@ SweepParams<T> make_params(asm_problem *p, const PrecBuffers &b, const WsLayout 
     sp.blocks = p->d_blocks;
     sp.pd.rec = (const T *)b.rec;
     sp.pd.pk = (const T *)b.pk;
-    sp.pd.Ut = (const T *)b.Ut;
-    sp.pd.Um = (const T *)b.Um;
+    sp.pd.Ue = (const T *)b.Ue;
+    sp.pd.Ux = (const T *)b.Ux;
     char *ws = (char *)p->ws;
     sp.F = (T *)(ws + L.F);
     sp.ldF = L.ldF;
@@ -984,7 +989,7 @@ SweepParams<T> make_params(asm_problem *p, const PrecBuffers &b, const WsLayout 
     return sp;
 }
 
-// The sweep kernels of one (precision, chains per warp, register budget, prior).
+// The sweep kernels of one (precision, chains per warp, prior).
 struct SweepFns {
     cudaError_t (*launch64)(const SweepParams<double> *, const WorkItem *, RunCtrl *, const LaunchShape &, int, int,
                             cudaStream_t);
@@ -1002,12 +1007,10 @@ SweepFns sweep_fns(int precision, const LaunchShape &sh)
     const int ci = sh.C == 1 ? 0 : sh.C == 2 ? 1 : 2;
 #define F64(NAME) SweepFns{launch_sweeps_##NAME, nullptr, sweep_ctas_per_sm_##NAME}
 #define F32(NAME) SweepFns{nullptr, launch_sweeps_##NAME, sweep_ctas_per_sm_##NAME}
-    static const SweepFns f64[2][3] = {{F64(f64_c1_m1), F64(f64_c2_m1), F64(f64_c4_m1)},
-                                       {F64(f64_c1_m2), F64(f64_c2_m2), F64(f64_c4_m2)}};
-    static const SweepFns f32[2][3] = {{F32(f32_c1_m1), F32(f32_c2_m1), F32(f32_c4_m1)},
-                                       {F32(f32_c1_m2), F32(f32_c2_m2), F32(f32_c4_m2)}};
-    if (precision == ASM_FP64) return sh.prior ? F64(f64_prior) : f64[sh.minb == 2][ci];
-    return sh.prior ? F32(f32_prior) : f32[sh.minb == 2][ci];
+    static const SweepFns f64[3] = {F64(f64_c1), F64(f64_c2), F64(f64_c4)};
+    static const SweepFns f32[3] = {F32(f32_c1), F32(f32_c2), F32(f32_c4)};
+    if (precision == ASM_FP64) return sh.prior ? F64(f64_prior) : f64[ci];
+    return sh.prior ? F32(f32_prior) : f32[ci];
 #undef F64
 #undef F32
 }
@@ -1074,11 +1077,9 @@ ShapeChoice pick_shape(bool f64, int kv, int chains, const std::vector<double> &
 // states; a ring of kRingRecords of the largest records; more packet slots; the
 // rest of the ring.  For a batch the shape covers the largest problem.
 template <class T>
-bool plan_shape(LaunchShape &sh, const ShapeChoice &pick, const PlanNeeds &nd, long long chains, int kv, int minb,
-                bool prior)
+bool plan_shape(LaunchShape &sh, const ShapeChoice &pick, const PlanNeeds &nd, long long chains, int kv, bool prior)
 {
     const int C = pick.C;
-    sh.minb = prior ? 1 : minb;   // the prior's kernels exist for one CTA per SM
     sh.prior = prior ? 1 : 0;
     sh.C = C;
     sh.wait_limit = kWaitLimit;
@@ -1099,7 +1100,8 @@ bool plan_shape(LaunchShape &sh, const ShapeChoice &pick, const PlanNeeds &nd, l
     const bool stage_u = std::getenv("ASM_NO_U_STAGE") == nullptr;
     constexpr size_t kBarBytes = 8 * (2 * kMaxRingDepth + 2 * kMaxPacketSlots);
     const size_t head = align_up((size_t)nd.head, 128);
-    auto stage_of = [&](int rps) { return align_up((size_t)rps * nd.max_rec * sizeof(T), 128); };
+    // at least eight rows of a streamed tile of 32 columns
+    auto stage_of = [&](int rps) { return std::max(align_up((size_t)rps * nd.max_rec * sizeof(T), 128), 256 * sizeof(T)); };
     for (int consumers = pick.consumers; consumers >= 1; --consumers) {
         LaunchShape probe = sh;   // no dynamic shared memory: the register limit alone
         probe.consumers = consumers;
@@ -1292,9 +1294,8 @@ int run_all(asm_problem *h, int chains, long long s_begin, long long s_end, long
     for (asm_problem *u : us) cost.push_back((double)u->N * (1.0 + u->max_nb / 2000.0));
     const ShapeChoice pick =
         pick_shape(sizeof(T) == 8, kv, chains, cost, prior ? 1 : h->team ? 32 / h->team : 0, want_consumers);
-    const int minb = h->tuned_minb ? h->tuned_minb : 1;
     LaunchShape sh{};
-    if (!plan_shape<T>(sh, pick, nd, all_chains, kv, minb, prior)) return ASM_ERR_TOO_LARGE;
+    if (!plan_shape<T>(sh, pick, nd, all_chains, kv, prior)) return ASM_ERR_TOO_LARGE;
     const SweepFns fns = sweep_fns(h->precision, sh);
     bool stall = h->test_stall;
     for (asm_problem *u : us) stall = stall || u->test_stall;
@@ -1321,7 +1322,6 @@ int run_all(asm_problem *h, int chains, long long s_begin, long long s_end, long
     h->last_consumers = sh.consumers;
     h->last_ctas = ctas;
     h->last_items = sh.n_items;
-    h->last_minb = sh.minb;
     const size_t rsmem = sizeof(double) * (size_t)nd.max_N;
     if (const int rc = refresh_smem(refresh_all_kernel<T>, rsmem); rc != ASM_OK) return rc;
     // the mixed path refreshes on the tensor cores (3xTF32) unless asked for FP64 CUDA cores
@@ -1381,7 +1381,7 @@ int run_all(asm_problem *h, int chains, long long s_begin, long long s_end, long
             key.consumers = sh.consumers;
             key.depth = sh.depth;
             key.n_items = sh.n_items;
-            key.minb = sh.minb + 4 * sh.prior + 8 * sh.stall;
+            key.kind = sh.prior + 2 * sh.stall;
             key.pbytes = sh.pbytes;
             key.pslots = sh.pslots;
             key.rps = sh.rps;
@@ -1566,7 +1566,7 @@ int asm_setup(const asm_desc *ds, asm_problem **out)
         nb += ds->level_nblocks[l];
     }
     p->n_blocks = nb;
-    long long oU = 0, oRec = 0, oPk = 0;
+    long long oUe = 0, oUx = 0, oRec = 0, oPk = 0;
     for (int l = 0; l < ds->n_levels; ++l) {
         const int *st = ds->block_start + p->level_first[l];
         for (int b = 0; b < ds->level_nblocks[l]; ++b) {
@@ -1578,7 +1578,8 @@ int asm_setup(const asm_desc *ds, asm_problem **out)
             B.np = std::min(M, B.n);
             B.rs = B.n <= kRowAlignSmall ? kRowAlignSmall : round_up_int(B.n, kRowAlign);
             B.last = b + 1 == ds->level_nblocks[l];
-            B.offU = oU; oU += (long long)B.np * M;
+            B.offUe = oUe; oUe += (long long)((B.np + 31) / 32) * M * entry_cols(B.np);
+            B.offUx = oUx; oUx += (long long)((M + 31) / 32) * B.np * 32;
             B.usr = M | 1;
             B.recstride = 2 * B.rs + 4;   // elements; the mode data take 3
             B.offRec = oRec; oRec += (long long)B.n * B.recstride;
@@ -1589,7 +1590,7 @@ int asm_setup(const asm_desc *ds, asm_problem **out)
             p->max_np = std::max(p->max_np, B.np);
         }
     }
-    p->totU = oU; p->totRec = oRec; p->totPk = oPk;
+    p->totUe = oUe; p->totUx = oUx; p->totRec = oRec; p->totPk = oPk;
     p->w.assign(N, 1.0);
     if (ds->w) {
         if (!all_finite(ds->w, N)) { asm_destroy(p); return ASM_ERR_NONFINITE; }
@@ -1926,7 +1927,7 @@ int asm_tune(asm_problem *p, int chains, int precision, void *d_workspace, size_
     if (!d_workspace || workspace_bytes < RL.total || ((uintptr_t)d_workspace & 255)) return ASM_ERR_WORKSPACE;
     if (p->ev_used && drain_events(p) != ASM_OK) return ASM_ERR_CUDA;
     bind_workspace(p, d_workspace, workspace_bytes, RL, (cudaStream_t)stream);
-    const int team0 = p->team, cons0 = p->tuned_consumers, minb0 = p->tuned_minb;
+    const int team0 = p->team, cons0 = p->tuned_consumers;
     const bool timing0 = p->timing;
     p->timing = false;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1934,7 +1935,7 @@ int asm_tune(asm_problem *p, int chains, int precision, void *d_workspace, size_
         if (e0) cudaEventDestroy(e0);
         return ASM_ERR_CUDA;
     }
-    int best_team = team0, best_cons = cons0, best_minb = minb0, rc = ASM_OK;
+    int best_team = team0, best_cons = cons0, rc = ASM_OK;
     float best = 0.f;
     bool any = false;
     bool prior = false;
@@ -1942,13 +1943,12 @@ int asm_tune(asm_problem *p, int chains, int precision, void *d_workspace, size_
         prior = prior || (precision == ASM_FP64 ? u->b64.prior_am1 : u->b32.prior_am1) != nullptr;
     const int teams[] = {32, 16, 8};
     const int conss[] = {0, 2, 3, 4, 5, 6, 7};   // 0: the built-in heuristic
-    for (int trial = 0; trial < 3 * 7 * 2; ++trial) {
-        const int S = teams[trial / 14], c = conss[(trial / 2) % 7], mb = 1 + trial % 2;
-        if (prior && (S != 32 || mb != 1)) continue;   // its kernels: one chain per warp, one CTA per SM
+    for (int trial = 0; trial < 3 * 7; ++trial) {
+        const int S = teams[trial / 7], c = conss[trial % 7];
+        if (prior && S != 32) continue;   // its kernels: one chain per warp
         {
             p->team = S;
             p->tuned_consumers = c;
-            p->tuned_minb = mb;
             // fresh chains, one sweep to warm up, then the timed sweeps
             rc = start_chains(p, chains, precision, 0x74756e65ull, false);
             if (rc != ASM_OK) break;
@@ -1971,7 +1971,6 @@ int asm_tune(asm_problem *p, int chains, int precision, void *d_workspace, size_
                 best = ms;
                 best_team = S;
                 best_cons = c;
-                best_minb = mb;
                 any = true;
             }
         }
@@ -1986,15 +1985,13 @@ int asm_tune(asm_problem *p, int chains, int precision, void *d_workspace, size_
     if (rc != ASM_OK || !any) {
         p->team = team0;
         p->tuned_consumers = cons0;
-        p->tuned_minb = minb0;
         return rc != ASM_OK ? rc : ASM_ERR_TOO_LARGE;
     }
     p->team = best_team;
     p->tuned_consumers = best_cons;
-    p->tuned_minb = best_minb;
     if (team_out) *team_out = best_team;
     if (consumers_out) *consumers_out = best_cons;
-    if (min_blocks_out) *min_blocks_out = best_minb;
+    if (min_blocks_out) *min_blocks_out = 1;
     return ASM_OK;
 }
 
@@ -2230,7 +2227,7 @@ int asm_status(asm_problem *p, asm_stats *out)
     out->consumers_per_cta = p->last_consumers;
     out->ctas = p->last_ctas;
     out->work_items = p->last_items;
-    out->min_blocks = p->last_minb;
+    out->min_blocks = 1;
     return ASM_OK;
 }
 

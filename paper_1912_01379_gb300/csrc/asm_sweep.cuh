@@ -814,6 +814,13 @@ __device__ __forceinline__ bool u_staged(const LaunchShape &sh, const BlockDesc 
 {
     return packet_bytes<T>(sh, B) > (unsigned)((kPacketHeader + B.rs) * sizeof(T));
 }
+// Streamed U: columns of an entry tile (modes; 32, or fewer for small blocks) and rows per ring stage.
+__device__ __forceinline__ int entry_width(int np) { return np > 16 ? 32 : np > 8 ? 16 : np > 4 ? 8 : 4; }
+template <class T>
+__device__ __forceinline__ int stream_rows(int stage_bytes, int width)
+{
+    return (stage_bytes / (int)(width * sizeof(T))) & ~7;
+}
 // Records of a block per ring stage.
 template <class T>
 __device__ __forceinline__ int records_per_stage(const LaunchShape &sh, int recstride)
@@ -881,8 +888,9 @@ struct Regions {
 // The producer warp.  Per block visit one bulk copy of the visit packet (block
 // descriptor, bounds row of the first mode, U where it fits) into the next
 // packet slot, then the block's move records, as many to a ring stage as fit,
-// one bulk copy per stage; each after every consumer warp has released the
-// slot's previous contents.  The ring positions run on across the CTA's items.
+// one bulk copy per stage, before and after them the tiles of U for the
+// projections where it did not fit; each copy after every consumer warp has
+// released the slot's previous contents.  The ring positions run on across the CTA's items.
 // --------------------------------------------------------------------------
 template <class T>
 __device__ __forceinline__ void produce(const SweepParams<T> &p, const LaunchShape &sh, const SweepRange &rg,
@@ -910,18 +918,33 @@ __device__ __forceinline__ void produce(const SweepParams<T> &p, const LaunchSha
         mbar_expect_tx(R.pfull + rp.pslot, pbytes);
         bulk_g2s(R.packets + (size_t)rp.pslot * sh.pbytes, p.pd.pk + B.offPk, pbytes, R.pfull + rp.pslot);
         packet_next(rp, P);
-        const int rps = records_per_stage<T>(sh, B.recstride);
-        for (int j = 0; j < B.n; j += rps) {
-            if (rp.g >= (unsigned)D && !mbar_wait(R.empty + rp.slot, rp.phase ^ 1u, sh.wait_limit)) {
+        // one bulk copy into the next ring stage
+        auto stage = [&](const T *src, size_t elements) {
+            if (failed || (rp.g >= (unsigned)D && !mbar_wait(R.empty + rp.slot, rp.phase ^ 1u, sh.wait_limit))) {
                 failed = true;
-                break;
+                return;
             }
-            const unsigned bytes = (unsigned)(min(rps, B.n - j) * B.recstride * sizeof(T));
+            const unsigned bytes = (unsigned)(elements * sizeof(T));
             mbar_expect_tx(R.full + rp.slot, bytes);
-            bulk_g2s(R.stages + (size_t)rp.slot * sh.stage_bytes, p.pd.rec + B.offRec + (size_t)j * B.recstride, bytes,
-                     R.full + rp.slot);
+            bulk_g2s(R.stages + (size_t)rp.slot * sh.stage_bytes, src, bytes, R.full + rp.slot);
             ring_next(rp, D);
-        }
+        };
+        // tiles of a streamed projection: columns [32 t, 32 t + width) x K rows, tile after tile
+        auto stream = [&](const T *src, int K, int cols, int width) {
+            const int rows = stream_rows<T>(sh.stage_bytes, width);
+            for (int col0 = 0; col0 < cols && !failed; col0 += 32)
+                for (int k = 0; k < K && !failed; k += rows) {
+                    const int n = min(rows, K - k);
+                    stage(src, (size_t)n * width);
+                    src += (size_t)n * width;
+                }
+        };
+        const bool streamed = !u_staged<T>(sh, B);
+        if (streamed) stream(p.pd.Ue + B.offUe, p.M, B.np, entry_width(B.np));
+        const int rps = records_per_stage<T>(sh, B.recstride);
+        for (int j = 0; j < B.n && !failed; j += rps)
+            stage(p.pd.rec + B.offRec + (size_t)j * B.recstride, (size_t)min(rps, B.n - j) * B.recstride);
+        if (streamed) stream(p.pd.Ux + B.offUx, B.np, p.M, 32);
         done = c.done;
     }
     if (failed) {
@@ -959,15 +982,14 @@ struct MoveCounts {
 };
 
 // c = U_b^T r~ for the warp's chains: partial sum i of eight takes the terms m = i mod 8
-// in increasing m, the rest goes to sum 0, then a fixed tree; so the sums are the same from
-// shared or global memory, for any C.  Blocks of up to eight modes spread the eight
+// in increasing m, the rest goes to sum 0, then a fixed tree; so the sums are the same for
+// any C, from a packet or streamed.  Blocks of up to eight modes spread the eight
 // partial sums over lanes (four modes at a time): with a lane per mode most lanes idle.
-template <class T, int C, int KVC, bool WIDE>
-__device__ __forceinline__ void project_entry(const WarpChains<T, C> &wc, const T *Us, const T *Um, int np, int usr, int M,
-                                              int lane)
+template <class T, int C>
+__device__ __forceinline__ void project_entry(const WarpChains<T, C> &wc, const T *Us, int np, int usr, int M, int lane)
 {
     constexpr int VEC = VecOf<T>::n;
-    if (Us && np <= 8) {
+    if (np <= 8) {
         const int i = lane & 7;
 #pragma unroll
         for (int c = 0; c < C; ++c) {
@@ -989,176 +1011,173 @@ __device__ __forceinline__ void project_entry(const WarpChains<T, C> &wc, const 
         }
         return;
     }
-    if (Us) {
-        constexpr int JJ = C == 1 ? 2 : 1;   // modes of a lane at a time
-        for (int j = lane; j < np; j += 32 * JJ) {
-            T a[C * JJ][8];
+    constexpr int JJ = C == 1 ? 2 : 1;   // modes of a lane at a time
+    for (int j = lane; j < np; j += 32 * JJ) {
+        T a[C * JJ][8];
 #pragma unroll
-            for (int x = 0; x < C * JJ; ++x)
+        for (int x = 0; x < C * JJ; ++x)
 #pragma unroll
-                for (int i = 0; i < 8; ++i) a[x][i] = T(0);
-            const T *u[JJ];
+            for (int i = 0; i < 8; ++i) a[x][i] = T(0);
+        const T *u[JJ];
 #pragma unroll
-            for (int x = 0; x < JJ; ++x) u[x] = Us + (size_t)(j + 32 * x < np ? j + 32 * x : j) * usr;
-            int m = 0;
-            for (; m + 7 < M; m += 8) {
+        for (int x = 0; x < JJ; ++x) u[x] = Us + (size_t)(j + 32 * x < np ? j + 32 * x : j) * usr;
+        int m = 0;
+        for (; m + 7 < M; m += 8) {
 #pragma unroll
-                for (int v = 0; v < 8; v += VEC) {
-                    T r[C][VEC];
+            for (int v = 0; v < 8; v += VEC) {
+                T r[C][VEC];
 #pragma unroll
-                    for (int c = 0; c < C; ++c) lds_v(wc.r_(c) + m + v, r[c]);
+                for (int c = 0; c < C; ++c) lds_v(wc.r_(c) + m + v, r[c]);
 #pragma unroll
-                    for (int k = 0; k < VEC; ++k)
+                for (int k = 0; k < VEC; ++k)
 #pragma unroll
-                        for (int x = 0; x < JJ; ++x) {
-                            const T uu = u[x][m + v + k];
+                    for (int x = 0; x < JJ; ++x) {
+                        const T uu = u[x][m + v + k];
 #pragma unroll
-                            for (int c = 0; c < C; ++c) a[c * JJ + x][v + k] = m_fma(uu, r[c][k], a[c * JJ + x][v + k]);
-                        }
-                }
+                        for (int c = 0; c < C; ++c) a[c * JJ + x][v + k] = m_fma(uu, r[c][k], a[c * JJ + x][v + k]);
+                    }
             }
-            for (; m < M; ++m)
-#pragma unroll
-                for (int c = 0; c < C; ++c)
-#pragma unroll
-                    for (int x = 0; x < JJ; ++x) a[c * JJ + x][0] = m_fma(u[x][m], wc.r_(c)[m], a[c * JJ + x][0]);
+        }
+        for (; m < M; ++m)
 #pragma unroll
             for (int c = 0; c < C; ++c)
 #pragma unroll
-                for (int x = 0; x < JJ; ++x) {
-                    const T(&b)[8] = a[c * JJ + x];
-                    if (x == 0 || j + 32 * x < np)
-                        wc.c_(c)[j + 32 * x] = ((b[0] + b[1]) + (b[2] + b[3])) + ((b[4] + b[5]) + (b[6] + b[7]));
-                }
-        }
-        return;
-    }
-    // U in global memory (grid-major): sixteen loads in flight, eight in the 128-register kernels of wide tiles
-    constexpr int NL = WIDE || KVC <= 8 ? 16 : 8;
-    for (int j = lane; j < np; j += 32) {
-        T a[C][8];
+                for (int x = 0; x < JJ; ++x) a[c * JJ + x][0] = m_fma(u[x][m], wc.r_(c)[m], a[c * JJ + x][0]);
 #pragma unroll
         for (int c = 0; c < C; ++c)
 #pragma unroll
-            for (int i = 0; i < 8; ++i) a[c][i] = T(0);
-        int m = 0;
-        for (; m + NL - 1 < M; m += NL) {
-            T x[NL];
-#pragma unroll
-            for (int i = 0; i < NL; ++i) x[i] = __ldg(Um + (size_t)(m + i) * np + j);
-#pragma unroll
-            for (int i = 0; i < NL; ++i)
-#pragma unroll
-                for (int c = 0; c < C; ++c) a[c][i & 7] = m_fma(x[i], wc.r_(c)[m + i], a[c][i & 7]);
-        }
-        for (; m + 7 < M; m += 8) {
-            T x[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) x[i] = __ldg(Um + (size_t)(m + i) * np + j);
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int c = 0; c < C; ++c) a[c][i] = m_fma(x[i], wc.r_(c)[m + i], a[c][i]);
-        }
-        for (; m < M; ++m) {
-            const T x = __ldg(Um + (size_t)m * np + j);
-#pragma unroll
-            for (int c = 0; c < C; ++c) a[c][0] = m_fma(x, wc.r_(c)[m], a[c][0]);
-        }
-#pragma unroll
-        for (int c = 0; c < C; ++c)
-            wc.c_(c)[j] = ((a[c][0] + a[c][1]) + (a[c][2] + a[c][3])) + ((a[c][4] + a[c][5]) + (a[c][6] + a[c][7]));
+            for (int x = 0; x < JJ; ++x) {
+                const T(&b)[8] = a[c * JJ + x];
+                if (x == 0 || j + 32 * x < np)
+                    wc.c_(c)[j + 32 * x] = ((b[0] + b[1]) + (b[2] + b[3])) + ((b[4] + b[5]) + (b[6] + b[7]));
+            }
     }
 }
 
 // r~ -= U_b w for the warp's chains (lanes split the data points; partial sum i of eight
 // takes the modes j = i mod 8 as at entry).
-template <class T, int C, int KVC, bool WIDE>
-__device__ __forceinline__ void project_exit(const WarpChains<T, C> &wc, const T *Us, const T *Ut, int np, int usr, int M,
-                                             int lane)
+template <class T, int C>
+__device__ __forceinline__ void project_exit(const WarpChains<T, C> &wc, const T *Us, int np, int usr, int M, int lane)
 {
     constexpr int VEC = VecOf<T>::n;
     constexpr int MM = C == 1 ? 2 : 1;   // data points of a lane at a time
-    if (Us) {
-        for (int m = lane; m < M; m += 32 * MM) {
-            T a[C * MM][8];
+    for (int m = lane; m < M; m += 32 * MM) {
+        T a[C * MM][8];
 #pragma unroll
-            for (int x = 0; x < C * MM; ++x)
+        for (int x = 0; x < C * MM; ++x)
 #pragma unroll
-                for (int i = 0; i < 8; ++i) a[x][i] = T(0);
-            int mm[MM];
+            for (int i = 0; i < 8; ++i) a[x][i] = T(0);
+        int mm[MM];
 #pragma unroll
-            for (int x = 0; x < MM; ++x) mm[x] = m + 32 * x < M ? m + 32 * x : m;
-            int j = 0;
-            for (; j + 7 < np; j += 8) {
-                const T *u = Us + (size_t)j * usr;
+        for (int x = 0; x < MM; ++x) mm[x] = m + 32 * x < M ? m + 32 * x : m;
+        int j = 0;
+        for (; j + 7 < np; j += 8) {
+            const T *u = Us + (size_t)j * usr;
 #pragma unroll
-                for (int v = 0; v < 8; v += VEC) {
-                    T w[C][VEC];
+            for (int v = 0; v < 8; v += VEC) {
+                T w[C][VEC];
 #pragma unroll
-                    for (int c = 0; c < C; ++c) lds_v(wc.w_(c) + j + v, w[c]);
+                for (int c = 0; c < C; ++c) lds_v(wc.w_(c) + j + v, w[c]);
 #pragma unroll
-                    for (int k = 0; k < VEC; ++k)
+                for (int k = 0; k < VEC; ++k)
 #pragma unroll
-                        for (int x = 0; x < MM; ++x) {
-                            const T uu = u[(v + k) * usr + mm[x]];
+                    for (int x = 0; x < MM; ++x) {
+                        const T uu = u[(v + k) * usr + mm[x]];
 #pragma unroll
-                            for (int c = 0; c < C; ++c) a[c * MM + x][v + k] = m_fma(uu, w[c][k], a[c * MM + x][v + k]);
-                        }
-                }
+                        for (int c = 0; c < C; ++c) a[c * MM + x][v + k] = m_fma(uu, w[c][k], a[c * MM + x][v + k]);
+                    }
             }
-            for (; j < np; ++j)
-#pragma unroll
-                for (int c = 0; c < C; ++c)
-#pragma unroll
-                    for (int x = 0; x < MM; ++x)
-                        a[c * MM + x][0] = m_fma(Us[(size_t)j * usr + mm[x]], wc.w_(c)[j], a[c * MM + x][0]);
+        }
+        for (; j < np; ++j)
 #pragma unroll
             for (int c = 0; c < C; ++c)
 #pragma unroll
-                for (int x = 0; x < MM; ++x) {
-                    const T(&b)[8] = a[c * MM + x];
-                    if (x == 0 || m + 32 * x < M)
-                        wc.r_(c)[m + 32 * x] -= ((b[0] + b[1]) + (b[2] + b[3])) + ((b[4] + b[5]) + (b[6] + b[7]));
-                }
-        }
-        return;
+                for (int x = 0; x < MM; ++x)
+                    a[c * MM + x][0] = m_fma(Us[(size_t)j * usr + mm[x]], wc.w_(c)[j], a[c * MM + x][0]);
+#pragma unroll
+        for (int c = 0; c < C; ++c)
+#pragma unroll
+            for (int x = 0; x < MM; ++x) {
+                const T(&b)[8] = a[c * MM + x];
+                if (x == 0 || m + 32 * x < M)
+                    wc.r_(c)[m + 32 * x] -= ((b[0] + b[1]) + (b[2] + b[3])) + ((b[4] + b[5]) + (b[6] + b[7]));
+            }
     }
-    constexpr int NL = WIDE || KVC <= 8 ? 16 : 8;
-    for (int m = lane; m < M; m += 32) {
+}
+
+// The columns of a projection whose U does not fit a packet, streamed through the record
+// ring in tiles of 32 columns (lane = column): sum over the K rows k of U[k][col] vec[k],
+// partial sum i of eight taking the rows k = i mod 8, the rest to sum 0, as above; stored
+// to out (entry) or subtracted from it (exit).  vec and out are chain 0's, chain c's lie
+// c tw elements on.  Every warp of the CTA reads the same stage; reads of U from global
+// memory by each warp were bound by their latency with eight loads in flight per lane
+// (N = 2000, M = 400, 2048 chains, U of 0.2 MB for a block of 125 points and 0.64 MB for
+// the whole grid: 2.39 ms a sweep, 1.35 streamed; 24 problems of 100 to 1000 points: 0.382,
+// 0.313).  Not inlined, so that kernels whose blocks bring U with their packets keep
+// their instruction cache.  In and out: the ring position (stage, phase); ok: no bounded
+// wait gave up.
+struct StreamPos {
+    int slot;
+    unsigned phase;
+    bool ok;
+};
+template <class T, int C>
+__device__ __noinline__ StreamPos project_stream(const T *vec, T *out, int tw, bool subtract, unsigned long long *full,
+                                                 unsigned long long *empty, const unsigned char *stages, int stage_bytes,
+                                                 int depth, int wait_limit, int K, int cols, int width, StreamPos at)
+{
+    constexpr int VEC = VecOf<T>::n;
+    const int lane = threadIdx.x & 31;
+    const int rows = stream_rows<T>(stage_bytes, width);
+    for (int col0 = 0; col0 < cols; col0 += 32) {
         T a[C][8];
 #pragma unroll
         for (int c = 0; c < C; ++c)
 #pragma unroll
             for (int i = 0; i < 8; ++i) a[c][i] = T(0);
-        int j = 0;
-        for (; j + NL - 1 < np; j += NL) {
-            T x[NL];
+        for (int k = 0; k < K;) {
+            if (!warp_wait(full + at.slot, at.phase, wait_limit)) {
+                at.ok = false;
+                return at;
+            }
+            const T *u = reinterpret_cast<const T *>(stages + (size_t)at.slot * stage_bytes) + (lane < width ? lane : 0);
+            const int kend = min(K, k + rows);
+#pragma unroll 2
+            for (; k + 7 < kend; k += 8, u += 8 * width) {
 #pragma unroll
-            for (int i = 0; i < NL; ++i) x[i] = __ldg(Ut + (size_t)(j + i) * M + m);
+                for (int v = 0; v < 8; v += VEC) {
+                    T x[C][VEC];
 #pragma unroll
-            for (int i = 0; i < NL; ++i)
+                    for (int c = 0; c < C; ++c) lds_v(vec + c * tw + k + v, x[c]);
 #pragma unroll
-                for (int c = 0; c < C; ++c) a[c][i & 7] = m_fma(x[i], wc.w_(c)[j + i], a[c][i & 7]);
+                    for (int i = 0; i < VEC; ++i) {
+                        const T uu = u[(v + i) * width];
+#pragma unroll
+                        for (int c = 0; c < C; ++c) a[c][v + i] = m_fma(uu, x[c][i], a[c][v + i]);
+                    }
+                }
+            }
+            for (; k < kend; ++k, u += width)
+#pragma unroll
+                for (int c = 0; c < C; ++c) a[c][0] = m_fma(u[0], vec[c * tw + k], a[c][0]);
+            __syncwarp();
+            mbar_arrive_lane0(empty + at.slot, lane);
+            if (++at.slot == depth) {
+                at.slot = 0;
+                at.phase ^= 1u;
+            }
         }
-        for (; j + 7 < np; j += 8) {
-            T x[8];
+        const int col = col0 + lane;
+        if (col < cols) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) x[i] = __ldg(Ut + (size_t)(j + i) * M + m);
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int c = 0; c < C; ++c) a[c][i] = m_fma(x[i], wc.w_(c)[j + i], a[c][i]);
+            for (int c = 0; c < C; ++c) {
+                const T x = ((a[c][0] + a[c][1]) + (a[c][2] + a[c][3])) + ((a[c][4] + a[c][5]) + (a[c][6] + a[c][7]));
+                if (subtract) out[c * tw + col] -= x;
+                else out[c * tw + col] = x;
+            }
         }
-        for (; j < np; ++j) {
-            const T x = __ldg(Ut + (size_t)j * M + m);
-#pragma unroll
-            for (int c = 0; c < C; ++c) a[c][0] = m_fma(x, wc.w_(c)[j], a[c][0]);
-        }
-#pragma unroll
-        for (int c = 0; c < C; ++c)
-            wc.r_(c)[m] -= ((a[c][0] + a[c][1]) + (a[c][2] + a[c][3])) + ((a[c][4] + a[c][5]) + (a[c][6] + a[c][7]));
     }
+    return at;
 }
 
 // --------------------------------------------------------------------------
@@ -1465,7 +1484,7 @@ struct Visit {
 // A consumer warp: its C chains of chain group `group` (consumers x C chains) of
 // problem p for the launch's sweeps.
 // --------------------------------------------------------------------------
-template <class T, int KV, int C, bool PRIOR, bool WIDE>
+template <class T, int KV, int C, bool PRIOR>
 __device__ __forceinline__ void consume(const SweepParams<T> &p, const LaunchShape &sh, const SweepRange &rg, int group,
                                         unsigned char *smem_raw, const Regions &R, RingPos &rp, bool &failed)
 {
@@ -1541,9 +1560,25 @@ __device__ __forceinline__ void consume(const SweepParams<T> &p, const LaunchSha
             last = uni(B.last) != 0;
             const int bn = uni(B.n), np = uni(B.np), usr = M | 1;
             const T *Us = uni((int)u_staged<T>(sh, B)) ? pk + kPacketHeader + B.rs : nullptr;
-            project_entry<T, C, KV * C, WIDE>(wc, Us, p.pd.Um + B.offU, np, usr, M, lane);
+            // a projection through the record ring, from vec to out
+            auto streamed = [&](int vec, int out, bool subtract, int K, int cols, int width) {
+                const StreamPos at = project_stream<T, C>(wc.sm + vec, wc.sm + out, wc.tw, subtract, R.full, R.empty, R.stages,
+                                                          sh.stage_bytes, sh.depth, sh.wait_limit, K, cols, width,
+                                                          StreamPos{rp.slot, rp.phase, true});
+                rp.slot = uni(at.slot);
+                rp.phase = uni(at.phase);
+                return uni((int)at.ok) != 0;
+            };
+            bool ok = true;
+            if (Us)
+                project_entry<T, C>(wc, Us, np, usr, M, lane);
+            else
+                ok = streamed(wc.off_r, 0, false, M, np, entry_width(np));
+            if (!ok) {
+                failed = true;
+                break;
+            }
             __syncwarp();
-            bool ok;
             if (bn <= 16 * VEC)
                 ok = Visit<T, KV, C, PRIOR, 1, VEC / 2>::run(p, sh, R, rp, wc, n, B, pk, Us, s, keep, trace, win, win_end,
                                                              lane, sd2, sf2);
@@ -1561,7 +1596,12 @@ __device__ __forceinline__ void consume(const SweepParams<T> &p, const LaunchSha
                 break;
             }
             __syncwarp();
-            project_exit<T, C, KV * C, WIDE>(wc, Us, p.pd.Ut + B.offU, np, usr, M, lane);
+            if (Us)
+                project_exit<T, C>(wc, Us, np, usr, M, lane);
+            else if (!streamed(wc.off_w, wc.off_r, true, np, M, 32)) {
+                failed = true;
+                break;
+            }
             // release the packet to the producer (one arrival per warp)
             __syncwarp();
             mbar_arrive_lane0(R.pempty + rp.pslot, lane);
@@ -1633,8 +1673,8 @@ __device__ __forceinline__ void consume(const SweepParams<T> &p, const LaunchSha
 // warp `consumers` produces visit packets and move records.  CTAs pull items
 // from ctrl->queue; an item's parameters are copied from probs into shared memory.
 // --------------------------------------------------------------------------
-template <class T, int KV, int C, int MINB, bool PRIOR>
-__global__ void __launch_bounds__(32 * (kMaxConsumers + 1), MINB)
+template <class T, int KV, int C, bool PRIOR>
+__global__ void __launch_bounds__(32 * (kMaxConsumers + 1), 1)
 sweep_kernel(const SweepParams<T> *__restrict__ probs, const WorkItem *__restrict__ items, RunCtrl *ctrl,
              const __grid_constant__ LaunchShape shape)
 {
@@ -1681,51 +1721,50 @@ sweep_kernel(const SweepParams<T> *__restrict__ probs, const WorkItem *__restric
         if (wcta == shape.consumers)
             produce(sp, shape, rg, R, rp, failed);
         else
-            consume<T, KV, C, PRIOR, (MINB > 1)>(sp, shape, rg, w.group, smem_raw, R, rp, failed);
+            consume<T, KV, C, PRIOR>(sp, shape, rg, w.group, smem_raw, R, rp, failed);
         __syncthreads();   // the item is finished before sp and s_item change
     }
 }
 
-template <class T, int KV, int C, int MINB, bool PRIOR>
+template <class T, int KV, int C, bool PRIOR>
 struct SweepKernel {
     static size_t smem(const LaunchShape &sh) { return (size_t)sh.off_stages + (size_t)sh.depth * sh.stage_bytes; }
     static cudaError_t launch(const SweepParams<T> *probs, const WorkItem *items, RunCtrl *ctrl, const LaunchShape &sh,
                               int ctas, cudaStream_t stream)
     {
-        const cudaError_t e = cudaFuncSetAttribute(sweep_kernel<T, KV, C, MINB, PRIOR>,
+        const cudaError_t e = cudaFuncSetAttribute(sweep_kernel<T, KV, C, PRIOR>,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(sh));
         if (e != cudaSuccess) return e;
-        sweep_kernel<T, KV, C, MINB, PRIOR>
+        sweep_kernel<T, KV, C, PRIOR>
             <<<(unsigned)ctas, 32 * (sh.consumers + 1), smem(sh), stream>>>(probs, items, ctrl, sh);
         return cudaGetLastError();
     }
     static int per_sm(const LaunchShape &sh)
     {
         int n = 0;
-        if (cudaFuncSetAttribute(sweep_kernel<T, KV, C, MINB, PRIOR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(sweep_kernel<T, KV, C, PRIOR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem(sh)) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, sweep_kernel<T, KV, C, MINB, PRIOR>,
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, sweep_kernel<T, KV, C, PRIOR>,
                                                           32 * (sh.consumers + 1), smem(sh)) != cudaSuccess)
             return 0;
         return n;
     }
 };
 
-// dispatch over the register tile (kv) for one chain count per warp, residency MINB
-// (CTAs per SM the registers are budgeted for) and prior flag
-template <class T, int C, int MINB, bool PRIOR, int... KVs>
+// dispatch over the register tile (kv) for one chain count per warp and prior flag
+template <class T, int C, bool PRIOR, int... KVs>
 struct SweepDispatch {
     static cudaError_t launch(const SweepParams<T> *probs, const WorkItem *items, RunCtrl *ctrl, const LaunchShape &sh,
                               int kv, int ctas, cudaStream_t s)
     {
         cudaError_t e = cudaErrorInvalidValue;
-        ((kv == KVs ? (e = SweepKernel<T, KVs, C, MINB, PRIOR>::launch(probs, items, ctrl, sh, ctas, s), 0) : 0), ...);
+        ((kv == KVs ? (e = SweepKernel<T, KVs, C, PRIOR>::launch(probs, items, ctrl, sh, ctas, s), 0) : 0), ...);
         return e;
     }
     static int per_sm(const LaunchShape &sh, int kv)
     {
         int n = 0;
-        ((kv == KVs ? (n = SweepKernel<T, KVs, C, MINB, PRIOR>::per_sm(sh), 0) : 0), ...);
+        ((kv == KVs ? (n = SweepKernel<T, KVs, C, PRIOR>::per_sm(sh), 0) : 0), ...);
         return n;
     }
 };

@@ -1,8 +1,8 @@
-// FP32 chain state (the mixed-precision path), 1 chain per warp: sweep kernels budgeted for one CTA per SM (up to 255 registers per thread).
+// FP32 chain state (the mixed-precision path), 1 chain per warp: sweep kernels.
 #include "asm_sweep.cuh"
 
 namespace asmgb {
 
-ASM_DEFINE_SWEEP_LAUNCHER(float, f32_c1_m1, 1, 1, false, 1, 2, 4, 8, 16)
+ASM_DEFINE_SWEEP_LAUNCHER(float, f32_c1, 1, false, 1, 2, 4, 8, 16)
 
 }  // namespace asmgb

@@ -1,8 +1,8 @@
-// FP64 chain state: sweep kernels with the gamma prior's acceptance step, one chain per warp, one CTA per SM.
+// FP64 chain state: sweep kernels with the gamma prior's acceptance step, one chain per warp.
 #include "asm_sweep.cuh"
 
 namespace asmgb {
 
-ASM_DEFINE_SWEEP_LAUNCHER(double, f64_prior, 1, 1, true, 1, 2, 4, 8, 16, 32)
+ASM_DEFINE_SWEEP_LAUNCHER(double, f64_prior, 1, true, 1, 2, 4, 8, 16, 32)
 
 }  // namespace asmgb
