@@ -17,6 +17,14 @@ constexpr int kPacketHeader = 32;
 // Residual refresh period of the sweep loop (sweeps).
 constexpr int kRefreshPeriod = 64;
 
+// Row stride of U in a packet: FP32 4 x odd, so that 16-byte loads of a row per lane are free
+// of bank conflicts, FP64 odd, for 8-byte ones.  Packets are laid out for the larger of the two.
+template <class T>
+__host__ __device__ constexpr int packet_row(int M)
+{
+    return sizeof(T) == 4 ? ((M + 3) / 4 | 1) * 4 : M | 1;
+}
+
 // One block of one level, as the device sees it.  Offsets are in elements of
 // the precision-specific arrays.
 struct BlockDesc {
@@ -26,8 +34,10 @@ struct BlockDesc {
     int ng, nz;      // modes before ng are Gaussian (d > 0), from nz on flat (d = 0 in this precision)
     int rs;          // row stride of V/R rows
     int recstride;   // elements per move record: 2 rs + 4
-    int usr;         // row stride of U in the packet: M | 1 (odd: conflict-free column reads)
+    int usr;         // elements a packet provides per row of U (the larger precision's stride)
     int last;        // 1: the last block of its level
+    int pkn;         // elements of the visit packet with U (saturated)
+    float inv_rec;   // 1 / recstride
     long long offUe, offUx;   // U in tiles of 32 columns for the streamed projections: entry
                               // (columns are modes, M rows each), exit (data points, np rows)
     long long offRec;  // move records of the block: n records of recstride elements
@@ -219,13 +229,13 @@ constexpr int kStepTraceMax = 4096;
 constexpr int kMaxConsumers = 7;
 // Deepest ring of move records (stages) a launch may use.
 constexpr int kMaxRingDepth = 48;
-// Move records of the largest block per ring stage: up to kMaxLargeRecords where shared
+// Move records of the largest block per ring stage: about kStageBytes of them where shared
 // memory allows, at least kRecordsPerStage while three stages fit (a stage costs a consumer
-// its wait, its release and the start of its loop); smaller blocks put up to
-// kMaxRecordsPerStage in a stage of that size.
+// some 450 cycles: its wait, its release and the start of its loop); smaller blocks put up
+// to kMaxRecordsPerStage in a stage of that size.
+constexpr int kStageBytes = 32 * 1024;
 constexpr int kRecordsPerStage = 4;
-constexpr int kMaxLargeRecords = 8;
-constexpr int kMaxRecordsPerStage = 16;
+constexpr int kMaxRecordsPerStage = 64;
 // Most slots of the ring of visit packets.
 constexpr int kMaxPacketSlots = 8;
 // Largest kv (16-byte vectors per lane and chain): 64 elements per lane.

@@ -894,7 +894,7 @@ int build_precision(asm_problem *p, const HostFactors &hf, PrecBuffers &out)
         bounds_row(0, k + kPacketHeader);
         for (int j = 0; j < B.np; ++j)
             for (int m = 0; m < M; ++m)
-                k[kPacketHeader + B.rs + (size_t)j * B.usr + m] = (T)hU[(size_t)j * M + m];
+                k[kPacketHeader + B.rs + (size_t)j * packet_row<T>(M) + m] = (T)hU[(size_t)j * M + m];
     }
     int rc;
     if ((rc = upload(&out.rec, rec)) || (rc = upload(&out.pk, pk)) || (rc = upload(&out.Ue, Ue)) ||
@@ -1121,7 +1121,8 @@ bool plan_shape(LaunchShape &sh, const ShapeChoice &pick, const PlanNeeds &nd, l
         if (rps == 0) {   // as many as leave room for everything else, at least kRecordsPerStage
             size_t extras = per_word * nr * (sizeof(T) == 4 ? 3 : 1);
             if (stage_u && !nd.packets.empty()) extras += 2 * (align_up((size_t)nd.packets.back(), 128) - head);
-            for (rps = kMaxLargeRecords; rps > kRecordsPerStage; --rps)
+            rps = std::min(kMaxRecordsPerStage, std::max(kRecordsPerStage, kStageBytes / (int)(nd.max_rec * sizeof(T))));
+            for (; rps > kRecordsPerStage; --rps)
                 if (used + extras + min_stages * stage_of(rps) <= budget) break;
         }
         while (rps > 1 && used + min_stages * stage_of(rps) > budget) --rps;
@@ -1580,8 +1581,10 @@ int asm_setup(const asm_desc *ds, asm_problem **out)
             B.last = b + 1 == ds->level_nblocks[l];
             B.offUe = oUe; oUe += (long long)((B.np + 31) / 32) * M * entry_cols(B.np);
             B.offUx = oUx; oUx += (long long)((M + 31) / 32) * B.np * 32;
-            B.usr = M | 1;
+            B.usr = std::max(packet_row<float>(M), packet_row<double>(M));
+            B.pkn = (int)std::min<long long>(kPacketHeader + B.rs + (long long)B.np * B.usr, 1 << 28);
             B.recstride = 2 * B.rs + 4;   // elements; the mode data take 3
+            B.inv_rec = 1.0f / (float)B.recstride;
             B.offRec = oRec; oRec += (long long)B.n * B.recstride;
             B.offPk = oPk; oPk += (kPacketHeader + B.rs + (long long)B.np * B.usr + 3) / 4 * 4;   // 16-byte aligned
             p->max_rec = std::max(p->max_rec, B.recstride);

@@ -488,13 +488,15 @@ __device__ __forceinline__ float narrow_offset(float a, float w, float u, int &c
     const float lam = a + 0.5f * w;
     const float x = lam * w;
     float t = m_abs(x) < 1e-3f ? u * w * (1.0f - 0.5f * x * (1.0f - u))   // the series for small lam w
-                               : -m_log1p(u * m_expm1(-x)) / lam;
+                               : m_abs(lam) < 1e30f ? div_by(-m_log1p(u * m_expm1(-x)), lam, __frcp_rn(lam))
+                                                    : -m_log1p(u * m_expm1(-x)) / lam;
     t = m_min(m_max(t, 0.0f), w);
     if (w * w <= 4e-7f) return t;
     const float target = __fmul_rn(u, __fmul_rn(0.5f * w, narrow_sum(a, w)));
     int it = 0;
     for (; it < GL::nmax; ++it) {
-        const float step = fmaf(0.5f * t, narrow_sum(a, t), -target) / m_exp(-t * (a + 0.5f * t));
+        const float den = m_exp(-t * (a + 0.5f * t));   // in [e^-1/2, e^1/2]
+        const float step = div_by(fmaf(0.5f * t, narrow_sum(a, t), -target), den, __frcp_rn(den));
         t = m_min(m_max(t - step, 0.0f), w);
         if (w <= 0.2f || m_abs(step) <= GL::tol * t || t == 0.0f) break;
     }
@@ -759,16 +761,6 @@ __device__ __forceinline__ double draw_team(double c, double d, double invd, dou
     return open ? fmin(fmax(delta, lo), hi) : 0.0;
 }
 
-// --------------------------------------------------------------------------
-// Position in the stream of blocks and moves of a launch (sweep, level, block).
-// --------------------------------------------------------------------------
-struct BlockCursor {
-    long long s, s_end;     // sweep, end of the launch's range
-    int bi, nb;             // block within the level, blocks of the level
-    const BlockDesc *bd;    // blocks of the level
-    bool done;
-};
-
 // The launch's sweep range, read from the device control block.
 struct SweepRange {
     long long sweep0, nsweeps, burn_in;
@@ -802,17 +794,16 @@ __device__ __forceinline__ void packet_next(RingPos &r, int slots)
     }
 }
 
-// Bytes of a block's visit packet: header and first bounds row alone, or with U where it fits a slot.
+// Whether a block's U comes with its visit packet, and the packet's bytes.
 template <class T>
-__device__ __forceinline__ unsigned packet_bytes(const LaunchShape &sh, const BlockDesc &B)
+__device__ __forceinline__ bool u_staged(const LaunchShape &sh, int pkn)
 {
-    const unsigned whole = (unsigned)((kPacketHeader + B.rs + (long long)B.np * B.usr) * (long long)sizeof(T) + 15) & ~15u;
-    return whole <= (unsigned)sh.pbytes ? whole : (unsigned)((kPacketHeader + B.rs) * sizeof(T));
+    return pkn <= sh.pbytes / (int)sizeof(T);
 }
 template <class T>
-__device__ __forceinline__ bool u_staged(const LaunchShape &sh, const BlockDesc &B)
+__device__ __forceinline__ unsigned packet_bytes(const LaunchShape &sh, int pkn, int rs)
 {
-    return packet_bytes<T>(sh, B) > (unsigned)((kPacketHeader + B.rs) * sizeof(T));
+    return u_staged<T>(sh, pkn) ? (unsigned)(pkn * sizeof(T) + 15) & ~15u : (unsigned)((kPacketHeader + rs) * sizeof(T));
 }
 // Streamed U: columns of an entry tile (modes; 32, or fewer for small blocks) and rows per ring stage.
 __device__ __forceinline__ int entry_width(int np) { return np > 16 ? 32 : np > 8 ? 16 : np > 4 ? 8 : 4; }
@@ -821,11 +812,14 @@ __device__ __forceinline__ int stream_rows(int stage_bytes, int width)
 {
     return (stage_bytes / (int)(width * sizeof(T))) & ~7;
 }
-// Records of a block per ring stage.
+// Records of a block per ring stage: floor(stage / record) by the block's reciprocal (an
+// integer division costs each visit of a small block about as much as a flat move).  The
+// product is off by less than 64 2^-23, and a quotient that is not whole stays 1/4100 (the
+// longest record) away from the next whole number, so 1e-4 makes the floor exact.
 template <class T>
-__device__ __forceinline__ int records_per_stage(const LaunchShape &sh, int recstride)
+__device__ __forceinline__ int records_per_stage(const LaunchShape &sh, float inv_rec)
 {
-    return min(kMaxRecordsPerStage, sh.stage_bytes / (int)(recstride * sizeof(T)));
+    return min(kMaxRecordsPerStage, (int)((float)(sh.stage_bytes / (int)sizeof(T)) * inv_rec + 1e-4f));
 }
 
 __device__ __forceinline__ int level_of_sweep(long long s, unsigned long long seed, unsigned long long pid,
@@ -835,26 +829,6 @@ __device__ __forceinline__ int level_of_sweep(long long s, unsigned long long se
     philox4x64_10(l0, l1, l2, l3, seed, 0ull);
     int level = (int)(uniform_from<double>(l0) * n_levels);
     return level >= n_levels ? n_levels - 1 : level;
-}
-
-template <class T>
-__device__ __forceinline__ void cursor_start_sweep(BlockCursor &c, const SweepParams<T> &p)
-{
-    const int level = level_of_sweep(c.s, p.seed, p.problem_id, p.n_levels);
-    c.nb = p.level_nblocks[level];
-    c.bd = p.blocks + p.level_first[level];
-    c.bi = 0;
-}
-
-template <class T>
-__device__ __forceinline__ void cursor_advance(BlockCursor &c, const SweepParams<T> &p)
-{
-    if (++c.bi < c.nb) return;
-    if (++c.s >= c.s_end) {
-        c.done = true;
-        return;
-    }
-    cursor_start_sweep(c, p);
 }
 
 // Arrival by lane 0 of the warp only, as a predicated instruction (no branch).
@@ -890,64 +864,109 @@ struct Regions {
 // packet slot, then the block's move records, as many to a ring stage as fit,
 // one bulk copy per stage, before and after them the tiles of U for the
 // projections where it did not fit; each copy after every consumer warp has
-// released the slot's previous contents.  The ring positions run on across the CTA's items.
+// released the slot's previous contents.  Lane 0 issues; the lanes hold the
+// descriptors of the next 32 blocks of the level, read while the copies before
+// them are issued (a descriptor read from global memory per visit made the
+// producer the slowest warp of a level of one-point blocks).  The ring positions
+// run on across the CTA's items.
 // --------------------------------------------------------------------------
 template <class T>
 __device__ __forceinline__ void produce(const SweepParams<T> &p, const LaunchShape &sh, const SweepRange &rg,
                                         const Regions &R, RingPos &rp, bool &failed)
 {
-    if ((threadIdx.x & 31) != 0 || rg.nsweeps <= 0 || failed || sh.stall) return;
-    const int D = sh.depth, P = sh.pslots;
-    BlockCursor c;
-    c.s = rg.sweep0;
-    c.s_end = rg.sweep0 + rg.nsweeps;
-    c.done = false;
-    cursor_start_sweep(c, p);
+    const long long nsweeps = uni(rg.nsweeps), sweep0 = uni(rg.sweep0);
+    if (nsweeps <= 0 || failed || sh.stall) return;
+    const int lane = threadIdx.x & 31;
+    const int D = sh.depth, P = sh.pslots, M = uni(p.M);
     const unsigned g0 = rp.g, pg0 = rp.pg;
-    BlockDesc next = c.bd[c.bi];
-    bool done = false;
-    while (!done && !failed) {
-        const BlockDesc B = next;
-        cursor_advance(c, p);
-        if (!c.done) next = c.bd[c.bi];   // in flight while this block's copies are issued
-        if (rp.pg >= (unsigned)P && !mbar_wait(R.pempty + rp.pslot, rp.pphase ^ 1u, sh.wait_limit)) {
+    // the blocks [base, base + 32) of sweep s, lane i's in B
+    struct Batch {
+        long long s;
+        int base, nb, first;
+        BlockDesc B;
+    };
+    auto load = [&](Batch &b) {   // the batch's descriptors (read-only data)
+        const int i = min(b.base + lane, b.nb - 1);
+        b.B = p.blocks[b.first + i];
+    };
+    auto start = [&](Batch &b, long long s) {
+        const int level = level_of_sweep(s, p.seed, p.problem_id, p.n_levels);
+        b.s = s;
+        b.base = 0;
+        b.nb = uni(p.level_nblocks[level]);
+        b.first = uni(p.level_first[level]);
+        load(b);
+    };
+    auto advance = [&](Batch &b) {
+        b.base += 32;
+        if (b.base < b.nb) load(b);
+        else if (b.s + 1 < sweep0 + nsweeps) start(b, b.s + 1);
+        else b.s = -1;
+    };
+    // one bulk copy into the next ring stage (lane 0)
+    auto stage = [&](const T *src, unsigned bytes) {
+        if (failed || (rp.g >= (unsigned)D && !mbar_wait(R.empty + rp.slot, rp.phase ^ 1u, sh.wait_limit))) {
             failed = true;
-            break;
+            return;
         }
-        const unsigned pbytes = packet_bytes<T>(sh, B);
-        mbar_expect_tx(R.pfull + rp.pslot, pbytes);
-        bulk_g2s(R.packets + (size_t)rp.pslot * sh.pbytes, p.pd.pk + B.offPk, pbytes, R.pfull + rp.pslot);
-        packet_next(rp, P);
-        // one bulk copy into the next ring stage
-        auto stage = [&](const T *src, size_t elements) {
-            if (failed || (rp.g >= (unsigned)D && !mbar_wait(R.empty + rp.slot, rp.phase ^ 1u, sh.wait_limit))) {
-                failed = true;
-                return;
+        mbar_expect_tx(R.full + rp.slot, bytes);
+        bulk_g2s(R.stages + (size_t)rp.slot * sh.stage_bytes, src, bytes, R.full + rp.slot);
+        ring_next(rp, D);
+    };
+    // tiles of a streamed projection: columns [32 t, 32 t + width) x K rows, tile after tile
+    auto stream = [&](const T *src, int K, int cols, int width) {
+        const int rows = stream_rows<T>(sh.stage_bytes, width);
+        for (int col0 = 0; col0 < cols && !failed; col0 += 32)
+            for (int k = 0; k < K && !failed; k += rows) {
+                const int n = min(rows, K - k);
+                stage(src, (unsigned)(n * width * sizeof(T)));
+                src += (size_t)n * width;
             }
-            const unsigned bytes = (unsigned)(elements * sizeof(T));
-            mbar_expect_tx(R.full + rp.slot, bytes);
-            bulk_g2s(R.stages + (size_t)rp.slot * sh.stage_bytes, src, bytes, R.full + rp.slot);
-            ring_next(rp, D);
-        };
-        // tiles of a streamed projection: columns [32 t, 32 t + width) x K rows, tile after tile
-        auto stream = [&](const T *src, int K, int cols, int width) {
-            const int rows = stream_rows<T>(sh.stage_bytes, width);
-            for (int col0 = 0; col0 < cols && !failed; col0 += 32)
-                for (int k = 0; k < K && !failed; k += rows) {
-                    const int n = min(rows, K - k);
-                    stage(src, (size_t)n * width);
-                    src += (size_t)n * width;
+    };
+    Batch cur;
+    start(cur, sweep0);
+    while (cur.s >= 0 && !failed) {
+        // this batch's blocks: what lane 0 needs of each, from its lane
+        const int count = min(32, cur.nb - cur.base);
+        const int n_ = cur.B.n, np_ = cur.B.np, rb_ = cur.B.recstride * (int)sizeof(T);
+        const int rps_ = records_per_stage<T>(sh, cur.B.inv_rec);
+        const unsigned pb_ = packet_bytes<T>(sh, cur.B.pkn, cur.B.rs);
+        const int staged_ = u_staged<T>(sh, cur.B.pkn);
+        const long long pk_ = cur.B.offPk, rec_ = cur.B.offRec, ue_ = cur.B.offUe, ux_ = cur.B.offUx;
+        advance(cur);   // in flight while the copies of this batch are issued
+        for (int i = 0; i < count && !failed; ++i) {
+            const int n = __shfl_sync(0xffffffffu, n_, i), rps = __shfl_sync(0xffffffffu, rps_, i),
+                      rb = __shfl_sync(0xffffffffu, rb_, i), staged = __shfl_sync(0xffffffffu, staged_, i);
+            const unsigned pb = __shfl_sync(0xffffffffu, pb_, i);
+            const long long pk = __shfl_sync(0xffffffffu, pk_, i), rec = __shfl_sync(0xffffffffu, rec_, i);
+            int np = 0;
+            long long ue = 0, ux = 0;
+            if (!staged) {
+                np = __shfl_sync(0xffffffffu, np_, i);
+                ue = __shfl_sync(0xffffffffu, ue_, i);
+                ux = __shfl_sync(0xffffffffu, ux_, i);
+            }
+            if (lane == 0) {
+                if (rp.pg >= (unsigned)P && !mbar_wait(R.pempty + rp.pslot, rp.pphase ^ 1u, sh.wait_limit)) {
+                    failed = true;
+                } else {
+                    mbar_expect_tx(R.pfull + rp.pslot, pb);
+                    bulk_g2s(R.packets + (size_t)rp.pslot * sh.pbytes, p.pd.pk + pk, pb, R.pfull + rp.pslot);
+                    packet_next(rp, P);
                 }
-        };
-        const bool streamed = !u_staged<T>(sh, B);
-        if (streamed) stream(p.pd.Ue + B.offUe, p.M, B.np, entry_width(B.np));
-        const int rps = records_per_stage<T>(sh, B.recstride);
-        for (int j = 0; j < B.n && !failed; j += rps)
-            stage(p.pd.rec + B.offRec + (size_t)j * B.recstride, (size_t)min(rps, B.n - j) * B.recstride);
-        if (streamed) stream(p.pd.Ux + B.offUx, B.np, p.M, 32);
-        done = c.done;
+                if (!staged) stream(p.pd.Ue + ue, M, np, entry_width(np));
+                const char *src = reinterpret_cast<const char *>(p.pd.rec + rec);
+                for (int j = 0; j < n && !failed; j += rps) {
+                    const unsigned bytes = (unsigned)(min(rps, n - j) * rb);
+                    stage(reinterpret_cast<const T *>(src), bytes);
+                    src += bytes;
+                }
+                if (!staged) stream(p.pd.Ux + ux, np, M, 32);
+            }
+            failed = uni((int)failed) != 0;
+        }
     }
-    if (failed) {
+    if (failed && lane == 0) {
         // the copies already issued must land before the CTA may exit
         const unsigned from = rp.g > g0 + (unsigned)D ? rp.g - D : g0;
         for (unsigned k = from; k < rp.g; ++k)
@@ -957,6 +976,7 @@ __device__ __forceinline__ void produce(const SweepParams<T> &p, const LaunchSha
             mbar_wait(R.pfull + (k % (unsigned)P), (k / (unsigned)P) & 1u, sh.wait_limit);
         atomicAdd(&p.counters->timeouts, 1ull);
     }
+    __syncwarp();
 }
 
 // The C chains of a consumer warp: shared memory and state of each.
@@ -985,24 +1005,33 @@ struct MoveCounts {
 // in increasing m, the rest goes to sum 0, then a fixed tree; so the sums are the same for
 // any C, from a packet or streamed.  Blocks of up to eight modes spread the eight
 // partial sums over lanes (four modes at a time): with a lane per mode most lanes idle.
+// FP32: U's rows in the packet are 4 x odd elements apart, so that 16-byte loads of a row per
+// lane meet no bank conflict (hierarchy of 64 points, 1024 chains: 0.0693 -> 0.0650 ms a sweep).
 template <class T, int C>
 __device__ __forceinline__ void project_entry(const WarpChains<T, C> &wc, const T *Us, int np, int usr, int M, int lane)
 {
     constexpr int VEC = VecOf<T>::n;
     if (np <= 8) {
-        const int i = lane & 7;
+        const int i = lane & 7, m8 = M & ~7;
 #pragma unroll
         for (int c = 0; c < C; ++c) {
             const T *r = wc.r_(c);
             for (int j0 = 0; j0 < np; j0 += 4) {
                 const int j = j0 + (lane >> 3);
                 const T *u = Us + (size_t)min(j, np - 1) * usr;
+                T tu[7], tr[7];   // the last M mod 8 terms, loaded ahead
+#pragma unroll
+                for (int k = 0; k < 7; ++k) {
+                    const bool in = i == 0 && m8 + k < M;
+                    tu[k] = in ? u[m8 + k] : T(0);
+                    tr[k] = in ? r[m8 + k] : T(0);
+                }
                 T a = T(0);
-                int m = 0;
-#pragma unroll 4
-                for (; m + 7 < M; m += 8) a = m_fma(u[m + i], r[m + i], a);
-                if (i == 0)
-                    for (; m < M; ++m) a = m_fma(u[m], r[m], a);
+#pragma unroll 8
+                for (int m = i; m < m8; m += 8) a = m_fma(u[m], r[m], a);
+#pragma unroll
+                for (int k = 0; k < 7; ++k)
+                    if (i == 0 && m8 + k < M) a = m_fma(tu[k], tr[k], a);
                 a += __shfl_xor_sync(0xffffffffu, a, 1);
                 a += __shfl_xor_sync(0xffffffffu, a, 2);
                 a += __shfl_xor_sync(0xffffffffu, a, 4);
@@ -1029,13 +1058,19 @@ __device__ __forceinline__ void project_entry(const WarpChains<T, C> &wc, const 
 #pragma unroll
                 for (int c = 0; c < C; ++c) lds_v(wc.r_(c) + m + v, r[c]);
 #pragma unroll
-                for (int k = 0; k < VEC; ++k)
+                for (int x = 0; x < JJ; ++x) {
+                    T uu[VEC];
+                    if constexpr (sizeof(T) == 4) {
+                        lds_v(u[x] + m + v, uu);
+                    } else {   // rows of an odd stride
 #pragma unroll
-                    for (int x = 0; x < JJ; ++x) {
-                        const T uu = u[x][m + v + k];
-#pragma unroll
-                        for (int c = 0; c < C; ++c) a[c * JJ + x][v + k] = m_fma(uu, r[c][k], a[c * JJ + x][v + k]);
+                        for (int k = 0; k < VEC; ++k) uu[k] = u[x][m + v + k];
                     }
+#pragma unroll
+                    for (int k = 0; k < VEC; ++k)
+#pragma unroll
+                        for (int c = 0; c < C; ++c) a[c * JJ + x][v + k] = m_fma(uu[k], r[c][k], a[c * JJ + x][v + k]);
+                }
             }
         }
         for (; m < M; ++m)
@@ -1314,7 +1349,7 @@ struct Visit {
 #pragma unroll
             for (int c = 0; c < C; ++c) kk[c].fold(lk[c], hk[c]);
         }
-        const int rps = records_per_stage<T>(sh, recstride);
+        const int rps = records_per_stage<T>(sh, uni(B.inv_rec));
         // modes j < ng are Gaussian, those from nz on flat; in between both occur (never, when
         // the singular values are sorted)
         const int ng = uni(B.ng), nz = uni(B.nz);
@@ -1558,8 +1593,8 @@ __device__ __forceinline__ void consume(const SweepParams<T> &p, const LaunchSha
             const T *pk = reinterpret_cast<const T *>(R.packets + (size_t)rp.pslot * sh.pbytes);
             const BlockDesc &B = *reinterpret_cast<const BlockDesc *>(pk);
             last = uni(B.last) != 0;
-            const int bn = uni(B.n), np = uni(B.np), usr = M | 1;
-            const T *Us = uni((int)u_staged<T>(sh, B)) ? pk + kPacketHeader + B.rs : nullptr;
+            const int bn = uni(B.n), np = uni(B.np), usr = packet_row<T>(M);
+            const T *Us = u_staged<T>(sh, uni(B.pkn)) ? pk + kPacketHeader + uni(B.rs) : nullptr;
             // a projection through the record ring, from vec to out
             auto streamed = [&](int vec, int out, bool subtract, int K, int cols, int width) {
                 const StreamPos at = project_stream<T, C>(wc.sm + vec, wc.sm + out, wc.tw, subtract, R.full, R.empty, R.stages,
