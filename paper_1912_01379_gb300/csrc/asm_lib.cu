@@ -452,6 +452,7 @@ struct asm_problem {
     float *d_Kth32 = nullptr;
     double *d_w = nullptr, *d_dw = nullptr;   // weights and dw/dtheta (P x N)
     double *d_vjp = nullptr;               // scratch of asm_backward: v', v, u (N each), y (M), g (P)
+    double *d_result = nullptr;            // results of asm_average and asm_mc_error: (3 + 2 kBinLevels) N, on first use
     bool moments = false;
     long long nsnap = 0;                   // chain snapshots in the moments
     PrecBuffers b64, b32;
@@ -1999,6 +2000,16 @@ int asm_tune(asm_problem *p, int chains, int precision, void *d_workspace, size_
 }
 
 namespace {
+// The handle's result buffer (a device allocation per result call cost a tenth of a short
+// run; the stream orders its uses, and a handle is used by one thread at a time).
+double *result_buffer(asm_problem *p)
+{
+    if (!p->d_result &&
+        cudaMalloc(&p->d_result, sizeof(double) * (3 + 2 * (size_t)kBinLevels) * (size_t)p->N) != cudaSuccess)
+        p->d_result = nullptr;
+    return p->d_result;
+}
+
 // Reads the run's device counters (synchronises the stream).
 int read_counters(asm_problem *p, Counters *c)
 {
@@ -2021,16 +2032,10 @@ int asm_average(asm_problem *p, double *mean_A, double *sem_A, double *ess, doub
     if (!p) return ASM_ERR_ARG;
     if (!p->kids.empty()) return ASM_ERR_ARG;   // a batch: asm_average_at
     if (!p->have_run || p->kept < 1) return ASM_ERR_STATE;
-    {
-        Counters c{};
-        const int rc0 = read_counters(p, &c);
-        if (rc0 != ASM_OK) return rc0;
-        if (c.timeouts) return ASM_ERR_TIMEOUT;
-    }
     const WsLayout L = ws_layout(p, p->chains, p->precision);
     const int N = p->N;
-    double *d = nullptr;
-    if (cudaMalloc(&d, sizeof(double) * 3 * N) != cudaSuccess) return ASM_ERR_CUDA;
+    double *d = result_buffer(p);
+    if (!d) return ASM_ERR_CUDA;
     char *ws = (char *)p->ws;
     ++p->other_launches;
     const bool open32 = p->precision != ASM_FP64;   // FP32 state: sums of the open 64-sweep block
@@ -2038,13 +2043,12 @@ int asm_average(asm_problem *p, double *mean_A, double *sem_A, double *ess, doub
         (const double *)(ws + L.S1), (const double *)(ws + L.S2), open32 ? (const float *)(ws + L.P1) : nullptr,
         open32 ? (const float *)(ws + L.P2) : nullptr, L.ldF, p->chains, N, (double)p->kept, d, d + N, d + 2 * N);
     std::vector<double> h((size_t)3 * N);
-    int rc = ASM_OK;
+    Counters c{};
     if (cudaGetLastError() != cudaSuccess ||
-        cudaMemcpyAsync(h.data(), d, sizeof(double) * 3 * N, cudaMemcpyDeviceToHost, p->stream) != cudaSuccess ||
-        cudaStreamSynchronize(p->stream) != cudaSuccess)
-        rc = ASM_ERR_CUDA;
-    cudaFree(d);
-    if (rc != ASM_OK) return rc;
+        cudaMemcpyAsync(h.data(), d, sizeof(double) * 3 * N, cudaMemcpyDeviceToHost, p->stream) != cudaSuccess)
+        return ASM_ERR_CUDA;
+    if (const int rc = read_counters(p, &c); rc != ASM_OK) return rc;   // synchronises
+    if (c.timeouts) return ASM_ERR_TIMEOUT;
     for (int n = 0; n < N; ++n) {
         const double mu = h[n], s2 = h[N + n], m2 = h[2 * N + n];
         const double var = std::max(m2 - mu * mu, 0.0);
@@ -2062,16 +2066,11 @@ int asm_mc_error(asm_problem *p, int k, double *ess, double *sem_fbar, double *s
     if (!p || k < 0 || k >= asm_problem_count(p)) return ASM_ERR_ARG;
     asm_problem *u = p->kids.empty() ? p : p->kids[(size_t)k];
     if (!p->have_run || !u->have_run || u->kept < 1) return ASM_ERR_STATE;
-    {
-        Counters c{};
-        if (read_counters_all(p, &c) != ASM_OK) return ASM_ERR_CUDA;
-        if (c.timeouts) return ASM_ERR_TIMEOUT;
-    }
     const WsLayout L = ws_layout(u, u->chains, u->precision);
     const int N = u->N, chains = u->chains;
     const size_t nk = (size_t)kBinLevels * N;
-    double *d = nullptr;
-    if (cudaMalloc(&d, sizeof(double) * (3 * (size_t)N + 2 * nk)) != cudaSuccess) return ASM_ERR_CUDA;
+    double *d = result_buffer(u);
+    if (!d) return ASM_ERR_CUDA;
     const char *ws = (const char *)u->ws;
     const bool open32 = u->precision != ASM_FP64;
     reduce_kernel<<<col_ctas(N), kColThreads, 0, p->stream>>>(
@@ -2083,14 +2082,15 @@ int asm_mc_error(asm_problem *p, int k, double *ess, double *sem_fbar, double *s
     p->other_launches += 2;
     std::vector<double> h(3 * (size_t)N + 2 * nk);
     int nb = 0;
-    int rc = ASM_OK;
     if (cudaGetLastError() != cudaSuccess ||
         cudaMemcpyAsync(h.data(), d, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, p->stream) != cudaSuccess ||
-        cudaMemcpyAsync(&nb, ws + L.bcount, sizeof(int), cudaMemcpyDeviceToHost, p->stream) != cudaSuccess ||
-        cudaStreamSynchronize(p->stream) != cudaSuccess)
-        rc = ASM_ERR_CUDA;
-    cudaFree(d);
-    if (rc != ASM_OK) return rc;
+        cudaMemcpyAsync(&nb, ws + L.bcount, sizeof(int), cudaMemcpyDeviceToHost, p->stream) != cudaSuccess)
+        return ASM_ERR_CUDA;
+    {
+        Counters c{};
+        if (read_counters_all(p, &c) != ASM_OK) return ASM_ERR_CUDA;   // synchronises
+        if (c.timeouts) return ASM_ERR_TIMEOUT;
+    }
     const double *A1 = h.data() + 3 * N, *A2 = A1 + nk;
     for (int l = 0; l < kBinLevels; ++l)
         if (bins_per_chain) bins_per_chain[l] = nb >> l;
@@ -2164,20 +2164,16 @@ int asm_chain_state(asm_problem *p, double *f, double *chi2)
     if (!p) return ASM_ERR_ARG;
     if (!p->kids.empty()) return ASM_ERR_ARG;
     if (!p->have_run) return ASM_ERR_STATE;
-    {
-        Counters c{};
-        const int rc0 = read_counters(p, &c);
-        if (rc0 != ASM_OK) return rc0;
-        if (c.timeouts) return ASM_ERR_TIMEOUT;
-    }
     const WsLayout L = ws_layout(p, p->chains, p->precision);
     const size_t es = p->precision == ASM_FP64 ? 8 : 4;
     const char *ws = (const char *)p->ws;
     std::vector<unsigned char> hF((size_t)p->chains * L.ldF * es), hR((size_t)p->chains * L.ldR * es);
     if (cudaMemcpyAsync(hF.data(), ws + L.F, hF.size(), cudaMemcpyDeviceToHost, p->stream) != cudaSuccess ||
-        cudaMemcpyAsync(hR.data(), ws + L.R, hR.size(), cudaMemcpyDeviceToHost, p->stream) != cudaSuccess ||
-        cudaStreamSynchronize(p->stream) != cudaSuccess)
+        cudaMemcpyAsync(hR.data(), ws + L.R, hR.size(), cudaMemcpyDeviceToHost, p->stream) != cudaSuccess)
         return ASM_ERR_CUDA;
+    Counters c{};
+    if (const int rc = read_counters(p, &c); rc != ASM_OK) return rc;   // synchronises
+    if (c.timeouts) return ASM_ERR_TIMEOUT;
     for (int q = 0; q < p->chains; ++q) {
         if (f)
             for (int n = 0; n < p->N; ++n) {
@@ -2394,7 +2390,7 @@ void asm_destroy(asm_problem *p)
     for (asm_problem *u : p->kids) asm_destroy(u);
     p->kids.clear();
     void *ptrs[] = {p->d_level_first, p->d_level_nblocks, p->d_blocks, p->d_KtT, p->d_gt, p->d_Khi, p->d_Klo, p->d_L,
-                    p->d_Kth64, p->d_Kth32, p->d_w, p->d_dw, p->d_vjp};
+                    p->d_Kth64, p->d_Kth32, p->d_w, p->d_dw, p->d_vjp, p->d_result};
     for (void *x : ptrs)
         if (x) cudaFree(x);
     free_prec(p->b64);
