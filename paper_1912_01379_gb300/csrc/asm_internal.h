@@ -123,7 +123,7 @@ struct LaunchShape {
     int rps;                          // the largest block's move records per stage
     int pslots, pbytes;               // visit packets: slots and bytes of one
     int off_bars, off_packets, off_stages;  // byte offsets in dynamic shared memory
-    int cpad;                         // shared-memory stride of the c/w buffers (>= max np)
+    int cpad;                         // shared-memory elements of the c / w buffer (>= max np)
     int mpad;                         // shared-memory stride of the residual (>= max M)
     int fpad;                         // chain state in shared memory (>= max N; 0: in global memory)
     int npad;                         // shared-memory sums of the kept sweeps per chain (>= max N;

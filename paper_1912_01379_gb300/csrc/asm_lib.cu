@@ -1069,7 +1069,7 @@ ShapeChoice pick_shape(bool f64, int kv, int chains, const std::vector<double> &
     return best;
 }
 
-// Shared memory of the sweep kernel: per chain c, w, r~ and the uniforms of a window of
+// Shared memory of the sweep kernel: per chain c / w, r~ and the uniforms of a window of
 // 128 moves (with a prior as many for the acceptances), the barriers, the packet slots
 // and the record stages.  CTAs per SM: as many as the work needs and the registers allow
 // (the persistent kernel queues the rest).  What the budget leaves goes, in this order, to: a ring of at least
@@ -1112,8 +1112,8 @@ bool plan_shape(LaunchShape &sh, const ShapeChoice &pick, const PlanNeeds &nd, l
         if (by_regs < 1) return false;   // no kernel for this tile
         const long long ctas = (total_warps + consumers - 1) / consumers;
         const int per_sm = (int)std::min<long long>(by_regs, std::max<long long>(1, (ctas + kSMs - 1) / kSMs));
-        const size_t budget = std::min<size_t>(220 * 1024 / per_sm, 224 * 1024);
-        const int base_words = 2 * sh.cpad + sh.mpad + (prior ? 256 : 128);
+        const size_t budget = per_sm > 1 ? 220 * 1024 / per_sm : 227 * 1024 - 512;   // 512: the static part
+        const int base_words = sh.cpad + sh.mpad + (prior ? 256 : 128);
         const size_t per_word = (size_t)consumers * C * sizeof(T);
         size_t used = per_word * base_words + kBarBytes + 256 + 2 * head;
         const int nr = round_up_int(nd.max_N, 32);
@@ -1128,16 +1128,21 @@ bool plan_shape(LaunchShape &sh, const ShapeChoice &pick, const PlanNeeds &nd, l
         }
         while (rps > 1 && used + min_stages * stage_of(rps) > budget) --rps;
         int depth = min_stages;
+        int slots = 2;
         if (used + depth * stage_of(rps) > budget) depth = 2;
+        if (consumers == 1 && used + depth * stage_of(rps) > budget) {   // the largest problems: one packet at a time
+            slots = 1;
+            used -= head;
+        }
         if (used + depth * stage_of(rps) > budget) continue;
         used += depth * stage_of(rps);
         size_t slot = head;
-        if (stage_u)
+        if (stage_u && slots == 2)
             for (int b : nd.packets) {
                 const size_t bb = align_up((size_t)b, 128);
                 if (bb > slot && used + 2 * (bb - head) <= budget) slot = bb;
             }
-        used += 2 * (slot - head);
+        used += slots * (slot - head);
         sh.npad = sh.fpad = 0;
         if (sizeof(T) == 4 && std::getenv("ASM_NO_SMEM_SUMS") == nullptr && used + 2 * per_word * nr <= budget) {
             sh.npad = nr;
@@ -1154,7 +1159,6 @@ bool plan_shape(LaunchShape &sh, const ShapeChoice &pick, const PlanNeeds &nd, l
             }
         };
         deepen(kRingRecords);
-        int slots = 2;
         while (slots < kMaxPacketSlots && used + slot <= budget) {
             ++slots;
             used += slot;

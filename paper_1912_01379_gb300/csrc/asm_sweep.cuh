@@ -14,7 +14,7 @@
 //
 // One move of mode j (Sec. IV.B, "sample e_i' from a univariate Gaussian ...
 // truncated to the interval for which f' >= 0"):
-//   [lo, hi]  = interval of delta from the previous pass (team minima of the
+//   [lo, hi]  = interval of delta from the previous pass (warp minima of the
 //               bound keys, see BoundKey)
 //   delta     ~ N(c_j/d_j, 1/d_j^2) on [lo, hi] by the inverse CDF (flat if d_j = 0)
 //   pass      f += delta V_j, clamp at 0, and the bounds of mode j+1 in the same
@@ -986,9 +986,9 @@ struct WarpChains {
     bool active[C];
     T *sm;                 // chain 0's shared memory; chain c at sm + c * team_words
     int tw;
-    int off_w, off_r, off_u, off_f, off_p;   // words: c at 0, w, r~, uniforms, f, sums
+    int off_r, off_u, off_f, off_p;   // words: c and w at 0, r~, uniforms, f, sums
     __device__ __forceinline__ T *c_(int c) const { return sm + (size_t)c * tw; }
-    __device__ __forceinline__ T *w_(int c) const { return c_(c) + off_w; }
+    __device__ __forceinline__ T *w_(int c) const { return c_(c); }
     __device__ __forceinline__ T *r_(int c) const { return c_(c) + off_r; }
     __device__ __forceinline__ T *u_(int c) const { return c_(c) + off_u; }
 };
@@ -1570,14 +1570,14 @@ __device__ __forceinline__ void consume(const SweepParams<T> &p, const LaunchSha
     const int lane = threadIdx.x & 31;
     const int wcta = uni((int)(threadIdx.x >> 5));
     WarpChains<T, C> wc;
-    // per chain in shared memory: c (cpad), w (cpad), r~ (mpad), the uniforms of the current
-    // window of 128 moves (with a prior 128 more) and, where they fit, the chain state (fpad)
-    // and the sums of f and f^2 over this launch's kept sweeps (FP32, npad each)
+    // per chain in shared memory: c and w (cpad: w_j takes c_j's place, which move j has
+    // read), r~ (mpad), the uniforms of the current window of 128 moves (with a prior 128
+    // more) and, where they fit, the chain state (fpad) and the sums of f and f^2 over this
+    // launch's kept sweeps (FP32, npad each)
     wc.tw = sh.team_words;
     wc.sm = reinterpret_cast<T *>(smem_raw) + (size_t)(wcta * C) * sh.team_words;
-    wc.off_w = sh.cpad;
-    wc.off_r = 2 * sh.cpad;
-    wc.off_u = 2 * sh.cpad + sh.mpad;
+    wc.off_r = sh.cpad;
+    wc.off_u = sh.cpad + sh.mpad;
     wc.off_f = wc.off_u + (PRIOR ? 256 : 128);
     wc.off_p = wc.off_f + sh.fpad;
     // FP32 chain state: the kept-sweep sums of the current kBinSweeps-sweep block (aligned
@@ -1675,7 +1675,7 @@ __device__ __forceinline__ void consume(const SweepParams<T> &p, const LaunchSha
             __syncwarp();
             if (Us)
                 project_exit<T, C>(wc, Us, np, usr, M, lane);
-            else if (!streamed(wc.off_w, wc.off_r, true, np, M, 32)) {
+            else if (!streamed(0, wc.off_r, true, np, M, 32)) {
                 failed = true;
                 break;
             }
