@@ -39,49 +39,40 @@ __global__ void init_kernel(T *F, int ldF, int N, double f0, double *S1, double 
     }
 }
 
-// r~ = g~ - K~ f in FP64 for every chain (one CTA per chain); chi2 = |r~|^2.
-// Records the largest relative change of chi2 against the tracked residual.
-template <class T>
-__global__ void refresh_kernel(int M, int N, const double *__restrict__ KtT, const double *__restrict__ gt,
-                               const T *__restrict__ F, int ldF, T *R, int ldR, double *chi2,
-                               Counters *cnt, int track_drift)
+// r~ = g~ - K~ f of the common start f = f0 in FP64, one thread per data point.  Every
+// chain starts there, so it is formed once and copied; per chain it took 1.5 ms of
+// FP64 arithmetic for 8192 chains of M = 400, N = 250.  The loads of a few rows are in flight
+// ahead of the chain of multiply-adds.
+__global__ void start_residual_kernel(int M, int N, const double *__restrict__ KtT, const double *__restrict__ gt,
+                                      double f0, double *__restrict__ r0)
 {
-    extern __shared__ double fs[];
-    __shared__ double red_old[32], red_new[32];
-    const int q = blockIdx.x;
-    for (int n = threadIdx.x; n < N; n += blockDim.x) fs[n] = (double)F[(size_t)q * ldF + n];
-    __syncthreads();
-    double so = 0.0, sn = 0.0;
-    for (int m = threadIdx.x; m < M; m += blockDim.x) {
-        double a = gt[m];
-        for (int n = 0; n < N; ++n) a -= KtT[(size_t)n * M + m] * fs[n];
-        const double old = (double)R[(size_t)q * ldR + m];
-        so += old * old;
-        sn += a * a;
-        R[(size_t)q * ldR + m] = (T)a;
-    }
-    for (int off = 16; off; off >>= 1) {
-        so += __shfl_xor_sync(0xffffffffu, so, off);
-        sn += __shfl_xor_sync(0xffffffffu, sn, off);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        red_old[threadIdx.x >> 5] = so;
-        red_new[threadIdx.x >> 5] = sn;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double a = 0.0, b = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { a += red_old[w]; b += red_new[w]; }
-        if (chi2) chi2[q] = b;
-        if (track_drift) {
-            const double drift = fabs(a - b) / fmax(b, 1e-300);
-            atomicMax(&cnt->drift_bits, (unsigned long long)__double_as_longlong(drift));
-        }
-    }
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m >= M) return;
+    double a = gt[m];
+#pragma unroll 16
+    for (int n = 0; n < N; ++n) a -= KtT[(size_t)n * M + m] * f0;
+    r0[m] = a;
 }
 
-// The same refresh for every chain of every problem of a launch: CTA b handles
-// chain b % chains of problem b / chains (parameters from the launch's table).
+// The start's residual and chi^2 = |r~|^2 to every chain, one warp per chain.
+template <class T>
+__global__ void start_chains_kernel(int M, const double *__restrict__ r0, T *R, int ldR, double *chi2, int chains)
+{
+    const int q = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (q >= chains) return;
+    double s = 0.0;
+    for (int m = lane; m < M; m += 32) {
+        const double r = r0[m];
+        s += r * r;
+        R[(size_t)q * ldR + m] = (T)r;
+    }
+    for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (lane == 0) chi2[q] = s;
+}
+
+// r~ = g~ - K~ f in FP64 for every chain of every problem of a launch (one CTA per chain;
+// CTA b handles chain b % chains of problem b / chains, parameters from the launch's table);
+// chi2 = |r~|^2.  Records the largest relative change of chi2 against the tracked residual.
 template <class T>
 __global__ void refresh_all_kernel(const SweepParams<T> *__restrict__ probs, int chains, int track_drift)
 {
@@ -1485,12 +1476,13 @@ int init_chains(asm_problem *p, const WsLayout &L, int chains)
     if (sizeof(T) == 4 && cudaMemsetAsync(ws + L.P1, 0, L.Dpart - L.P1, p->stream) != cudaSuccess)
         return ASM_ERR_CUDA;
     p->nsnap = 0;
-    if (const int rc = refresh_smem(refresh_kernel<T>, sizeof(double) * p->N); rc != ASM_OK) return rc;
-    refresh_kernel<T><<<chains, 128, sizeof(double) * p->N, p->stream>>>(
-        p->M, p->N, p->d_KtT, p->d_gt, (const T *)(ws + L.F), L.ldF, (T *)(ws + L.R), L.ldR,
-        (double *)(ws + L.chi2), (Counters *)(ws + L.counters), 0);
+    if (const int rc = refresh_smem(refresh_all_kernel<T>, sizeof(double) * p->N); rc != ASM_OK) return rc;
+    start_residual_kernel<<<(p->M + 63) / 64, 64, 0, p->stream>>>(p->M, p->N, p->d_KtT, p->d_gt, (double)(T)p->f0,
+                                                                  (double *)(ws + L.rref));
+    start_chains_kernel<T><<<(chains + 7) / 8, 256, 0, p->stream>>>(p->M, (const double *)(ws + L.rref), (T *)(ws + L.R),
+                                                                    L.ldR, (double *)(ws + L.chi2), chains);
     if (cudaGetLastError() != cudaSuccess) return ASM_ERR_CUDA;
-    p->other_launches += 2;
+    p->other_launches += 3;
     return ASM_OK;
 }
 
