@@ -1014,6 +1014,34 @@ struct PlanNeeds {
     std::vector<int> packets;        // bytes of every block's packet with U
 };
 
+constexpr size_t kBarBytes = 8 * (2 * kMaxRingDepth + 2 * kMaxPacketSlots);
+constexpr size_t kSmemLimit = 227 * 1024 - 512;   // of a CTA; 512: the static part
+
+// Shared-memory elements of a chain without the sums and the state.
+int chain_words(const PlanNeeds &nd, bool prior)
+{
+    return round_up_int(std::max(nd.max_np, 1), 32) + round_up_int(std::max(nd.max_M, 1), 32) + (prior ? 256 : 128);
+}
+
+// Bytes of a ring stage of rps of the largest records: at least eight rows of a streamed tile of 32 columns.
+template <class T>
+size_t stage_size(const PlanNeeds &nd, int rps)
+{
+    return std::max(align_up((size_t)rps * nd.max_rec * sizeof(T), 128), 256 * sizeof(T));
+}
+
+// The most chain warps of C chains that a CTA's shared memory holds with the smallest ring (0: none).
+template <class T>
+int warps_that_fit(const PlanNeeds &nd, int C, bool prior)
+{
+    int w = 0;
+    while (w < kMaxConsumers && (w + 1) * C * sizeof(T) * chain_words(nd, prior) + kBarBytes + 256 +
+                                        (w ? 2 : 1) * align_up((size_t)nd.head, 128) + 2 * stage_size<T>(nd, 1) <=
+                                    kSmemLimit)
+        ++w;
+    return w;
+}
+
 // Chains per warp (C) and chain warps per CTA (w) of a launch: the pair with the shortest
 // estimated run.  The chains of a warp share its row loads and its draws but also its issue
 // slots, and up to four warps have a sub-partition each, so a CTA's time (in units of C = 1,
@@ -1024,11 +1052,13 @@ struct PlanNeeds {
 // sweep for C = 1, 2, 4: 1024 chains 0.083, 0.106, 0.150; 2048: 0.163, 0.134, 0.162; 5000: 0.402,
 // 0.384, 0.438; 8192: 0.642, 0.522, 0.469), and few chains per warp where a batch's largest problem
 // bounds its time (8 problems x 256 chains: 0.31, 0.40, 0.50).  One CTA per SM: with two (128
-// registers per thread) no size was faster.  c, w > 0: given.
+// registers per thread) no size was faster.  c, w > 0: given.  fit: the most warps that shared
+// memory holds for C = 1, 2, 4 (long residuals, M in the thousands, leave few).
 struct ShapeChoice {
     int C, consumers;
 };
-ShapeChoice pick_shape(bool f64, int kv, int chains, const std::vector<double> &cost, int c, int w)
+ShapeChoice pick_shape(bool f64, int kv, int chains, const std::vector<double> &cost, int c, int w,
+                       const int (&fit)[3])
 {
     static const double kCta[3][kMaxConsumers] = {{0.79, 0.79, 0.80, 0.82, 0.96, 0.98, 1.00},
                                                   {1.17, 1.17, 1.19, 1.27, 1.51, 1.56, 1.60},
@@ -1044,8 +1074,10 @@ ShapeChoice pick_shape(bool f64, int kv, int chains, const std::vector<double> &
     for (int i = 0; i < 3; ++i) {
         const int C = 1 << i;
         if (c > 0 ? C != c : (C == 2 && kv > 16) || (C == 4 && kv > (f64 ? 4 : 8))) continue;   // the widest tiles: no registers
-        for (int x = 1; x <= kMaxConsumers; ++x) {
-            if (w > 0 ? x != w : cost.size() > 1 && x < 4) continue;   // a batch's small CTAs would share SMs
+        if (c == 0 && C > 1 && fit[i] < std::max(w, 1)) continue;
+        const int most = w > 0 ? w : std::max(fit[i], 1);
+        const int least = w > 0 ? w : cost.size() > 1 ? std::min(4, most) : 1;   // a batch's small CTAs would share SMs
+        for (int x = least; x <= most; ++x) {
             const double items = (double)((chains + x * C - 1) / (x * C));
             const double load = cost.size() == 1
                                     ? std::ceil(items / kSMs) * longest
@@ -1090,10 +1122,8 @@ bool plan_shape(LaunchShape &sh, const ShapeChoice &pick, const PlanNeeds &nd, l
     const int want_rps = env("ASM_RECORDS_PER_STAGE", 1, 8, 0);
     const int max_depth = env("ASM_RING_DEPTH", 2, kMaxRingDepth, kMaxRingDepth);
     const bool stage_u = std::getenv("ASM_NO_U_STAGE") == nullptr;
-    constexpr size_t kBarBytes = 8 * (2 * kMaxRingDepth + 2 * kMaxPacketSlots);
     const size_t head = align_up((size_t)nd.head, 128);
-    // at least eight rows of a streamed tile of 32 columns
-    auto stage_of = [&](int rps) { return std::max(align_up((size_t)rps * nd.max_rec * sizeof(T), 128), 256 * sizeof(T)); };
+    auto stage_of = [&](int rps) { return stage_size<T>(nd, rps); };
     for (int consumers = pick.consumers; consumers >= 1; --consumers) {
         LaunchShape probe = sh;   // no dynamic shared memory: the register limit alone
         probe.consumers = consumers;
@@ -1102,13 +1132,15 @@ bool plan_shape(LaunchShape &sh, const ShapeChoice &pick, const PlanNeeds &nd, l
         const int by_regs = sweep_fns(sizeof(T) == 8 ? ASM_FP64 : ASM_MIXED, probe).per_sm(probe, kv);
         if (by_regs < 1) return false;   // no kernel for this tile
         const long long ctas = (total_warps + consumers - 1) / consumers;
-        const int per_sm = (int)std::min<long long>(by_regs, std::max<long long>(1, (ctas + kSMs - 1) / kSMs));
-        const size_t budget = per_sm > 1 ? 220 * 1024 / per_sm : 227 * 1024 - 512;   // 512: the static part
-        const int base_words = sh.cpad + sh.mpad + (prior ? 256 : 128);
+        int per_sm = (int)std::min<long long>(by_regs, std::max<long long>(1, (ctas + kSMs - 1) / kSMs));
+        const int base_words = chain_words(nd, prior);
         const size_t per_word = (size_t)consumers * C * sizeof(T);
         size_t used = per_word * base_words + kBarBytes + 256 + 2 * head;
         const int nr = round_up_int(nd.max_N, 32);
         const int min_stages = std::min(kMinStages, max_depth);
+        // CTAs that share an SM leave each a part of its shared memory: fewer of them where that is too little
+        while (per_sm > 1 && used + 2 * stage_of(1) > 220 * 1024 / (size_t)per_sm) --per_sm;
+        const size_t budget = per_sm > 1 ? 220 * 1024 / per_sm : kSmemLimit;
         int rps = want_rps;
         if (rps == 0) {   // as many as leave room for everything else, at least kRecordsPerStage
             size_t extras = per_word * nr * (sizeof(T) == 4 ? 3 : 1);
@@ -1289,8 +1321,9 @@ int run_all(asm_problem *h, int chains, long long s_begin, long long s_end, long
     }
     std::vector<double> cost;   // relative time of a problem's sweep: wide blocks cost more per move
     for (asm_problem *u : us) cost.push_back((double)u->N * (1.0 + u->max_nb / 2000.0));
+    const int fit[3] = {warps_that_fit<T>(nd, 1, prior), warps_that_fit<T>(nd, 2, prior), warps_that_fit<T>(nd, 4, prior)};
     const ShapeChoice pick =
-        pick_shape(sizeof(T) == 8, kv, chains, cost, prior ? 1 : h->team ? 32 / h->team : 0, want_consumers);
+        pick_shape(sizeof(T) == 8, kv, chains, cost, prior ? 1 : h->team ? 32 / h->team : 0, want_consumers, fit);
     LaunchShape sh{};
     if (!plan_shape<T>(sh, pick, nd, all_chains, kv, prior)) return ASM_ERR_TOO_LARGE;
     const SweepFns fns = sweep_fns(h->precision, sh);

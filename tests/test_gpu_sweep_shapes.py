@@ -70,3 +70,18 @@ def test_block_widths_and_shapes(M, N, levels):
             other = _states(p, dec, shape, precision, 66)
             for a, b in zip(first, other):
                 assert np.array_equal(a, b), (shape, precision)
+
+
+def test_long_residuals():
+    """Thousands of data points leave shared memory for a few chains only, down to one warp of
+    one chain on an SM: every chain count is taken and gives the few chains' states."""
+    p = W.small_problem(7000, 24, seed=77, levels=[[0], [0, 12]])
+    for precision, chains in ((asm.ASM_FP64, (13, 500, 2300)), (asm.ASM_MIXED, (13, 2300))):
+        gp = asm.Problem(p.K, p.G, p.C, p.levels, w=p.w)
+        states = []
+        for n in chains:
+            gp.sample(n, 0, 2, 17, precision=precision)
+            states.append([x[:13].copy() for x in gp.chain_state()])
+            assert gp.status()["timeouts"] == 0
+        for f, chi2 in states[1:]:
+            assert np.array_equal(f, states[0][0]) and np.array_equal(chi2, states[0][1])
