@@ -457,7 +457,9 @@ __device__ __forceinline__ void pair_of(F f, T x0, T x1, const TeamLanes<G> &tl,
 
 // n / d, correctly rounded, from r = the correctly rounded 1 / d (Markstein 1990: the
 // remainder is exact in a fused multiply-add; the second step makes it correct where the
-// first product was off by more than an ulp).  For d well inside the normal range.
+// first product was off by more than an ulp).  For normal d, r and n / d, with |n| >= 2^-100,
+// so that the remainder, a multiple of 2^-48 |n|, is a number too; or n = +0.  A subnormal
+// quotient can lie halfway between two numbers, and then it came out an ulp off.
 __device__ __forceinline__ float div_by(float n, float d, float r)
 {
     const float q0 = __fmul_rn(n, r);
@@ -487,8 +489,10 @@ __device__ __forceinline__ float narrow_offset(float a, float w, float u, int &c
     using GL = GaussLegendre<float>;
     const float lam = a + 0.5f * w;
     const float x = lam * w;
+    // beyond the series the dividend is at least 2^-34 (u >= 2^-24, |x| >= 1e-3) and |lam| >= 1.4e-3
+    // (w < 0.71): a normal quotient up to lam = 1e27
     float t = m_abs(x) < 1e-3f ? u * w * (1.0f - 0.5f * x * (1.0f - u))   // the series for small lam w
-                               : m_abs(lam) < 1e30f ? div_by(-m_log1p(u * m_expm1(-x)), lam, __frcp_rn(lam))
+                               : m_abs(lam) < 1e27f ? div_by(-m_log1p(u * m_expm1(-x)), lam, __frcp_rn(lam))
                                                     : -m_log1p(u * m_expm1(-x)) / lam;
     t = m_min(m_max(t, 0.0f), w);
     if (w * w <= 4e-7f) return t;
