@@ -69,8 +69,11 @@ enum { ASM_FP64 = 0, ASM_MIXED = 1 };   /* precision of asm_sample */
  * depends on them, every chain does the same arithmetic under every launch
  * shape; values outside the ranges below are ignored):
  *   ASM_TEAM_LANES         8, 16 or 32: lanes per chain of a handle, i.e. 4, 2 or
- *                          1 chains per warp (with a gamma prior always 1), read
- *                          by asm_setup (asm_tune replaces it);
+ *                          1 chains per warp (with a gamma prior always 1; where
+ *                          no kernel runs as many on the handle's blocks, or
+ *                          shared memory does not hold them, the heuristic
+ *                          chooses), read by asm_setup (calls that asm_tune has
+ *                          timed take its choice instead);
  *   ASM_CONSUMERS_PER_CTA  1..7: chain warps per CTA of every sweep launch
  *                          (takes precedence over the heuristic and asm_tune);
  *   ASM_RING_DEPTH         2..48: stages of the move-record ring (default: as
@@ -164,8 +167,8 @@ typedef struct {
  * that level U_j = K~ V_j / d_j is not resolvable in FP64 while the likelihood
  * is flat along V_j over its positivity interval).  On success *out receives a new handle (free with asm_destroy);
  * on failure *out is NULL and nothing stays allocated.  The environment variable
- * ASM_TEAM_LANES = 8, 16 or 32, read here, fixes the lanes per chain of the
- * handle's sweep launches (testing; other values are ignored, asm_tune overrides it). */
+ * ASM_TEAM_LANES = 8, 16 or 32, read here, asks for the lanes per chain of the
+ * handle's sweep launches (testing; other values are ignored, see above). */
 int asm_setup(const asm_desc *d, asm_problem **out);
 
 /* Set-up of n independent problems as one batch handle (each problem as in
@@ -200,8 +203,10 @@ int asm_problem_count(const asm_problem *p);
  * that share every row it loads) times chain warps per
  * CTA in {heuristic, 2, 3, 4, 5, 6, 7}, where it fits -- on one warm-up and three
  * timed sweeps of fresh trial chains in the caller's workspace (same layout
- * and size rule as asm_sample), and keeps the fastest for later asm_sample
- * calls on p.  The shape changes no result: every chain does the same
+ * and size rule as asm_sample), and keeps the fastest for later sampling
+ * calls on p with this precision and number of chains (one choice per
+ * precision, the last; other calls run as on an untuned handle).  The shape
+ * changes no result: every chain does the same
  * arithmetic in the same order under every shape.  The workspace's contents
  * are overwritten, so the next asm_sample must start fresh chains
  * (ASM_SAMPLE_CONTINUE then fails with ASM_ERR_STATE).  Synchronises

@@ -265,7 +265,7 @@ class _Handle:
 
     def tune(self, chains, precision=ASM_MIXED, stream=None, workspace=None):
         """asm_tune: picks the fastest launch shape (lanes per chain, chain warps
-        per CTA) for `chains` chains; returns
+        per CTA) for later calls with `chains` chains in this precision; returns
         (team_lanes, consumers, min_blocks)."""
         torch, workspace = self._workspace(chains, precision, workspace)
         s = stream if stream is not None else torch.cuda.current_stream()

@@ -241,5 +241,7 @@ constexpr int kMaxPacketSlots = 8;
 // Largest kv (16-byte vectors per lane and chain): 64 elements per lane.
 constexpr int kMaxKvF32 = 16;
 constexpr int kMaxKvF64 = 32;
+// Largest kv with a kernel of C chains per warp (the lists in asm_sweep_*.cu).
+constexpr int max_kv(bool f64, int C) { return C == 4 ? 8 : C == 2 ? 16 : f64 ? kMaxKvF64 : kMaxKvF32; }
 
 }  // namespace asmgb

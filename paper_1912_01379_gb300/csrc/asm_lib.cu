@@ -454,7 +454,19 @@ struct asm_problem {
     void *ws = nullptr;       // this problem's section of it
     size_t ws_bytes = 0;
     int chains = 0, precision = -1;
-    int team = 0;   // lanes per chain, 32 / (chains per warp): 32, 16 or 8 (0: the built-in heuristic)
+    // Launch shape wanted: lanes per chain, 32 / (chains per warp), 32, 16 or 8, and chain warps per
+    // CTA (0: the built-in heuristic)
+    struct Want {
+        int team = 0, consumers = 0;
+        int chains = 0;   // tuned: the number of chains it was timed with
+    };
+    Want want;              // ASM_TEAM_LANES
+    // By precision: asm_tune's last choice, for the calls it was timed for.  Kernels of several chains
+    // per warp end at other block widths in the other precision, and the fastest shape of one number of chains
+    // can be a slow one of another (8192 chains of 400 points, FP32, ms a sweep: 0.60 with the one chain
+    // per warp that 1024 chains run best with, 0.43 with four).
+    Want tuned[2];
+    bool trial = false;     // asm_tune is timing tuned[precision]: a shape that does not fit is refused
     long long sweeps_done = 0, kept = 0;
     long long kept_since = 0;   // every sweep from this one on has been accumulated
     unsigned long long seed = 0;
@@ -462,8 +474,6 @@ struct asm_problem {
     unsigned long long next_problem_id = 0, next_chain_offset = 0;
     cudaStream_t stream = nullptr;
     bool have_run = false;
-    // launch shape chosen by asm_tune (0: the built-in heuristic)
-    int tuned_consumers = 0;
     // one refresh period (advance the range, sweep, refresh) as a CUDA graph
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t gexec = nullptr;
@@ -1073,7 +1083,7 @@ ShapeChoice pick_shape(bool f64, int kv, int chains, const std::vector<double> &
     }
     for (int i = 0; i < 3; ++i) {
         const int C = 1 << i;
-        if (c > 0 ? C != c : (C == 2 && kv > 16) || (C == 4 && kv > (f64 ? 4 : 8))) continue;   // the widest tiles: no registers
+        if (c > 0 ? C != c : kv > max_kv(f64, C) || (f64 && C == 4 && kv > 4)) continue;   // the widest tiles: no registers
         if (c == 0 && C > 1 && fit[i] < std::max(w, 1)) continue;
         const int most = w > 0 ? w : std::max(fit[i], 1);
         const int least = w > 0 ? w : cost.size() > 1 ? std::min(4, most) : 1;   // a batch's small CTAs would share SMs
@@ -1314,7 +1324,8 @@ int run_all(asm_problem *h, int chains, long long s_begin, long long s_end, long
     const int kv = pick_kv(max_nb, vec, sizeof(T) == 8 ? kMaxKvF64 : kMaxKvF32);
     if (kv < 0) return ASM_ERR_TOO_LARGE;
     const long long all_chains = (long long)chains * (long long)us.size();
-    int want_consumers = h->tuned_consumers;
+    const asm_problem::Want want = h->tuned[h->precision].chains == chains ? h->tuned[h->precision] : h->want;
+    int want_consumers = want.consumers;
     if (const char *e = std::getenv("ASM_CONSUMERS_PER_CTA")) {   // tuning override
         const int v = std::atoi(e);
         if (v >= 1 && v <= kMaxConsumers) want_consumers = v;
@@ -1322,8 +1333,12 @@ int run_all(asm_problem *h, int chains, long long s_begin, long long s_end, long
     std::vector<double> cost;   // relative time of a problem's sweep: wide blocks cost more per move
     for (asm_problem *u : us) cost.push_back((double)u->N * (1.0 + u->max_nb / 2000.0));
     const int fit[3] = {warps_that_fit<T>(nd, 1, prior), warps_that_fit<T>(nd, 2, prior), warps_that_fit<T>(nd, 4, prior)};
-    const ShapeChoice pick =
-        pick_shape(sizeof(T) == 8, kv, chains, cost, prior ? 1 : h->team ? 32 / h->team : 0, want_consumers, fit);
+    int want_C = prior ? 1 : want.team ? 32 / want.team : 0;
+    if (want_C > 1 && (kv > max_kv(sizeof(T) == 8, want_C) || fit[want_C == 2 ? 1 : 2] < 1)) {
+        if (h->trial) return ASM_ERR_TOO_LARGE;
+        want_C = 0;   // no kernel for the blocks, or no room for its chains: the heuristic's
+    }
+    const ShapeChoice pick = pick_shape(sizeof(T) == 8, kv, chains, cost, want_C, want_consumers, fit);
     LaunchShape sh{};
     if (!plan_shape<T>(sh, pick, nd, all_chains, kv, prior)) return ASM_ERR_TOO_LARGE;
     const SweepFns fns = sweep_fns(h->precision, sh);
@@ -1757,7 +1772,7 @@ int asm_setup(const asm_desc *ds, asm_problem **out)
     const char *team = std::getenv("ASM_TEAM_LANES");
     if (team) {
         const int t = std::atoi(team);
-        if (t == 8 || t == 16 || t == 32) p->team = t;
+        if (t == 8 || t == 16 || t == 32) p->want.team = t;
     }
     *out = p;
     return ASM_OK;
@@ -1960,7 +1975,7 @@ int asm_tune(asm_problem *p, int chains, int precision, void *d_workspace, size_
     if (!d_workspace || workspace_bytes < RL.total || ((uintptr_t)d_workspace & 255)) return ASM_ERR_WORKSPACE;
     if (p->ev_used && drain_events(p) != ASM_OK) return ASM_ERR_CUDA;
     bind_workspace(p, d_workspace, workspace_bytes, RL, (cudaStream_t)stream);
-    const int team0 = p->team, cons0 = p->tuned_consumers;
+    const asm_problem::Want tuned0 = p->tuned[precision];
     const bool timing0 = p->timing;
     p->timing = false;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1968,7 +1983,7 @@ int asm_tune(asm_problem *p, int chains, int precision, void *d_workspace, size_
         if (e0) cudaEventDestroy(e0);
         return ASM_ERR_CUDA;
     }
-    int best_team = team0, best_cons = cons0, rc = ASM_OK;
+    int best_team = 0, best_cons = 0, rc = ASM_OK;
     float best = 0.f;
     bool any = false;
     bool prior = false;
@@ -1976,12 +1991,12 @@ int asm_tune(asm_problem *p, int chains, int precision, void *d_workspace, size_
         prior = prior || (precision == ASM_FP64 ? u->b64.prior_am1 : u->b32.prior_am1) != nullptr;
     const int teams[] = {32, 16, 8};
     const int conss[] = {0, 2, 3, 4, 5, 6, 7};   // 0: the built-in heuristic
+    p->trial = true;
     for (int trial = 0; trial < 3 * 7; ++trial) {
         const int S = teams[trial / 7], c = conss[trial % 7];
         if (prior && S != 32) continue;   // its kernels: one chain per warp
         {
-            p->team = S;
-            p->tuned_consumers = c;
+            p->tuned[precision] = {S, c, chains};
             // fresh chains, one sweep to warm up, then the timed sweeps
             rc = start_chains(p, chains, precision, 0x74756e65ull, false);
             if (rc != ASM_OK) break;
@@ -2011,17 +2026,16 @@ int asm_tune(asm_problem *p, int chains, int precision, void *d_workspace, size_
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
+    p->trial = false;
     p->timing = timing0;
     // the workspace now holds trial chains: the next asm_sample starts afresh
     p->have_run = false;
     for (asm_problem *u : p->kids) u->have_run = false;
     if (rc != ASM_OK || !any) {
-        p->team = team0;
-        p->tuned_consumers = cons0;
+        p->tuned[precision] = tuned0;
         return rc != ASM_OK ? rc : ASM_ERR_TOO_LARGE;
     }
-    p->team = best_team;
-    p->tuned_consumers = best_cons;
+    p->tuned[precision] = {best_team, best_cons, chains};
     if (team_out) *team_out = best_team;
     if (consumers_out) *consumers_out = best_cons;
     if (min_blocks_out) *min_blocks_out = 1;
@@ -2408,7 +2422,7 @@ int asm_setup_batch(int n, const asm_desc *d, asm_problem **out)
         b->M = std::max(b->M, u->M);
         b->N = std::max(b->N, u->N);
     }
-    b->team = b->kids[0]->team;
+    b->want = b->kids[0]->want;
     *out = b;
     return ASM_OK;
 }
