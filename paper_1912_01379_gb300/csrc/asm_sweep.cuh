@@ -145,8 +145,6 @@ template <> struct BoundKey<float> {
     static constexpr S lo0 = (S)0xff800000;   // -inf
     static constexpr U hi0 = 0x7f800000u;     // +inf
     static __device__ __forceinline__ S bits(float x) { return __float_as_int(x); }
-    static __device__ __forceinline__ float lo_of(S k) { return __int_as_float(k); }
-    static __device__ __forceinline__ float hi_of(U k) { return __uint_as_float(k); }
 };
 template <> struct BoundKey<double> {
     using S = long long;
@@ -154,8 +152,6 @@ template <> struct BoundKey<double> {
     static constexpr S lo0 = (S)0xfff0000000000000ull;
     static constexpr U hi0 = 0x7ff0000000000000ull;
     static __device__ __forceinline__ S bits(double x) { return __double_as_longlong(x); }
-    static __device__ __forceinline__ double lo_of(S k) { return __longlong_as_double(k); }
-    static __device__ __forceinline__ double hi_of(U k) { return __longlong_as_double((long long)k); }
 };
 // max(x, +0) (NaN gives +0).  FP64 as an integer test of the high word: a DSETP
 // would occupy the FP64 pipe, which issues one warp instruction per 64 cycles and
@@ -1357,8 +1353,8 @@ struct Visit {
     // false: a bounded wait gave up
     static __device__ __forceinline__ bool run(const SweepParams<T> &p, const LaunchShape &sh, const Regions &R, RingPos &rp,
                                                const WarpChains<T, C> &wc, MoveCounts<C> &n, const BlockDesc &B,
-                                               const T *pk, const T *Us, long long s, bool keep, bool trace, int &win,
-                                               int &win_end, int lane, T (&sd2)[C], T (&sf2)[C])
+                                               const T *pk, long long s, bool keep, bool trace, int &win, int &win_end,
+                                               int lane, T (&sd2)[C], T (&sf2)[C])
     {
         const int bn = uni(B.n), bstart = uni(B.start), rs = uni(B.rs), np = uni(B.np), recstride = 2 * rs + 4;
         const int kcnt = (bn + 32 * VE - 1) / (32 * VE);
@@ -1661,16 +1657,16 @@ __device__ __forceinline__ void consume(const SweepParams<T> &p, const LaunchSha
             }
             __syncwarp();
             if (bn <= 16 * VEC)
-                ok = Visit<T, KV, C, PRIOR, 1, VEC / 2>::run(p, sh, R, rp, wc, n, B, pk, Us, s, keep, trace, win, win_end,
+                ok = Visit<T, KV, C, PRIOR, 1, VEC / 2>::run(p, sh, R, rp, wc, n, B, pk, s, keep, trace, win, win_end,
                                                              lane, sd2, sf2);
             else if (KV == 1 || bn <= 32 * VEC)
-                ok = Visit<T, KV, C, PRIOR, 1, VEC>::run(p, sh, R, rp, wc, n, B, pk, Us, s, keep, trace, win, win_end, lane,
+                ok = Visit<T, KV, C, PRIOR, 1, VEC>::run(p, sh, R, rp, wc, n, B, pk, s, keep, trace, win, win_end, lane,
                                                          sd2, sf2);
             else if (KV == 2 || bn > 32 * VEC * (KV - 1))
-                ok = Visit<T, KV, C, PRIOR, KV, VEC>::run(p, sh, R, rp, wc, n, B, pk, Us, s, keep, trace, win, win_end, lane,
+                ok = Visit<T, KV, C, PRIOR, KV, VEC>::run(p, sh, R, rp, wc, n, B, pk, s, keep, trace, win, win_end, lane,
                                                           sd2, sf2);
             else
-                ok = Visit<T, KV, C, PRIOR, 0, VEC>::run(p, sh, R, rp, wc, n, B, pk, Us, s, keep, trace, win, win_end, lane,
+                ok = Visit<T, KV, C, PRIOR, 0, VEC>::run(p, sh, R, rp, wc, n, B, pk, s, keep, trace, win, win_end, lane,
                                                          sd2, sf2);
             if (!ok) {
                 failed = true;
