@@ -79,8 +79,12 @@ enum { ASM_FP64 = 0, ASM_MIXED = 1 };   /* precision of asm_sample */
  *   ASM_RING_DEPTH         2..48: stages of the move-record ring (default: as
  *                          many as shared memory holds, at most 48);
  *   ASM_RECORDS_PER_STAGE  1..8: move records of the largest block per ring stage
- *                          (default 4: one barrier wait and release per stage;
- *                          smaller blocks put more records in a stage);
+ *                          (default: about 32 KB of them, 1 to 64 as shared memory
+ *                          allows; one barrier wait and release per stage; smaller
+ *                          blocks put more records, up to 64, in a stage);
+ *   ASM_NO_SMEM_SUMS       set: the FP32 kept-sweep sums stay in the workspace
+ *                          during a launch (default: in shared memory where they
+ *                          fit);
  *   ASM_NO_U_STAGE         set: U of every block is streamed through the record
  *                          ring for the projections instead of coming with the
  *                          block's visit packet. */

@@ -887,7 +887,7 @@ int build_precision(asm_problem *p, const HostFactors &hf, PrecBuffers &out)
             r[2 * B.rs + 1] = hd[j] > 0.0 ? (T)(1.0 / hd[j]) : T(0);
             r[2 * B.rs + 2] = (T)hf.dres[b][j];
         }
-        // visit packet: descriptor, R_0, U with odd row stride
+        // visit packet: descriptor, R_0, U with a row stride free of bank conflicts (packet_row)
         T *k = &pk[B.offPk];
         BlockDesc D = B;   // with this precision's runs of Gaussian and flat modes
         while (D.ng < B.n && (T)hd[D.ng] != T(0)) ++D.ng;
@@ -1055,13 +1055,19 @@ int warps_that_fit(const PlanNeeds &nd, int C, bool prior)
 // Chains per warp (C) and chain warps per CTA (w) of a launch: the pair with the shortest
 // estimated run.  The chains of a warp share its row loads and its draws but also its issue
 // slots, and up to four warps have a sub-partition each, so a CTA's time (in units of C = 1,
-// w = 7) is kCta[C][w] below: blocked modes, N = 400, one CTA per SM, FP32 (1.0 = 0.083 ms a sweep;
-// FP64 scales alike, 1.0 = 1.32 ms).  A problem's items then take ceil(items / SMs) waves, those of
+// w = 7) is kCta[C][w] below: blocked modes, N = 400, one CTA per SM, FP32 (1.0 = 0.083 ms a sweep when
+// it was taken, 0.077 now).  A problem's items then take ceil(items / SMs) waves, those of
 // a batch (uneven, longest first) the longest item or the mean load of an SM and part of the longest.  So one chain per warp up to one wave
 // of 1064 chains, two up to 2128, four beyond, except where a last wave would be nearly empty (ms a
-// sweep for C = 1, 2, 4: 1024 chains 0.083, 0.106, 0.150; 2048: 0.163, 0.134, 0.162; 5000: 0.402,
-// 0.384, 0.438; 8192: 0.642, 0.522, 0.469), and few chains per warp where a batch's largest problem
-// bounds its time (8 problems x 256 chains: 0.31, 0.40, 0.50).  One CTA per SM: with two (128
+// sweep for C = 1, 2, 4: 1024 chains 0.077, 0.091, 0.138; 2048: 0.150, 0.124, 0.149; 4096: 0.300, 0.246, 0.218;
+// 8192: 0.598, 0.489, 0.434; 5000, with the first kernels: 0.402, 0.384, 0.438), and few chains per warp where a batch's
+// largest problem bounds its time (8 problems x 256 chains: 0.31, 0.40, 0.50).
+// In FP32 the rule took the fastest C for each of eight problems (hierarchies of 64 and 128 points, one-point blocks, plain
+// modes, blocks of 50 to 400 points) at 256 to 8192 chains.  FP64, bound by its pipe, gains more from shared draws: there the
+// rule was up to 20 % from the fastest where draws are most of the work (hierarchy of 64 points, 1024 chains, C = 1, 2, 4:
+// 0.751, 0.627, 0.772; 2048: 1.48, 1.04, 0.925), and 6 to 18 % on blocks of 257 to 512 points from 4096 chains on (blocked
+// modes, 4096: 4.95, 3.98, 3.39), where four chains per warp win although that kernel spills (a stack of 184 bytes a thread) and only
+// asm_tune takes it.  One CTA per SM: with two (128
 // registers per thread) no size was faster.  c, w > 0: given.  fit: the most warps that shared
 // memory holds for C = 1, 2, 4 (long residuals, M in the thousands, leave few).
 struct ShapeChoice {

@@ -399,9 +399,12 @@ __device__ __forceinline__ void lds_mode(const double *p, double &d, double &inv
 // at most w^2/8 across the interval, so one or two steps converge where the flat start
 // t = u w needed four.  The offset keeps its relative accuracy however narrow the
 // interval is.  In FP32 the start is the answer when w^2 / 8, the curvature's bound on
-// the relative error of the exponential law's CDF, lies below 2^-23 (w <= 6e-4: the weak
-// modes whose intervals are a tiny fraction of their Gaussian's width), and one Newton
-// step is when w <= 0.2: Newton's error is quadratic in the start's, which is below
+// the relative error of the exponential law's CDF, lies below 5e-8 (w <= 6e-4: the weak
+// modes whose intervals are a tiny fraction of their Gaussian's width); with the series
+// that stands for the exponential law below |lam w| = 1e-3 and leaves out terms of up to
+// (lam w)^2 / 6 = 1.7e-7, the start is within 2.2e-7 relative (2.0e-7 measured at 2 million
+// (a, w, u), 3.3e-8 beyond the series), half the FP32 tolerance.  One Newton
+// step is the answer when w <= 0.2: Newton's error is quadratic in the start's, which is below
 // w^2/12 relative, and one step leaves at most 1.5e-7 relative over the narrow regime
 // with w <= 0.2 (measured against the root of a 64-point rule at 4 million (a, w, u)),
 // below the FP32 tolerance.
