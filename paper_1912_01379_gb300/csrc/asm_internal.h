@@ -194,7 +194,7 @@ size_t refresh_tc_smem(int max_bn);        // dynamic shared memory of one CTA
 constexpr int kRefreshTcLdK = 32;          // ldK is a multiple of this (one k-tile)
 cudaError_t launch_split_k(const double *KtT, int M, int N, int ldK, float *Khi, float *Klo, cudaStream_t s);
 // Reference state of every problem's tensor-core refresh: fref over tiles of 32
-// grid points, then r_ref over tiles of 64 data points (two launches).
+// grid points, then r_ref over tiles of 128 data points (two launches).
 cudaError_t launch_refresh_ref(const SweepParams<float> *probs, int n_problems, int chains, int max_N, int max_M,
                                cudaStream_t s);
 // Contractions of the backward pass (asm_moments.cu).  D: chains x ldD snapshot

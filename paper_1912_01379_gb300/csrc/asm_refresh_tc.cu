@@ -195,31 +195,18 @@ __global__ void refresh_fref_kernel(const SweepParams<float> *__restrict__ probs
     }
 }
 
-// r_ref = g~ - K~ fref in FP64, one thread per data point: a chain of N multiply-adds of
-// 64 cycles each.  fref is converted once per CTA (a conversion takes the FP64 pipe as
-// long as the multiply-add), and the loads of sixteen rows are in flight ahead of the chain,
-// which waited for memory before: 70 us at N = 400.
-constexpr int kRrefThreads = 64;
-constexpr int kRrefTile = 256;
-__global__ void __launch_bounds__(kRrefThreads) refresh_rref_kernel(const SweepParams<float> *__restrict__ probs)
+// r_ref = g~ - K~ fref in FP64, one thread per data point: a chain of N multiply-adds.
+// 36 us at M = 100, N = 400, 24 at 400 x 250 and 347 at 400 x 2000, with K~ in L2; fref
+// converted once per CTA through shared memory, with sixteen rows' loads ahead of the chain
+// and 64 threads per CTA, took 46, 31 and 559.
+__global__ void refresh_rref_kernel(const SweepParams<float> *__restrict__ probs)
 {
-    __shared__ double fs[kRrefTile];
     const SweepParams<float> &p = probs[blockIdx.y];
-    if (blockIdx.x * kRrefThreads >= (unsigned)p.M) return;   // (uniform per CTA)
-    const int m = blockIdx.x * kRrefThreads + threadIdx.x, M = p.M, N = p.N;
-    const bool in = m < M;
-    const double *__restrict__ K = p.KtT + (in ? m : 0);
-    const float *__restrict__ fref = p.fref;
-    double a = p.gt[in ? m : 0];
-    for (int n0 = 0; n0 < N; n0 += kRrefTile) {
-        const int nt = min(kRrefTile, N - n0);
-        __syncthreads();   // the previous tile has been read
-        for (int k = threadIdx.x; k < nt; k += kRrefThreads) fs[k] = (double)fref[n0 + k];
-        __syncthreads();
-#pragma unroll 16
-        for (int k = 0; k < nt; ++k) a -= K[(size_t)(n0 + k) * M] * fs[k];
-    }
-    if (in) p.rref[m] = a;
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m >= p.M) return;
+    double a = p.gt[m];
+    for (int n = 0; n < p.N; ++n) a -= p.KtT[(size_t)n * p.M + m] * (double)p.fref[n];
+    p.rref[m] = a;
 }
 
 __global__ void __launch_bounds__(kTcThreads, 1)
@@ -458,8 +445,7 @@ cudaError_t launch_refresh_ref(const SweepParams<float> *probs, int n_problems, 
                                cudaStream_t s)
 {
     refresh_fref_kernel<<<dim3((unsigned)((max_N + 31) / 32), (unsigned)n_problems), 256, 0, s>>>(probs, chains);
-    refresh_rref_kernel<<<dim3((unsigned)((max_M + kRrefThreads - 1) / kRrefThreads), (unsigned)n_problems), kRrefThreads, 0,
-                          s>>>(probs);
+    refresh_rref_kernel<<<dim3((unsigned)((max_M + 127) / 128), (unsigned)n_problems), 128, 0, s>>>(probs);
     return cudaGetLastError();
 }
 
