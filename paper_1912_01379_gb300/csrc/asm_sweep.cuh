@@ -1269,25 +1269,27 @@ struct Visit {
 
     // Gamma prior (Eq. compat): the draw is a proposal, accepted with probability
     // min(1, prod ((f + delta V)_+ / f)^(a - 1)) over the block.  Where the tile leaves registers
-    // (kCachePrior) a visit keeps a - 1 and the logarithms of its points there: an accepted
-    // proposal's logarithms are the next move's current ones, so a move takes one logarithm per
-    // point instead of two and reads nothing from global memory (ragged blocks of 20 points and a
-    // level of 101, 250 chains: 0.100 -> 0.066 ms a sweep).
-    static constexpr bool kCachePrior = PRIOR && KK * VE * sizeof(T) <= 64;
+    // a visit keeps a - 1 there (kKeepShape), and the logarithms of its points too (kKeepLogs): an
+    // accepted proposal's logarithms are the next move's current ones, so a move takes one logarithm
+    // per point instead of two and reads nothing from global memory (250 chains, ms a sweep: ragged
+    // blocks of 20 points and a level of 101, FP32, 0.100 -> 0.066; one of 520, 2.07 -> 1.18; of 100 to 300, FP64,
+    // 6.8 -> 4.2; with a - 1 alone: one of 1100, FP32, 8.4 -> 5.6; one of 600, FP64, both 23.1).
+    static constexpr bool kKeepLogs = PRIOR && KK * VE * sizeof(T) <= 128;
+    static constexpr bool kKeepShape = PRIOR && KK * VE * sizeof(T) <= 256;
     struct PriorState {
-        T am1[kCachePrior ? KK : 1][kCachePrior ? VE : 1], lg[kCachePrior ? KK : 1][kCachePrior ? VE : 1];
+        T am1[kKeepShape ? KK : 1][kKeepShape ? VE : 1], lg[kKeepLogs ? KK : 1][kKeepLogs ? VE : 1];
     };
     static __device__ __forceinline__ void prior_start(const SweepParams<T> &p, const T (&f)[C][KK][VE], int bn, int bstart,
                                                        int lane, PriorState &ps)
     {
-        if constexpr (kCachePrior) {
+        if constexpr (kKeepShape) {
 #pragma unroll
             for (int k = 0; k < KK; ++k)
 #pragma unroll
                 for (int v = 0; v < VE; ++v) {
                     const int nl = VE * (32 * k + lane) + v;
                     ps.am1[k][v] = nl < bn ? __ldg(p.prior_am1 + bstart + nl) : T(0);
-                    ps.lg[k][v] = ps.am1[k][v] != T(0) ? m_log(f[0][k][v]) : T(0);
+                    if constexpr (kKeepLogs) ps.lg[k][v] = ps.am1[k][v] != T(0) ? m_log(f[0][k][v]) : T(0);
                 }
         }
     }
@@ -1298,7 +1300,7 @@ struct Visit {
         if (delta[0] == T(0)) return;
         const T log_ua = m_log(ua);
         T lsum = T(0);
-        T l1[kCachePrior ? KK : 1][kCachePrior ? VE : 1];
+        T l1[kKeepLogs ? KK : 1][kKeepLogs ? VE : 1];
         unsigned zflags = 0u;   // 1: a proposed value is 0, 2: a current value is 0
 #pragma unroll
         for (int k = 0; k < KK; ++k) {
@@ -1313,28 +1315,21 @@ struct Visit {
 #pragma unroll
                 for (int v = 0; v < VE; ++v) {
                     const int nl = VE * (32 * k + lane) + v;
-                    if constexpr (kCachePrior) {
-                        const T am1 = ps.am1[k][v], x0 = f[0][k][v];
-                        const T x1 = m_max(m_fma(delta[0], vv[v], x0), T(0));
-                        l1[k][v] = T(0);
-                        if (am1 != T(0)) {
-                            l1[k][v] = m_log(x1);
-                            if (x1 == T(0)) zflags |= 1u;
-                            else if (x0 == T(0)) zflags |= 2u;
-                            else lsum += am1 * (l1[k][v] - ps.lg[k][v]);
-                        }
-                    } else if (nl < bn) {
-                        const T am1 = __ldg(p.prior_am1 + bstart + nl);
-                        if (am1 != T(0)) {
-                            const T x0 = f[0][k][v];
-                            const T x1 = m_max(m_fma(delta[0], vv[v], x0), T(0));
-                            if (x1 == T(0)) zflags |= 1u;
-                            else if (x0 == T(0)) zflags |= 2u;
-                            else lsum += am1 * (m_log(x1) - m_log(x0));
-                        }
+                    T am1;
+                    if constexpr (kKeepShape) am1 = ps.am1[k][v];
+                    else am1 = nl < bn ? __ldg(p.prior_am1 + bstart + nl) : T(0);
+                    const T x0 = f[0][k][v];
+                    const T x1 = m_max(m_fma(delta[0], vv[v], x0), T(0));
+                    if constexpr (kKeepLogs) l1[k][v] = T(0);
+                    if (am1 != T(0)) {
+                        if constexpr (kKeepLogs) l1[k][v] = m_log(x1);
+                        if (x1 == T(0)) zflags |= 1u;
+                        else if (x0 == T(0)) zflags |= 2u;
+                        else if constexpr (kKeepLogs) lsum += am1 * (l1[k][v] - ps.lg[k][v]);
+                        else lsum += am1 * (m_log(x1) - m_log(x0));
                     }
                 }
-            } else if constexpr (kCachePrior) {
+            } else if constexpr (kKeepLogs) {
 #pragma unroll
                 for (int v = 0; v < VE; ++v) l1[k][v] = T(0);
             }
@@ -1345,7 +1340,7 @@ struct Visit {
         if (!(log_ua < lr)) {
             delta[0] = T(0);
             ++rej[0];
-        } else if constexpr (kCachePrior) {
+        } else if constexpr (kKeepLogs) {
 #pragma unroll
             for (int k = 0; k < KK; ++k)
 #pragma unroll

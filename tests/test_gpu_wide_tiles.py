@@ -3,9 +3,9 @@
 * Blocks of 513 to 2048 points: the states and counters of one chain per warp, bit for
   bit, from the kernels of two and four (where one exists for the width).
 * The prior's kernel keeps a - 1 and the logarithms of a block's points in registers
-  where the tile leaves room and reads them anew at every move elsewhere.  The tile
-  follows the handle's largest block, so that a problem takes the one form alone and
-  the other in a batch with a wider problem: the same states bit for bit.
+  (up to 1024 points in FP32, 512 in FP64), a - 1 alone (2048, 1024) or neither.  The
+  tile follows the handle's largest block, so that a problem takes the one form alone
+  and another in a batch with a wider problem: the same states bit for bit.
 * The most data points that one warp of one chain leaves room for (a single packet slot,
   a ring of two stages, U streamed), and one more.  Rows of zeros add nothing to a
   chain's sums, so that the same problem without them, which has packets with U and a deep
@@ -101,7 +101,10 @@ def test_wide_blocks(N):
 # the narrow problem's blocks fill its own tile wholly or in part; the wide one raises the tile
 @pytest.mark.parametrize("precision,levels,N,wide", [
     (asm.ASM_MIXED, [[0], [0, 300]], 500, 520), (asm.ASM_MIXED, [[0, 200]], 340, 600),
-    (asm.ASM_FP64, [[0], [0, 150]], 250, 260), (asm.ASM_FP64, [[0, 100]], 170, 300)])
+    (asm.ASM_FP64, [[0], [0, 150]], 250, 260), (asm.ASM_FP64, [[0, 100]], 170, 300),
+    (asm.ASM_MIXED, [[0], [0, 300]], 500, 1100), (asm.ASM_MIXED, [[0], [0, 560]], 900, 1030),
+    (asm.ASM_FP64, [[0], [0, 150]], 250, 520), (asm.ASM_FP64, [[0, 300]], 500, 1030),
+    (asm.ASM_FP64, [[0], [0, 300]], 600, 1030)])
 def test_prior_in_registers_and_from_memory(precision, levels, N, wide):
     def spec(n, lv, seed):
         p = W.small_problem(12, n, seed=seed, levels=lv, noise=3e-3)
