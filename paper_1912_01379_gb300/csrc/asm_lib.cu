@@ -174,7 +174,10 @@ __global__ void bin_kernel(const SweepParams<T> *__restrict__ probs, int chains,
 // column, serial over the chains, was bound by memory latency and left the GPU
 // idle: 7.08 ms for the score products of 4096 chains x 200 points x 8
 // parameters and 3.65 ms for the means of a result call.  The groups are added
-// in a fixed order, so a result does not depend on the schedule.
+// in a fixed order, so a result does not depend on the schedule.  Up to 28 chains leave
+// whole warps without one, whose zeros cost FP64 additions all the same: the CTA
+// then has a warp per four chains, and the same sums (one chain: asm_average on 400
+// points 45 -> 39 us, asm_mc_error on 2000 points 79 -> 63).
 constexpr int kColTile = 8;
 constexpr int kColThreads = 256;
 constexpr int kColRows = kColThreads / kColTile;
@@ -188,7 +191,9 @@ __device__ __forceinline__ double column_total(double v, double (*part)[kColTile
     if ((threadIdx.x & 31) < kColTile) part[threadIdx.x >> 5][threadIdx.x & 7] = v;
     __syncthreads();
     double t = part[0][threadIdx.x & 7];
-    for (int k = 1; k < kColThreads / 32; ++k) t += part[k][threadIdx.x & 7];
+#pragma unroll
+    for (int k = 1; k < kColThreads / 32; ++k)
+        if (k < (int)(blockDim.x >> 5)) t += part[k][threadIdx.x & 7];
     return t;
 }
 
@@ -211,8 +216,10 @@ __global__ void __launch_bounds__(kColThreads) bin_reduce_kernel(const double *_
             b += acc2[(size_t)q * cols + i];
         }
     }
-    a = column_total(a, part);
-    b = column_total(b, part);
+    if (__syncthreads_or(any)) {   // (uniform per CTA)
+        a = column_total(a, part);
+        b = column_total(b, part);
+    }
     if (i < cols && threadIdx.x < kColTile) {
         out[i] = a;
         out[(size_t)cols + i] = b;
@@ -398,6 +405,7 @@ __global__ void vjp_theta_kernel(const double *Sfs, const double *Ss, const doub
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 int round_up_int(int x, int a) { return (x + a - 1) / a * a; }
 unsigned col_ctas(size_t cols) { return (unsigned)((cols + kColTile - 1) / kColTile); }   // CTAs of the column sums
+unsigned col_threads(int chains) { return 32u * (unsigned)std::min(kColThreads / 32, (chains - 1) / 4 + 1); }   // of each
 
 struct WsLayout {
     size_t counters, F, R, S1, S2, chi2;
@@ -1237,7 +1245,7 @@ int moment_update(asm_problem *p, const WsLayout &L, int chains)
     const T *Fraw = (const T *)(ws + L.F);
     double *shift = (double *)(ws + L.shift);
     if (p->nsnap == 0) {   // centre every snapshot on the first one's mean (keeps FP32 GEMMs accurate)
-        shift_kernel<T><<<col_ctas(N), kColThreads, 0, p->stream>>>(Fraw, L.ldF, chains, N, shift);
+        shift_kernel<T><<<col_ctas(N), col_threads(chains), 0, p->stream>>>(Fraw, L.ldF, chains, N, shift);
         ++p->other_launches;
         if (p->P > 0) {
             kshift_kernel<<<(M * p->P + 127) / 128, 128, 0, p->stream>>>(p->d_Kth64, shift, M, N, p->P,
@@ -1266,7 +1274,7 @@ int moment_update(asm_problem *p, const WsLayout &L, int chains)
             return ASM_ERR_CUDA;
         p->other_launches += 2;
     }
-    moment_sums_kernel<T><<<dim3((unsigned)p->P + 1, col_ctas(N)), kColThreads, 0, p->stream>>>(
+    moment_sums_kernel<T><<<dim3((unsigned)p->P + 1, col_ctas(N)), col_threads(chains), 0, p->stream>>>(
         F, L.ldF, (const double *)(ws + L.Sq), chains, N, p->P, (double *)(ws + L.Sf), (double *)(ws + L.Sfs),
         (double *)(ws + L.Ss));
     ++p->other_launches;
@@ -2088,7 +2096,7 @@ int asm_average(asm_problem *p, double *mean_A, double *sem_A, double *ess, doub
     char *ws = (char *)p->ws;
     ++p->other_launches;
     const bool open32 = p->precision != ASM_FP64;   // FP32 state: sums of the open 64-sweep block
-    reduce_kernel<<<col_ctas(N), kColThreads, 0, p->stream>>>(
+    reduce_kernel<<<col_ctas(N), col_threads(p->chains), 0, p->stream>>>(
         (const double *)(ws + L.S1), (const double *)(ws + L.S2), open32 ? (const float *)(ws + L.P1) : nullptr,
         open32 ? (const float *)(ws + L.P2) : nullptr, L.ldF, p->chains, N, (double)p->kept, d, d + N, d + 2 * N);
     std::vector<double> h((size_t)3 * N);
@@ -2122,10 +2130,10 @@ int asm_mc_error(asm_problem *p, int k, double *ess, double *sem_fbar, double *s
     if (!d) return ASM_ERR_CUDA;
     const char *ws = (const char *)u->ws;
     const bool open32 = u->precision != ASM_FP64;
-    reduce_kernel<<<col_ctas(N), kColThreads, 0, p->stream>>>(
+    reduce_kernel<<<col_ctas(N), col_threads(chains), 0, p->stream>>>(
         (const double *)(ws + L.S1), (const double *)(ws + L.S2), open32 ? (const float *)(ws + L.P1) : nullptr,
         open32 ? (const float *)(ws + L.P2) : nullptr, L.ldF, chains, N, (double)u->kept, d, d + N, d + 2 * N);
-    bin_reduce_kernel<<<col_ctas(nk), kColThreads, 0, p->stream>>>(
+    bin_reduce_kernel<<<col_ctas(nk), col_threads(chains), 0, p->stream>>>(
         (const double *)(ws + L.bacc1), (const double *)(ws + L.bacc2), (const int *)(ws + L.bcount), chains, N,
         d + 3 * N);
     p->other_launches += 2;
@@ -2310,7 +2318,7 @@ int asm_sample_noalloc(asm_problem *p, int chains, long burn_in, long sweeps, ui
     const WsLayout L = ws_layout(p, chains, precision);
     const char *ws = (const char *)p->ws;
     const bool open32 = precision != ASM_FP64;
-    reduce_kernel<<<col_ctas(p->N), kColThreads, 0, p->stream>>>(
+    reduce_kernel<<<col_ctas(p->N), col_threads(chains), 0, p->stream>>>(
         (const double *)(ws + L.S1), (const double *)(ws + L.S2), open32 ? (const float *)(ws + L.P1) : nullptr,
         open32 ? (const float *)(ws + L.P2) : nullptr, L.ldF, chains, p->N, (double)sweeps, d_mean_fbar, d_sem2_fbar,
         d_m2_fbar);
