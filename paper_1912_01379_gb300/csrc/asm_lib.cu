@@ -2221,16 +2221,19 @@ int asm_chain_state(asm_problem *p, double *f, double *chi2)
     if (!p) return ASM_ERR_ARG;
     if (!p->kids.empty()) return ASM_ERR_ARG;
     if (!p->have_run) return ASM_ERR_STATE;
+    {
+        Counters c{};
+        if (const int rc = read_counters(p, &c); rc != ASM_OK) return rc;
+        if (c.timeouts) return ASM_ERR_TIMEOUT;
+    }
     const WsLayout L = ws_layout(p, p->chains, p->precision);
     const size_t es = p->precision == ASM_FP64 ? 8 : 4;
     const char *ws = (const char *)p->ws;
     std::vector<unsigned char> hF((size_t)p->chains * L.ldF * es), hR((size_t)p->chains * L.ldR * es);
     if (cudaMemcpyAsync(hF.data(), ws + L.F, hF.size(), cudaMemcpyDeviceToHost, p->stream) != cudaSuccess ||
-        cudaMemcpyAsync(hR.data(), ws + L.R, hR.size(), cudaMemcpyDeviceToHost, p->stream) != cudaSuccess)
+        cudaMemcpyAsync(hR.data(), ws + L.R, hR.size(), cudaMemcpyDeviceToHost, p->stream) != cudaSuccess ||
+        cudaStreamSynchronize(p->stream) != cudaSuccess)
         return ASM_ERR_CUDA;
-    Counters c{};
-    if (const int rc = read_counters(p, &c); rc != ASM_OK) return rc;   // synchronises
-    if (c.timeouts) return ASM_ERR_TIMEOUT;
     for (int q = 0; q < p->chains; ++q) {
         if (f)
             for (int n = 0; n < p->N; ++n) {
